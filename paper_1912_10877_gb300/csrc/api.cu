@@ -54,8 +54,8 @@ int ensure_ws(qs_state* s, Workspace& w, size_t bytes) {
 
 int expect_raw(const void* data, int dtype, int n, int nreg, const qs_observable* o, qs_state* ws_owner,
                double* host_out);
-int measure_one(void* data, int dtype, int n, const double* host_u, int nshots, int64_t* host_out,
-                int collapse, qs_state* owner, const uint64_t* seed, uint64_t k0);
+int measure_regs(void* data, int dtype, int n, int nreg, const double* host_u, int nshots, int64_t* host_out,
+                 int collapse, qs_state* owner, const uint64_t* seed, uint64_t k0);
 int reset_basis(qs_state* s, const uint64_t* host_basis);
 int backward(qs_state* s, const qs_circuit* c, const double* params, const qs_observable* o, int ckpt_every,
              const void* ckpts, void* work, double* host_grad, double* host_loss);
@@ -496,28 +496,33 @@ int qs_backward_tiled(qs_state* s, const qs_circuit* c, const double* params, co
   return fused_backward(s, c, params, o, work, grad, loss, tile_qubits);
 }
 
+// registers of one size together, those of an uneven batch one by one
+static int measure_all(qs_state* s, const double* u, int nshots, int64_t* out, int collapse, const uint64_t* seed) {
+  if (s->uniform)
+    return measure_regs(s->data, s->dtype, s->nq[0], s->nreg, u, nshots, out, collapse, s, seed, 0);
+  const size_t ab = amp_bytes(s->dtype);
+  for (int r = 0; r < s->nreg; ++r) {
+    const size_t k0 = (size_t)r * nshots;
+    QS_TRY(measure_regs((char*)s->data + ab * s->off[r], s->dtype, s->nq[r], 1, u ? u + k0 : nullptr, nshots, out + k0,
+                        collapse, s, seed, k0));
+  }
+  return QS_OK;
+}
+
 int qs_measure(qs_state* s, const double* u, int nshots, int64_t* out, int collapse) {
   if (!s || !u || !out) return fail(QS_EINVAL, "null argument");
   if (nshots < 1) return fail(QS_EINVAL, "nshots must be >= 1");
   if (collapse && nshots != 1) return fail(QS_EINVAL, "collapse needs nshots == 1");
   for (int i = 0; i < nshots * s->nreg; ++i)
     if (!(u[i] >= 0.0 && u[i] < 1.0)) return fail(QS_EINVAL, "uniform %d not in [0, 1)", i);
-  const size_t ab = amp_bytes(s->dtype);
-  for (int r = 0; r < s->nreg; ++r)
-    QS_TRY(measure_one((char*)s->data + ab * s->off[r], s->dtype, s->nq[r], u + (size_t)r * nshots, nshots,
-                       out + (size_t)r * nshots, collapse, s, nullptr, 0));
-  return QS_OK;
+  return measure_all(s, u, nshots, out, collapse, nullptr);
 }
 
 int qs_measure_seeded(qs_state* s, uint64_t seed, int nshots, int64_t* out, int collapse) {
   if (!s || !out) return fail(QS_EINVAL, "null argument");
   if (nshots < 1) return fail(QS_EINVAL, "nshots must be >= 1");
   if (collapse && nshots != 1) return fail(QS_EINVAL, "collapse needs nshots == 1");
-  const size_t ab = amp_bytes(s->dtype);
-  for (int r = 0; r < s->nreg; ++r)
-    QS_TRY(measure_one((char*)s->data + ab * s->off[r], s->dtype, s->nq[r], nullptr, nshots,
-                       out + (size_t)r * nshots, collapse, s, &seed, (uint64_t)r * (uint64_t)nshots));
-  return QS_OK;
+  return measure_all(s, nullptr, nshots, out, collapse, &seed);
 }
 
 }  // extern "C"

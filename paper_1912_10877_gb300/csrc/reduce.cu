@@ -306,63 +306,240 @@ int apply_observable_c128(const double2* psi, double2* lam, int n, const qs_obse
 
 constexpr int kF = 1024;
 
-template <typename T>
-__device__ __forceinline__ double prob(const T* p, uint64_t i) {
-  const double2 a = ld_amp(p, i);
-  return __dadd_rn(__dmul_rn(a.x, a.x), __dmul_rn(a.y, a.y));
+// A float as a double without the conversion instruction, which runs on the FP64
+// unit, this part's scarcest (1/64 of the FP32 rate): the exponent is rebased and
+// the mantissa moved by integer instructions, a subnormal scaled to a normal one
+// first.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t sign = __float_as_uint(x) & 0x80000000u;
+  const bool tiny = (__float_as_uint(x) & 0x7fffffffu) < 0x00800000u;
+  const uint32_t m = __float_as_uint(tiny ? __fmul_rn(x, 16777216.f) : x) & 0x7fffffffu;
+  const uint32_t bias = tiny ? 0x38000000u - (24u << 20) : m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+  const uint32_t hi = m ? (m >> 3) + bias : 0u;
+  return __hiloint2double((int)(hi | sign), (int)(m << 29));
+}
+
+// What a fold adds up: |amplitude|^2 by the contract, or a level's sums.  The
+// square of a float is exact in FP64, so one fused multiply-add rounds re*re +
+// im*im once, as the contract's multiply, multiply and add do: 2 FP64
+// operations instead of 5 with the conversions.
+__device__ __forceinline__ double prob(float2 v) {
+  const double x = widen(v.x), y = widen(v.y);
+  return __fma_rn(x, x, __dmul_rn(y, y));
+}
+__device__ __forceinline__ double prob(double2 v) { return __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)); }
+__device__ __forceinline__ double prob(double v) { return v; }
+
+// Left folds of equal blocks.  A block's fold is one chain of dependent FP64
+// adds, so a CTA gives each of up to 32 blocks a lane of one warp and lets all
+// its warps load the values (coalesced, the next chunk while the present one
+// is folded), form the probabilities and put them in shared memory.
+//   bound: the FP64 rate (3 operations an amplitude) when the blocks fill the
+//   GPU, the chain's latency (1024 adds of 87 clocks) when they do not; the
+//   fold warp differs between the CTAs of an SM so that each of its FP64 units
+//   gets its share.  Measured, n = 25 complex64: 210 us (a thread a block reading
+//   the state directly: 449 us; with conversion instructions here: 346 us).  One
+//   block, n = 10: 58 us (198 us).
+// `start`: the value a block's fold begins with; RUN: also every running sum.
+constexpr int kFoldCta = 128;
+constexpr int kFoldElems = 1024;  // values of a chunk over all blocks of the CTA
+
+// the exclusive prefix of block b of a register that has `per` of them: inner[b - 1],
+// or outer[g - 1] for the first block of group g of 1024 (mask: the bits of a block's
+// place in its group), 0 for the register's first
+struct FoldStart {
+  const double* inner;
+  const double* outer;
+  uint64_t per, mask, outer_per;
+};
+__device__ __forceinline__ double start_of(const FoldStart& s, uint64_t b) {
+  const uint64_t r = b / s.per, k = b - r * s.per;
+  if (s.inner && (k & s.mask)) return s.inner[b - 1];
+  if (!s.outer || k < kF) return 0.0;
+  return s.outer[r * s.outer_per + k / kF - 1];
 }
 
 template <typename T>
-__global__ void k_level0(const T* __restrict__ psi, uint64_t dim, uint64_t nb0, double* __restrict__ s0) {
-  const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= nb0) return;
-  const uint64_t lo = b * kF, hi = lo + kF < dim ? lo + kF : dim;
-  double a = prob(psi, lo);
-  for (uint64_t i = lo + 1; i < hi; ++i) a = __dadd_rn(a, prob(psi, i));
-  s0[b] = a;
-}
+struct FoldChunk {
+  T v[kFoldElems / kFoldCta];
+};
 
-__global__ void k_level1(const double* __restrict__ s0, uint64_t nb0, uint64_t nb1, double* __restrict__ s1) {
-  const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= nb1) return;
-  const uint64_t lo = c * kF, hi = lo + kF < nb0 ? lo + kF : nb0;
-  double a = s0[lo];
-  for (uint64_t b = lo + 1; b < hi; ++b) a = __dadd_rn(a, s0[b]);
-  s1[c] = a;
-}
-
-// the walk of the contract: first j whose running sum exceeds t, else the last
-// positive value, else the last; acc carries the exclusive prefix
-template <typename F>
-__device__ uint64_t walk(F value, uint64_t len, double t, double& acc) {
-  double a = acc, a_last = acc;
-  int64_t last = -1;
-  for (uint64_t j = 0; j < len; ++j) {
-    const double v = value(j);
-    const double nxt = __dadd_rn(a, v);
-    if (nxt > t) { acc = a; return j; }
-    if (v > 0.0) { last = (int64_t)j; a_last = a; }
-    a = nxt;
+// values j0 .. j0 + 2^chl - 1 of blocks first[g] (in units of len values), thread by thread
+template <typename T, typename First>
+__device__ __forceinline__ void fold_load(FoldChunk<T>& c, const T* __restrict__ src, First first, int elems, int chl,
+                                          uint64_t len, uint64_t j0) {
+#pragma unroll
+  for (int k = 0; k < kFoldElems / kFoldCta; ++k) {
+    const int e = threadIdx.x + k * kFoldCta;
+    if (e < elems) c.v[k] = src[first(e >> chl) * len + j0 + (uint64_t)(e & ((1 << chl) - 1))];
   }
-  if (last >= 0) { acc = a_last; return (uint64_t)last; }
+}
+template <typename T>
+__device__ __forceinline__ void fold_put(double* buf, const FoldChunk<T>& c, int elems, int chl) {
+#pragma unroll
+  for (int k = 0; k < kFoldElems / kFoldCta; ++k) {
+    const int e = threadIdx.x + k * kFoldCta;
+    if (e < elems) buf[(e >> chl) * ((1 << chl) + 1) + (e & ((1 << chl) - 1))] = prob(c.v[k]);
+  }
+}
+
+// B: values read ahead of the adds (a divisor of the chunk)
+template <typename T, bool RUN, int B>
+__global__ void __launch_bounds__(kFoldCta)
+k_fold(const T* __restrict__ src, uint64_t nblocks, uint64_t len, int gl, int chl, const FoldStart st,
+       double* __restrict__ sums, double* __restrict__ run) {
+  __shared__ double buf[2][kFoldElems + 32];
+  const uint64_t b0 = (uint64_t)blockIdx.x << gl;
+  const int G = (int)(nblocks - b0 < (1ull << gl) ? nblocks - b0 : (1ull << gl)), elems = G << chl;
+  const int pitch = (1 << chl) + 1, lane = threadIdx.x & 31;
+  const bool folds = (int)(threadIdx.x >> 5) == (int)(blockIdx.x % (kFoldCta / 32)) && lane < G;
+  auto first = [&](int g) { return b0 + (uint64_t)g; };
+  double a = folds ? start_of(st, b0 + lane) : 0.0;
+  FoldChunk<T> c;
+  fold_load(c, src, first, elems, chl, len, 0);
+  fold_put(buf[0], c, elems, chl);
+  __syncthreads();
+  const uint64_t nch = len >> chl;
+  // running sums replace their values in the chunk's buffer; a thread stores
+  // the slots of the chunk before the last that it then refills itself
+  auto flush = [&](const double* b, uint64_t ch) {
+#pragma unroll
+    for (int k = 0; k < kFoldElems / kFoldCta; ++k) {
+      const int e = threadIdx.x + k * kFoldCta, g = e >> chl, j = e & ((1 << chl) - 1);
+      if (e < elems) run[(b0 + g) * len + (ch << chl) + j] = b[g * pitch + j];
+    }
+  };
+  for (uint64_t ch = 0; ch < nch; ++ch) {
+    double* cur = buf[ch & 1];
+    double* nxt = buf[(ch + 1) & 1];
+    if (ch + 1 < nch) fold_load(c, src, first, elems, chl, len, (ch + 1) << chl);
+    if (folds) {
+      double* row = cur + lane * pitch;
+      for (int j = 0; j < (1 << chl); j += B) {
+        double v[B];
+#pragma unroll
+        for (int k = 0; k < B; ++k) v[k] = row[j + k];
+#pragma unroll
+        for (int k = 0; k < B; ++k) v[k] = a = __dadd_rn(a, v[k]);
+        if (RUN) {
+#pragma unroll
+          for (int k = 0; k < B; ++k) row[j + k] = v[k];
+        }
+      }
+    }
+    if (RUN && ch > 0) flush(nxt, ch - 1);
+    if (ch + 1 < nch) fold_put(nxt, c, elems, chl);
+    __syncthreads();
+  }
+  if (RUN) flush(buf[(nch - 1) & 1], nch - 1);
+  if (sums && folds) sums[b0 + lane] = a;
+}
+
+// Where the running sums of the three levels lie.  r2 is over the level-1 sums
+// (NULL: one level-1 block, whose prefix is 0), r1 over the level-0 sums (NULL:
+// one level-0 block), r0 over the probabilities (NULL: folded per shot).
+struct SampleArgs {
+  const double *s1, *s0, *r2, *r1, *r0, *u;
+  int64_t* out;
+  uint64_t dim, nb0, nb1;
+  int nshots;
+  uint64_t total;  // shots of all registers
+};
+
+// The walk of the contract: the first value whose running sum exceeds t, else the
+// last positive one, else the last.  The running sums of non-negative values do
+// not decrease, so the first is found by bisection (a sum that is not finite
+// makes the total and t so as well, and no sum exceeds that).
+template <typename V>
+__device__ __forceinline__ uint64_t walk(const double* __restrict__ run, uint64_t len, double t, V value) {
+  uint64_t lo = 0, hi = len;
+  while (lo < hi) {
+    const uint64_t mid = (lo + hi) >> 1;
+    if (run[mid] > t) hi = mid;
+    else lo = mid + 1;
+  }
+  if (lo < len) return lo;
+  for (uint64_t j = len; j-- > 0;)
+    if (value(j) > 0.0) return j;
   return len - 1;
 }
 
+// level-0 block of shot s (of its register r) and the target t
+__device__ __forceinline__ uint64_t shot_block(const SampleArgs& a, uint64_t r, double t) {
+  uint64_t c = 0;
+  if (a.r2) c = walk(a.r2 + r * a.nb1, a.nb1, t, [&](uint64_t j) { return a.s1[r * a.nb1 + j]; });
+  if (!a.r1) return 0;
+  const uint64_t k0 = c * kF, k1 = k0 + kF < a.nb0 ? k0 + kF : a.nb0;
+  return k0 + walk(a.r1 + r * a.nb0 + k0, k1 - k0, t, [&](uint64_t j) { return a.s0[r * a.nb0 + k0 + j]; });
+}
+__device__ __forceinline__ double shot_target(const SampleArgs& a, uint64_t s, uint64_t r) {
+  const double total = a.r2   ? a.r2[(r + 1) * a.nb1 - 1]
+                       : a.r1 ? a.r1[(r + 1) * a.nb0 - 1]
+                              : a.r0[(r + 1) * a.dim - 1];
+  return __dmul_rn(a.u[s], total);
+}
+
+// every running sum at hand: three bisections a shot (240 registers x 1024 shots at
+// n = 10: 9.5 us; a serial walk a shot, one launch a register, took 366 us each)
 template <typename T>
-__global__ void k_sample(const T* __restrict__ psi, uint64_t dim, const double* __restrict__ s0, uint64_t nb0,
-                         const double* __restrict__ s1, uint64_t nb1, const double* __restrict__ u, int nshots,
-                         int64_t* __restrict__ out) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nshots) return;
-  double total = s1[0];
-  for (uint64_t c = 1; c < nb1; ++c) total = __dadd_rn(total, s1[c]);
-  const double t = __dmul_rn(u[s], total);
-  double acc = 0.0;
-  const uint64_t c = walk([&](uint64_t j) { return s1[j]; }, nb1, t, acc);
-  const uint64_t b0 = c * kF, b1 = b0 + kF < nb0 ? b0 + kF : nb0;
-  const uint64_t b = b0 + walk([&](uint64_t j) { return s0[b0 + j]; }, b1 - b0, t, acc);
-  const uint64_t i0 = b * kF, i1 = i0 + kF < dim ? i0 + kF : dim;
-  out[s] = (int64_t)(i0 + walk([&](uint64_t j) { return prob(psi, i0 + j); }, i1 - i0, t, acc));
+__global__ void __launch_bounds__(128) k_sample(const T* __restrict__ psi, const SampleArgs a) {
+  const uint64_t s = (uint64_t)blockIdx.x * 128 + threadIdx.x;
+  if (s >= a.total) return;
+  const uint64_t r = s / a.nshots;
+  const double t = shot_target(a, s, r);
+  const uint64_t b = shot_block(a, r, t), i0 = b * kF, i1 = i0 + kF < a.dim ? i0 + kF : a.dim;
+  const T* p = psi + r * a.dim + i0;
+  a.out[s] = (int64_t)(i0 + walk(a.r0 + r * a.dim + i0, i1 - i0, t, [&](uint64_t j) { return prob(p[j]); }));
+}
+
+// fewer shots than blocks: a lane a shot folds its own block of probabilities
+// from the block's prefix (k_fold's layout, with the blocks that the shots fall into;
+// 4096 shots at n = 25: 112 us, 621 us as a serial walk of every level a thread)
+template <typename T>
+__global__ void __launch_bounds__(kFoldCta) k_sample_fold(const T* __restrict__ psi, const FoldStart st, const SampleArgs a) {
+  __shared__ double buf[2][kFoldElems + 32];
+  __shared__ uint64_t blk[32];
+  constexpr int CHL = 5;
+  const uint64_t s0 = (uint64_t)blockIdx.x * 32;
+  const int G = (int)(a.total - s0 < 32 ? a.total - s0 : 32), elems = G << CHL;
+  const int lane = threadIdx.x & 31;
+  const bool folds = (int)(threadIdx.x >> 5) == (int)(blockIdx.x % (kFoldCta / 32)) && lane < G;
+  uint64_t r = 0, b = 0;
+  double t = 0.0, acc = 0.0;
+  if (folds) {
+    r = (s0 + lane) / a.nshots;
+    t = shot_target(a, s0 + lane, r);
+    b = shot_block(a, r, t);
+    blk[lane] = r * a.nb0 + b;
+    acc = start_of(st, r * a.nb0 + b);
+  }
+  __syncthreads();
+  auto first = [&](int g) { return blk[g]; };
+  FoldChunk<T> c;
+  fold_load(c, psi, first, elems, CHL, kF, 0);
+  fold_put(buf[0], c, elems, CHL);
+  __syncthreads();
+  int found = -1, last = -1;
+  for (int ch = 0; ch < kF / 32; ++ch) {
+    if (ch + 1 < kF / 32) fold_load(c, psi, first, elems, CHL, kF, (uint64_t)(ch + 1) << CHL);
+    if (folds) {
+      const double* row = buf[ch & 1] + lane * 33;
+#pragma unroll 8
+      for (int j = 0; j < 32; ++j) {
+        const double v = row[j];
+        acc = __dadd_rn(acc, v);
+        // signs of the comparisons by the bit patterns (none is negative), off the FP64 unit;
+        // a t that is not finite is never exceeded
+        if (found < 0 && __double_as_longlong(acc) > __double_as_longlong(t) && !(__double2hiint(t) >= 0x7ff00000))
+          found = ch * 32 + j;
+        const long long vb = __double_as_longlong(v);
+        if (vb > 0 && vb <= 0x7ff0000000000000ll) last = ch * 32 + j;
+      }
+    }
+    if (ch + 1 < kF / 32) fold_put(buf[(ch + 1) & 1], c, elems, CHL);
+    __syncthreads();
+  }
+  if (folds) a.out[s0 + lane] = (int64_t)(b * kF + (found >= 0 ? found : last >= 0 ? last : kF - 1));
 }
 
 template <typename T>
@@ -382,31 +559,107 @@ __global__ void k_collapse_write(T* psi, uint64_t dim, int64_t x, const double2*
   st_amp(psi, i, i == (uint64_t)x ? *keep : make_double2(0.0, 0.0));
 }
 
-// one register at `data` with 2^n amplitudes
-// samples of one register with device uniforms into device indices; scratch:
-// sample_scratch_doubles(n) doubles (block sums of the three-level walk)
-size_t sample_scratch_doubles(int n) {
-  const uint64_t dim = 1ull << n;
-  const uint64_t nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF;
-  return (size_t)(nb0 + nb1);
+// samples of nreg registers of 2^n amplitudes (back to back) with device uniforms
+// [nreg][nshots] into device indices; scratch: sample_scratch_doubles() doubles
+constexpr uint64_t kRunDoubles = 1ull << 25;  // running sums of the probabilities in scratch: at most 256 MiB
+
+// The running sums of every probability cost a second pass over the state and
+// 8 bytes an amplitude, a shot without them folds 1024 probabilities: they are
+// formed once a level-0 block gets a shot or more on the average, or when a
+// register is a single block (whose fold is the running sum).
+static bool keep_runs(int n, int nshots) {
+  const uint64_t dim = 1ull << n, nb0 = (dim + kF - 1) / kF;
+  return nb0 == 1 || (nb0 <= (uint64_t)nshots && dim <= kRunDoubles);
+}
+// registers sampled together
+static int sample_group(int n, int nreg) {
+  return (int)std::min<uint64_t>((uint64_t)nreg, std::max<uint64_t>(1, kRunDoubles >> n));
 }
 
-int sample_dev(const void* data, int dtype, int n, const double* dev_u, int nshots, int64_t* dev_out,
+size_t sample_scratch_doubles(int n, int nreg, int nshots) {
+  const uint64_t dim = 1ull << n, nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF;
+  const uint64_t levels = (nb0 > 1 ? 2 * nb0 : 0) + (nb1 > 1 ? 2 * nb1 : 0);
+  return (size_t)((levels + (keep_runs(n, nshots) ? dim : 0)) * (uint64_t)sample_group(n, nreg));
+}
+
+template <typename T, bool RUN>
+static int launch_fold(const T* src, uint64_t nblocks, uint64_t len, const FoldStart& st, double* sums, double* run,
+                       cudaStream_t stream) {
+  // as many blocks a CTA (up to a warp of chains) as leave two CTAs an SM
+  int gl = 0;
+  while (gl < 5 && (nblocks >> (gl + 1)) >= 304) ++gl;
+  int chl = 10 - gl;
+  while ((1ull << chl) > len) --chl;
+  const uint64_t grid = (nblocks + (1ull << gl) - 1) >> gl;
+  if (grid > 0x7fffffffull) return fail(QS_EUNSUPPORTED, "register too large to sample");
+  if (chl >= 3) k_fold<T, RUN, 8><<<(unsigned)grid, kFoldCta, 0, stream>>>(src, nblocks, len, gl, chl, st, sums, run);
+  else k_fold<T, RUN, 1><<<(unsigned)grid, kFoldCta, 0, stream>>>(src, nblocks, len, gl, chl, st, sums, run);
+  QS_LAUNCHED();
+  return QS_OK;
+}
+
+template <typename T>
+static int sample_regs(const T* psi, int n, int nreg, const double* dev_u, int nshots, int64_t* dev_out, double* scratch,
+                       cudaStream_t st) {
+  const uint64_t dim = 1ull << n, R = (uint64_t)nreg;
+  const uint64_t nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF, len0 = std::min<uint64_t>(dim, kF);
+  const bool runs = keep_runs(n, nshots);
+  SampleArgs a;
+  memset(&a, 0, sizeof(a));
+  a.u = dev_u;
+  a.out = dev_out;
+  a.dim = dim;
+  a.nb0 = nb0;
+  a.nb1 = nb1;
+  a.nshots = nshots;
+  a.total = R * (uint64_t)nshots;
+  FoldStart zero;
+  memset(&zero, 0, sizeof(zero));
+  zero.per = 1;
+  FoldStart st0 = zero;  // prefixes of the level-0 blocks
+  if (nb0 > 1) {
+    double* s0 = scratch;
+    double* r1 = s0 + R * nb0;
+    scratch = r1 + R * nb0;
+    QS_TRY((launch_fold<T, false>(psi, R * nb0, len0, zero, s0, nullptr, st)));
+    FoldStart st1 = zero;  // prefixes of the level-1 blocks
+    if (nb1 > 1) {
+      double* s1 = scratch;
+      double* r2 = s1 + R * nb1;
+      scratch = r2 + R * nb1;
+      QS_TRY((launch_fold<double, false>(s0, R * nb1, kF, zero, s1, nullptr, st)));
+      QS_TRY((launch_fold<double, true>(s1, R, nb1, zero, nullptr, r2, st)));
+      a.s1 = s1;
+      a.r2 = r2;
+      st1 = FoldStart{r2, nullptr, nb1, ~0ull, 0};
+    }
+    QS_TRY((launch_fold<double, true>(s0, R * nb1, std::min<uint64_t>(nb0, kF), st1, nullptr, r1, st)));
+    a.s0 = s0;
+    a.r1 = r1;
+    st0 = FoldStart{r1, a.r2, nb0, kF - 1, nb1};
+  }
+  if (runs) {
+    QS_TRY((launch_fold<T, true>(psi, R * nb0, len0, st0, nullptr, scratch, st)));
+    a.r0 = scratch;
+    k_sample<T><<<(unsigned)((a.total + 127) / 128), 128, 0, st>>>(psi, a);
+  } else {
+    k_sample_fold<T><<<(unsigned)((a.total + 31) / 32), kFoldCta, 0, st>>>(psi, st0, a);
+  }
+  QS_LAUNCHED();
+  return QS_OK;
+}
+
+int sample_dev(const void* data, int dtype, int n, int nreg, const double* dev_u, int nshots, int64_t* dev_out,
                double* scratch, cudaStream_t st) {
-  const uint64_t dim = 1ull << n;
-  const uint64_t nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF;
-  double* s0 = scratch;
-  double* s1 = s0 + nb0;
-  if (dtype == QS_C64) k_level0<float2><<<(unsigned)((nb0 + 127) / 128), 128, 0, st>>>((const float2*)data, dim, nb0, s0);
-  else k_level0<double2><<<(unsigned)((nb0 + 127) / 128), 128, 0, st>>>((const double2*)data, dim, nb0, s0);
-  QS_LAUNCHED();
-  k_level1<<<(unsigned)((nb1 + 127) / 128), 128, 0, st>>>(s0, nb0, nb1, s1);
-  QS_LAUNCHED();
-  if (dtype == QS_C64)
-    k_sample<float2><<<(nshots + 127) / 128, 128, 0, st>>>((const float2*)data, dim, s0, nb0, s1, nb1, dev_u, nshots, dev_out);
-  else
-    k_sample<double2><<<(nshots + 127) / 128, 128, 0, st>>>((const double2*)data, dim, s0, nb0, s1, nb1, dev_u, nshots, dev_out);
-  QS_LAUNCHED();
+  const int group = sample_group(n, nreg);
+  for (int r = 0; r < nreg; r += group) {
+    const int k = std::min(group, nreg - r);
+    const char* p = (const char*)data + ((amp_bytes(dtype) * (size_t)r) << n);
+    const double* u = dev_u + (size_t)r * nshots;
+    int64_t* out = dev_out + (size_t)r * nshots;
+    if (dtype == QS_C64) QS_TRY(sample_regs((const float2*)p, n, k, u, nshots, out, scratch, st));
+    else QS_TRY(sample_regs((const double2*)p, n, k, u, nshots, out, scratch, st));
+  }
   return QS_OK;
 }
 
@@ -414,62 +667,51 @@ int sample_dev(const void* data, int dtype, int n, const double* dev_u, int nsho
 // (Steele, Lea and Flood 2014): state seed + k * 0x9E3779B97F4A7C15, then the
 // 64-bit finaliser (xor-shift 30, multiply, xor-shift 27, multiply, xor-shift
 // 31); u = top 53 bits / 2^53.  Shot j of this call is draw k0 + j + 1.
-__global__ void k_seeded_uniforms(uint64_t seed, uint64_t k0, int nshots, double* __restrict__ u) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_seeded_uniforms(uint64_t seed, uint64_t k0, uint64_t nshots, double* __restrict__ u) {
+  const uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= nshots) return;
-  uint64_t x = seed + (k0 + (uint64_t)j + 1ull) * 0x9E3779B97F4A7C15ull;
+  uint64_t x = seed + (k0 + j + 1ull) * 0x9E3779B97F4A7C15ull;
   x = (x ^ (x >> 30)) * 0xBF58476D1CE4E5B9ull;
   x = (x ^ (x >> 27)) * 0x94D049BB133111EBull;
   x ^= x >> 31;
   u[j] = (double)(x >> 11) * 0x1.0p-53;
 }
 
-int measure_one(void* data, int dtype, int n, const double* host_u, int nshots, int64_t* host_out,
-                int collapse, qs_state* owner, const uint64_t* seed, uint64_t k0) {
+// nreg registers of 2^n amplitudes back to back; the uniforms are host_u or drawn
+// from seed (shot j of register r: draw k0 + r nshots + j + 1)
+int measure_regs(void* data, int dtype, int n, int nreg, const double* host_u, int nshots, int64_t* host_out,
+                 int collapse, qs_state* owner, const uint64_t* seed, uint64_t k0) {
   cudaStream_t st = owner->stream;
   const uint64_t dim = 1ull << n;
-  const uint64_t nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF;
-  const size_t need = sizeof(double) * (nb0 + nb1) + sizeof(double) * nshots + sizeof(int64_t) * nshots + 64;
-  QS_TRY(ensure_ws(owner, owner->ws, need + 256));
-  char* w = (char*)owner->ws.ptr;
-  double* s0 = (double*)w;
-  double* s1 = s0 + nb0;
-  double* du = s1 + nb1;
-  int64_t* dout = (int64_t*)(du + nshots);
-  double2* keep = (double2*)(((uintptr_t)(dout + nshots) + 15) & ~(uintptr_t)15);
+  const size_t shots = (size_t)nreg * nshots, scr = sample_scratch_doubles(n, nreg, nshots);
+  QS_TRY(ensure_ws(owner, owner->ws, sizeof(double) * (scr + shots) + sizeof(int64_t) * shots + sizeof(double2) + 256));
+  double* dscr = (double*)owner->ws.ptr;
+  double* du = dscr + scr;
+  int64_t* dout = (int64_t*)(du + shots);
+  double2* keep = (double2*)(((uintptr_t)(dout + shots) + 15) & ~(uintptr_t)15);
   if (seed) {
-    k_seeded_uniforms<<<(nshots + 127) / 128, 128, 0, st>>>(*seed, k0, nshots, du);
+    k_seeded_uniforms<<<(unsigned)((shots + 127) / 128), 128, 0, st>>>(*seed, k0, shots, du);
     QS_LAUNCHED();
   } else {
-    QS_CUDA(cudaMemcpyAsync(du, host_u, sizeof(double) * nshots, cudaMemcpyHostToDevice, st));
+    QS_CUDA(cudaMemcpyAsync(du, host_u, sizeof(double) * shots, cudaMemcpyHostToDevice, st));
   }
-  if (dtype == QS_C64) {
-    k_level0<float2><<<(unsigned)((nb0 + 127) / 128), 128, 0, st>>>((const float2*)data, dim, nb0, s0);
-  } else {
-    k_level0<double2><<<(unsigned)((nb0 + 127) / 128), 128, 0, st>>>((const double2*)data, dim, nb0, s0);
-  }
-  QS_LAUNCHED();
-  k_level1<<<(unsigned)((nb1 + 127) / 128), 128, 0, st>>>(s0, nb0, nb1, s1);
-  QS_LAUNCHED();
-  if (dtype == QS_C64)
-    k_sample<float2><<<(nshots + 127) / 128, 128, 0, st>>>((const float2*)data, dim, s0, nb0, s1, nb1, du, nshots, dout);
-  else
-    k_sample<double2><<<(nshots + 127) / 128, 128, 0, st>>>((const double2*)data, dim, s0, nb0, s1, nb1, du, nshots, dout);
-  QS_LAUNCHED();
-  QS_CUDA(cudaMemcpyAsync(host_out, dout, sizeof(int64_t) * nshots, cudaMemcpyDeviceToHost, st));
+  QS_TRY(sample_dev(data, dtype, n, nreg, du, nshots, dout, dscr, st));
+  QS_CUDA(cudaMemcpyAsync(host_out, dout, sizeof(int64_t) * shots, cudaMemcpyDeviceToHost, st));
   QS_CUDA(cudaStreamSynchronize(st));
-  if (collapse) {
-    const int64_t x = host_out[0];
+  if (!collapse) return QS_OK;
+  for (int r = 0; r < nreg; ++r) {
+    const int64_t x = host_out[r];
+    char* reg = (char*)data + amp_bytes(dtype) * dim * r;
     if (dtype == QS_C64) {
-      k_collapse_scale<float2><<<1, 1, 0, st>>>((float2*)data, x, keep);
-      k_collapse_write<float2><<<(unsigned)((dim + 255) / 256), 256, 0, st>>>((float2*)data, dim, x, keep);
+      k_collapse_scale<float2><<<1, 1, 0, st>>>((float2*)reg, x, keep);
+      k_collapse_write<float2><<<(unsigned)((dim + 255) / 256), 256, 0, st>>>((float2*)reg, dim, x, keep);
     } else {
-      k_collapse_scale<double2><<<1, 1, 0, st>>>((double2*)data, x, keep);
-      k_collapse_write<double2><<<(unsigned)((dim + 255) / 256), 256, 0, st>>>((double2*)data, dim, x, keep);
+      k_collapse_scale<double2><<<1, 1, 0, st>>>((double2*)reg, x, keep);
+      k_collapse_write<double2><<<(unsigned)((dim + 255) / 256), 256, 0, st>>>((double2*)reg, dim, x, keep);
     }
     QS_LAUNCHED();
-    QS_CUDA(cudaStreamSynchronize(st));
   }
+  QS_CUDA(cudaStreamSynchronize(st));
   return QS_OK;
 }
 

@@ -1,0 +1,48 @@
+"""The sampler's routes against the oracle, index for index: registers below, at and
+above a level-0 block (1024 amplitudes) and a level-1 block (2^20), with fewer and
+more shots than level-0 blocks, one register and a batch."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def sparse_state(n, seed):
+    """A state with long runs of zeros (blocks without weight, at both ends too)."""
+    psi = W.haar_state(n, seed=seed)
+    keep = W.rng(seed + 1).random(1 << n) < 0.01
+    keep[: 1 << max(0, n - 2)] = False
+    keep[-(1 << max(0, n - 3)):] = False
+    keep[(1 << n) // 2] = True
+    psi[~keep] = 0
+    return psi
+
+
+@pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
+@pytest.mark.parametrize("n,nreg,nshots", [(1, 3, 5), (4, 1, 1), (9, 40, 33), (10, 5, 300), (11, 3, 1), (11, 3, 2),
+                                           (13, 7, 64), (14, 2, 15), (20, 1, 100), (20, 1, 2000), (21, 2, 50),
+                                           (21, 1, 5000)])
+def test_samples_equal_the_oracles(dt, n, nreg, nshots):
+    from paper_1912_10877_gb300 import qsim
+    u = W.shot_uniforms(nshots, seed=n, nreg=nreg)
+    u[:, 0] = 0.0
+    u[:, -1] = np.nextafter(1.0, 0.0)
+    for make in (W.haar_state, sparse_state):
+        psi = np.concatenate([make(n, seed=7 * n + r) for r in range(nreg)])
+        st = qsim.State([n] * nreg, dtype=dt).upload(psi)
+        amps = st.numpy().astype(np.complex128).reshape(nreg, -1)
+        got = st.measure(u)
+        for r in range(nreg):
+            assert np.array_equal(got[r], oracle.sample(amps[r], n, u[r])), (make.__name__, r)
+
+
+def test_register_without_weight():
+    from paper_1912_10877_gb300 import qsim
+    for n in (3, 12):
+        st = qsim.State(n, dtype=torch.complex64).upload(np.zeros(1 << n))
+        u = W.shot_uniforms(8, seed=1)
+        assert np.array_equal(st.measure(u)[0], oracle.sample(np.zeros(1 << n, np.complex128), n, u[0]))
