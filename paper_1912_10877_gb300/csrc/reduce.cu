@@ -4,107 +4,271 @@
 // expect (Sec. "Forward Mode"): O = sum_t c_t P_t with P_t a Pauli string.
 // For a basis state, P|i> = i^{nY} (-1)^{popc(i & z)} |i ^ x>, so
 // <psi|P|psi> = sum_i ph(i) conj(psi_{i^x}) psi_i.  Terms are grouped by their
-// x mask; one streaming pass per group reads each amplitude (or each pair
-// (i, i^x) once, counting it twice) and accumulates every term of the group in
-// FP64.  The sum is pairwise: a thread adds at most kSerialItems items in
-// order (the serial base case), warps and blocks combine by balanced trees,
-// and a second kernel folds the per-block partials of every term by a
-// balanced tree as well (fixed shapes, so results are reproducible run to
-// run).  Error bound: (kSerialItems + log2 of the item count) * 2^-53 of the
-// sum of the absolute terms.
+// x mask; each group reads each amplitude (or each pair (i, i^x) once, counting
+// it twice) and adds it weighted with the group's coefficients in FP64.  The sum
+// is pairwise: a thread adds at most 16 items in order (the serial base case),
+// threads, warps and blocks combine by balanced trees, and a second kernel folds
+// the per-block partials (64 at most in order) and the groups by balanced trees
+// as well (fixed shapes, so results are reproducible run to run).
 //
 // measure (Sec. "Instructions on Quantum Registers"): the deterministic
 // contract of qsim.h -- FP64 probabilities with separately rounded multiply
 // and add, left folds over level-0 blocks of 1024 probabilities and level-1
 // blocks of 1024 level-0 sums, and a three-level walk per shot.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <map>
+#include <vector>
 
 #include "common.cuh"
 
 namespace qs {
 
 constexpr int kRedThreads = 256;
-constexpr int kSerialItems = 64;  // serial base case of the pairwise expectation sums
-constexpr int kGroupTerms = 16;   // terms of one x-mask group handled per launch
 constexpr int kObsChunk = 64;     // terms per lambda = O psi launch
 
-struct TermGroup {
-  int nt;
-  int item_log2;
-  int h;                 // highest bit of x (-1 if x == 0)
-  uint64_t x;
-  uint64_t z[kGroupTerms];
-  int ny[kGroupTerms];   // number of Y factors mod 4
-};
-
-__device__ __forceinline__ double2 ld_amp(const float2* p, uint64_t i) {
-  const float2 v = p[i];
-  return make_double2((double)v.x, (double)v.y);
+// A float as a double without the conversion instruction, which runs on the FP64
+// unit, this part's scarcest (1/64 of the FP32 rate): the exponent is rebased and
+// the mantissa moved by integer instructions, a subnormal scaled to a normal one
+// first.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t sign = __float_as_uint(x) & 0x80000000u;
+  const bool tiny = (__float_as_uint(x) & 0x7fffffffu) < 0x00800000u;
+  const uint32_t m = __float_as_uint(tiny ? __fmul_rn(x, 16777216.f) : x) & 0x7fffffffu;
+  const uint32_t bias = tiny ? 0x38000000u - (24u << 20) : m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+  const uint32_t hi = m ? (m >> 3) + bias : 0u;
+  return __hiloint2double((int)(hi | sign), (int)(m << 29));
 }
-__device__ __forceinline__ double2 ld_amp(const double2* p, uint64_t i) { return p[i]; }
 
-__device__ __forceinline__ double term_value(int ny, double s, double zr, double zi) {
-  switch (ny & 3) {
-    case 0: return s * zr;
-    case 1: return -s * zi;
-    case 2: return -s * zr;
-    default: return s * zi;
+__device__ __forceinline__ double2 widen(float2 v) { return make_double2(widen(v.x), widen(v.y)); }
+__device__ __forceinline__ double2 widen(double2 v) { return v; }
+template <typename T>
+__device__ __forceinline__ double2 ld_amp(const T* p, uint64_t i) { return widen(p[i]); }
+
+// Expectation sums: a block of 256 threads covers kBlockAmps amplitudes (64 a
+// thread, or 32 pairs), the terms' coefficients inside the sum, and writes one
+// partial sum for each slot (a launch's unit).  FP64 products of this part run
+// at 1/64 of the FP32 rate, so both kernels are written for their FP64
+// operations: floats are widened by integer instructions, the signs of a term
+// are bit patterns of the index whose low bits a thread keeps for all its items
+// and whose high bits are worked out once a block.
+constexpr int kBlockAmps = 16384;
+constexpr int kZLo = 10;     // index bits a thread of k_expect_z keeps fixed
+constexpr int kZTerms = 64;  // terms of a k_expect_z launch
+constexpr int kZMixed = 32;  // of them, terms with qubits on both sides of bit kZLo
+
+__device__ __forceinline__ double flip(double c, uint32_t neg) {  // neg & 1: -c
+  return __hiloint2double(__double2hiint(c) ^ (int)(neg << 31), __double2loint(c));
+}
+
+__device__ __forceinline__ void block_partial(double acc, double* out) {
+  __shared__ double red[kRedThreads / 32];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    static_assert(kRedThreads / 32 == 8, "block tree below is written for 8 warps");
+    *out = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
   }
 }
 
-// grid (blocks_per_reg, nreg); partials[(reg * nt_total + term_base + t) * nblk + block]
+// Z strings: sum_i W(i) |psi_i|^2 with W(i) = sum_t c_t (-1)^popcount(i & z_t).
+// Terms on qubits below kZLo are a constant of the thread's item, terms above a
+// value of the chunk of 2^kZLo amplitudes; only those that span both are added
+// item by item.  4 FP64 operations an amplitude and one a mixed term, where a sum a
+// term took 2 and one for every term.  Bound by them: 24 strings Z_i Z_{i+1} at
+// n = 25 complex64 368 us (two launches of 610 us before).
+struct ZTerms {
+  int nlo, nhi, nmix;
+  uint64_t z[kZTerms];  // low terms, high ones, mixed ones
+  double c[kZTerms];
+};
+
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads)
-k_expect_group(const T* __restrict__ psi, uint64_t reg_stride, TermGroup g, double* __restrict__ partials,
-               int nt_total, int term_base) {
-  const int nblk = gridDim.x;
-  const uint64_t r = blockIdx.y;
-  const T* p = psi + r * reg_stride;
-  const uint64_t items = 1ull << g.item_log2;
-  double acc[kGroupTerms];
+k_expect_z(const T* __restrict__ psi, int n, const __grid_constant__ ZTerms g, double* __restrict__ partials,
+           int nslots, int slot) {
+  constexpr int CH = kBlockAmps >> kZLo;         // chunks of a block
+  constexpr int I = (1 << kZLo) / kRedThreads;   // items of a thread in a chunk
+  __shared__ double high[CH];
+  __shared__ uint32_t mixhi[CH];
+  const uint64_t dim = 1ull << n, nvb = (dim + kBlockAmps - 1) / kBlockAmps;
+  const T* p = psi + blockIdx.y * dim;
+  const int tid = threadIdx.x, nl = g.nlo + g.nhi, nt = nl + g.nmix;
+  double low[I], acc[I];
+  uint32_t mixlo[I];
 #pragma unroll
-  for (int t = 0; t < kGroupTerms; ++t) acc[t] = 0.0;
-  for (uint64_t j = (uint64_t)blockIdx.x * kRedThreads + threadIdx.x; j < items;
-       j += (uint64_t)nblk * kRedThreads) {
-    uint64_t i = j;
-    if (g.h >= 0) i = ((j >> g.h) << (g.h + 1)) | (j & ((1ull << g.h) - 1ull));
-    const double2 a = ld_amp(p, i);
-    double zr, zi;
-    if (g.h >= 0) {
-      const double2 b = ld_amp(p, i ^ g.x);
-      zr = b.x * a.x + b.y * a.y;
-      zi = b.x * a.y - b.y * a.x;
-    } else {
-      zr = a.x * a.x + a.y * a.y;
-      zi = 0.0;
+  for (int k = 0; k < I; ++k) {
+    const uint32_t lo = tid + k * kRedThreads;
+    low[k] = acc[k] = 0.0;
+    mixlo[k] = 0;
+    for (int t = 0; t < g.nlo; ++t) low[k] += flip(g.c[t], __popc(lo & (uint32_t)g.z[t]));
+    for (int t = nl; t < nt; ++t) mixlo[k] |= (__popc(lo & (uint32_t)g.z[t] & ((1u << kZLo) - 1)) & 1u) << (t - nl);
+  }
+  for (uint64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
+    __syncthreads();
+    if (tid < 2 * CH) {
+      const int ch = tid & (CH - 1);
+      const uint64_t hi = (vb * CH + ch) << kZLo;
+      if (tid < CH) {
+        double w = 0.0;
+        for (int t = g.nlo; t < nl; ++t) w += flip(g.c[t], __popcll(hi & g.z[t]));
+        high[ch] = w;
+      } else {
+        uint32_t m = 0;
+        for (int t = nl; t < nt; ++t) m |= (__popcll(hi & g.z[t]) & 1u) << (t - nl);
+        mixhi[ch] = m;
+      }
     }
+    __syncthreads();
+    const uint64_t i0 = vb * kBlockAmps + tid;
+    const int chunks = dim >= kBlockAmps ? CH : (int)((dim + (1 << kZLo) - 1) >> kZLo);
+#pragma unroll 2
+    for (int ch = 0; ch < chunks; ++ch) {
+      const double h = high[ch];
+      const uint32_t mh = mixhi[ch];
 #pragma unroll
-    for (int t = 0; t < kGroupTerms; ++t) {
-      if (t < g.nt) {
-        const double s = (__popcll(i & g.z[t]) & 1) ? -1.0 : 1.0;
-        acc[t] += term_value(g.ny[t], s, zr, zi);
+      for (int k = 0; k < I; ++k) {
+        const uint64_t i = i0 + ((uint64_t)ch << kZLo) + k * kRedThreads;
+        if (i >= dim) continue;
+        const double2 a = ld_amp(p, i);
+        double w = low[k] + h;
+        const uint32_t m = mixlo[k] ^ mh;
+        for (int t = 0; t < g.nmix; ++t) w += flip(g.c[nl + t], m >> t);
+        acc[k] = fma(w, fma(a.x, a.x, a.y * a.y), acc[k]);
       }
     }
   }
-  __shared__ double red[kRedThreads / 32][kGroupTerms];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int t = 0; t < kGroupTerms; ++t) {
-    double v = acc[t];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp][t] = v;
+  double v = 0.0;
+  static_assert(I == 4, "the thread's tree below is written for 4 items");
+  v = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+  block_partial(v, partials + ((size_t)blockIdx.y * nslots + slot) * gridDim.x + blockIdx.x);
+}
+
+// Strings with X or Y factors.  The terms of one x mask share their pairs (i, i ^ x),
+// i without x's highest bit h: with zr + i zi = conj(psi_{i^x}) psi_i a pair adds
+// 2 (Wr zr + Wi zi), where a term puts its +-c into Wr (an even number of Y factors)
+// or Wi (an odd one).  A unit is up to kXTerms terms of one mask: their signs index a
+// table of Wr and Wi, and a lone term without sign (an X string) needs 2 FP64
+// operations a pair.  The units of an observable run in one launch (blockIdx.z).
+// Bound by the FP64 operations: 25 strings X_i at n = 25 complex64 1.63 ms, 65 us
+// each (610 us each as launches that ran 16 predicated terms a pair).
+constexpr int kXTerms = 4;
+constexpr int kXUnits = 36;
+struct XUnit {
+  uint64_t x;
+  uint64_t z[kXTerms];  // over pair numbers: bit h taken out
+  double c[kXTerms];
+  int8_t ny[kXTerms];   // number of Y factors mod 4
+  int16_t h, nt;
+};
+struct XUnits {
+  XUnit u[kXUnits];
+};
+
+template <typename T> struct Pairs { double2 a0, b0, a1, b1; };  // pairs j and j + 1
+
+// vec: the registers start on 16-byte boundaries
+template <typename T>
+__device__ __forceinline__ Pairs<T> ld_pairs(const T* __restrict__ p, uint64_t j, int h, uint64_t x, bool vec) {
+  Pairs<T> r;
+  const uint64_t i = ((j >> h) << (h + 1)) | (j & ((1ull << h) - 1ull));
+  const uint64_t step = h ? 1 : 2;  // from pair j to j + 1
+  if constexpr (sizeof(T) == 8) {
+    if (vec) {
+      const float4 u = *reinterpret_cast<const float4*>(p + i);
+      const float4 v = *reinterpret_cast<const float4*>(p + (h ? ((i ^ x) & ~1ull) : i + 2));
+      const double2 u0 = widen(make_float2(u.x, u.y)), u1 = widen(make_float2(u.z, u.w));
+      const double2 v0 = widen(make_float2(v.x, v.y)), v1 = widen(make_float2(v.z, v.w));
+      if (h == 0) return {u0, u1, v0, v1};
+      return (x & 1) ? Pairs<T>{u0, v1, u1, v0} : Pairs<T>{u0, v0, u1, v1};
+    }
   }
-  __syncthreads();
-  if (threadIdx.x < g.nt) {
-    static_assert(kRedThreads / 32 == 8, "block tree below is written for 8 warps");
-    const int t = threadIdx.x;
-    const double v = ((red[0][t] + red[1][t]) + (red[2][t] + red[3][t])) +
-                     ((red[4][t] + red[5][t]) + (red[6][t] + red[7][t]));
-    const double f = g.h >= 0 ? 2.0 : 1.0;
-    partials[((r * nt_total) + term_base + threadIdx.x) * nblk + blockIdx.x] = f * v;
+  r.a0 = ld_amp(p, i);
+  r.b0 = ld_amp(p, i ^ x);
+  r.a1 = ld_amp(p, i + step);
+  r.b1 = ld_amp(p, (i + step) ^ x);
+  return r;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kRedThreads)
+k_expect_x(const T* __restrict__ psi, int n, const __grid_constant__ XUnits g, double* __restrict__ partials,
+           int nslots, int slot0, int vec) {
+  constexpr int STEPS = kBlockAmps / 2 / (2 * kRedThreads);
+  __shared__ double tabr[1 << kXTerms], tabi[1 << kXTerms];
+  __shared__ uint32_t pathi[STEPS];
+  const XUnit& U = g.u[blockIdx.z];
+  const int tid = threadIdx.x, h = U.h, nt = U.nt;
+  const uint64_t x = U.x, dim = 1ull << n, items = dim >> 1, nvb = (dim + kBlockAmps - 1) / kBlockAmps;
+  const T* p = psi + blockIdx.y * dim;
+  bool real = false, imag = false;
+  for (int t = 0; t < nt; ++t) ((U.ny[t] & 1) ? imag : real) = true;
+  const bool plain = nt == 1 && !imag && U.z[0] == 0;
+  if (tid < (1 << kXTerms)) {
+    double wr = 0.0, wi = 0.0;
+    for (int t = 0; t < nt; ++t) {
+      // i^ny z: zr, -zi, -zr, zi
+      const double c = flip(U.c[t], ((uint32_t)tid >> t) ^ (U.ny[t] == 1 || U.ny[t] == 2));
+      if (U.ny[t] & 1) wi += c;
+      else wr += c;
+    }
+    tabr[tid] = wr;
+    tabi[tid] = wi;
   }
+  uint32_t lo0 = 0, lo1 = 0;  // sign patterns of the thread's two pairs of a step
+  for (int t = 0; t < nt; ++t) {
+    lo0 |= (__popc((uint32_t)(2 * tid) & (uint32_t)U.z[t]) & 1u) << t;
+    lo1 |= (__popc((uint32_t)(2 * tid + 1) & (uint32_t)U.z[t]) & 1u) << t;
+  }
+  double acc0 = 0.0, acc1 = 0.0;
+  for (uint64_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
+    const uint64_t j0 = vb * (kBlockAmps / 2);
+    __syncthreads();
+    if (tid < STEPS) {
+      uint32_t m = 0;
+      for (int t = 0; t < nt; ++t) m |= (__popcll((j0 + (uint64_t)tid * 2 * kRedThreads) & U.z[t]) & 1u) << t;
+      pathi[tid] = m;
+    }
+    __syncthreads();
+    if (items == 1) {  // a one-qubit register: one pair
+      if (tid == 0) {
+        const double2 a = ld_amp(p, 0), b = ld_amp(p, 1);
+        acc0 = tabr[0] * (b.x * a.x + b.y * a.y) + tabi[0] * (b.x * a.y - b.y * a.x);
+      }
+      continue;
+    }
+    const int steps = items >= kBlockAmps / 2 ? STEPS : (int)((items + 2 * kRedThreads - 1) / (2 * kRedThreads));
+    auto load = [&](int s) { return ld_pairs(p, j0 + (uint64_t)(s * 2 * kRedThreads + 2 * tid), h, x, vec != 0); };
+    auto on = [&](int s) { return j0 + (uint64_t)(s * 2 * kRedThreads + 2 * tid) < items; };
+    if (plain) {
+#pragma unroll 4
+      for (int s = 0; s < steps; ++s) {
+        if (!on(s)) continue;
+        const Pairs<T> q = load(s);
+        acc0 = fma(q.b0.x, q.a0.x, fma(q.b0.y, q.a0.y, acc0));
+        acc1 = fma(q.b1.x, q.a1.x, fma(q.b1.y, q.a1.y, acc1));
+      }
+    } else {
+#pragma unroll 4
+      for (int s = 0; s < steps; ++s) {
+        if (!on(s)) continue;
+        const Pairs<T> q = load(s);
+        const uint32_t m0 = lo0 ^ pathi[s], m1 = lo1 ^ pathi[s];
+        if (real) {
+          acc0 = fma(tabr[m0], fma(q.b0.x, q.a0.x, q.b0.y * q.a0.y), acc0);
+          acc1 = fma(tabr[m1], fma(q.b1.x, q.a1.x, q.b1.y * q.a1.y), acc1);
+        }
+        if (imag) {
+          acc0 = fma(tabi[m0], fma(q.b0.x, q.a0.y, -q.b0.y * q.a0.x), acc0);
+          acc1 = fma(tabi[m1], fma(q.b1.x, q.a1.y, -q.b1.y * q.a1.x), acc1);
+        }
+      }
+    }
+  }
+  const double c = plain && items > 1 ? 2.0 * U.c[0] : 2.0;
+  block_partial(c * (acc0 + acc1),
+                partials + ((size_t)blockIdx.y * nslots + slot0 + blockIdx.z) * gridDim.x + blockIdx.x);
 }
 
 // Pairwise sum in index order of the values add()ed one by one: a binary
@@ -133,46 +297,111 @@ struct PairwiseAcc {
   }
 };
 
-constexpr int kFoldThreads = 256;
+constexpr int kFoldThreads = 1024;
+constexpr int kFoldRow = 2048;  // partial sums a warp takes at a time
 
-// Pairwise sum of v[0..len) by one CTA of kFoldThreads threads: contiguous
-// chunks per thread (binary counter), then a shared-memory tree.  Every thread
-// receives the result.
-__device__ double block_pairwise(const double* __restrict__ v, int64_t len, double* sh) {
-  const int64_t chunk = (len + kFoldThreads - 1) / kFoldThreads;
-  const int64_t lo = (int64_t)threadIdx.x * chunk, hi = lo + chunk < len ? lo + chunk : len;
-  PairwiseAcc acc;
-  for (int64_t i = lo; i < hi; ++i) acc.add(v[i]);
-  sh[threadIdx.x] = acc.total();
-  __syncthreads();
-  for (int w = kFoldThreads / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] = sh[threadIdx.x] + sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  const double r = sh[0];
-  __syncthreads();
-  return r;
-}
-
-// one CTA per register: every term's block partials folded pairwise, then the
-// terms' c_t * v_t pairwise in term order.
+// one CTA per register, one warp per slot: the slot's block partials in rows of
+// kFoldRow (64 a lane in four chains, then a tree), the rows pairwise; then the
+// warps' slots (one CTA summing every term's partials in turn took 180 us for 49
+// terms at n = 25; this 21 us for their 26 slots)
 __global__ void __launch_bounds__(kFoldThreads)
-k_expect_final(const double* __restrict__ partials, int nblk, int nt_total, const double* __restrict__ coeff,
-               double* __restrict__ out) {
-  __shared__ double sh[kFoldThreads];
-  const int r = blockIdx.x;
-  PairwiseAcc terms;
-  for (int t = 0; t < nt_total; ++t) {
-    const double v = block_pairwise(partials + ((size_t)r * nt_total + t) * nblk, nblk, sh);
-    terms.add(coeff[t] * v);
+k_expect_final(const double* __restrict__ partials, int nblk, int nslots, double* __restrict__ out) {
+  __shared__ double sh[kFoldThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  PairwiseAcc slots;
+  for (int t = warp; t < nslots; t += kFoldThreads / 32) {
+    const double* row = partials + ((size_t)blockIdx.x * nslots + t) * nblk;
+    PairwiseAcc rows;
+    double v = 0.0;
+    for (int64_t r0 = 0; r0 < nblk; r0 += kFoldRow) {
+      double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+      for (int k = 0; k < kFoldRow / 32 / 4; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int64_t i = r0 + (k * 4 + q) * 32 + lane;
+          if (i < nblk) a[q] += row[i];
+        }
+      v = (a[0] + a[1]) + (a[2] + a[3]);
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (nblk > kFoldRow) rows.add(v);
+    }
+    slots.add(nblk > kFoldRow ? rows.total() : v);
   }
-  if (threadIdx.x == 0) out[r] = terms.total();
+  if (lane == 0) sh[warp] = slots.total();
+  __syncthreads();
+  if (warp == 0) {
+    double v = sh[lane];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) out[blockIdx.x] = v;
+  }
 }
 
-// blocks per register for the pairwise expectation: at most kSerialItems items per thread
-static int expect_blocks(uint64_t items) {
-  const uint64_t per_block = (uint64_t)kRedThreads * kSerialItems;
-  return (int)std::max<uint64_t>(1, (items + per_block - 1) / per_block);
+// blocks per register for the pairwise expectation
+static int expect_blocks(uint64_t dim) { return (int)std::max<uint64_t>(1, (dim + kBlockAmps - 1) / kBlockAmps); }
+
+// Slots (partial sums per block) of terms ordered by x mask, and their launches into
+// partials[nreg][slots][nblk]; partials == NULL: only the count
+static int expect_launch(const void* psi, int dtype, int n, int nreg, const qs_pauli_term* const* terms, int nt,
+                         double* partials, int nblk, int nslots, int* slots, cudaStream_t st) {
+  const dim3 grid((unsigned)nblk, (unsigned)nreg);
+  int slot = 0, t = 0;
+  // Z strings
+  while (t < nt && !terms[t]->x_mask) {
+    ZTerms g;
+    memset(&g, 0, sizeof(g));
+    const int t0 = t;
+    const uint64_t lo = (1ull << kZLo) - 1;
+    auto kind = [&](const qs_pauli_term* q) { return !(q->z_mask & ~lo) ? 0 : !(q->z_mask & lo) ? 1 : 2; };
+    while (t < nt && !terms[t]->x_mask && t - t0 < kZTerms && (kind(terms[t]) != 2 || g.nmix < kZMixed))
+      g.nmix += kind(terms[t++]) == 2;
+    int at = 0;
+    g.nmix = 0;
+    for (int k = 0; k < 3; ++k)
+      for (int q = t0; q < t; ++q) {
+        if (kind(terms[q]) != k) continue;
+        g.z[at] = terms[q]->z_mask;
+        g.c[at++] = terms[q]->coeff;
+        ++(k == 0 ? g.nlo : k == 1 ? g.nhi : g.nmix);
+      }
+    if (partials) {
+      if (dtype == QS_C64)
+        k_expect_z<float2><<<grid, kRedThreads, 0, st>>>((const float2*)psi, n, g, partials, nslots, slot);
+      else
+        k_expect_z<double2><<<grid, kRedThreads, 0, st>>>((const double2*)psi, n, g, partials, nslots, slot);
+      QS_LAUNCHED();
+    }
+    ++slot;
+  }
+  // the others
+  const int vec = ((uintptr_t)psi & 15) == 0;
+  while (t < nt) {
+    XUnits g;
+    memset(&g, 0, sizeof(g));
+    int nu = 0;
+    for (; t < nt && nu < kXUnits; ++nu) {
+      XUnit& u = g.u[nu];
+      u.x = terms[t]->x_mask;
+      u.h = (int16_t)(63 - __builtin_clzll(u.x));
+      for (; t < nt && terms[t]->x_mask == u.x && u.nt < kXTerms; ++t, ++u.nt) {
+        const uint64_t z = terms[t]->z_mask, low = (1ull << u.h) - 1;
+        u.z[u.nt] = (z & low) | ((z >> 1) & ~low);
+        u.c[u.nt] = terms[t]->coeff;
+        u.ny[u.nt] = (int8_t)(__builtin_popcountll(u.x & z) & 3);
+      }
+    }
+    if (partials) {
+      const dim3 gx(grid.x, grid.y, (unsigned)nu);
+      if (dtype == QS_C64)
+        k_expect_x<float2><<<gx, kRedThreads, 0, st>>>((const float2*)psi, n, g, partials, nslots, slot, vec);
+      else
+        k_expect_x<double2><<<gx, kRedThreads, 0, st>>>((const double2*)psi, n, g, partials, nslots, slot, vec);
+      QS_LAUNCHED();
+    }
+    slot += nu;
+  }
+  *slots = slot;
+  return QS_OK;
 }
 
 struct ObsChunk {
@@ -209,68 +438,30 @@ k_apply_obs(const double2* __restrict__ psi, double2* __restrict__ lam, uint64_t
 
 // ------------------------------------------------------------------ host side
 
-static int grouped(const qs_observable* o, std::vector<std::pair<uint64_t, std::vector<int>>>& groups) {
-  std::map<uint64_t, std::vector<int>> m;
-  for (int t = 0; t < (int)o->terms.size(); ++t) m[o->terms[t].x_mask].push_back(t);
-  groups.assign(m.begin(), m.end());
-  return QS_OK;
-}
-
 // expectation of registers stored at `data` (uniform: nreg x 2^n, else one register)
 int expect_raw(const void* data, int dtype, int n, int nreg, const qs_observable* o, qs_state* ws_owner,
                double* host_out) {
   cudaStream_t st = ws_owner->stream;
-  const int nt_total = (int)o->terms.size();
+  std::vector<const qs_pauli_term*> terms;
   for (const auto& t : o->terms) {
     if (n < 64 && ((t.x_mask | t.z_mask) >> n)) return fail(QS_EINVAL, "observable acts on a qubit >= n=%d", n);
+    terms.push_back(&t);
   }
-  std::vector<std::pair<uint64_t, std::vector<int>>> groups;
-  grouped(o, groups);
-  const uint64_t dim = 1ull << n;
-  // every group's items: 2^n (x = 0) or 2^(n-1) pairs; the grid covers the larger
-  const int nblk = expect_blocks(dim);
-  const size_t part_bytes = sizeof(double) * (size_t)nreg * std::max(1, nt_total) * nblk;
-  const size_t coeff_off = (part_bytes + 255) / 256 * 256;
-  const size_t out_off = coeff_off + (sizeof(double) * std::max(1, nt_total) + 255) / 256 * 256;
+  std::stable_sort(terms.begin(), terms.end(),
+                   [](const qs_pauli_term* a, const qs_pauli_term* b) { return a->x_mask < b->x_mask; });
+  const int nt = (int)terms.size(), nblk = expect_blocks(1ull << n), group = std::min(nreg, 65535);
+  int nslots = 0;
+  QS_TRY(expect_launch(data, dtype, n, nreg, terms.data(), nt, nullptr, nblk, 0, &nslots, st));
+  const size_t out_off = (sizeof(double) * (size_t)group * std::max(1, nslots) * nblk + 255) / 256 * 256;
   QS_TRY(ensure_ws(ws_owner, ws_owner->ws, out_off + sizeof(double) * nreg));
   double* partials = (double*)ws_owner->ws.ptr;
-  double* dcoeff = (double*)((char*)ws_owner->ws.ptr + coeff_off);
   double* dev_out = (double*)((char*)ws_owner->ws.ptr + out_off);
-  // coefficients in the global term order of the partials layout below
-  std::vector<double> coeff;
-  std::vector<int> order;
-  for (auto& g : groups)
-    for (int t : g.second) { order.push_back(t); coeff.push_back(o->terms[t].coeff); }
-  if (nt_total > 0)
-    QS_CUDA(cudaMemcpyAsync(dcoeff, coeff.data(), sizeof(double) * nt_total, cudaMemcpyHostToDevice, st));
-  int base = 0;
-  for (auto& g : groups) {
-    const auto& ids = g.second;
-    for (size_t c0 = 0; c0 < ids.size(); c0 += kGroupTerms) {
-      TermGroup tg;
-      memset(&tg, 0, sizeof(tg));
-      tg.x = g.first;
-      tg.h = g.first ? 63 - __builtin_clzll(g.first) : -1;
-      tg.item_log2 = g.first ? n - 1 : n;
-      tg.nt = (int)std::min<size_t>(kGroupTerms, ids.size() - c0);
-      for (int t = 0; t < tg.nt; ++t) {
-        const auto& term = o->terms[ids[c0 + t]];
-        tg.z[t] = term.z_mask;
-        tg.ny[t] = __builtin_popcountll(term.x_mask & term.z_mask) & 3;
-      }
-      dim3 grid(nblk, nreg);
-      if (dtype == QS_C64)
-        k_expect_group<float2><<<grid, kRedThreads, 0, st>>>((const float2*)data, dim, tg, partials, nt_total, base);
-      else
-        k_expect_group<double2><<<grid, kRedThreads, 0, st>>>((const double2*)data, dim, tg, partials, nt_total, base);
-      QS_LAUNCHED();
-      base += tg.nt;
-    }
-  }
-  if (nt_total == 0) {
-    QS_CUDA(cudaMemsetAsync(dev_out, 0, sizeof(double) * nreg, st));
-  } else {
-    k_expect_final<<<nreg, kFoldThreads, 0, st>>>(partials, nblk, nt_total, dcoeff, dev_out);
+  if (nt == 0) QS_CUDA(cudaMemsetAsync(dev_out, 0, sizeof(double) * nreg, st));
+  for (int r = 0; nt > 0 && r < nreg; r += group) {
+    const int k = std::min(group, nreg - r);
+    const char* p = (const char*)data + ((amp_bytes(dtype) * (size_t)r) << n);
+    QS_TRY(expect_launch(p, dtype, n, k, terms.data(), nt, partials, nblk, nslots, &nslots, st));
+    k_expect_final<<<k, kFoldThreads, 0, st>>>(partials, nblk, nslots, dev_out + r);
     QS_LAUNCHED();
   }
   QS_CUDA(cudaMemcpyAsync(host_out, dev_out, sizeof(double) * nreg, cudaMemcpyDeviceToHost, st));
@@ -306,26 +497,13 @@ int apply_observable_c128(const double2* psi, double2* lam, int n, const qs_obse
 
 constexpr int kF = 1024;
 
-// A float as a double without the conversion instruction, which runs on the FP64
-// unit, this part's scarcest (1/64 of the FP32 rate): the exponent is rebased and
-// the mantissa moved by integer instructions, a subnormal scaled to a normal one
-// first.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t sign = __float_as_uint(x) & 0x80000000u;
-  const bool tiny = (__float_as_uint(x) & 0x7fffffffu) < 0x00800000u;
-  const uint32_t m = __float_as_uint(tiny ? __fmul_rn(x, 16777216.f) : x) & 0x7fffffffu;
-  const uint32_t bias = tiny ? 0x38000000u - (24u << 20) : m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
-  const uint32_t hi = m ? (m >> 3) + bias : 0u;
-  return __hiloint2double((int)(hi | sign), (int)(m << 29));
-}
-
 // What a fold adds up: |amplitude|^2 by the contract, or a level's sums.  The
 // square of a float is exact in FP64, so one fused multiply-add rounds re*re +
 // im*im once, as the contract's multiply, multiply and add do: 2 FP64
 // operations instead of 5 with the conversions.
 __device__ __forceinline__ double prob(float2 v) {
-  const double x = widen(v.x), y = widen(v.y);
-  return __fma_rn(x, x, __dmul_rn(y, y));
+  const double2 w = widen(v);
+  return __fma_rn(w.x, w.x, __dmul_rn(w.y, w.y));
 }
 __device__ __forceinline__ double prob(double2 v) { return __dadd_rn(__dmul_rn(v.x, v.x), __dmul_rn(v.y, v.y)); }
 __device__ __forceinline__ double prob(double v) { return v; }
@@ -776,23 +954,6 @@ constexpr int kStaticMaxDevices = 64;
 
 static __device__ __align__(256) double g_static_partials[kStaticPartials];
 
-struct StaticCoeffs {
-  double c[kStaticTerms];
-};
-
-__global__ void __launch_bounds__(kFoldThreads)
-k_expect_final_static(const double* __restrict__ partials, int nblk, int nt_total,
-                      const __grid_constant__ StaticCoeffs co, double* __restrict__ out) {
-  __shared__ double sh[kFoldThreads];
-  const int r = blockIdx.x;
-  PairwiseAcc terms;
-  for (int t = 0; t < nt_total; ++t) {
-    const double v = block_pairwise(partials + ((size_t)r * nt_total + t) * nblk, nblk, sh);
-    terms.add(co.c[t] * v);
-  }
-  if (threadIdx.x == 0) out[r] = terms.total();
-}
-
 // device address of g_static_partials on the current device, resolved once per
 // device (host code must not use the symbol's host-side name as an address)
 static double* g_static_addr[kStaticMaxDevices];
@@ -851,34 +1012,14 @@ extern "C" int qs_expect_static(const void* dev_amps, int dtype, int nqubits, in
     order[j] = t;
   }
   const uint64_t dim = 1ull << nqubits;
-  long long nblk = expect_blocks(dim);
-  nblk = std::max(1LL, std::min(nblk, (long long)kStaticPartials / ((long long)nreg * nterms)));
-  StaticCoeffs co;
-  memset(&co, 0, sizeof(co));
-  int base = 0;
-  while (base < nterms) {
-    const uint64_t x = host_terms[order[base]].x_mask;
-    TermGroup tg;
-    memset(&tg, 0, sizeof(tg));
-    tg.x = x;
-    tg.h = x ? 63 - __builtin_clzll(x) : -1;
-    tg.item_log2 = x ? nqubits - 1 : nqubits;
-    while (base + tg.nt < nterms && tg.nt < kGroupTerms && host_terms[order[base + tg.nt]].x_mask == x) {
-      const qs_pauli_term& term = host_terms[order[base + tg.nt]];
-      tg.z[tg.nt] = term.z_mask;
-      tg.ny[tg.nt] = __builtin_popcountll(term.x_mask & term.z_mask) & 3;
-      co.c[base + tg.nt] = term.coeff;
-      ++tg.nt;
-    }
-    dim3 grid((unsigned)nblk, nreg);
-    if (dtype == QS_C64)
-      k_expect_group<float2><<<grid, kRedThreads, 0, st>>>((const float2*)dev_amps, dim, tg, partials, nterms, base);
-    else
-      k_expect_group<double2><<<grid, kRedThreads, 0, st>>>((const double2*)dev_amps, dim, tg, partials, nterms, base);
-    QS_LAUNCHED();
-    base += tg.nt;
-  }
-  k_expect_final_static<<<nreg, kFoldThreads, 0, st>>>(partials, (int)nblk, nterms, co, dev_out);
+  const qs_pauli_term* terms[kStaticTerms];
+  for (int t = 0; t < nterms; ++t) terms[t] = &host_terms[order[t]];
+  int nslots = 0;
+  QS_TRY(expect_launch(dev_amps, dtype, nqubits, nreg, terms, nterms, nullptr, 1, 0, &nslots, st));
+  const int nblk = (int)std::max<long long>(
+      1, std::min<long long>(expect_blocks(dim), (long long)kStaticPartials / ((long long)nreg * nslots)));
+  QS_TRY(expect_launch(dev_amps, dtype, nqubits, nreg, terms, nterms, partials, nblk, nslots, &nslots, st));
+  k_expect_final<<<nreg, kFoldThreads, 0, st>>>(partials, nblk, nslots, dev_out);
   if (cudaPeekAtLastError() != cudaSuccess) g_static_addr[cur_dev] = nullptr;  // resolve again next call
   QS_LAUNCHED();
   return QS_OK;
