@@ -18,6 +18,7 @@
 // register's gradient lives in shared memory (FP64) and is written once.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <numeric>
 
@@ -26,7 +27,7 @@
 namespace qs {
 
 constexpr int kMaxRegParams = 2048;
-constexpr int kMaxPhaseOps = 64;
+constexpr int kMaxPhaseOps = 64;   // gates with a parameter in a phase (its gradient sums)
 constexpr int kBatchTile = kMaxTileBits;
 
 struct GSpec {           // one circuit gate of one register
@@ -72,6 +73,7 @@ struct BArgs {
   const TOp* bops;
   const float2* dtab;    // TK_DIAG16 factor tables
   const DRun* druns;     // TK_DIAGRUN entries
+  const float4* rtab;    // TK_DIAGRUN tables (kRunTab a run)
   const BTerm* terms;
   double* loss;
   double* grad;
@@ -110,6 +112,8 @@ __device__ __forceinline__ float recj(float2 p, float2 q) { return fmaf(p.x, q.x
 // (a, b) <- U (a, b) for the structured kinds; U row-major in u0..u3
 // a diagonal whose first entry is exactly 1 (shift, controlled phases): only b changes
 constexpr int TK_DIAGB = 16;
+// a real 2x2
+constexpr int TK_REAL = 17;
 
 template <int KIND>
 __device__ __forceinline__ void pair_apply(float2& a, float2& b, float2 u0, float2 u1, float2 u2, float2 u3) {
@@ -129,6 +133,10 @@ __device__ __forceinline__ void pair_apply(float2& a, float2& b, float2 u0, floa
     const float c = u0.x, p = u1.x, q = u2.x;
     const float2 na = make_float2(fmaf(c, a.x, p * b.x), fmaf(c, a.y, p * b.y));
     const float2 nb = make_float2(fmaf(q, a.x, c * b.x), fmaf(q, a.y, c * b.y));
+    a = na; b = nb;
+  } else if (KIND == TK_REAL) {
+    const float2 na = make_float2(fmaf(u0.x, a.x, u1.x * b.x), fmaf(u0.x, a.y, u1.x * b.y));
+    const float2 nb = make_float2(fmaf(u2.x, a.x, u3.x * b.x), fmaf(u2.x, a.y, u3.x * b.y));
     a = na; b = nb;
   } else {
     const float2 na = cmaf(u1, b, cmulf(u0, a));
@@ -217,43 +225,86 @@ __device__ __forceinline__ void mul_by_bit(float2 (&x)[1 << RB], float2 p0, floa
   for (int j = 0; j < (1 << RB); ++j) x[j] = cmulf(x[j], ((j >> T) & 1) ? p1 : p0);
 }
 
-// a TK_DIAGRUN op: the products p0, p1 of its entries' factors where their
-// controls hold (selects, no branch on the thread's bits), then one pass over
-// the amplitudes by phase bit t
-template <int RB>
-__device__ __forceinline__ void diag_run(float2 (&x)[1 << RB], const TOp& op, const DRun* runs, uint32_t gb) {
-  float2 p0 = make_float2(1.f, 0.f), p1 = p0;
-  const DRun* e = runs + op.param;
-#pragma unroll 2
-  for (uint32_t k = 0; k < op.count; ++k) {
-    const uint4* w = reinterpret_cast<const uint4*>(e + k);
-    const uint4 a = w[0], b = w[1];  // tmask, tval, gate, tq | u0, u3
-    const float2 u0 = make_float2(__uint_as_float(b.x), __uint_as_float(b.y));
-    const float2 u3 = make_float2(__uint_as_float(b.z), __uint_as_float(b.w));
-    const bool on = (gb & a.x) == a.y;
-    float2 f0 = u0, f1 = u3;
-    if (a.w != 0xffffffffu) {  // target outside the phase: one factor by its bit
-      f0 = ((gb >> (a.w & 31u)) & 1u) ? u3 : u0;
-      f1 = f0;
-    }
-    const float2 q0 = cmulf(p0, f0), q1 = cmulf(p1, f1);
-    p0 = on ? q0 : p0;
-    p1 = on ? q1 : p1;
+// x_j *= p1 where bit T of j is 1
+template <int RB, int T>
+__device__ __forceinline__ void mul_bit1(float2 (&x)[1 << RB], float2 p1) {
+#pragma unroll
+  for (int j = 0; j < (1 << RB); ++j)
+    if ((j >> T) & 1) x[j] = cmulf(x[j], p1);
+}
+
+// one entry of a run where its controls hold, by a thread of index bits gb
+__device__ __forceinline__ void run_entry(const DRun* e, uint32_t gb, float2& p0, float2& p1) {
+  const uint4* w = reinterpret_cast<const uint4*>(e);
+  const uint4 a = w[0], b = w[1];  // tmask, tval, gate, tq | u0, u3
+  const float2 u0 = make_float2(__uint_as_float(b.x), __uint_as_float(b.y));
+  const float2 u3 = make_float2(__uint_as_float(b.z), __uint_as_float(b.w));
+  const bool on = (gb & a.x) == a.y;
+  float2 f0 = u0, f1 = u3;
+  if (a.w != 0xffffffffu) {  // target outside the phase: one factor by its bit
+    f0 = ((gb >> (a.w & 31u)) & 1u) ? u3 : u0;
+    f1 = f0;
   }
-  switch (op.t) {
-    case 0: mul_by_bit<RB, 0>(x, p0, p1); break;
-    case 1: mul_by_bit<RB, 1>(x, p0, p1); break;
-    case 2: if constexpr (RB > 2) mul_by_bit<RB, 2>(x, p0, p1); break;
-    default: if constexpr (RB > 3) mul_by_bit<RB, 3>(x, p0, p1); break;
+  const float2 q0 = cmulf(p0, f0), q1 = cmulf(p1, f1);
+  p0 = on ? q0 : p0;
+  p1 = on ? q1 : p1;
+}
+
+// What a TK_DIAGRUN op reads besides its record: the pass's entries, its runs' tables
+// and, in the tile engine, the products of each run's tile-id entries for this tile.  In
+// shared memory, so that the op loops carry one pointer for it.
+struct RunCtx {
+  const DRun* entries;
+  const float4* tab;
+  const float4* tile;  // NULL: those entries are applied thread by thread
+};
+
+// a TK_DIAGRUN op: the products p0, p1 of its entries' factors, then one pass over the
+// amplitudes by phase bit t.  The table look-ups replace up to n - 4 entries tested and
+// multiplied by every thread (QFT of 29 qubits,
+// first pass: 20.7 -> 11.0 ms, with the phases no longer cut at 64 gates).
+template <int RB>
+__device__ __forceinline__ void diag_run(float2 (&x)[1 << RB], const TOp& op, const RunCtx& rc, uint32_t gb) {
+  const int run = __float_as_int(op.cfac2);
+  const float4* tab = rc.tab + run * kRunTab;
+  const float4 a = tab[threadIdx.x & 31], b = tab[32 + (threadIdx.x >> 5)];
+  float2 p0 = make_float2(1.f, 0.f);
+  float2 p1 = cmulf(make_float2(a.z, a.w), make_float2(b.z, b.w));
+  const bool one0 = op.gen == 1;
+  if (!one0) p0 = cmulf(make_float2(a.x, a.y), make_float2(b.x, b.y));
+  uint32_t k = 0;
+  if (rc.tile) {
+    const float4 t = rc.tile[run];
+    if (!one0) p0 = cmulf(p0, make_float2(t.x, t.y));
+    p1 = cmulf(p1, make_float2(t.z, t.w));
+    k = op.shared;
+  }
+  const DRun* e = rc.entries + op.param;
+  for (; k < op.count; ++k) run_entry(e + k, gb, p0, p1);
+  if (one0) {
+    switch (op.t) {
+      case 0: mul_bit1<RB, 0>(x, p1); break;
+      case 1: mul_bit1<RB, 1>(x, p1); break;
+      case 2: if constexpr (RB > 2) mul_bit1<RB, 2>(x, p1); break;
+      default: if constexpr (RB > 3) mul_bit1<RB, 3>(x, p1); break;
+    }
+  } else {
+    switch (op.t) {
+      case 0: mul_by_bit<RB, 0>(x, p0, p1); break;
+      case 1: mul_by_bit<RB, 1>(x, p0, p1); break;
+      case 2: if constexpr (RB > 2) mul_by_bit<RB, 2>(x, p0, p1); break;
+      default: if constexpr (RB > 3) mul_by_bit<RB, 3>(x, p0, p1); break;
+    }
   }
 }
 
 // Forward op forms by TOp::var: 0 out-of-phase diagonal, 1 diagonal table,
 // 2 + t controlled swap, 6 + t / 10 + t diagonal without / with phase-local
 // controls, 14 + t / 18 + t dense without / with them (t: target phase bit),
-// 22 a run of diagonal gates (TK_DIAGRUN)
+// 22 a run of diagonal gates (TK_DIAGRUN), 23 + t dense and real without controls (H:
+// half the multiply-adds)
 enum { FV_DIAGOUT = 0, FV_DIAG16 = 1, FV_SWAP = 2, FV_DIAG = 6, FV_DIAGC = 10, FV_DENSE = 14, FV_DENSEC = 18,
-       FV_DIAGRUN = 22 };
+       FV_DIAGRUN = 22, FV_REAL = 23 };
 
 template <int RB, int T, int KIND, bool CTRL, bool COMP>
 __device__ __forceinline__ void fwd_form(float2 (&x)[1 << RB], const TOp& op, const float2* lo) {
@@ -273,11 +324,15 @@ __device__ __forceinline__ void fwd_form(float2 (&x)[1 << RB], const TOp& op, co
 
 template <int RB, bool COMP>
 __device__ __forceinline__ void apply_fwd_var(float2 (&x)[1 << RB], const TOp& op, const float2* lo,
-                                              const DRun* runs, uint32_t gb) {
+                                              const RunCtx& rc, uint32_t gb) {
   switch (op.var) {
     case FV_DIAGRUN:
-      if constexpr (!COMP) diag_run<RB>(x, op, runs, gb);
+      if constexpr (!COMP) diag_run<RB>(x, op, rc, gb);
       break;
+    case FV_REAL + 0: if constexpr (!COMP) fwd_form<RB, 0, TK_REAL, false, COMP>(x, op, lo); break;
+    case FV_REAL + 1: if constexpr (!COMP) fwd_form<RB, 1, TK_REAL, false, COMP>(x, op, lo); break;
+    case FV_REAL + 2: if constexpr (!COMP) fwd_form<RB, 2, TK_REAL, false, COMP>(x, op, lo); break;
+    case FV_REAL + 3: if constexpr (!COMP) fwd_form<RB, 3, TK_REAL, false, COMP>(x, op, lo); break;
     case FV_SWAP + 0: fwd_form<RB, 0, TK_SWAP, true, COMP>(x, op, lo); break;
     case FV_SWAP + 1: fwd_form<RB, 1, TK_SWAP, true, COMP>(x, op, lo); break;
     case FV_SWAP + 2: fwd_form<RB, 2, TK_SWAP, true, COMP>(x, op, lo); break;
@@ -604,11 +659,22 @@ __device__ __forceinline__ float apply_bwd_ff(ffc (&x)[1 << RB], ffc (&l)[1 << R
 
 constexpr int kWarps = kTileThreads / 32;
 
+// The functions below that are not inlined take shared memory as byte offsets into the
+// dynamic array: through a generic pointer every access costs 64-bit address
+// arithmetic and a generic load (with the phase index arithmetic below: 8 % fewer
+// instructions in a QFT pass, batch of 1024 registers 112 -> 107 ms).
+template <typename T>
+__device__ __forceinline__ T* sh(uint32_t off) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  return reinterpret_cast<T*>(smraw + off);
+}
+
 struct BShared {
   double grad[kMaxRegParams];
   float red[kMaxPhaseOps * kWarps];
   double lred[kWarps];
   uint32_t rowoff[1 << (kMaxTileBits - kRowBits)];  // register offset of each 32-amplitude tile row (current pass)
+  RunCtx rc;
   int reg;
 };
 
@@ -636,8 +702,10 @@ __device__ __forceinline__ uint64_t tile_base(uint64_t tile, const TPass& p, int
 constexpr int kLdChunk = 8;
 
 template <bool TWO>
-__device__ __noinline__ void load_tiles(float2* sm0, const float2* src0, float2* sm1, const float2* src1,
-                                        const uint32_t* rowoff, int m) {
+__device__ __noinline__ void load_tiles(uint32_t o0, const float2* src0, uint32_t o1, const float2* src1,
+                                        uint32_t rows, int m) {
+  float2 *sm0 = sh<float2>(o0), *sm1 = sh<float2>(o1);
+  const uint32_t* rowoff = sh<uint32_t>(rows);
   const uint32_t nq = 1u << (m - 1);  // float4 per tile
   constexpr int C = TWO ? kLdChunk / 2 : kLdChunk;
   for (uint32_t q0 = 0; q0 < nq; q0 += C * kTileThreads) {
@@ -668,8 +736,9 @@ __device__ __noinline__ void load_tiles(float2* sm0, const float2* src0, float2*
 }
 
 template <bool TWO>
-__device__ __noinline__ void store_tiles(const float2* sm0, float2* dst0, const float2* sm1, float2* dst1,
-                                         const uint32_t* rowoff, int m) {
+__device__ __noinline__ void store_tiles(uint32_t o0, float2* dst0, uint32_t o1, float2* dst1, uint32_t rows, int m) {
+  const float2 *sm0 = sh<float2>(o0), *sm1 = sh<float2>(o1);
+  const uint32_t* rowoff = sh<uint32_t>(rows);
   const uint32_t nq = 1u << (m - 1);
   for (uint32_t q = threadIdx.x; q < nq; q += kTileThreads) {
     const uint32_t off = rowoff[q >> 4] + 2 * (q & 15);
@@ -683,17 +752,19 @@ __device__ __noinline__ void store_tiles(const float2* sm0, float2* dst0, const 
   }
 }
 
-__device__ __forceinline__ void load_tile(float2* sm, const float2* src, const uint32_t* rowoff, int m) {
-  load_tiles<false>(sm, src, nullptr, nullptr, rowoff, m);
+__device__ __forceinline__ void load_tile(uint32_t sm, const float2* src, uint32_t rows, int m) {
+  load_tiles<false>(sm, src, 0, nullptr, rows, m);
 }
-__device__ __forceinline__ void store_tile(const float2* sm, float2* dst, const uint32_t* rowoff, int m) {
-  store_tiles<false>(sm, dst, nullptr, nullptr, rowoff, m);
+__device__ __forceinline__ void store_tile(uint32_t sm, float2* dst, uint32_t rows, int m) {
+  store_tiles<false>(sm, dst, 0, nullptr, rows, m);
 }
 
 // double-float tiles of psi and lambda (one float4 = hi.re, hi.im, lo.re, lo.im
 // per amplitude, in global and shared memory)
-__device__ __noinline__ void load_tiles_ff(float4* sm0, const float4* src0, float4* sm1, const float4* src1,
-                                           const uint32_t* rowoff, int m) {
+__device__ __noinline__ void load_tiles_ff(uint32_t o0, const float4* src0, uint32_t o1, const float4* src1,
+                                           uint32_t rows, int m) {
+  float4 *sm0 = sh<float4>(o0), *sm1 = sh<float4>(o1);
+  const uint32_t* rowoff = sh<uint32_t>(rows);
   const uint32_t cnt = 1u << m;
   constexpr int C = kLdChunk / 2;
   for (uint32_t q0 = 0; q0 < cnt; q0 += C * kTileThreads) {
@@ -718,8 +789,9 @@ __device__ __noinline__ void load_tiles_ff(float4* sm0, const float4* src0, floa
   }
 }
 
-__device__ __noinline__ void store_tiles_ff(const float4* sm0, float4* dst0, const float4* sm1, float4* dst1,
-                                            const uint32_t* rowoff, int m) {
+__device__ __noinline__ void store_tiles_ff(uint32_t o0, float4* dst0, uint32_t o1, float4* dst1, uint32_t rows, int m) {
+  const float4 *sm0 = sh<float4>(o0), *sm1 = sh<float4>(o1);
+  const uint32_t* rowoff = sh<uint32_t>(rows);
   const uint32_t cnt = 1u << m;
   for (uint32_t q = threadIdx.x; q < cnt; q += kTileThreads) {
     const uint32_t off = rowoff[q >> kRowBits] + (q & 31u);
@@ -728,17 +800,20 @@ __device__ __noinline__ void store_tiles_ff(const float4* sm0, float4* dst0, con
   }
 }
 
-__device__ __forceinline__ uint32_t phase_base(uint32_t tid, const TPhase& ph, int nthreadbits) {
-  uint32_t b = 0;
-  for (int k = 0; k < nthreadbits; ++k) b |= ((tid >> k) & 1u) << ph.tpos[k];
+// Tile-local index of a thread's first amplitude: zeros put in at the phase's register
+// bits (keep[k]: the bits below the k-th of them; rb steps of two instructions)
+template <int RB>
+__device__ __forceinline__ uint32_t phase_base(uint32_t tid, const TPhase& ph) {
+  uint32_t b = tid;
+#pragma unroll
+  for (int k = 0; k < RB; ++k) b += b & ~(uint32_t)ph.keep[k];
   return b;
 }
 
-// global register index bits of this thread's amplitudes outside the phase
-__device__ __forceinline__ uint32_t thread_global(uint32_t tid, const TPhase& ph, int nthreadbits, uint32_t tbase) {
-  uint32_t b = tbase;
-  for (int k = 0; k < nthreadbits; ++k) b |= ((tid >> k) & 1u) << ph.tq[k];
-  return b;
+// global register index bits of this thread's amplitudes outside the phase: its place
+// in the tile's rows (register qubits 0..4 are the tile's bits 0..4)
+__device__ __forceinline__ uint32_t thread_global(uint32_t base, const uint32_t* rowoff, uint32_t tbase) {
+  return tbase + rowoff[base >> kRowBits] + (base & 31u);
 }
 
 // shared-memory slot of amplitude j of a phase: swz is linear over XOR, so
@@ -773,7 +848,7 @@ __device__ __forceinline__ TOp load_op(const TOp* p) {
   r.gen = (uint8_t)(a.y & 0xffu);
   r.shared = (uint8_t)((a.y >> 8) & 0xffu);
   r.var = (uint8_t)((a.y >> 16) & 0xffu);
-  r.pad = 0;
+  r.pad = (uint8_t)(a.y >> 24);
   r.param = (int32_t)a.z;
   r.cfac2 = __uint_as_float(a.w);
   r.tmask = b.x;
@@ -861,14 +936,15 @@ __device__ __forceinline__ void diag_masked(float2 (&x)[1 << RB], float2 f, int 
 // diagonal table); out-of-phase diagonal factors are then applied one by one
 template <int RB, bool COMP, bool RESLOT>
 __device__ __forceinline__ void phase_fwd_body(float2* sm, const TPhase* php, const TOp* fops, const float2* dtab,
-                                               const float2* flo, const float2* dtlo, const DRun* runs, int m,
-                                               uint32_t tbase) {
+                                               const float2* flo, const float2* dtlo, const RunCtx& rc,
+                                               const uint32_t* rowoff, int m, uint32_t tbase) {
   constexpr int A = 1 << RB;
   const TPhase& ph = *php;
   const int ntb = m - RB;
   if (threadIdx.x < (1u << ntb)) {
-    const PhaseSlots ps = phase_slots(swz(phase_base(threadIdx.x, ph, ntb)), ph);
-    const uint32_t gb = thread_global(threadIdx.x, ph, ntb, tbase);
+    const uint32_t base = phase_base<RB>(threadIdx.x, ph);
+    const PhaseSlots ps = phase_slots(swz(base), ph);
+    const uint32_t gb = thread_global(base, rowoff, tbase);
     float2 x[A];
 #pragma unroll
     for (int j = 0; j < A; ++j) x[j] = sm[slot(ps, j)];
@@ -907,7 +983,7 @@ __device__ __forceinline__ void phase_fwd_body(float2* sm, const TPhase* php, co
           for (int j = 0; j < A; ++j) x[j] = cmulf(x[j], t[j]);
         }
       } else {
-        apply_fwd_var<RB, COMP>(x, cur, COMP ? flo + 4 * oi : nullptr, runs, gb);
+        apply_fwd_var<RB, COMP>(x, cur, COMP ? flo + 4 * oi : nullptr, rc, gb);
       }
     }
     if (!COMP && has_pend) {
@@ -917,7 +993,7 @@ __device__ __forceinline__ void phase_fwd_body(float2* sm, const TPhase* php, co
     // RESLOT: the slot offsets again (from shared memory) rather than live
     // through the op loop (fewer spills in k_batch; slower in the tile engine,
     // whose loop does not spill)
-    const PhaseSlots ps2 = RESLOT ? phase_slots(swz(phase_base(threadIdx.x, ph, ntb)), ph) : ps;
+    const PhaseSlots ps2 = RESLOT ? phase_slots(swz(phase_base<RB>(threadIdx.x, ph)), ph) : ps;
 #pragma unroll
     for (int j = 0; j < A; ++j) sm[slot(ps2, j)] = x[j];
   }
@@ -930,11 +1006,12 @@ __device__ __forceinline__ void phase_fwd_body(float2* sm, const TPhase* php, co
 // k_batch spilled several times as much (ptxas -v) as two copies do; SITE 2
 // is the tile engine's pass.
 template <int RB, bool COMP, int SITE = 0>
-__device__ __noinline__ void run_tile_fwd(float2* sm, const TPhase* ph, int nphase, const TOp* fops,
-                                          const float2* dtab, const float2* flo, const float2* dtlo,
-                                          const DRun* runs, int m, uint32_t tbase) {
+__device__ __noinline__ void run_tile_fwd(uint32_t sm, const TPhase* ph, int nphase, const TOp* fops,
+                                          const float2* dtab, const float2* flo, const float2* dtlo, uint32_t rc,
+                                          uint32_t rows, int m, uint32_t tbase) {
   for (int f = 0; f < nphase; ++f)
-    phase_fwd_body<RB, COMP, SITE != 2>(sm, ph + f, fops, dtab, flo, dtlo, runs, m, tbase);
+    phase_fwd_body<RB, COMP, SITE != 2>(sh<float2>(sm), ph + f, fops, dtab, flo, dtlo, *sh<RunCtx>(rc),
+                                        sh<uint32_t>(rows), m, tbase);
 }
 
 // backward of an out-of-phase diagonal gate: the generator is diagonal on the
@@ -1025,7 +1102,7 @@ __device__ __forceinline__ void fold_phase_grad(const TPhase& ph, const TOp* bop
     const int t = base + (int)threadIdx.x;
     const int o = t >> 4, w = t & 15;
     const bool valid = o < nbop && bops[bop0 + o].gen != GEN_NONE;
-    float s = valid ? red[o * kWarps + w] : 0.f, e = 0.f;
+    float s = valid ? red[bops[bop0 + o].pad * kWarps + w] : 0.f, e = 0.f;
 #pragma unroll
     for (int d = 8; d > 0; d >>= 1) {
       const float so = __shfl_xor_sync(0xffffffffu, s, d), eo = __shfl_xor_sync(0xffffffffu, e, d);
@@ -1046,7 +1123,7 @@ __device__ __forceinline__ void fold_phase_grad(const TPhase& ph, const TOp* bop
       const TOp& op = bops[bop0 + q];
       if (op.gen == GEN_NONE || !op.shared) continue;
       double v = 0.0;
-      for (int w = 0; w < kWarps; ++w) v += (double)red[q * kWarps + w];
+      for (int w = 0; w < kWarps; ++w) v += (double)red[op.pad * kWarps + w];
       gacc[op.param] += (double)op.cfac2 * v;
     }
   }
@@ -1055,7 +1132,7 @@ __device__ __forceinline__ void fold_phase_grad(const TPhase& ph, const TOp* bop
 
 template <int RB>
 __device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPhase* php, const TOp* bops, int m,
-                                               float* red, double* gacc, uint32_t tbase) {
+                                               const uint32_t* rowoff, float* red, double* gacc, uint32_t tbase) {
   // the phase record is read where it lies (the pass's shared-memory copy when
   // staged): with 2 x 2^RB live amplitudes per thread there are no registers
   // to spare for a copy of it
@@ -1066,8 +1143,9 @@ __device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPh
   const bool active = threadIdx.x < (1u << ntb);
   const int nbop = ph.nbop, bop0 = ph.bop0;
   float2 x[A], l[A];
-  const uint32_t gb = active ? thread_global(threadIdx.x, ph, ntb, tbase) : 0u;
-  const PhaseSlots ps = phase_slots(active ? swz(phase_base(threadIdx.x, ph, ntb)) : 0u, ph);
+  const uint32_t base = active ? phase_base<RB>(threadIdx.x, ph) : 0u;
+  const uint32_t gb = thread_global(base, rowoff, tbase);
+  const PhaseSlots ps = phase_slots(swz(base), ph);
   if (active) {
 #pragma unroll
     for (int j = 0; j < A; ++j) {
@@ -1083,7 +1161,7 @@ __device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPh
     float part = 0.f;
     if (active && (gb & op.tmask) == op.tval)
       part = op.kind == TK_DIAGOUT ? diagout_bwd<RB>(x, l, op, gb) : apply_bwd_var<RB>(x, l, op);
-    if (op.gen != GEN_NONE) warp_partial(part, o, pend, pend_o, red, lane, warp);
+    if (op.gen != GEN_NONE) warp_partial(part, op.pad, pend, pend_o, red, lane, warp);
   }
   flush_partial(pend, pend_o, red, lane, warp);
   if (active) {
@@ -1101,14 +1179,21 @@ __device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPh
 // All phases of a pass on one tile, last phase first: one call per tile, so
 // that the callers' loop state is saved once per tile rather than per phase
 template <int RB>
-__device__ __noinline__ void run_tile_bwd(float2* sx, float2* sl, const TPhase* ph, int nphase, const TOp* bops,
-                                          int m, float* red, double* gacc, uint32_t tbase) {
-  for (int f = nphase - 1; f >= 0; --f) phase_bwd_body<RB>(sx, sl, ph + f, bops, m, red, gacc, tbase);
+__device__ __noinline__ void run_tile_bwd(uint32_t sx, uint32_t sl, const TPhase* ph, int nphase, const TOp* bops,
+                                          int m, uint32_t rows, uint32_t red, uint32_t gacc, uint32_t tbase) {
+  for (int f = nphase - 1; f >= 0; --f)
+    phase_bwd_body<RB>(sh<float2>(sx), sh<float2>(sl), ph + f, bops, m, sh<uint32_t>(rows), sh<float>(red),
+                       sh<double>(gacc), tbase);
 }
 
 template <int RB>
-__device__ __noinline__ void run_phase_bwd_ff(float4* sx, float4* sl, const TPhase* php, const TOp* bops,
-                                              const float2* blo, int m, float* red, double* gacc, uint32_t tbase) {
+__device__ __noinline__ void run_phase_bwd_ff(uint32_t ox, uint32_t ol, const TPhase* php, const TOp* bops,
+                                              const float2* blo, int m, uint32_t rows, uint32_t ored, uint32_t ogacc,
+                                              uint32_t tbase) {
+  float4 *sx = sh<float4>(ox), *sl = sh<float4>(ol);
+  const uint32_t* rowoff = sh<uint32_t>(rows);
+  float* red = sh<float>(ored);
+  double* gacc = sh<double>(ogacc);
   constexpr int A = 1 << RB;
   const TPhase& ph = *php;
   const int ntb = m - RB;
@@ -1116,8 +1201,9 @@ __device__ __noinline__ void run_phase_bwd_ff(float4* sx, float4* sl, const TPha
   const bool active = threadIdx.x < (1u << ntb);
   const int nbop = ph.nbop, bop0 = ph.bop0;
   ffc x[A], l[A];
-  const uint32_t gb = active ? thread_global(threadIdx.x, ph, ntb, tbase) : 0u;
-  const PhaseSlots ps = phase_slots(active ? swz(phase_base(threadIdx.x, ph, ntb)) : 0u, ph);
+  const uint32_t base = active ? phase_base<RB>(threadIdx.x, ph) : 0u;
+  const uint32_t gb = thread_global(base, rowoff, tbase);
+  const PhaseSlots ps = phase_slots(swz(base), ph);
   if (active) {
 #pragma unroll
     for (int j = 0; j < A; ++j) {
@@ -1138,7 +1224,7 @@ __device__ __noinline__ void run_phase_bwd_ff(float4* sx, float4* sl, const TPha
     if (active && (gb & op.tmask) == op.tval)
       part = op.kind == TK_DIAGOUT ? diagout_bwd_ff<RB>(x, l, op, blo + 4 * oi, gb)
                                    : apply_bwd_ff<RB>(x, l, op, blo + 4 * oi);
-    if (op.gen != GEN_NONE) warp_partial(part, o, pend, pend_o, red, lane, warp);
+    if (op.gen != GEN_NONE) warp_partial(part, op.pad, pend, pend_o, red, lane, warp);
   }
   flush_partial(pend, pend_o, red, lane, warp);
   if (active) {
@@ -1211,61 +1297,62 @@ __device__ void block_loss(double e, BShared& S, double* out) {
 // functions: a phase call then sees only the loop's few live values, and the
 // phase functions keep their amplitudes in registers.
 template <int RB>
-__device__ __noinline__ void batch_bwd_resident(float2* sx, float2* sl, const TPass* P, int npass, int m,
-                                                const TPhase* phases, const TOp* bops, float* red, double* gacc) {
+__device__ __noinline__ void batch_bwd_resident(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m,
+                                                const TPhase* phases, const TOp* bops, uint32_t rows, uint32_t red,
+                                                uint32_t gacc) {
   for (int pi = npass - 1; pi >= 0; --pi)
-    run_tile_bwd<RB>(sx, sl, phases + P[pi].phase0, P[pi].nphase, bops, m, red, gacc, 0u);
+    run_tile_bwd<RB>(sx, sl, phases + P[pi].phase0, P[pi].nphase, bops, m, rows, red, gacc, 0u);
 }
 
 template <int RB>
-__device__ __noinline__ void batch_bwd_resident_ff(float4* sx, float4* sl, const TPass* P, int npass, int m,
+__device__ __noinline__ void batch_bwd_resident_ff(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m,
                                                    const TPhase* phases, const TOp* bops, const float2* blo,
-                                                   float* red, double* gacc) {
+                                                   uint32_t rows, uint32_t red, uint32_t gacc) {
   for (int pi = npass - 1; pi >= 0; --pi) {
     const int ph0 = P[pi].phase0;
     for (int f = P[pi].nphase - 1; f >= 0; --f)
-      run_phase_bwd_ff<RB>(sx, sl, phases + ph0 + f, bops, blo, m, red, gacc, 0u);
+      run_phase_bwd_ff<RB>(sx, sl, phases + ph0 + f, bops, blo, m, rows, red, gacc, 0u);
   }
 }
 
 template <int RB>
-__device__ __noinline__ void batch_bwd_streamed(float2* sx, float2* sl, const TPass* P, int npass, int m, int g,
+__device__ __noinline__ void batch_bwd_streamed(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m, int g,
                                                 float2* wp, float2* wl, const TPhase* phases, const TOp* bops,
-                                                uint32_t* rowoff, float* red, double* gacc, unsigned char* stage) {
+                                                uint32_t rows, uint32_t red, uint32_t gacc, unsigned char* stage) {
   const uint64_t ntile = 1ull << g;
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
-    set_rows(rowoff, p, m);
+    set_rows(sh<uint32_t>(rows), p, m);
     const StagedPass sp = stage_pass<false>(p, phases, bops, stage);
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
-      load_tiles<true>(sx, wp + tb, sl, wl + tb, rowoff, m);
+      load_tiles<true>(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
-      run_tile_bwd<RB>(sx, sl, sp.ph, p.nphase, sp.ops, m, red, gacc, (uint32_t)tb);
-      store_tiles<true>(sx, wp + tb, sl, wl + tb, rowoff, m);
+      run_tile_bwd<RB>(sx, sl, sp.ph, p.nphase, sp.ops, m, rows, red, gacc, (uint32_t)tb);
+      store_tiles<true>(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
     }
   }
 }
 
 template <int RB>
-__device__ __noinline__ void batch_bwd_streamed_ff(float4* sx, float4* sl, const TPass* P, int npass, int m, int g,
+__device__ __noinline__ void batch_bwd_streamed_ff(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m, int g,
                                                    float4* wp, float4* wl, const TPhase* phases, const TOp* bops,
-                                                   const float2* blo, uint32_t* rowoff, float* red, double* gacc,
+                                                   const float2* blo, uint32_t rows, uint32_t red, uint32_t gacc,
                                                    unsigned char* stage) {
   const uint64_t ntile = 1ull << g;
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
-    set_rows(rowoff, p, m);
+    set_rows(sh<uint32_t>(rows), p, m);
     const StagedPass sp = stage_pass<false>(p, phases, bops, stage);
     const float2* lo = blo + 4 * (size_t)sp.first;
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
-      load_tiles_ff(sx, wp + tb, sl, wl + tb, rowoff, m);
+      load_tiles_ff(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
       for (int f = p.nphase - 1; f >= 0; --f)
-        run_phase_bwd_ff<RB>(sx, sl, sp.ph + f, sp.ops, lo, m, red, gacc, (uint32_t)tb);
-      store_tiles_ff(sx, wp + tb, sl, wl + tb, rowoff, m);
+        run_phase_bwd_ff<RB>(sx, sl, sp.ph + f, sp.ops, lo, m, rows, red, gacc, (uint32_t)tb);
+      store_tiles_ff(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
     }
   }
@@ -1282,36 +1369,40 @@ __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wa
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
 // issue the copies of one tile (2^m amplitudes) into sm (no wait)
-__device__ __forceinline__ void load_tile_async(float2* sm, const float2* src, const uint32_t* rowoff, int m) {
+__device__ __forceinline__ void load_tile_async(uint32_t o, const float2* src, uint32_t rows, int m) {
+  float2* sm = sh<float2>(o);
+  const uint32_t* rowoff = sh<uint32_t>(rows);
   const uint32_t n = 1u << m;
   for (uint32_t l = threadIdx.x; l < n; l += kTileThreads)
     cp_async8(sm + swz(l), src + rowoff[l >> kRowBits] + (l & 31u));
 }
 
 template <int RB, bool COMP>
-__device__ __noinline__ void batch_fwd_streamed(float2* sx, float2* sx2, float2* st, const TPass* P, int npass,
+__device__ __noinline__ void batch_fwd_streamed(uint32_t sx, uint32_t sx2, float2* st, const TPass* P, int npass,
                                                 int m, int g, const TPhase* phases, const TOp* fops,
                                                 const float2* dtab, const float2* flo, const float2* dtlo,
-                                                const DRun* druns, uint32_t* rowoff, unsigned char* stage) {
+                                                const DRun* druns, const float4* rtab, uint32_t rc, uint32_t rows,
+                                                unsigned char* stage) {
   const uint64_t ntile = 1ull << g;
   for (int pi = 0; pi < npass; ++pi) {
     const TPass& p = P[pi];
-    set_rows(rowoff, p, m);
+    set_rows(sh<uint32_t>(rows), p, m);
     const StagedPass sp = stage_pass<true>(p, phases, fops, stage, druns);
     const float2* lo = COMP ? flo + 4 * (size_t)sp.first : nullptr;
+    if (threadIdx.x == 0) *sh<RunCtx>(rc) = RunCtx{sp.runs, rtab + kRunTab * p.run0, nullptr};
     // two tile buffers (sx, sx2): the next tile's copies are in flight while
     // the current one is computed
-    load_tile_async(sx, st + tile_base(0, p, g), rowoff, m);
+    load_tile_async(sx, st + tile_base(0, p, g), rows, m);
     cp_async_commit();
     for (uint64_t t = 0; t < ntile; ++t) {
-      float2* cur = (t & 1) ? sx2 : sx;
-      if (t + 1 < ntile) load_tile_async((t & 1) ? sx : sx2, st + tile_base(t + 1, p, g), rowoff, m);
+      const uint32_t cur = (t & 1) ? sx2 : sx;
+      if (t + 1 < ntile) load_tile_async((t & 1) ? sx : sx2, st + tile_base(t + 1, p, g), rows, m);
       cp_async_commit();
       cp_async_wait_prev();
       __syncthreads();
       const uint64_t tb = tile_base(t, p, g);
-      run_tile_fwd<RB, COMP, 1>(cur, sp.ph, p.nphase, sp.ops, dtab, lo, dtlo, sp.runs, m, (uint32_t)tb);
-      store_tile(cur, st + tb, rowoff, m);
+      run_tile_fwd<RB, COMP, 1>(cur, sp.ph, p.nphase, sp.ops, dtab, lo, dtlo, rc, rows, m, (uint32_t)tb);
+      store_tile(cur, st + tb, rows, m);
       __syncthreads();
     }
     cp_async_wait_all();
@@ -1338,6 +1429,11 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
   float4* sxf = reinterpret_cast<float4*>(body + (size_t)8 * (1 << MT));   // double-float psi (precise)
   float4* slf = sxf + (1 << MT);                                           // double-float lambda (precise)
   unsigned char* stage = body + (size_t)(PREC ? 40 : 16) * (1 << MT);      // a pass's records (streamed registers)
+  // byte offsets of the above
+  const uint32_t ox = (uint32_t)(body - smraw), ol = ox + (uint32_t)sizeof(float2) * (1u << MT);
+  const uint32_t oxf = ol, olf = oxf + (uint32_t)sizeof(float4) * (1u << MT);
+  const uint32_t orows = (uint32_t)offsetof(BShared, rowoff), ored = (uint32_t)offsetof(BShared, red);
+  const uint32_t ograd = (uint32_t)offsetof(BShared, grad), orc = (uint32_t)offsetof(BShared, rc);
   const int tid = threadIdx.x;
   for (;;) {
     if (tid == 0) S.reg = atomicAdd(a.counter, 1);
@@ -1359,21 +1455,25 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
       if (a.flags & BF_RESET) {
         for (uint32_t l = tid; l < (1u << m); l += blockDim.x) sx[swz(l)] = make_float2(l == 0 ? 1.f : 0.f, 0.f);
       } else {
-        load_tile(sx, st, S.rowoff, m);
+        load_tile(ox, st, orows, m);
       }
       __syncthreads();
-      for (int pi = 0; pi < R.npass; ++pi)
-        run_tile_fwd<RB, PREC>(sx, a.phases + P[pi].phase0, P[pi].nphase, a.fops, a.dtab, a.flo, a.dtlo,
-                               a.druns + P[pi].drun0, m, 0u);
-      store_tile(sx, st, S.rowoff, m);  // psi_N
+      for (int pi = 0; pi < R.npass; ++pi) {
+        if (!PREC) {
+          if (tid == 0) S.rc = RunCtx{a.druns + P[pi].drun0, a.rtab + kRunTab * P[pi].run0, nullptr};
+          __syncthreads();
+        }
+        run_tile_fwd<RB, PREC>(ox, a.phases + P[pi].phase0, P[pi].nphase, a.fops, a.dtab, a.flo, a.dtlo, orc, orows, m, 0u);
+      }
+      store_tile(ox, st, orows, m);  // psi_N
       if (PREC) {
         block_loss(expect_tile_ff(sx, sxf, slf, 0, S.rowoff, m, a.terms + R.term0, R.nterm), S, a.loss + reg);
         __syncthreads();
-        if (grad) batch_bwd_resident_ff<RB>(sxf, slf, P, R.npass, m, a.phases, a.bops, a.blo, S.red, S.grad);
+        if (grad) batch_bwd_resident_ff<RB>(oxf, olf, P, R.npass, m, a.phases, a.bops, a.blo, orows, ored, ograd);
       } else {
         block_loss(expect_tile(sx, sl, 0, S.rowoff, m, a.terms + R.term0, R.nterm), S, a.loss + reg);
         __syncthreads();
-        if (grad) batch_bwd_resident<RB>(sx, sl, P, R.npass, m, a.phases, a.bops, S.red, S.grad);
+        if (grad) batch_bwd_resident<RB>(ox, ol, P, R.npass, m, a.phases, a.bops, orows, ored, ograd);
       }
     } else {
       // ---- tiles streamed through global memory
@@ -1381,24 +1481,24 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
         for (uint64_t i = tid; i < (1ull << n); i += blockDim.x) st[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
         __syncthreads();
       }
-      batch_fwd_streamed<RB, PREC>(sx, PREC ? reinterpret_cast<float2*>(sxf) : sl, st, P, R.npass, m, g, a.phases,
-                                   a.fops, a.dtab, a.flo, a.dtlo, a.druns, S.rowoff, stage);
+      batch_fwd_streamed<RB, PREC>(ox, ol, st, P, R.npass, m, g, a.phases,
+                                   a.fops, a.dtab, a.flo, a.dtlo, a.druns, a.rtab, orc, orows, stage);
       // expectation, lambda = O psi, and the work copy of psi for the uncompute
       double e = 0.0;
       const TPass& p0 = P[0];
       set_rows(S.rowoff, p0, m);
       for (uint64_t t = 0; t < ntile; ++t) {
         const uint64_t tb = tile_base(t, p0, g);
-        load_tile(sx, st + tb, S.rowoff, m);
+        load_tile(ox, st + tb, orows, m);
         __syncthreads();
         if (PREC) {
           e += expect_tile_ff(sx, sxf, slf, tb, S.rowoff, m, a.terms + R.term0, R.nterm);
           __syncthreads();
-          if (grad) store_tiles_ff(sxf, a.wpsif + R.work_off + tb, slf, a.wlamf + R.work_off + tb, S.rowoff, m);
+          if (grad) store_tiles_ff(oxf, a.wpsif + R.work_off + tb, olf, a.wlamf + R.work_off + tb, orows, m);
         } else {
           e += expect_tile(sx, sl, tb, S.rowoff, m, a.terms + R.term0, R.nterm);
           __syncthreads();
-          if (grad) store_tiles<true>(sx, a.wpsi + R.work_off + tb, sl, a.wlam + R.work_off + tb, S.rowoff, m);
+          if (grad) store_tiles<true>(ox, a.wpsi + R.work_off + tb, ol, a.wlam + R.work_off + tb, orows, m);
         }
         __syncthreads();
       }
@@ -1406,11 +1506,11 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
       __syncthreads();
       if (grad) {
         if (PREC)
-          batch_bwd_streamed_ff<RB>(sxf, slf, P, R.npass, m, g, a.wpsif + R.work_off, a.wlamf + R.work_off, a.phases,
-                                    a.bops, a.blo, S.rowoff, S.red, S.grad, stage);
+          batch_bwd_streamed_ff<RB>(oxf, olf, P, R.npass, m, g, a.wpsif + R.work_off, a.wlamf + R.work_off, a.phases,
+                                    a.bops, a.blo, orows, ored, ograd, stage);
         else
-          batch_bwd_streamed<RB>(sx, sl, P, R.npass, m, g, a.wpsi + R.work_off, a.wlam + R.work_off, a.phases,
-                                 a.bops, S.rowoff, S.red, S.grad, stage);
+          batch_bwd_streamed<RB>(ox, ol, P, R.npass, m, g, a.wpsi + R.work_off, a.wlam + R.work_off, a.phases,
+                                 a.bops, orows, ored, ograd, stage);
       }
     }
     __syncthreads();
@@ -1446,11 +1546,34 @@ struct FArgs {
   const TOp* fops;
   const float2* dtab;
   const DRun* druns;
+  const float4* rtab;
+  const int2* runs;        // first tile-id entry (in the pass) and their count, a run
   int m, g;
   uint64_t ntile;          // tiles per register
   uint64_t reg_stride;     // amplitudes per register
   int nreg;
 };
+
+constexpr int kTileRuns = 48;  // runs of a pass whose tables and tile products shared memory holds
+constexpr size_t kRunBytes = sizeof(float4) * kTileRuns * (kRunTab + 2) + sizeof(RunCtx);
+
+// products of the tile-id entries of the pass's runs for the tile at tb: 16 lanes a run
+__device__ __forceinline__ void tile_products(float4* out, const DRun* entries, const int2* runs, int nrun, uint32_t tb) {
+  for (int r0 = 0; r0 < nrun; r0 += kTileThreads / 16) {
+    const int r = r0 + (int)threadIdx.x / 16;
+    float2 p0 = make_float2(1.f, 0.f), p1 = p0;
+    if (r < nrun) {
+      const int2 e = runs[r];
+      for (int k = threadIdx.x & 15; k < e.y; k += 16) run_entry(entries + e.x + k, tb, p0, p1);
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      p0 = cmulf(p0, make_float2(__shfl_xor_sync(0xffffffffu, p0.x, o), __shfl_xor_sync(0xffffffffu, p0.y, o)));
+      p1 = cmulf(p1, make_float2(__shfl_xor_sync(0xffffffffu, p1.x, o), __shfl_xor_sync(0xffffffffu, p1.y, o)));
+    }
+    if (r < nrun && (threadIdx.x & 15) == 0) out[r] = make_float4(p0.x, p0.y, p1.x, p1.y);
+  }
+}
 
 // One pass over every register of a uniform batch: CTA-strided over tiles,
 // each tile staged in shared memory once and run through all phases of the pass.
@@ -1466,6 +1589,16 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_pass(FArgs a) {
   const TPass& p = *a.pass;
   set_rows(rowoff, p, a.m);
   const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, stage, a.druns);
+  // the runs' tables, and their tile products for this tile and the one before
+  const bool held = p.nrun <= kTileRuns;
+  float4* rtile = reinterpret_cast<float4*>(stage + kStageBytes);
+  float4* rtab = rtile + 2 * kTileRuns;
+  RunCtx* rc = reinterpret_cast<RunCtx*>(rtab + kTileRuns * kRunTab);
+  const uint32_t obuf = (uint32_t)(reinterpret_cast<unsigned char*>(sbuf) - smraw);
+  const uint32_t orc = (uint32_t)(reinterpret_cast<unsigned char*>(rc) - smraw);
+  constexpr uint32_t kTileBytes = sizeof(float2) << kBatchTile;
+  if (held)
+    for (int i = threadIdx.x; i < p.nrun * kRunTab; i += blockDim.x) rtab[i] = a.rtab[kRunTab * p.run0 + i];
   const uint64_t total = a.ntile * (uint64_t)a.nreg;
   auto tile_src = [&](uint64_t t, uint64_t& tb) {
     const uint64_t r = t / a.ntile, tl = t - r * a.ntile;
@@ -1473,22 +1606,25 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_pass(FArgs a) {
     return a.state + r * a.reg_stride + tb;
   };
   uint64_t tb = 0;
-  if (blockIdx.x < total) load_tile_async(sbuf, tile_src(blockIdx.x, tb), rowoff, a.m);
+  if (blockIdx.x < total) load_tile_async(obuf, tile_src(blockIdx.x, tb), 0, a.m);
   cp_async_commit();
   int i = 0;
   for (uint64_t t = blockIdx.x; t < total; t += gridDim.x, ++i) {
-    float2* sx = sbuf + (size_t)(i & 1) * (1 << kBatchTile);
+    const uint32_t sx = obuf + (i & 1) * kTileBytes;
     const uint64_t tn = t + gridDim.x;
     if (tn < total) {
       uint64_t tbn;
-      load_tile_async(sbuf + (size_t)((i + 1) & 1) * (1 << kBatchTile), tile_src(tn, tbn), rowoff, a.m);
+      load_tile_async(obuf + ((i + 1) & 1) * kTileBytes, tile_src(tn, tbn), 0, a.m);
     }
     cp_async_commit();
+    float2* base = tile_src(t, tb);
+    float4* rt = held ? rtile + (i & 1) * kTileRuns : nullptr;
+    if (held) tile_products(rt, sp.runs, a.runs + p.run0, p.nrun, (uint32_t)tb);
+    if (threadIdx.x == 0) *rc = RunCtx{sp.runs, held ? rtab : a.rtab + kRunTab * p.run0, rt};
     cp_async_wait_prev();  // this tile's copies (all groups but the one just issued)
     __syncthreads();
-    float2* base = tile_src(t, tb);
-    run_tile_fwd<kRB, false, 2>(sx, sp.ph, p.nphase, sp.ops, a.dtab, nullptr, nullptr, sp.runs, a.m, (uint32_t)tb);
-    store_tile(sx, base, rowoff, a.m);
+    run_tile_fwd<kRB, false, 2>(sx, sp.ph, p.nphase, sp.ops, a.dtab, nullptr, nullptr, orc, 0, a.m, (uint32_t)tb);
+    store_tile(sx, base, 0, a.m);
     __syncthreads();
   }
   cp_async_wait_all();
@@ -1523,12 +1659,13 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_bwd_pass(FBArgs a) {
   for (int i = threadIdx.x; i < a.nparam; i += blockDim.x) gacc[i] = 0.0;
   set_rows(rowoff, p, a.m);
   const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage);
+  auto at = [&](const void* q) { return (uint32_t)((const unsigned char*)q - smraw); };
   for (uint64_t t = blockIdx.x; t < a.ntile; t += gridDim.x) {
     const uint64_t tb = tile_base(t, p, a.g);
-    load_tiles<true>(sx, a.wpsi + tb, sl, a.wlam + tb, rowoff, a.m);
+    load_tiles<true>(at(sx), a.wpsi + tb, at(sl), a.wlam + tb, 0, a.m);
     __syncthreads();
-    run_tile_bwd<kRB>(sx, sl, sp.ph, p.nphase, sp.ops, a.m, red, gacc, (uint32_t)tb);
-    store_tiles<true>(sx, a.wpsi + tb, sl, a.wlam + tb, rowoff, a.m);
+    run_tile_bwd<kRB>(at(sx), at(sl), sp.ph, p.nphase, sp.ops, a.m, 0, at(red), at(gacc), (uint32_t)tb);
+    store_tiles<true>(at(sx), a.wpsi + tb, at(sl), a.wlam + tb, 0, a.m);
     __syncthreads();
   }
   for (int i = threadIdx.x; i < a.nparam; i += blockDim.x) a.partials[(size_t)blockIdx.x * a.nparam + i] = gacc[i];
@@ -1598,8 +1735,11 @@ struct PrepArgs {
   TOp* bops;
   float2* dtab;
   DRun* druns;
+  const DRun* tabent;      // lane and warp entries of the runs: masks over table index bits
+  const int4* tabs;        // per run: first of them, lane entries, warp entries
+  float4* rtab;
   const double* params;
-  int nfop, nbop, ndiag, ndrun;
+  int nfop, nbop, ndiag, ndrun, nrun;
 };
 
 __device__ void gate_mat(const GSpec& gs, const double* params, double2 (&U)[4]) {
@@ -1690,6 +1830,25 @@ __global__ void k_batch_prep(PrepArgs a) {
     gate_mat(a.gspec[e.gate], a.params, U);
     e.u0 = hi_of(U[0]);
     e.u3 = hi_of(U[3]);
+  } else if (i < a.nfop + a.nbop + a.ndiag + a.ndrun + a.nrun * kRunTab) {
+    // an entry of a run's table: the products over the members whose controls hold at
+    // this lane (or warp), formed in FP64 and rounded once
+    const int k = i - a.nfop - a.nbop - a.ndiag - a.ndrun, run = k / kRunTab, at = k % kRunTab;
+    const int4 t = a.tabs[run];
+    const uint32_t bits = at < 32 ? at : at - 32;
+    const int e0 = at < 32 ? t.x : t.x + t.y, n = at < 32 ? t.y : t.z;
+    double2 p0 = make_double2(1.0, 0.0), p1 = p0;
+    for (int q = 0; q < n; ++q) {
+      const DRun& e = a.tabent[e0 + q];
+      if ((bits & e.tmask) != e.tval) continue;
+      double2 U[4];
+      gate_mat(a.gspec[e.gate], a.params, U);
+      const bool scalar = e.tq != 0xffffffffu, one = scalar && ((bits >> e.tq) & 1u);
+      p0 = zmul(p0, one ? U[3] : U[0]);
+      p1 = zmul(p1, scalar && !one ? U[0] : U[3]);
+    }
+    const float2 h0 = hi_of(p0), h1 = hi_of(p1);
+    a.rtab[k] = make_float4(h0.x, h0.y, h1.x, h1.y);
   }
 }
 
@@ -1721,6 +1880,11 @@ struct qs_batch_program {
   int ndiag = 0;
   qs::DRun* druns = nullptr;  // TK_DIAGRUN entries
   int ndrun = 0;
+  qs::DRun* tabent = nullptr;  // those formed into tables
+  int4* tabs = nullptr;
+  int2* runs = nullptr;
+  float4* rtab = nullptr;
+  int nrun = 0;
   int* counter = nullptr;
   float2* wpsi = nullptr;
   float2* wlam = nullptr;
@@ -1743,6 +1907,8 @@ struct qs_batch_program {
   std::vector<qs::TPass> host_passes;
   double* dparams = nullptr;
   int64_t dparams_n = 0;
+  // SWAP networks before and after the passes (k_bitswap), the phases' share of npass
+  std::vector<std::pair<int, int>> pre_swaps, post_swaps;
 };
 
 namespace qs {
@@ -1784,7 +1950,7 @@ static void free_program(qs_batch_program* p) {
                     cudaSetDevice(p->device) == cudaSuccess;
   void* ptrs[] = {p->regs, p->order, p->passes, p->phases, p->fops, p->bops, p->terms, p->gspec, p->fmem,
                   p->bgate, p->dmem, p->dref, p->dtab, p->counter, p->wpsi, p->wlam, p->dparams,
-                  p->flo, p->blo, p->dtlo, p->wpsif, p->wlamf, p->druns};
+                  p->flo, p->blo, p->dtlo, p->wpsif, p->wlamf, p->druns, p->tabent, p->tabs, p->runs, p->rtab};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (swap) cudaSetDevice(cur);
@@ -1838,7 +2004,9 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   std::vector<int32_t> bgate;
   std::vector<DMem> dmems;
   std::vector<DRef> drefs;
-  std::vector<DRun> druns;
+  std::vector<DRun> druns, tabent;
+  std::vector<int4> tabs;
+  std::vector<int2> runs;
   P->nreg = nreg;
   P->nq.resize(nreg);
   P->param_off.assign(nreg + 1, 0);
@@ -1906,6 +2074,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
         if (std::find(p.tbits.begin(), p.tbits.end(), qb) == p.tbits.end()) tp.gbits[ng++] = (uint8_t)qb;
       tp.phase0 = (int)phases.size();
       tp.drun0 = (int)druns.size();
+      tp.run0 = (int)runs.size();
       tp.nphase = (int)p.phases.size();
       for (const HostPhase& ph : p.phases) {
         TPhase t;
@@ -1920,6 +2089,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
         t.fop0 = (int)fops.size();
         std::vector<int> last(rb, -1);   // forward op index (in fops) open for fusion per phase bit
         int dg = -1;                     // open TK_DIAG16 table of this phase
+        int nval = 0;                    // backward ops with a gradient sum
         // TK_DIAGRUN runs of this phase (complex64 path): the op each opened,
         // its entries, the run open per phase bit and the latest run opened
         std::vector<int> run_op;
@@ -1969,6 +2139,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
               bops[q].shared = 1;
               b.shared = 1;
             }
+          if (b.gen != GEN_NONE) b.pad = (uint8_t)nval++;
           bops.push_back(b);
           bgate.push_back(g0 + gi);
           // forward op.  A diagonal gate with its target outside the phase is a
@@ -2085,24 +2256,72 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
             fmem[run_op[r]].g[0] = e.gate;
             continue;
           }
+          // entries by where their qubits lie: lane bits, warp bits, tile-id bits, several
+          const int ntb = m - rb;
+          uint32_t lanes = 0, warps = 0, tile = 0;
+          for (int k = 0; k < ntb; ++k) (k < 5 ? lanes : warps) |= 1u << t.tq[k];
+          for (int k = 0; k < ng; ++k) tile |= 1u << tp.gbits[k];
+          auto local = [&](uint32_t q, int k0) {  // register qubits as table index bits
+            uint32_t v = 0;
+            for (int k = k0; k < std::min(ntb, k0 == 0 ? 5 : ntb); ++k) v |= ((q >> t.tq[k]) & 1u) << (k - k0);
+            return v;
+          };
+          std::vector<DRun> part[4];
+          for (const DRun& e : run_ent[r]) {
+            const uint32_t q = e.tmask | (e.tq != 0xffffffffu ? 1u << e.tq : 0u);
+            const int kind = !(q & ~lanes) ? 0 : !(q & ~warps) ? 1 : !(q & ~tile) ? 2 : 3;
+            DRun f = e;
+            if (kind < 2) {
+              const int k0 = kind == 0 ? 0 : 5;
+              f.tmask = local(e.tmask, k0);
+              f.tval = local(e.tval, k0);
+              if (e.tq != 0xffffffffu) f.tq = (uint32_t)__builtin_ctz(local(1u << e.tq, k0));
+            }
+            part[kind == 2 && part[2].size() >= 255 ? 3 : kind].push_back(f);
+          }
+          bool one0 = true;
+          for (const DRun& e : run_ent[r]) {
+            const int k = gspec[e.gate].kind;
+            one0 = one0 && e.tq == 0xffffffffu &&
+                   (k == QS_GATE_SHIFT || k == QS_GATE_Z || k == QS_GATE_S || k == QS_GATE_SDG || k == QS_GATE_T ||
+                    k == QS_GATE_TDG || k == QS_GATE_I);
+          }
+          const int run = (int)runs.size() - tp.run0;
           ro.param = (int)druns.size() - tp.drun0;
-          ro.count = (uint32_t)run_ent[r].size();
-          druns.insert(druns.end(), run_ent[r].begin(), run_ent[r].end());
+          ro.count = (uint32_t)(part[2].size() + part[3].size());
+          ro.shared = (uint8_t)part[2].size();
+          ro.gen = one0 ? 1 : 0;
+          std::memcpy(&ro.cfac2, &run, sizeof(run));
+          runs.push_back(make_int2(ro.param, (int)part[2].size()));
+          tabs.push_back(make_int4((int)tabent.size(), (int)part[0].size(), (int)part[1].size(), 0));
+          for (int k = 0; k < 2; ++k) tabent.insert(tabent.end(), part[k].begin(), part[k].end());
+          for (int k = 2; k < 4; ++k) druns.insert(druns.end(), part[k].begin(), part[k].end());
         }
         t.nbop = (int)bops.size() - t.bop0;
         t.nfop = (int)fops.size() - t.fop0;
         t.nshared = 0;
         for (int q = t.bop0; q < (int)bops.size(); ++q) t.nshared += bops[q].shared ? 1 : 0;
-        if (t.nbop > kMaxPhaseOps) return fail(QS_EUNSUPPORTED, "phase with %d ops", t.nbop);
         phases.push_back(t);
         cost += (double)(1ll << n) * (1 + 0.02 * t.nbop);
       }
       tp.ndrun = (int)druns.size() - tp.drun0;
+      tp.nrun = (int)runs.size() - tp.run0;
       passes.push_back(tp);
     }
     R.cost = cost;
   }
-  for (TOp& f : fops) f.var = fwd_variant(f);
+  for (size_t i = 0; i < fops.size(); ++i) {
+    TOp& f = fops[i];
+    f.var = fwd_variant(f);
+    bool real = !precise && f.kind == TK_DENSE && !f.cmask;
+    for (int k = 0; real && k < fmem[i].count; ++k) {
+      const GSpec& gs = gspec[fmem[i].g[k]];
+      real = gs.kind == QS_GATE_H || gs.kind == QS_GATE_RY || gs.kind == QS_GATE_X || gs.kind == QS_GATE_Z ||
+             gs.kind == QS_GATE_I ||
+             (gs.kind == QS_GATE_MATRIX && gs.mat[0].y == 0 && gs.mat[1].y == 0 && gs.mat[2].y == 0 && gs.mat[3].y == 0);
+    }
+    if (real) f.var = (uint8_t)(FV_REAL + f.t);
+  }
   for (TOp& b : bops) b.var = bwd_variant(b);
   // decreasing cost order
   std::vector<int32_t> order(nreg);
@@ -2127,7 +2346,12 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   QS_TRY(upload(&P->dref, drefs));
   P->ndiag = (int)drefs.size();
   P->ndrun = (int)druns.size();
+  P->nrun = (int)runs.size();
   QS_TRY(upload(&P->druns, druns.empty() ? std::vector<DRun>(1) : druns));
+  QS_TRY(upload(&P->tabent, tabent));
+  QS_TRY(upload(&P->tabs, tabs));
+  QS_TRY(upload(&P->runs, runs));
+  QS_TRY(upload(&P->rtab, std::vector<float4>((size_t)kRunTab * runs.size())));
   QS_TRY(upload(&P->dtab, std::vector<float2>(16 * std::max<size_t>(1, drefs.size()))));
   QS_TRY(upload(&P->counter, std::vector<int>(1, 0)));
   if (work > 0 && !precise) {
@@ -2149,7 +2373,8 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   }
   P->host_passes = passes;
   if (P->fused_only) {
-    P->smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + 2 * sizeof(float2) * (1 << kBatchTile) + kStageBytes;
+    P->smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + 2 * sizeof(float2) * (1 << kBatchTile) + kStageBytes +
+              kRunBytes;
     QS_CUDA(cudaFuncSetAttribute(k_fused_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P->smem));
     int dev = 0, sms = 0, per_sm = 0;
     QS_CUDA(cudaGetDevice(&dev));
@@ -2187,12 +2412,16 @@ static int launch_prep(const qs_batch_program* P, const double* dev_params, bool
   pa.bops = P->bops;
   pa.dtab = P->dtab;
   pa.druns = P->druns;
+  pa.tabent = P->tabent;
+  pa.tabs = P->tabs;
+  pa.rtab = P->rtab;
+  pa.nrun = P->nrun;
   pa.params = dev_params;
   pa.nfop = P->nfop;
   pa.nbop = bwd ? P->nbop : 0;
   pa.ndiag = P->ndiag;
   pa.ndrun = P->ndrun;
-  const int tot = pa.nfop + pa.nbop + pa.ndiag + pa.ndrun;
+  const int tot = pa.nfop + pa.nbop + pa.ndiag + pa.ndrun + pa.nrun * kRunTab;
   if (tot > 0) {
     k_batch_prep<<<(tot + 255) / 256, 256, 0, st>>>(pa);
     QS_LAUNCHED();
@@ -2202,13 +2431,15 @@ static int launch_prep(const qs_batch_program* P, const double* dev_params, bool
 
 // ------------------------------------------------------------------ host: fused forward of one circuit
 
-// SWAP(a, b) = CX(a->b) CX(b->a) CX(a->b), each also carrying the SWAP's own controls
-static void expand_swaps(const qs_circuit* c, qs_circuit* out) {
+// SWAP(a, b) = CX(a->b) CX(b->a) CX(a->b), each also carrying the SWAP's own controls;
+// gates first .. last - 1 of c
+static void expand_swaps(const qs_circuit* c, size_t first, size_t last, qs_circuit* out) {
   out->nqubits = c->nqubits;
   out->nparams = c->nparams;
   out->mats = c->mats;
   out->gates.clear();
-  for (const qs_gate_desc& g : c->gates) {
+  for (size_t i = first; i < last; ++i) {
+    const qs_gate_desc& g = c->gates[i];
     if (g.kind != QS_GATE_SWAP) {
       out->gates.push_back(g);
       continue;
@@ -2229,6 +2460,46 @@ static void expand_swaps(const qs_circuit* c, qs_circuit* out) {
   }
 }
 
+// The tile engine's plan of a circuit: SWAP networks (uncontrolled, on disjoint
+// qubits) at its start and its end as passes of their own where that takes no more
+// passes than their controlled X gates inside the others (a pass that only moves
+// amplitudes runs at the copy rate, one that tests controls at half of it), and the
+// tile passes of what lies between.
+struct TilePlan {
+  size_t first = 0, last = 0;  // gates of the tile passes
+  std::vector<HostPass> passes;
+  qs_circuit mid;              // those gates, SWAPs expanded
+};
+
+static int plan_tiles(const qs_circuit* c, int M, TilePlan* out) {
+  const int n = c->nqubits, m = std::min(n, M);
+  const size_t ng = c->gates.size();
+  out->first = 0;
+  out->last = ng;
+  expand_swaps(c, 0, ng, &out->mid);
+  QS_TRY(plan_passes(&out->mid, n, m, kMaxPhaseOps, out->passes));
+  if (n < kBitSwapMinQubits) return QS_OK;
+  uint64_t used = 0;
+  auto network = [&](const qs_gate_desc& g) {
+    const uint64_t q = g.kind == QS_GATE_SWAP && !g.ctrl_mask ? (1ull << g.locs[0]) | (1ull << g.locs[1]) : 0;
+    if (!q || (q & used)) return false;
+    used |= q;
+    return true;
+  };
+  size_t first = 0, last = ng;
+  while (last > 0 && network(c->gates[last - 1])) --last;
+  used = 0;
+  while (first < last && network(c->gates[first])) ++first;
+  if (first == 0 && last == ng) return QS_OK;
+  TilePlan t;
+  t.first = first;
+  t.last = last;
+  expand_swaps(c, first, last, &t.mid);
+  QS_TRY(plan_passes(&t.mid, n, m, kMaxPhaseOps, t.passes));
+  if (t.passes.size() + (first > 0) + (last < ng) <= out->passes.size()) *out = t;
+  return QS_OK;
+}
+
 // the circuit's tile-engine schedule for tiles of M qubits, built once and cached
 // on the current device (a schedule built on another device is rebuilt here: its
 // tables are that device's memory)
@@ -2240,11 +2511,14 @@ static int ensure_schedule(const qs_circuit* c, int M) {
     free_program(c->fused);
     c->fused = nullptr;
   }
-  qs_circuit tmp;
-  expand_swaps(c, &tmp);
-  const qs_circuit* cp = &tmp;
+  TilePlan plan;
+  QS_TRY(plan_tiles(c, M, &plan));
+  const qs_circuit* cp = &plan.mid;
   qs_batch_program* P = new qs_batch_program();
   P->fused_only = true;
+  for (size_t i = 0; i < c->gates.size(); ++i)
+    if (i < plan.first || i >= plan.last)
+      (i < plan.first ? P->pre_swaps : P->post_swaps).emplace_back(c->gates[i].locs[0], c->gates[i].locs[1]);
   const int rc = build_program(1, &cp, nullptr, M, P);
   if (rc != QS_OK) {
     const std::string msg = qs_last_error();
@@ -2288,6 +2562,8 @@ int fused_forward(qs_state* s, const qs_circuit* c, const double* host_params, i
   a.fops = P->fops;
   a.dtab = P->dtab;
   a.druns = P->druns;
+  a.rtab = P->rtab;
+  a.runs = P->runs;
   a.m = m;
   a.g = g;
   a.ntile = 1ull << g;
@@ -2295,11 +2571,13 @@ int fused_forward(qs_state* s, const qs_circuit* c, const double* host_params, i
   a.nreg = s->nreg;
   const uint64_t tiles = a.ntile * (uint64_t)s->nreg;
   const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)P->blocks);
+  if (!P->pre_swaps.empty()) QS_TRY(launch_bitswap(a.state, n, s->nreg, P->pre_swaps, st));
   for (int64_t pi = 0; pi < P->npass; ++pi) {
     a.pass = P->passes + pi;
     k_fused_pass<<<grid, kTileThreads, P->smem, st>>>(a);
     QS_LAUNCHED();
   }
+  if (!P->post_swaps.empty()) QS_TRY(launch_bitswap(a.state, n, s->nreg, P->post_swaps, st));
   return QS_OK;
 }
 
@@ -2307,7 +2585,7 @@ void free_fused(qs_batch_program* p) { free_program(p); }
 
 int schedule_info(const qs_circuit* c, int tile_qubits, int* npasses, int* nphases) {
   QS_TRY(ensure_schedule(c, tile_qubits > 0 ? tile_qubits : kBatchTile));
-  if (npasses) *npasses = (int)c->fused->npass;
+  if (npasses) *npasses = (int)c->fused->npass + !c->fused->pre_swaps.empty() + !c->fused->post_swaps.empty();
   if (nphases) *nphases = (int)c->fused->nphase;
   return QS_OK;
 }
@@ -2317,18 +2595,31 @@ int tile_order(const qs_circuit* c, int tile_qubits, std::vector<int>& order, st
   if (M < kRowBits + kRB || M > kBatchTile) return fail(QS_EINVAL, "tile_qubits must be in %d..%d", kRowBits + kRB, kBatchTile);
   const int n = c->nqubits;
   if (n < kRowBits || n > 32) return fail(QS_EUNSUPPORTED, "%d qubits outside the tile engine's range", n);
-  qs_circuit tmp;
-  expand_swaps(c, &tmp);
-  std::vector<HostPass> hp;
-  QS_TRY(plan_passes(&tmp, n, std::min(n, M), kMaxPhaseOps, hp));
+  TilePlan plan;
+  QS_TRY(plan_tiles(c, M, &plan));
   order.clear();
   pass.clear();
-  for (size_t p = 0; p < hp.size(); ++p)
-    for (const HostPhase& ph : hp[p].phases)
+  int at = 0, p = 0;  // place in the expanded list, pass
+  auto network = [&](size_t first, size_t last) {
+    if (first == last) return;
+    for (size_t k = 0; k < 3 * (last - first); ++k) {
+      order.push_back(at++);
+      pass.push_back(p);
+    }
+    ++p;
+  };
+  network(0, plan.first);
+  const int mid = at;
+  for (const HostPass& hp : plan.passes) {
+    for (const HostPhase& ph : hp.phases)
       for (int gi : ph.gates) {
-        order.push_back(gi);
-        pass.push_back((int)p);
+        order.push_back(mid + gi);
+        pass.push_back(p);
       }
+    ++p;
+  }
+  at = mid + (int)plan.mid.gates.size();
+  network(plan.last, c->gates.size());
   return QS_OK;
 }
 
@@ -2420,6 +2711,10 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
   a.stage = stage ? 1 : 0;
   a.ntile = ntile;
   a.partials = partials;
+  auto swaps = [&](const std::vector<std::pair<int, int>>& net) -> int {  // its own inverse, on psi and lambda
+    return net.empty() ? QS_OK : launch_bitswap(wpsi, n, 2, net, st);
+  };
+  QS_TRY(swaps(P->post_swaps));
   for (int64_t pi = P->npass - 1; pi >= 0; --pi) {
     a.pass = P->passes + pi;
     k_fused_bwd_pass<<<grid, kTileThreads, smem, st>>>(a);
@@ -2621,6 +2916,7 @@ int qs_batch_run(qs_state* s, const qs_batch_program* p, const double* dev_param
   a.state = (float2*)s->data;
   a.dtab = p->dtab;
   a.druns = p->druns;
+  a.rtab = p->rtab;
   a.wpsi = p->wpsi;
   a.wlam = p->wlam;
   a.wpsif = p->wpsif;

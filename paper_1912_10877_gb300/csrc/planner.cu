@@ -32,12 +32,14 @@ bool gate_is_diagonal(const qs_circuit* c, const qs_gate_desc& g) {
 
 // greedy scan: take gates (in order) whose `fit` bits fit in `set` grown up to
 // `cap` bits, skipping (and blocking all qubits of) gates that do not fit or
-// depend on a skipped gate; at most `limit` gates are taken
-static void scan(const std::vector<int>& rem, const std::vector<uint64_t>& dep, const std::vector<uint64_t>& fit,
-                 uint64_t& set, int cap, size_t limit, std::vector<int>& taken, std::vector<int>& left) {
+// depend on a skipped gate; at most `limit` gates with a parameter are taken
+static void scan(const qs_circuit* c, const std::vector<int>& rem, const std::vector<uint64_t>& dep,
+                 const std::vector<uint64_t>& fit, uint64_t& set, int cap, size_t limit, std::vector<int>& taken,
+                 std::vector<int>& left) {
   uint64_t blocked = 0;
+  size_t params = 0;
   for (int gi : rem) {
-    if ((dep[gi] & blocked) || taken.size() >= limit) {
+    if ((dep[gi] & blocked) || params >= limit) {
       blocked |= dep[gi];
       left.push_back(gi);
       continue;
@@ -45,6 +47,7 @@ static void scan(const std::vector<int>& rem, const std::vector<uint64_t>& dep, 
     const uint64_t u = set | fit[gi];
     if (__builtin_popcountll(u) <= cap) {
       set = u;
+      params += c->gates[gi].param >= 0;
       taken.push_back(gi);
     } else {
       blocked |= dep[gi];
@@ -60,7 +63,7 @@ static std::vector<int> bits_of(uint64_t m) {
   return v;
 }
 
-int plan_passes(const qs_circuit* c, int n, int m, int max_phase_ops, std::vector<HostPass>& out, int rb) {
+int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::vector<HostPass>& out, int rb) {
   out.clear();
   if (m < kRowBits || m > n || m > kMaxTileBits)
     return fail(QS_EINVAL, "tile of %d qubits for a register of %d", m, n);
@@ -81,7 +84,7 @@ int plan_passes(const qs_circuit* c, int n, int m, int max_phase_ops, std::vecto
   while (!rem.empty()) {
     uint64_t B = seed;
     std::vector<int> taken, left;
-    scan(rem, dep, fit, B, m, (size_t)-1, taken, left);
+    scan(c, rem, dep, fit, B, m, (size_t)-1, taken, left);
     if (taken.empty()) return fail(QS_EUNSUPPORTED, "no gate fits a %d-qubit tile", m);
     for (int b = 0; __builtin_popcountll(B) < m && b < n; ++b) B |= 1ull << b;  // pad with low qubits
     HostPass P;
@@ -90,7 +93,7 @@ int plan_passes(const qs_circuit* c, int n, int m, int max_phase_ops, std::vecto
     while (!prem.empty()) {
       uint64_t R = 0;
       std::vector<int> pt, pl;
-      scan(prem, dep, fit, R, rb, (size_t)max_phase_ops, pt, pl);
+      scan(c, prem, dep, fit, R, rb, (size_t)max_phase_params, pt, pl);
       for (int b : P.tbits) {
         if (__builtin_popcountll(R) >= rb) break;
         R |= 1ull << b;
@@ -119,10 +122,10 @@ void phase_positions(const HostPass& p, const HostPhase& ph, TPhase* out, int rb
     for (int k = 0; k < rb; ++k)
       if (ph.rbits[k] == qb) inR = true;
     if (inR) {
+      out->keep[nr] = (uint16_t)((1u << l) - 1);
       out->rpos[nr++] = (uint8_t)l;
     } else {
-      out->tq[nt] = (uint8_t)qb;
-      out->tpos[nt++] = (uint8_t)l;
+      out->tq[nt++] = (uint8_t)qb;
     }
   }
   for (int j = 0; j < (1 << rb); ++j) {

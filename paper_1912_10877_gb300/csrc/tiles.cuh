@@ -16,6 +16,8 @@
 // with it.
 #pragma once
 
+#include <utility>
+
 #include "common.cuh"
 
 namespace qs {
@@ -37,7 +39,7 @@ struct TOp {
   uint8_t gen;    // backward ops: generator code (GEN_*), 0 = no parameter
   uint8_t shared; // backward ops: the parameter also appears in another op of the phase
   uint8_t var;    // forward ops: the specialised form (fwd_variant), one jump per op
-  uint8_t pad;
+  uint8_t pad;    // backward ops with a generator: their place among the phase's gradient sums
   int32_t param;  // register-local parameter index (forward TK_DIAG16: table index), -1 = none
   float cfac2;    // 2 c for U = exp(-i theta c H)
   uint32_t tmask; // controls outside the phase (register qubit bits)
@@ -59,6 +61,8 @@ struct TOp {
 // applied to the amplitudes once
 enum { TK_DENSE = 0, TK_SWAP = 1, TK_DIAG = 2, TK_RX = 3, TK_RY = 4, TK_DIAG16 = 5, TK_DIAGOUT = 6, TK_DIAGRUN = 7 };
 
+constexpr int kRunTab = 48;  // entries of a run's table: 32 lanes, then 16 warps (products for bit t = 0 and 1)
+
 struct DRun {
   uint32_t tmask, tval;  // its controls (register qubit bits), all outside the phase
   int32_t gate;          // gate spec index (the matrix is formed from the parameters on the device)
@@ -69,8 +73,8 @@ enum { GEN_NONE = 0, GEN_X = 1, GEN_Y = 2, GEN_Z = 3, GEN_P1 = 4, GEN_I = 5 };
 
 struct TPhase {
   uint8_t rpos[kRB];        // tile-local positions of the register bits (ascending; rb used)
-  uint8_t tpos[12];         // tile-local positions of the thread bits (ascending)
   uint8_t tq[12];           // register qubits of the thread bits
+  uint16_t keep[kRB];       // bits below each register bit (phase_base)
   uint16_t sroff[1 << kRB]; // swz(register offset of amplitude j): slot = swz(base) ^ sroff[j]
   int32_t fop0, nfop;       // forward ops (fused), applied in order
   int32_t bop0, nbop;       // backward ops (unfused), applied in reverse order
@@ -82,6 +86,7 @@ struct TPass {
   uint8_t gbits[32];        // register qubits of the tile-id bits (ascending)
   int32_t phase0, nphase;
   int32_t drun0, ndrun;     // the pass's TK_DIAGRUN entries
+  int32_t run0, nrun;       // the pass's TK_DIAGRUN ops
 };
 
 struct HostPhase {
@@ -96,16 +101,21 @@ struct HostPass {
 
 // Greedy commutation-aware scheduling: passes of m qubits (always containing
 // register qubits 0..4, so tile rows are contiguous), phases of exactly rb of
-// the pass's qubits.  Gates must be single-target; a non-diagonal gate's target
+// the pass's qubits with at most max_phase_params parameterised gates.  Gates must be single-target; a non-diagonal gate's target
 // lies in its phase, its controls and diagonal gates may be anywhere.  Returns
 // QS_OK or QS_EUNSUPPORTED.
-int plan_passes(const qs_circuit* c, int n, int m, int max_phase_ops, std::vector<HostPass>& out, int rb = kRB);
+int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::vector<HostPass>& out, int rb = kRB);
 
 // diagonal gates (fit in any phase: they only multiply amplitudes)
 bool gate_is_diagonal(const qs_circuit* c, const qs_gate_desc& g);
 
 // tile-local positions of a phase's register bits and thread bits
 void phase_positions(const HostPass& p, const HostPhase& ph, TPhase* out, int rb = kRB);
+
+// SWAP gates on disjoint qubit pairs as one pass over nreg complex64 registers of n
+// qubits (bitswap.cu)
+constexpr int kBitSwapMinQubits = 16;
+int launch_bitswap(float2* psi, int n, int nreg, const std::vector<std::pair<int, int>>& swaps, cudaStream_t st);
 
 // swizzled shared-memory slot of tile-local amplitude l (spreads the 8-byte
 // accesses of a half-warp over all banks for the phase patterns used here).
