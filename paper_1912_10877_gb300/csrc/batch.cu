@@ -21,13 +21,16 @@
 #include <cstddef>
 #include <cstring>
 #include <numeric>
+#include <unordered_map>
 
 #include "tiles.cuh"
 
 namespace qs {
 
 constexpr int kMaxRegParams = 2048;
-constexpr int kMaxPhaseOps = 64;   // gates with a parameter in a phase (its gradient sums)
+constexpr int kMaxPhaseOps = 64;    // gates with a parameter in a phase
+constexpr int kMaxPhaseVals = 128;  // sums of its backward ops
+constexpr int kMaxRun = 4;          // gates of a fused run
 constexpr int kBatchTile = kMaxTileBits;
 
 struct GSpec {           // one circuit gate of one register
@@ -37,9 +40,10 @@ struct GSpec {           // one circuit gate of one register
   double2 mat[4];        // MATRIX gates (1 target)
 };
 
-struct FMem {            // members of a fused forward op (applied in order)
+struct FMem {            // members of a fused op (applied in order)
   int32_t count;
-  int32_t g[4];          // global GSpec indices
+  int32_t g[kMaxRun];    // global GSpec indices
+  int32_t rec0;          // backward: first of its GMem records (TK_RUN), else -1
 };
 
 struct BReg {
@@ -71,6 +75,7 @@ struct BArgs {
   const TPhase* phases;
   const TOp* fops;
   const TOp* bops;
+  const GMem* gmem;
   const float2* dtab;    // TK_DIAG16 factor tables
   const DRun* druns;     // TK_DIAGRUN entries
   const float4* rtab;    // TK_DIAGRUN tables (kRunTab a run)
@@ -186,34 +191,44 @@ __device__ __forceinline__ void op_fwd_c(float2 (&x)[1 << RB], const TOp& op, co
   }
 }
 
-template <int RB, int T, bool COMP>
-__device__ __forceinline__ void op_fwd_k(float2 (&x)[1 << RB], const TOp& op, const float2* lo) {
-  if (COMP) {
-    if (op.kind == TK_SWAP) op_fwd<RB, T, TK_SWAP, true>(x, op);
-    else if (op.cmask == 0) {
-      if (op.kind == TK_DIAG) op_fwd_c<RB, T, TK_DIAG, false>(x, op, lo);
-      else op_fwd_c<RB, T, TK_DENSE, false>(x, op, lo);
-    } else {
-      if (op.kind == TK_DIAG) op_fwd_c<RB, T, TK_DIAG, true>(x, op, lo);
-      else op_fwd_c<RB, T, TK_DENSE, true>(x, op, lo);
+// A run's 2x2 with X on the same bit, before it (PRE) or after, where the X is
+// controlled: C >= 0: by phase bit C; else on every pair if `on`.  The X renames the
+// inputs or outputs of the pairs it acts on.
+template <int RB, int T, int C, bool PRE>
+__device__ __forceinline__ void op_fwd_x(float2 (&x)[1 << RB], const TOp& op, bool on) {
+  if constexpr (T < RB && C < RB && C != T) {
+    const bool sw = C < 0 && on;
+    constexpr int P = PRE ? 1 : 2;  // columns or rows trade places
+    const float2 u0 = sw ? op.u[P] : op.u[0], u1 = sw ? op.u[P ^ 1] : op.u[1];
+    const float2 u2 = sw ? op.u[P ^ 2] : op.u[2], u3 = sw ? op.u[P ^ 3] : op.u[3];
+#pragma unroll
+    for (int j = 0; j < (1 << RB); ++j) {
+      if (j & (1 << T)) continue;
+      const bool ren = C >= 0 && ((j >> (C < 0 ? 0 : C)) & 1);
+      const int k = j | (1 << T), ja = PRE && ren ? k : j, jb = PRE && ren ? j : k;
+      const float2 a = x[ja], b = x[jb];
+      const float2 na = cmaf(u1, b, cmulf(u0, a)), nb = cmaf(u3, b, cmulf(u2, a));
+      x[!PRE && ren ? k : j] = na;
+      x[!PRE && ren ? j : k] = nb;
     }
-    return;
   }
-  const bool one0 = op.u[0].x == 1.f && op.u[0].y == 0.f;  // uniform across the CTA
-  if (op.kind == TK_SWAP) op_fwd<RB, T, TK_SWAP, true>(x, op);
-  else if (op.cmask == 0) {
-    if (op.kind == TK_DIAG) {
-      if (one0) op_fwd<RB, T, TK_DIAGB, false>(x, op);
-      else op_fwd<RB, T, TK_DIAG, false>(x, op);
-    } else {
-      op_fwd<RB, T, TK_DENSE, false>(x, op);
-    }
-  } else {
-    if (op.kind == TK_DIAG) {
-      if (one0) op_fwd<RB, T, TK_DIAGB, true>(x, op);
-      else op_fwd<RB, T, TK_DIAG, true>(x, op);
-    } else {
-      op_fwd<RB, T, TK_DENSE, true>(x, op);
+}
+template <int RB, int T, int C, bool PRE>
+__device__ __forceinline__ void op_fwd_x_c(float2 (&x)[1 << RB], const TOp& op, const float2* lo, bool on) {
+  if constexpr (T < RB && C < RB && C != T) {
+    const bool sw = C < 0 && on;
+    constexpr int P = PRE ? 1 : 2;
+    const float2 u0 = sw ? op.u[P] : op.u[0], u1 = sw ? op.u[P ^ 1] : op.u[1];
+    const float2 u2 = sw ? op.u[P ^ 2] : op.u[2], u3 = sw ? op.u[P ^ 3] : op.u[3];
+    const float2 w0 = lo[sw ? P : 0], w1 = lo[sw ? P ^ 1 : 1], w2 = lo[sw ? P ^ 2 : 2], w3 = lo[sw ? P ^ 3 : 3];
+#pragma unroll
+    for (int j = 0; j < (1 << RB); ++j) {
+      if (j & (1 << T)) continue;
+      const bool ren = C >= 0 && ((j >> (C < 0 ? 0 : C)) & 1);
+      const int k = j | (1 << T), ja = PRE && ren ? k : j, jb = PRE && ren ? j : k;
+      const float2 na = cf_dot2(x[ja], u0, w0, x[jb], u1, w1), nb = cf_dot2(x[ja], u2, w2, x[jb], u3, w3);
+      x[!PRE && ren ? k : j] = na;
+      x[!PRE && ren ? j : k] = nb;
     }
   }
 }
@@ -302,9 +317,10 @@ __device__ __forceinline__ void diag_run(float2 (&x)[1 << RB], const TOp& op, co
 // 2 + t controlled swap, 6 + t / 10 + t diagonal without / with phase-local
 // controls, 14 + t / 18 + t dense without / with them (t: target phase bit),
 // 22 a run of diagonal gates (TK_DIAGRUN), 23 + t dense and real without controls (H:
-// half the multiply-adds)
+// half the multiply-adds), 27 + 10 t + (0, or 1 + control bit, then the
+// same with the X before) TK_DENSEX
 enum { FV_DIAGOUT = 0, FV_DIAG16 = 1, FV_SWAP = 2, FV_DIAG = 6, FV_DIAGC = 10, FV_DENSE = 14, FV_DENSEC = 18,
-       FV_DIAGRUN = 22, FV_REAL = 23 };
+       FV_DIAGRUN = 22, FV_REAL = 23, FV_DENSEX = 27 };
 
 template <int RB, int T, int KIND, bool CTRL, bool COMP>
 __device__ __forceinline__ void fwd_form(float2 (&x)[1 << RB], const TOp& op, const float2* lo) {
@@ -357,13 +373,43 @@ __device__ __forceinline__ void apply_fwd_var(float2 (&x)[1 << RB], const TOp& o
   }
 }
 
+// TK_DENSEX ops; on: the controls outside the phase hold
 template <int RB, bool COMP>
-__device__ __forceinline__ void apply_fwd(float2 (&x)[1 << RB], const TOp& op, const float2* lo) {
-  switch (op.t) {
-    case 0: op_fwd_k<RB, 0, COMP>(x, op, lo); break;
-    case 1: op_fwd_k<RB, 1, COMP>(x, op, lo); break;
-    case 2: if constexpr (RB > 2) op_fwd_k<RB, 2, COMP>(x, op, lo); break;
-    default: if constexpr (RB > 3) op_fwd_k<RB, 3, COMP>(x, op, lo); break;
+__device__ __forceinline__ void apply_densex(float2 (&x)[1 << RB], const TOp& op, const float2* lo, bool on) {
+  switch (op.var) {
+    case FV_DENSEX + 0: if constexpr (COMP) op_fwd_x_c<RB, 0, -1, false>(x, op, lo, on); else op_fwd_x<RB, 0, -1, false>(x, op, on); break;
+    case FV_DENSEX + 2: if constexpr (COMP) op_fwd_x_c<RB, 0, 1, false>(x, op, lo, on); else op_fwd_x<RB, 0, 1, false>(x, op, on); break;
+    case FV_DENSEX + 3: if constexpr (COMP) op_fwd_x_c<RB, 0, 2, false>(x, op, lo, on); else op_fwd_x<RB, 0, 2, false>(x, op, on); break;
+    case FV_DENSEX + 4: if constexpr (COMP) op_fwd_x_c<RB, 0, 3, false>(x, op, lo, on); else op_fwd_x<RB, 0, 3, false>(x, op, on); break;
+    case FV_DENSEX + 5: if constexpr (COMP) op_fwd_x_c<RB, 0, -1, true>(x, op, lo, on); else op_fwd_x<RB, 0, -1, true>(x, op, on); break;
+    case FV_DENSEX + 7: if constexpr (COMP) op_fwd_x_c<RB, 0, 1, true>(x, op, lo, on); else op_fwd_x<RB, 0, 1, true>(x, op, on); break;
+    case FV_DENSEX + 8: if constexpr (COMP) op_fwd_x_c<RB, 0, 2, true>(x, op, lo, on); else op_fwd_x<RB, 0, 2, true>(x, op, on); break;
+    case FV_DENSEX + 9: if constexpr (COMP) op_fwd_x_c<RB, 0, 3, true>(x, op, lo, on); else op_fwd_x<RB, 0, 3, true>(x, op, on); break;
+    case FV_DENSEX + 10: if constexpr (COMP) op_fwd_x_c<RB, 1, -1, false>(x, op, lo, on); else op_fwd_x<RB, 1, -1, false>(x, op, on); break;
+    case FV_DENSEX + 11: if constexpr (COMP) op_fwd_x_c<RB, 1, 0, false>(x, op, lo, on); else op_fwd_x<RB, 1, 0, false>(x, op, on); break;
+    case FV_DENSEX + 13: if constexpr (COMP) op_fwd_x_c<RB, 1, 2, false>(x, op, lo, on); else op_fwd_x<RB, 1, 2, false>(x, op, on); break;
+    case FV_DENSEX + 14: if constexpr (COMP) op_fwd_x_c<RB, 1, 3, false>(x, op, lo, on); else op_fwd_x<RB, 1, 3, false>(x, op, on); break;
+    case FV_DENSEX + 15: if constexpr (COMP) op_fwd_x_c<RB, 1, -1, true>(x, op, lo, on); else op_fwd_x<RB, 1, -1, true>(x, op, on); break;
+    case FV_DENSEX + 16: if constexpr (COMP) op_fwd_x_c<RB, 1, 0, true>(x, op, lo, on); else op_fwd_x<RB, 1, 0, true>(x, op, on); break;
+    case FV_DENSEX + 18: if constexpr (COMP) op_fwd_x_c<RB, 1, 2, true>(x, op, lo, on); else op_fwd_x<RB, 1, 2, true>(x, op, on); break;
+    case FV_DENSEX + 19: if constexpr (COMP) op_fwd_x_c<RB, 1, 3, true>(x, op, lo, on); else op_fwd_x<RB, 1, 3, true>(x, op, on); break;
+    case FV_DENSEX + 20: if constexpr (COMP) op_fwd_x_c<RB, 2, -1, false>(x, op, lo, on); else op_fwd_x<RB, 2, -1, false>(x, op, on); break;
+    case FV_DENSEX + 21: if constexpr (COMP) op_fwd_x_c<RB, 2, 0, false>(x, op, lo, on); else op_fwd_x<RB, 2, 0, false>(x, op, on); break;
+    case FV_DENSEX + 22: if constexpr (COMP) op_fwd_x_c<RB, 2, 1, false>(x, op, lo, on); else op_fwd_x<RB, 2, 1, false>(x, op, on); break;
+    case FV_DENSEX + 24: if constexpr (COMP) op_fwd_x_c<RB, 2, 3, false>(x, op, lo, on); else op_fwd_x<RB, 2, 3, false>(x, op, on); break;
+    case FV_DENSEX + 25: if constexpr (COMP) op_fwd_x_c<RB, 2, -1, true>(x, op, lo, on); else op_fwd_x<RB, 2, -1, true>(x, op, on); break;
+    case FV_DENSEX + 26: if constexpr (COMP) op_fwd_x_c<RB, 2, 0, true>(x, op, lo, on); else op_fwd_x<RB, 2, 0, true>(x, op, on); break;
+    case FV_DENSEX + 27: if constexpr (COMP) op_fwd_x_c<RB, 2, 1, true>(x, op, lo, on); else op_fwd_x<RB, 2, 1, true>(x, op, on); break;
+    case FV_DENSEX + 29: if constexpr (COMP) op_fwd_x_c<RB, 2, 3, true>(x, op, lo, on); else op_fwd_x<RB, 2, 3, true>(x, op, on); break;
+    case FV_DENSEX + 30: if constexpr (COMP) op_fwd_x_c<RB, 3, -1, false>(x, op, lo, on); else op_fwd_x<RB, 3, -1, false>(x, op, on); break;
+    case FV_DENSEX + 31: if constexpr (COMP) op_fwd_x_c<RB, 3, 0, false>(x, op, lo, on); else op_fwd_x<RB, 3, 0, false>(x, op, on); break;
+    case FV_DENSEX + 32: if constexpr (COMP) op_fwd_x_c<RB, 3, 1, false>(x, op, lo, on); else op_fwd_x<RB, 3, 1, false>(x, op, on); break;
+    case FV_DENSEX + 33: if constexpr (COMP) op_fwd_x_c<RB, 3, 2, false>(x, op, lo, on); else op_fwd_x<RB, 3, 2, false>(x, op, on); break;
+    case FV_DENSEX + 35: if constexpr (COMP) op_fwd_x_c<RB, 3, -1, true>(x, op, lo, on); else op_fwd_x<RB, 3, -1, true>(x, op, on); break;
+    case FV_DENSEX + 36: if constexpr (COMP) op_fwd_x_c<RB, 3, 0, true>(x, op, lo, on); else op_fwd_x<RB, 3, 0, true>(x, op, on); break;
+    case FV_DENSEX + 37: if constexpr (COMP) op_fwd_x_c<RB, 3, 1, true>(x, op, lo, on); else op_fwd_x<RB, 3, 1, true>(x, op, on); break;
+    case FV_DENSEX + 38: if constexpr (COMP) op_fwd_x_c<RB, 3, 2, true>(x, op, lo, on); else op_fwd_x<RB, 3, 2, true>(x, op, on); break;
+    default: break;
   }
 }
 
@@ -389,25 +435,44 @@ __device__ __forceinline__ float op_bwd(float2 (&x)[1 << RB], float2 (&l)[1 << R
   return acc;
 }
 
-template <int RB, int T, bool CTRL>
-__device__ __forceinline__ float op_bwd_c(float2 (&x)[1 << RB], float2 (&l)[1 << RB], const TOp& op) {
-  switch (op.gen) {
-    case GEN_X: return op_bwd<RB, T, TK_RX, 2, CTRL>(x, l, op, 0.f, 0.f);
-    case GEN_Y: return op_bwd<RB, T, TK_RY, 3, CTRL>(x, l, op, 0.f, 0.f);
-    case GEN_Z: return op_bwd<RB, T, TK_DIAG, 1, CTRL>(x, l, op, 1.f, -1.f);
-    case GEN_P1: return op_bwd<RB, T, TK_DIAG, 1, CTRL>(x, l, op, 0.f, 1.f);
-    default: return op_bwd<RB, T, TK_DIAG, 1, CTRL>(x, l, op, 1.f, 1.f);  // GEN_I
+// A TK_RUN op.  With (a, b) the pair at the end of the run (an X after it undone: the
+// pair swapped where it acted), the thread's shares of Im conj(l_a) x_a, Im conj(l_b) x_b,
+// Im<l|X|x>, Im<l|Y|x> to v; then the run's U^dagger (and an X before it undone: the
+// outputs swapped).  22 multiply-adds an amplitude for the whole run, where Rz Rx Rz gate
+// by gate took 32, three dispatches and three sums over the warp, and the X a fourth.
+template <int RB, int T, int C, bool PRE>
+__device__ __forceinline__ void op_bwd_run(float2 (&x)[1 << RB], float2 (&l)[1 << RB], const TOp& op, bool on,
+                                           float (&v)[4]) {
+  if constexpr (T < RB && C < RB && C != T) {
+    const bool sw = C < 0 && on;
+    constexpr int P = PRE ? 2 : 1;  // the outputs' rows or the inputs' columns trade places
+    const float2 u0 = sw ? op.u[P] : op.u[0], u1 = sw ? op.u[P ^ 1] : op.u[1];
+    const float2 u2 = sw ? op.u[P ^ 2] : op.u[2], u3 = sw ? op.u[P ^ 3] : op.u[3];
+    float va = 0.f, vb = 0.f, vx = 0.f, vy = 0.f;
+#pragma unroll
+    for (int j = 0; j < (1 << RB); ++j) {
+      if (j & (1 << T)) continue;
+      const bool ren = C >= 0 && ((j >> (C < 0 ? 0 : C)) & 1);
+      const int k = j | (1 << T), ja = !PRE && ren ? k : j, jb = !PRE && ren ? j : k;
+      const float2 xa = x[ja], xb = x[jb], la = l[ja], lb = l[jb];
+      va = fmaf(la.x, xa.y, fmaf(-la.y, xa.x, va));
+      vb = fmaf(lb.x, xb.y, fmaf(-lb.y, xb.x, vb));
+      vx = fmaf(la.x, xb.y, fmaf(-la.y, xb.x, vx));
+      vx = fmaf(lb.x, xa.y, fmaf(-lb.y, xa.x, vx));
+      vy = fmaf(lb.x, xa.x, fmaf(lb.y, xa.y, vy));
+      vy = fmaf(-la.x, xb.x, fmaf(-la.y, xb.y, vy));
+      const int oa = PRE && ren ? k : j, ob = PRE && ren ? j : k;
+      x[oa] = cmaf(u1, xb, cmulf(u0, xa));
+      x[ob] = cmaf(u3, xb, cmulf(u2, xa));
+      l[oa] = cmaf(u1, lb, cmulf(u0, la));
+      l[ob] = cmaf(u3, lb, cmulf(u2, la));
+    }
+    const bool neg = !PRE && sw;
+    v[0] = neg ? vb : va;
+    v[1] = neg ? va : vb;
+    v[2] = vx;
+    v[3] = neg ? -vy : vy;
   }
-}
-
-template <int RB, int T>
-__device__ __forceinline__ float op_bwd_t(float2 (&x)[1 << RB], float2 (&l)[1 << RB], const TOp& op) {
-  if (op.gen == GEN_NONE) {
-    if (op.kind == TK_SWAP) return op_bwd<RB, T, TK_SWAP, 0, true>(x, l, op, 0.f, 0.f);
-    if (op.kind == TK_DIAG) return op_bwd<RB, T, TK_DIAG, 0, true>(x, l, op, 0.f, 0.f);
-    return op_bwd<RB, T, TK_DENSE, 0, true>(x, l, op, 0.f, 0.f);
-  }
-  return op.cmask ? op_bwd_c<RB, T, true>(x, l, op) : op_bwd_c<RB, T, false>(x, l, op);
 }
 
 // backward op forms (TOp::var = 13 t + form): 0 controlled swap, 1 / 2 diagonal /
@@ -493,13 +558,47 @@ __device__ __forceinline__ float apply_bwd_var(float2 (&x)[1 << RB], float2 (&l)
   }
 }
 
+// TK_RUN forms: BV_RUN + 10 t + (0, or 1 + control bit of the X; then the same with the X
+// before the run)
+constexpr int BV_RUN = 64;
+
 template <int RB>
-__device__ __forceinline__ float apply_bwd(float2 (&x)[1 << RB], float2 (&l)[1 << RB], const TOp& op) {
-  switch (op.t) {
-    case 0: return op_bwd_t<RB, 0>(x, l, op);
-    case 1: return op_bwd_t<RB, 1>(x, l, op);
-    case 2: if constexpr (RB > 2) return op_bwd_t<RB, 2>(x, l, op); return 0.f;
-    default: if constexpr (RB > 3) return op_bwd_t<RB, 3>(x, l, op); return 0.f;
+__device__ __forceinline__ void apply_bwd_run(float2 (&x)[1 << RB], float2 (&l)[1 << RB], const TOp& op, bool on,
+                                              float (&v)[4]) {
+  switch (op.var) {
+    case BV_RUN + 0: op_bwd_run<RB, 0, -1, false>(x, l, op, on, v); break;
+    case BV_RUN + 2: op_bwd_run<RB, 0, 1, false>(x, l, op, on, v); break;
+    case BV_RUN + 3: op_bwd_run<RB, 0, 2, false>(x, l, op, on, v); break;
+    case BV_RUN + 4: op_bwd_run<RB, 0, 3, false>(x, l, op, on, v); break;
+    case BV_RUN + 5: op_bwd_run<RB, 0, -1, true>(x, l, op, on, v); break;
+    case BV_RUN + 7: op_bwd_run<RB, 0, 1, true>(x, l, op, on, v); break;
+    case BV_RUN + 8: op_bwd_run<RB, 0, 2, true>(x, l, op, on, v); break;
+    case BV_RUN + 9: op_bwd_run<RB, 0, 3, true>(x, l, op, on, v); break;
+    case BV_RUN + 10: op_bwd_run<RB, 1, -1, false>(x, l, op, on, v); break;
+    case BV_RUN + 11: op_bwd_run<RB, 1, 0, false>(x, l, op, on, v); break;
+    case BV_RUN + 13: op_bwd_run<RB, 1, 2, false>(x, l, op, on, v); break;
+    case BV_RUN + 14: op_bwd_run<RB, 1, 3, false>(x, l, op, on, v); break;
+    case BV_RUN + 15: op_bwd_run<RB, 1, -1, true>(x, l, op, on, v); break;
+    case BV_RUN + 16: op_bwd_run<RB, 1, 0, true>(x, l, op, on, v); break;
+    case BV_RUN + 18: op_bwd_run<RB, 1, 2, true>(x, l, op, on, v); break;
+    case BV_RUN + 19: op_bwd_run<RB, 1, 3, true>(x, l, op, on, v); break;
+    case BV_RUN + 20: op_bwd_run<RB, 2, -1, false>(x, l, op, on, v); break;
+    case BV_RUN + 21: op_bwd_run<RB, 2, 0, false>(x, l, op, on, v); break;
+    case BV_RUN + 22: op_bwd_run<RB, 2, 1, false>(x, l, op, on, v); break;
+    case BV_RUN + 24: op_bwd_run<RB, 2, 3, false>(x, l, op, on, v); break;
+    case BV_RUN + 25: op_bwd_run<RB, 2, -1, true>(x, l, op, on, v); break;
+    case BV_RUN + 26: op_bwd_run<RB, 2, 0, true>(x, l, op, on, v); break;
+    case BV_RUN + 27: op_bwd_run<RB, 2, 1, true>(x, l, op, on, v); break;
+    case BV_RUN + 29: op_bwd_run<RB, 2, 3, true>(x, l, op, on, v); break;
+    case BV_RUN + 30: op_bwd_run<RB, 3, -1, false>(x, l, op, on, v); break;
+    case BV_RUN + 31: op_bwd_run<RB, 3, 0, false>(x, l, op, on, v); break;
+    case BV_RUN + 32: op_bwd_run<RB, 3, 1, false>(x, l, op, on, v); break;
+    case BV_RUN + 33: op_bwd_run<RB, 3, 2, false>(x, l, op, on, v); break;
+    case BV_RUN + 35: op_bwd_run<RB, 3, -1, true>(x, l, op, on, v); break;
+    case BV_RUN + 36: op_bwd_run<RB, 3, 0, true>(x, l, op, on, v); break;
+    case BV_RUN + 37: op_bwd_run<RB, 3, 1, true>(x, l, op, on, v); break;
+    case BV_RUN + 38: op_bwd_run<RB, 3, 2, true>(x, l, op, on, v); break;
+    default: break;
   }
 }
 
@@ -624,6 +723,68 @@ __device__ __forceinline__ float op_bwd_ff(ffc (&x)[1 << RB], ffc (&l)[1 << RB],
   return acc;
 }
 
+// op_bwd_run with the double-float uncompute (sums from the hi parts)
+template <int RB, int T, int C, bool PRE>
+__device__ __forceinline__ void op_bwd_run_ff(ffc (&x)[1 << RB], ffc (&l)[1 << RB], const TOp& op, const float2* lo,
+                                              bool on, float (&v)[4]) {
+  if constexpr (T < RB && C < RB && C != T) {
+    const bool sw = C < 0 && on;
+    constexpr int P = PRE ? 2 : 1;
+    const float2 u[4] = {sw ? op.u[P] : op.u[0], sw ? op.u[P ^ 1] : op.u[1], sw ? op.u[P ^ 2] : op.u[2],
+                         sw ? op.u[P ^ 3] : op.u[3]};
+    const float2 w[4] = {lo[sw ? P : 0], lo[sw ? P ^ 1 : 1], lo[sw ? P ^ 2 : 2], lo[sw ? P ^ 3 : 3]};
+    float va = 0.f, vb = 0.f, vx = 0.f, vy = 0.f;
+#pragma unroll
+    for (int j = 0; j < (1 << RB); ++j) {
+      if (j & (1 << T)) continue;
+      const bool ren = C >= 0 && ((j >> (C < 0 ? 0 : C)) & 1);
+      const int k = j | (1 << T), ja = !PRE && ren ? k : j, jb = !PRE && ren ? j : k;
+      ffc xa = x[ja], xb = x[jb], la = l[ja], lb = l[jb];
+      va = fmaf(la.h.x, xa.h.y, fmaf(-la.h.y, xa.h.x, va));
+      vb = fmaf(lb.h.x, xb.h.y, fmaf(-lb.h.y, xb.h.x, vb));
+      vx = fmaf(la.h.x, xb.h.y, fmaf(-la.h.y, xb.h.x, vx));
+      vx = fmaf(lb.h.x, xa.h.y, fmaf(-lb.h.y, xa.h.x, vx));
+      vy = fmaf(lb.h.x, xa.h.x, fmaf(lb.h.y, xa.h.y, vy));
+      vy = fmaf(-la.h.x, xb.h.x, fmaf(-la.h.y, xb.h.y, vy));
+      pair_apply_ff<TK_DENSE>(xa, xb, u, w);
+      pair_apply_ff<TK_DENSE>(la, lb, u, w);
+      const int oa = PRE && ren ? k : j, ob = PRE && ren ? j : k;
+      x[oa] = xa; x[ob] = xb;
+      l[oa] = la; l[ob] = lb;
+    }
+    const bool neg = !PRE && sw;
+    v[0] = neg ? vb : va;
+    v[1] = neg ? va : vb;
+    v[2] = vx;
+    v[3] = neg ? -vy : vy;
+  }
+}
+template <int RB>
+__device__ __forceinline__ void apply_bwd_run_ff(ffc (&x)[1 << RB], ffc (&l)[1 << RB], const TOp& op, const float2* lo,
+                                                 bool on, float (&v)[4]) {
+  switch (op.var) {
+    case BV_RUN + 0: op_bwd_run_ff<RB, 0, -1, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 2: op_bwd_run_ff<RB, 0, 1, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 3: op_bwd_run_ff<RB, 0, 2, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 5: op_bwd_run_ff<RB, 0, -1, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 7: op_bwd_run_ff<RB, 0, 1, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 8: op_bwd_run_ff<RB, 0, 2, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 10: op_bwd_run_ff<RB, 1, -1, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 11: op_bwd_run_ff<RB, 1, 0, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 13: op_bwd_run_ff<RB, 1, 2, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 15: op_bwd_run_ff<RB, 1, -1, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 16: op_bwd_run_ff<RB, 1, 0, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 18: op_bwd_run_ff<RB, 1, 2, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 20: op_bwd_run_ff<RB, 2, -1, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 21: op_bwd_run_ff<RB, 2, 0, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 22: op_bwd_run_ff<RB, 2, 1, false>(x, l, op, lo, on, v); break;
+    case BV_RUN + 25: op_bwd_run_ff<RB, 2, -1, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 26: op_bwd_run_ff<RB, 2, 0, true>(x, l, op, lo, on, v); break;
+    case BV_RUN + 27: op_bwd_run_ff<RB, 2, 1, true>(x, l, op, lo, on, v); break;
+    default: break;
+  }
+}
+
 template <int RB, int T, bool CTRL>
 __device__ __forceinline__ float op_bwd_ff_c(ffc (&x)[1 << RB], ffc (&l)[1 << RB], const TOp& op, const float2* lo) {
   switch (op.gen) {
@@ -671,7 +832,7 @@ __device__ __forceinline__ T* sh(uint32_t off) {
 
 struct BShared {
   double grad[kMaxRegParams];
-  float red[kMaxPhaseOps * kWarps];
+  float red[kMaxPhaseVals * kWarps];
   double lred[kWarps];
   uint32_t rowoff[1 << (kMaxTileBits - kRowBits)];  // register offset of each 32-amplitude tile row (current pass)
   RunCtx rc;
@@ -848,7 +1009,7 @@ __device__ __forceinline__ TOp load_op(const TOp* p) {
   r.gen = (uint8_t)(a.y & 0xffu);
   r.shared = (uint8_t)((a.y >> 8) & 0xffu);
   r.var = (uint8_t)((a.y >> 16) & 0xffu);
-  r.pad = (uint8_t)(a.y >> 24);
+  r.val = (uint8_t)(a.y >> 24);
   r.param = (int32_t)a.z;
   r.cfac2 = __uint_as_float(a.w);
   r.tmask = b.x;
@@ -872,18 +1033,19 @@ __device__ __forceinline__ TOp load_op(const TOp* p) {
 // indices rebased to the pass's first op.  A pass larger than the staging
 // area keeps reading global memory.
 constexpr int kStagePhases = 32;
-constexpr int kStageOps = 512;
-constexpr int kStageRuns = 256;
+constexpr int kStageOps = 480;
+constexpr int kStageRecs = 256;  // forward: TK_DIAGRUN entries; backward: GMem records
 static_assert(sizeof(TOp) == 64 && sizeof(TOp) % 16 == 0, "TOp is copied as 16-byte words");
-static_assert(sizeof(DRun) == 32, "DRun is copied as 16-byte words");
+static_assert(sizeof(DRun) == 32 && sizeof(GMem) == 32, "records are copied as 16-byte words");
 constexpr size_t kStagePhaseBytes = (sizeof(TPhase) * kStagePhases + 15) & ~size_t(15);
-constexpr size_t kStageBytes = kStagePhaseBytes + sizeof(TOp) * kStageOps + sizeof(DRun) * kStageRuns;
+constexpr size_t kStageBytes = kStagePhaseBytes + sizeof(TOp) * kStageOps + sizeof(DRun) * kStageRecs;
 
 struct StagedPass {
   const TPhase* ph;  // the pass's first phase
   const TOp* ops;    // op table the phases index
   int first;         // index of ops[0] in the global op table (0 when not staged)
   const DRun* runs;  // the pass's TK_DIAGRUN entries (forward)
+  const GMem* mem;   // GMem records the ops index (backward)
 };
 
 // FWD: the forward ops (fop0 / nfop), else the backward ops (bop0 / nbop).
@@ -891,10 +1053,10 @@ struct StagedPass {
 // calls this (it ends with a barrier when it copies).
 template <bool FWD>
 __device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp* ops, unsigned char* buf,
-                                 const DRun* druns = nullptr) {
-  StagedPass r{phases + p.phase0, ops, 0, druns ? druns + p.drun0 : nullptr};
+                                 const DRun* druns, const GMem* gmem) {
+  StagedPass r{phases + p.phase0, ops, 0, FWD ? druns + p.drun0 : nullptr, gmem};
   if (!buf || p.nphase <= 0 || p.nphase > kStagePhases) return r;
-  if (FWD && druns && p.ndrun > kStageRuns) return r;
+  if (FWD && p.ndrun > kStageRecs) return r;
   const TPhase& f0 = phases[p.phase0];
   const TPhase& fl = phases[p.phase0 + p.nphase - 1];
   const int first = FWD ? f0.fop0 : f0.bop0;
@@ -912,16 +1074,14 @@ __device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp
     else q.bop0 -= first;
     sph[threadIdx.x] = q;
   }
-  const DRun* runs = nullptr;
-  if (FWD && druns) {
-    DRun* srun = reinterpret_cast<DRun*>(buf + kStagePhaseBytes + sizeof(TOp) * kStageOps);
-    const uint4* rs = reinterpret_cast<const uint4*>(druns + p.drun0);
-    uint4* rd = reinterpret_cast<uint4*>(srun);
-    for (int i = threadIdx.x; i < p.ndrun * 2; i += blockDim.x) rd[i] = rs[i];
-    runs = srun;
-  }
+  // a pass with more GMem records than the area holds reads those from global memory
+  uint4* rd = reinterpret_cast<uint4*>(buf + kStagePhaseBytes + sizeof(TOp) * kStageOps);
+  const bool recs = FWD || p.nmem <= kStageRecs;
+  const uint4* rs = FWD ? reinterpret_cast<const uint4*>(druns + p.drun0) : reinterpret_cast<const uint4*>(gmem + p.mem0);
+  for (int i = threadIdx.x; recs && i < (FWD ? p.ndrun : p.nmem) * 2; i += blockDim.x) rd[i] = rs[i];
   __syncthreads();
-  return StagedPass{sph, sop, first, runs};
+  if (FWD) return StagedPass{sph, sop, first, reinterpret_cast<const DRun*>(rd), nullptr};
+  return StagedPass{sph, sop, first, nullptr, recs ? reinterpret_cast<const GMem*>(rd) - p.mem0 : gmem};
 }
 
 // out-of-phase diagonal gate with phase-local controls: x_j *= f where (j & cm) == cv
@@ -955,7 +1115,12 @@ __device__ __forceinline__ void phase_fwd_body(float2* sm, const TPhase* php, co
     for (int o = 0; o < ph.nfop; ++o) {
       const int oi = ph.fop0 + o;
       const TOp cur = load_op(fops + oi);
-      if ((gb & cur.tmask) != cur.tval) continue;
+      const bool on = (gb & cur.tmask) == cur.tval;
+      if (cur.kind == TK_DENSEX) {
+        apply_densex<RB, COMP>(x, cur, COMP ? flo + 4 * oi : nullptr, on);
+        continue;
+      }
+      if (!on) continue;
       if (cur.kind == TK_DIAGOUT) {
         const bool b1 = (gb >> cur.t) & 1u;
         const float2 f = b1 ? cur.u[3] : cur.u[0];
@@ -1088,32 +1253,67 @@ __device__ __forceinline__ void flush_partial(float pend, int pend_o, float* red
   if (lane == 0) red[pend_o * kWarps + warp] = pend;
 }
 
+// warp sums of the four values of a TK_RUN op: each step halves the values a lane still
+// carries (6 shuffles, where four trees take 20); lanes 0, 8, 16, 24 hold one each
+__device__ __forceinline__ void warp_sums4(const float (&v)[4], float* red, int lane, int warp) {
+  const bool h = lane & 16, q = lane & 8;
+  float a = h ? v[2] : v[0], b = h ? v[3] : v[1];
+  a += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[2], 16);
+  b += __shfl_xor_sync(0xffffffffu, h ? v[1] : v[3], 16);
+  float c = q ? b : a;
+  c += __shfl_xor_sync(0xffffffffu, q ? a : b, 8);
+#pragma unroll
+  for (int s = 4; s > 0; s >>= 1) c += __shfl_xor_sync(0xffffffffu, c, s);
+  if ((lane & 7) == 0) red[(lane >> 3) * kWarps + warp] = c;
+}
+
 // fold the warp partials of every parameterised op of a phase: the 16 warp
-// partials of an op are summed by 16 lanes in a TwoSum tree (the double-float
+// partials of a sum are added by 16 lanes in a TwoSum tree (the double-float
 // sum s + e of the FP32 partials, exact to ~2^-48), one op per 16 lanes, all
-// ops at once; the leader adds (s + e) cfac2 to the FP64 accumulator.  Ops whose
-// parameter another op of the phase shares are added by one thread afterwards.
+// ops at once; then lane k of the 16 adds the op's k-th record, its combination of
+// the op's sums in double-float, to the FP64 accumulator.  Records whose
+// parameter another one of the phase shares are added by one thread afterwards.
 // (FP64 arithmetic runs at 1/64 of the FP32 rate here: summing in FP64 took
 // one warp thousands of cycles per phase while the others waited.)
-__device__ __forceinline__ void fold_phase_grad(const TPhase& ph, const TOp* bops, const float* red, double* gacc) {
+__device__ __forceinline__ void fold_phase_grad(const TPhase& ph, const TOp* bops, const GMem* gmem, const float* red,
+                                                double* gacc) {
   static_assert(kWarps == 16, "one op per 16 lanes");
   const int nbop = ph.nbop, bop0 = ph.bop0;
   for (int base = 0; base < nbop * kWarps; base += blockDim.x) {
     const int t = base + (int)threadIdx.x;
     const int o = t >> 4, w = t & 15;
-    const bool valid = o < nbop && bops[bop0 + o].gen != GEN_NONE;
-    float s = valid ? red[bops[bop0 + o].pad * kWarps + w] : 0.f, e = 0.f;
+    const TOp* op = bops + bop0 + (o < nbop ? o : 0);
+    const int recs = o < nbop ? (int)op->count : 0;
+    const bool run = recs && op->kind == TK_RUN;
+    const float* r = red + op->val * kWarps + w;
+    float s[4], e[4];
 #pragma unroll
-    for (int d = 8; d > 0; d >>= 1) {
-      const float so = __shfl_xor_sync(0xffffffffu, s, d), eo = __shfl_xor_sync(0xffffffffu, e, d);
-      float q, r;
-      two_sum(s, so, q, r);
-      s = q;
-      e = __fadd_rn(__fadd_rn(e, eo), r);
+    for (int k = 0; k < 4; ++k) {
+      s[k] = e[k] = 0.f;
+      if (k > 0 && !__any_sync(0xffffffffu, run)) continue;
+      if (k == 0 ? recs > 0 : run) s[k] = r[k * kWarps];
+#pragma unroll
+      for (int d = 8; d > 0; d >>= 1) {
+        const float so = __shfl_xor_sync(0xffffffffu, s[k], d), eo = __shfl_xor_sync(0xffffffffu, e[k], d);
+        float q, f;
+        two_sum(s[k], so, q, f);
+        s[k] = q;
+        e[k] = __fadd_rn(__fadd_rn(e[k], eo), f);
+      }
     }
-    if (w == 0 && valid) {
-      const TOp& op = bops[bop0 + o];
-      if (!op.shared) gacc[op.param] += (double)op.cfac2 * ((double)s + (double)e);
+    if (w < recs) {
+      const GMem m = gmem[op->param + w];
+      float hs = 0.f, he = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float p = __fmul_rn(m.c[k], s[k]);
+        const float pe = fmaf(m.c[k], e[k], fmaf(m.c[k], s[k], -p));
+        float q, f;
+        two_sum(hs, p, q, f);
+        hs = q;
+        he = __fadd_rn(he, __fadd_rn(f, pe));
+      }
+      if (!m.shared) gacc[m.param] += (double)hs + (double)he;
     }
   }
   __syncthreads();
@@ -1121,18 +1321,25 @@ __device__ __forceinline__ void fold_phase_grad(const TPhase& ph, const TOp* bop
   if (threadIdx.x == 0) {
     for (int q = 0; q < nbop; ++q) {
       const TOp& op = bops[bop0 + q];
-      if (op.gen == GEN_NONE || !op.shared) continue;
-      double v = 0.0;
-      for (int w = 0; w < kWarps; ++w) v += (double)red[op.pad * kWarps + w];
-      gacc[op.param] += (double)op.cfac2 * v;
+      for (int k = 0; k < (int)op.count; ++k) {
+        const GMem& m = gmem[op.param + k];
+        if (!m.shared) continue;
+        double g = 0.0;
+        for (int i = 0; i < (op.kind == TK_RUN ? 4 : 1); ++i) {
+          double v = 0.0;
+          for (int w = 0; w < kWarps; ++w) v += (double)red[(op.val + i) * kWarps + w];
+          g += (double)m.c[i] * v;
+        }
+        gacc[m.param] += g;
+      }
     }
   }
   __syncthreads();
 }
 
 template <int RB>
-__device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPhase* php, const TOp* bops, int m,
-                                               const uint32_t* rowoff, float* red, double* gacc, uint32_t tbase) {
+__device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPhase* php, const TOp* bops,
+                                               const GMem* gmem, int m, const uint32_t* rowoff, float* red, double* gacc, uint32_t tbase) {
   // the phase record is read where it lies (the pass's shared-memory copy when
   // staged): with 2 x 2^RB live amplitudes per thread there are no registers
   // to spare for a copy of it
@@ -1158,10 +1365,17 @@ __device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPh
   int pend_o = -1;
   for (int o = nbop - 1; o >= 0; --o) {
     const TOp op = load_op(bops + bop0 + o);
+    const bool on = (gb & op.tmask) == op.tval;
+    if (op.kind == TK_RUN) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (active) apply_bwd_run<RB>(x, l, op, on && op.cmask, v);
+      warp_sums4(v, red + op.val * kWarps, lane, warp);
+      continue;
+    }
     float part = 0.f;
-    if (active && (gb & op.tmask) == op.tval)
+    if (active && on)
       part = op.kind == TK_DIAGOUT ? diagout_bwd<RB>(x, l, op, gb) : apply_bwd_var<RB>(x, l, op);
-    if (op.gen != GEN_NONE) warp_partial(part, op.pad, pend, pend_o, red, lane, warp);
+    if (op.gen != GEN_NONE) warp_partial(part, op.val, pend, pend_o, red, lane, warp);
   }
   flush_partial(pend, pend_o, red, lane, warp);
   if (active) {
@@ -1173,23 +1387,23 @@ __device__ __forceinline__ void phase_bwd_body(float2* sx, float2* sl, const TPh
     }
   }
   __syncthreads();
-  fold_phase_grad(ph, bops, red, gacc);
+  fold_phase_grad(ph, bops, gmem, red, gacc);
 }
 
 // All phases of a pass on one tile, last phase first: one call per tile, so
 // that the callers' loop state is saved once per tile rather than per phase
 template <int RB>
 __device__ __noinline__ void run_tile_bwd(uint32_t sx, uint32_t sl, const TPhase* ph, int nphase, const TOp* bops,
-                                          int m, uint32_t rows, uint32_t red, uint32_t gacc, uint32_t tbase) {
+                                          const GMem* gmem, int m, uint32_t rows, uint32_t red, uint32_t gacc, uint32_t tbase) {
   for (int f = nphase - 1; f >= 0; --f)
-    phase_bwd_body<RB>(sh<float2>(sx), sh<float2>(sl), ph + f, bops, m, sh<uint32_t>(rows), sh<float>(red),
+    phase_bwd_body<RB>(sh<float2>(sx), sh<float2>(sl), ph + f, bops, gmem, m, sh<uint32_t>(rows), sh<float>(red),
                        sh<double>(gacc), tbase);
 }
 
 template <int RB>
 __device__ __noinline__ void run_phase_bwd_ff(uint32_t ox, uint32_t ol, const TPhase* php, const TOp* bops,
-                                              const float2* blo, int m, uint32_t rows, uint32_t ored, uint32_t ogacc,
-                                              uint32_t tbase) {
+                                              const GMem* gmem, const float2* blo, int m, uint32_t rows, uint32_t ored,
+                                              uint32_t ogacc, uint32_t tbase) {
   float4 *sx = sh<float4>(ox), *sl = sh<float4>(ol);
   const uint32_t* rowoff = sh<uint32_t>(rows);
   float* red = sh<float>(ored);
@@ -1220,11 +1434,18 @@ __device__ __noinline__ void run_phase_bwd_ff(uint32_t ox, uint32_t ol, const TP
   for (int o = nbop - 1; o >= 0; --o) {
     const int oi = bop0 + o;
     const TOp op = load_op(bops + oi);
+    const bool on = (gb & op.tmask) == op.tval;
+    if (op.kind == TK_RUN) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (active) apply_bwd_run_ff<RB>(x, l, op, blo + 4 * oi, on && op.cmask, v);
+      warp_sums4(v, red + op.val * kWarps, lane, warp);
+      continue;
+    }
     float part = 0.f;
-    if (active && (gb & op.tmask) == op.tval)
+    if (active && on)
       part = op.kind == TK_DIAGOUT ? diagout_bwd_ff<RB>(x, l, op, blo + 4 * oi, gb)
                                    : apply_bwd_ff<RB>(x, l, op, blo + 4 * oi);
-    if (op.gen != GEN_NONE) warp_partial(part, op.pad, pend, pend_o, red, lane, warp);
+    if (op.gen != GEN_NONE) warp_partial(part, op.val, pend, pend_o, red, lane, warp);
   }
   flush_partial(pend, pend_o, red, lane, warp);
   if (active) {
@@ -1236,7 +1457,7 @@ __device__ __noinline__ void run_phase_bwd_ff(uint32_t ox, uint32_t ol, const TP
     }
   }
   __syncthreads();
-  fold_phase_grad(ph, bops, red, gacc);
+  fold_phase_grad(ph, bops, gmem, red, gacc);
 }
 
 // the diagonal observable's weight w(i) = sum_t c_t (-1)^popcount(i & z_t)
@@ -1298,37 +1519,37 @@ __device__ void block_loss(double e, BShared& S, double* out) {
 // phase functions keep their amplitudes in registers.
 template <int RB>
 __device__ __noinline__ void batch_bwd_resident(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m,
-                                                const TPhase* phases, const TOp* bops, uint32_t rows, uint32_t red,
-                                                uint32_t gacc) {
+                                                const TPhase* phases, const TOp* bops, const GMem* gmem, uint32_t rows,
+                                                uint32_t red, uint32_t gacc) {
   for (int pi = npass - 1; pi >= 0; --pi)
-    run_tile_bwd<RB>(sx, sl, phases + P[pi].phase0, P[pi].nphase, bops, m, rows, red, gacc, 0u);
+    run_tile_bwd<RB>(sx, sl, phases + P[pi].phase0, P[pi].nphase, bops, gmem, m, rows, red, gacc, 0u);
 }
 
 template <int RB>
 __device__ __noinline__ void batch_bwd_resident_ff(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m,
-                                                   const TPhase* phases, const TOp* bops, const float2* blo,
-                                                   uint32_t rows, uint32_t red, uint32_t gacc) {
+                                                   const TPhase* phases, const TOp* bops, const GMem* gmem,
+                                                   const float2* blo, uint32_t rows, uint32_t red, uint32_t gacc) {
   for (int pi = npass - 1; pi >= 0; --pi) {
     const int ph0 = P[pi].phase0;
     for (int f = P[pi].nphase - 1; f >= 0; --f)
-      run_phase_bwd_ff<RB>(sx, sl, phases + ph0 + f, bops, blo, m, rows, red, gacc, 0u);
+      run_phase_bwd_ff<RB>(sx, sl, phases + ph0 + f, bops, gmem, blo, m, rows, red, gacc, 0u);
   }
 }
 
 template <int RB>
 __device__ __noinline__ void batch_bwd_streamed(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m, int g,
                                                 float2* wp, float2* wl, const TPhase* phases, const TOp* bops,
-                                                uint32_t rows, uint32_t red, uint32_t gacc, unsigned char* stage) {
+                                                const GMem* gmem, uint32_t rows, uint32_t red, uint32_t gacc, unsigned char* stage) {
   const uint64_t ntile = 1ull << g;
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<false>(p, phases, bops, stage);
+    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, nullptr, gmem);
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
       load_tiles<true>(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
-      run_tile_bwd<RB>(sx, sl, sp.ph, p.nphase, sp.ops, m, rows, red, gacc, (uint32_t)tb);
+      run_tile_bwd<RB>(sx, sl, sp.ph, p.nphase, sp.ops, sp.mem, m, rows, red, gacc, (uint32_t)tb);
       store_tiles<true>(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
     }
@@ -1338,20 +1559,20 @@ __device__ __noinline__ void batch_bwd_streamed(uint32_t sx, uint32_t sl, const 
 template <int RB>
 __device__ __noinline__ void batch_bwd_streamed_ff(uint32_t sx, uint32_t sl, const TPass* P, int npass, int m, int g,
                                                    float4* wp, float4* wl, const TPhase* phases, const TOp* bops,
-                                                   const float2* blo, uint32_t rows, uint32_t red, uint32_t gacc,
+                                                   const GMem* gmem, const float2* blo, uint32_t rows, uint32_t red, uint32_t gacc,
                                                    unsigned char* stage) {
   const uint64_t ntile = 1ull << g;
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<false>(p, phases, bops, stage);
+    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, nullptr, gmem);
     const float2* lo = blo + 4 * (size_t)sp.first;
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
       load_tiles_ff(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
       for (int f = p.nphase - 1; f >= 0; --f)
-        run_phase_bwd_ff<RB>(sx, sl, sp.ph + f, sp.ops, lo, m, rows, red, gacc, (uint32_t)tb);
+        run_phase_bwd_ff<RB>(sx, sl, sp.ph + f, sp.ops, sp.mem, lo, m, rows, red, gacc, (uint32_t)tb);
       store_tiles_ff(sx, wp + tb, sl, wl + tb, rows, m);
       __syncthreads();
     }
@@ -1387,7 +1608,7 @@ __device__ __noinline__ void batch_fwd_streamed(uint32_t sx, uint32_t sx2, float
   for (int pi = 0; pi < npass; ++pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<true>(p, phases, fops, stage, druns);
+    const StagedPass sp = stage_pass<true>(p, phases, fops, stage, druns, nullptr);
     const float2* lo = COMP ? flo + 4 * (size_t)sp.first : nullptr;
     if (threadIdx.x == 0) *sh<RunCtx>(rc) = RunCtx{sp.runs, rtab + kRunTab * p.run0, nullptr};
     // two tile buffers (sx, sx2): the next tile's copies are in flight while
@@ -1469,11 +1690,11 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
       if (PREC) {
         block_loss(expect_tile_ff(sx, sxf, slf, 0, S.rowoff, m, a.terms + R.term0, R.nterm), S, a.loss + reg);
         __syncthreads();
-        if (grad) batch_bwd_resident_ff<RB>(oxf, olf, P, R.npass, m, a.phases, a.bops, a.blo, orows, ored, ograd);
+        if (grad) batch_bwd_resident_ff<RB>(oxf, olf, P, R.npass, m, a.phases, a.bops, a.gmem, a.blo, orows, ored, ograd);
       } else {
         block_loss(expect_tile(sx, sl, 0, S.rowoff, m, a.terms + R.term0, R.nterm), S, a.loss + reg);
         __syncthreads();
-        if (grad) batch_bwd_resident<RB>(ox, ol, P, R.npass, m, a.phases, a.bops, orows, ored, ograd);
+        if (grad) batch_bwd_resident<RB>(ox, ol, P, R.npass, m, a.phases, a.bops, a.gmem, orows, ored, ograd);
       }
     } else {
       // ---- tiles streamed through global memory
@@ -1507,10 +1728,10 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
       if (grad) {
         if (PREC)
           batch_bwd_streamed_ff<RB>(oxf, olf, P, R.npass, m, g, a.wpsif + R.work_off, a.wlamf + R.work_off, a.phases,
-                                    a.bops, a.blo, orows, ored, ograd, stage);
+                                    a.bops, a.gmem, a.blo, orows, ored, ograd, stage);
         else
           batch_bwd_streamed<RB>(ox, ol, P, R.npass, m, g, a.wpsi + R.work_off, a.wlam + R.work_off, a.phases,
-                                 a.bops, orows, ored, ograd, stage);
+                                 a.bops, a.gmem, orows, ored, ograd, stage);
       }
     }
     __syncthreads();
@@ -1588,7 +1809,7 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_pass(FArgs a) {
   unsigned char* stage = reinterpret_cast<unsigned char*>(sbuf + 2 * (1 << kBatchTile));
   const TPass& p = *a.pass;
   set_rows(rowoff, p, a.m);
-  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, stage, a.druns);
+  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, stage, a.druns, nullptr);
   // the runs' tables, and their tile products for this tile and the one before
   const bool held = p.nrun <= kTileRuns;
   float4* rtile = reinterpret_cast<float4*>(stage + kStageBytes);
@@ -1641,6 +1862,8 @@ struct FBArgs {
   const TPass* pass;
   const TPhase* phases;
   const TOp* bops;
+  const GMem* gmem;
+  int vals;              // gradient sums of a phase, at most
   int m, g, nparam;
   int stage;             // 1: kStageBytes of shared memory after the tiles hold the pass's records
   uint64_t ntile;
@@ -1651,20 +1874,20 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_bwd_pass(FBArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   uint32_t* rowoff = reinterpret_cast<uint32_t*>(smraw);
   float* red = reinterpret_cast<float*>(rowoff + (1 << (kMaxTileBits - kRowBits)));
-  double* gacc = reinterpret_cast<double*>(red + kMaxPhaseOps * kWarps);
+  double* gacc = reinterpret_cast<double*>(red + a.vals * kWarps);
   float2* sx = reinterpret_cast<float2*>(gacc + ((a.nparam + 1) & ~1));
   float2* sl = sx + (1 << a.m);
   unsigned char* stage = a.stage ? reinterpret_cast<unsigned char*>(sl + (1 << a.m)) : nullptr;
   const TPass& p = *a.pass;
   for (int i = threadIdx.x; i < a.nparam; i += blockDim.x) gacc[i] = 0.0;
   set_rows(rowoff, p, a.m);
-  const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage);
+  const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage, nullptr, a.gmem);
   auto at = [&](const void* q) { return (uint32_t)((const unsigned char*)q - smraw); };
   for (uint64_t t = blockIdx.x; t < a.ntile; t += gridDim.x) {
     const uint64_t tb = tile_base(t, p, a.g);
     load_tiles<true>(at(sx), a.wpsi + tb, at(sl), a.wlam + tb, 0, a.m);
     __syncthreads();
-    run_tile_bwd<kRB>(at(sx), at(sl), sp.ph, p.nphase, sp.ops, a.m, 0, at(red), at(gacc), (uint32_t)tb);
+    run_tile_bwd<kRB>(at(sx), at(sl), sp.ph, p.nphase, sp.ops, sp.mem, a.m, 0, at(red), at(gacc), (uint32_t)tb);
     store_tiles<true>(at(sx), a.wpsi + tb, at(sl), a.wlam + tb, 0, a.m);
     __syncthreads();
   }
@@ -1725,7 +1948,8 @@ struct DRef {
 struct PrepArgs {
   const GSpec* gspec;
   const FMem* fmem;
-  const int32_t* bgate;
+  const FMem* bmem;
+  GMem* gmem;
   float2* flo;             // if not NULL: corrections of the forward matrices (precise path)
   float2* blo;             // backward U^dagger corrections
   float2* dtlo;            // diagonal table corrections
@@ -1800,8 +2024,51 @@ __global__ void k_batch_prep(PrepArgs a) {
       for (int k = 0; k < 4; ++k) a.flo[4 * i + k] = lo_of(A[k]);
   } else if (i < a.nfop + a.nbop) {
     const int j = i - a.nfop;
+    const FMem& bm = a.bmem[j];
     double2 U[4];
-    gate_mat(a.gspec[a.bgate[j]], a.params, U);
+    gate_mat(a.gspec[bm.g[bm.count - 1]], a.params, U);
+    if (bm.count > 1) {
+      // walk the run from its end: E is the product of the members passed, and a
+      // member's generator H becomes E H E^dagger at the end of the run
+      double2 E[4] = {make_double2(1, 0), make_double2(0, 0), make_double2(0, 0), make_double2(1, 0)};
+      int rec = bm.rec0;
+      for (int k = bm.count - 1; k >= 0; --k) {
+        const GSpec& gs = a.gspec[bm.g[k]];
+        if (bm.rec0 >= 0 && gs.param >= 0) {
+          // E H E^dagger for H = [[h0, h1], [conj(h1), h3]]
+          double f = 1.0, h0 = 0.0, h3 = 0.0;
+          double2 h1 = make_double2(0, 0);
+          switch (gs.kind) {
+            case QS_GATE_RX: h1.x = 1.0; break;
+            case QS_GATE_RY: h1.y = -1.0; break;
+            case QS_GATE_RZ: h0 = 1.0; h3 = -1.0; break;
+            case QS_GATE_SHIFT: f = -2.0; h3 = 1.0; break;
+            default: f = -2.0; h0 = h3 = 1.0; break;  // PHASE
+          }
+          auto row = [&](double2 p, double2 q, double2& r0, double2& r1) {  // (p, q) H
+            r0 = zadd(make_double2(p.x * h0, p.y * h0), zmul(q, make_double2(h1.x, -h1.y)));
+            r1 = zadd(zmul(p, h1), make_double2(q.x * h3, q.y * h3));
+          };
+          auto dot = [&](double2 p, double2 q, double2 u, double2 v) {  // p conj(u) + q conj(v)
+            return zadd(zmul(p, make_double2(u.x, -u.y)), zmul(q, make_double2(v.x, -v.y)));
+          };
+          double2 p0, p1, q0, q1;
+          row(E[0], E[1], p0, p1);
+          row(E[2], E[3], q0, q1);
+          const double2 m00 = dot(p0, p1, E[0], E[1]), m01 = dot(p0, p1, E[2], E[3]), m11 = dot(q0, q1, E[2], E[3]);
+          GMem& m = a.gmem[rec++];
+          m.c[0] = (float)(f * m00.x);
+          m.c[1] = (float)(f * m11.x);
+          m.c[2] = (float)(f * m01.x);
+          m.c[3] = (float)(-f * m01.y);
+        }
+        gate_mat(gs, a.params, U);
+        const double2 C0 = zadd(zmul(E[0], U[0]), zmul(E[1], U[2])), C1 = zadd(zmul(E[0], U[1]), zmul(E[1], U[3]));
+        const double2 C2 = zadd(zmul(E[2], U[0]), zmul(E[3], U[2])), C3 = zadd(zmul(E[2], U[1]), zmul(E[3], U[3]));
+        E[0] = C0; E[1] = C1; E[2] = C2; E[3] = C3;
+      }
+      for (int k = 0; k < 4; ++k) U[k] = E[k];
+    }
     // U^dagger
     const double2 D[4] = {make_double2(U[0].x, -U[0].y), make_double2(U[2].x, -U[2].y),
                           make_double2(U[1].x, -U[1].y), make_double2(U[3].x, -U[3].y)};
@@ -1873,7 +2140,8 @@ struct qs_batch_program {
   qs::BTerm* terms = nullptr;
   qs::GSpec* gspec = nullptr;
   qs::FMem* fmem = nullptr;
-  int32_t* bgate = nullptr;
+  qs::FMem* bmem = nullptr;
+  qs::GMem* gmem = nullptr;
   qs::DMem* dmem = nullptr;
   qs::DRef* dref = nullptr;
   float2* dtab = nullptr;
@@ -1949,7 +2217,7 @@ static void free_program(qs_batch_program* p) {
   const bool swap = p->device >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != p->device &&
                     cudaSetDevice(p->device) == cudaSuccess;
   void* ptrs[] = {p->regs, p->order, p->passes, p->phases, p->fops, p->bops, p->terms, p->gspec, p->fmem,
-                  p->bgate, p->dmem, p->dref, p->dtab, p->counter, p->wpsi, p->wlam, p->dparams,
+                  p->bmem, p->gmem, p->dmem, p->dref, p->dtab, p->counter, p->wpsi, p->wlam, p->dparams,
                   p->flo, p->blo, p->dtlo, p->wpsif, p->wlamf, p->druns, p->tabent, p->tabs, p->runs, p->rtab};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -1963,6 +2231,7 @@ static int max_tile(int rb) { return std::min(kBatchTile, 9 + rb); }
 // TOp::var of a backward op (bwd_form): 13 t + form
 static uint8_t bwd_variant(const TOp& b) {
   if (b.kind == TK_DIAGOUT) return 0xff;
+  if (b.kind == TK_RUN) return b.var;  // set where the op is built
   int f;
   if (b.gen == GEN_NONE) f = b.kind == TK_SWAP ? 0 : b.kind == TK_DIAG ? 1 : 2;
   else f = 3 + 2 * (b.gen - GEN_X) + (b.cmask ? 1 : 0);
@@ -1975,14 +2244,51 @@ static uint8_t fwd_variant(const TOp& f) {
     case TK_DIAGOUT: return FV_DIAGOUT;
     case TK_DIAG16: return FV_DIAG16;
     case TK_DIAGRUN: return FV_DIAGRUN;
+    case TK_DENSEX: return f.var;  // set where the op is built
     case TK_SWAP: return (uint8_t)(FV_SWAP + f.t);
     case TK_DIAG: return (uint8_t)((f.cmask ? FV_DIAGC : FV_DIAG) + f.t);
     default: return (uint8_t)((f.cmask ? FV_DENSEC : FV_DENSE) + f.t);
   }
 }
 
+// Gradient sums a phase may have.  The tiled gradient keeps them beside a double per
+// parameter in shared memory: circuits that nearly fill it keep to one sum a gate.
+static int phase_vals(int nparams) { return nparams > 11000 ? kMaxPhaseOps : kMaxPhaseVals; }
+
+// uncompute kind of a gate on a phase bit: the generator picks the structured form
+static uint8_t bwd_kind(int gen, bool diag, bool x) {
+  if (gen == GEN_X) return TK_RX;
+  if (gen == GEN_Y) return TK_RY;
+  if (gen != GEN_NONE) return TK_DIAG;
+  return x ? TK_SWAP : diag ? TK_DIAG : TK_DENSE;
+}
+
+// a run that TK_RUN takes: two gates or more, not all diagonal, one of them with a parameter
+static bool is_run(const qs_circuit* c, const int* gates, int count) {
+  bool diag = true, param = false;
+  for (int k = 0; k < count; ++k) {
+    diag = diag && gate_is_diagonal(c, c->gates[gates[k]]);
+    param = param || c->gates[gates[k]].param >= 0;
+  }
+  return count > 1 && !diag && param;
+}
+
+// The backward ops of a phase while they are put together: a run of gates, with the X it
+// takes along (gate x, -1: none; xop: as an op of its own), before or after it
+struct BGroup {
+  TOp op, xop;
+  int gates[kMaxRun];
+  int count, x;
+  bool dead, pre;
+};
+
+// sizes of the program's tables (fmem and bmem go with the ops, runs with tabs)
+struct Marks {
+  size_t passes, phases, fops, bops, gspec, dmems, drefs, druns, tabent, tabs, gmem;
+};
+
 static int build_program(int nreg, const qs_circuit* const* circs, const qs_observable* const* obs, int tile_qubits,
-                         qs_batch_program* P, int rb = kRB, bool precise = false) {
+                         qs_batch_program* P, int rb = kRB, bool precise = false, bool plain = false) {
   if (rb < kMinRB || rb > kRB) return fail(QS_EINVAL, "phase_qubits must be in %d..%d", kMinRB, kRB);
   if (precise && rb > 3) return fail(QS_EINVAL, "the precise path takes phases of at most 3 qubits");
   const int MT = max_tile(rb);
@@ -2001,7 +2307,8 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   std::vector<BTerm> terms;
   std::vector<GSpec> gspec;
   std::vector<FMem> fmem;
-  std::vector<int32_t> bgate;
+  std::vector<FMem> bmem;
+  std::vector<GMem> gmem;
   std::vector<DMem> dmems;
   std::vector<DRef> drefs;
   std::vector<DRun> druns, tabent;
@@ -2012,7 +2319,19 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   P->param_off.assign(nreg + 1, 0);
   P->amp_off.assign(nreg + 1, 0);
   int64_t work = 0;
+  std::vector<TOp> pf;   // a phase's ops while they are put together: one that moves to a
+  std::vector<FMem> pm;  // later place leaves a dead one behind
+  std::vector<BGroup> pb;
+  // registers of one circuit share its schedule: the tables of the first are copied
+  // with their indices moved
+  std::unordered_map<const qs_circuit*, int> first;
+  std::vector<Marks> marks(nreg + 1);
+  auto here = [&] {
+    return Marks{passes.size(), phases.size(), fops.size(), bops.size(), gspec.size(), dmems.size(), drefs.size(),
+                 druns.size(), tabent.size(), tabs.size(), gmem.size()};
+  };
   for (int r = 0; r < nreg; ++r) {
+    marks[r] = here();
     const qs_circuit* c = circs[r];
     const qs_observable* o = obs ? obs[r] : nullptr;
     if (!c || (!o && !P->fused_only)) return fail(QS_EINVAL, "register %d: null circuit or observable", r);
@@ -2025,13 +2344,15 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
     P->param_off[r + 1] = P->param_off[r] + c->nparams;
     P->amp_off[r + 1] = P->amp_off[r] + (1ll << n);
     const int m = std::min(n, M);
+    const auto seen = first.emplace(c, r);
+    const int r0 = seen.second ? -1 : seen.first->second;
     std::vector<HostPass> hp;
-    QS_TRY(plan_passes(c, n, m, kMaxPhaseOps, hp, rb));
+    if (r0 < 0) QS_TRY(plan_passes(c, n, m, kMaxPhaseOps, hp, rb, plain));
     BReg& R = regs[r];
     memset(&R, 0, sizeof(R));
     R.n = n;
     R.m = m;
-    R.npass = (int)hp.size();
+    R.npass = r0 < 0 ? (int)hp.size() : regs[r0].npass;
     R.pass0 = (int)passes.size();
     R.nparam = c->nparams;
     R.amp_off = P->amp_off[r];
@@ -2048,6 +2369,47 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
       }
     }
     R.nterm = o ? (int)o->terms.size() : 0;
+    if (r0 >= 0) {
+      const Marks &a = marks[r0], &z = marks[r0 + 1], d = marks[r];
+      auto moved = [](size_t from, size_t to) { return (int)to - (int)from; };
+      const int dg = moved(a.gspec, d.gspec), dm = moved(a.gmem, d.gmem);
+      auto copy = [](auto& v, size_t i0, size_t i1, auto fix) {
+        for (size_t i = i0; i < i1; ++i) {
+          auto e = v[i];
+          fix(e);
+          v.push_back(e);
+        }
+      };
+      copy(gspec, a.gspec, z.gspec, [&](GSpec& e) { if (e.param >= 0) e.param += (int)(P->param_off[r] - P->param_off[r0]); });
+      copy(passes, a.passes, z.passes, [&](TPass& e) {
+        e.phase0 += moved(a.phases, d.phases);
+        e.drun0 += moved(a.druns, d.druns);
+        e.run0 += moved(a.tabs, d.tabs);
+        e.mem0 += dm;
+      });
+      copy(phases, a.phases, z.phases, [&](TPhase& e) {
+        e.fop0 += moved(a.fops, d.fops);
+        e.bop0 += moved(a.bops, d.bops);
+      });
+      auto mems = [&](FMem& e) {
+        for (int k = 0; k < e.count; ++k) e.g[k] += dg;
+        if (e.rec0 >= 0) e.rec0 += dm;
+      };
+      copy(fops, a.fops, z.fops, [&](TOp& e) { if (e.kind == TK_DIAG16) e.param += moved(a.drefs, d.drefs); });
+      copy(fmem, a.fops, z.fops, mems);
+      copy(bops, a.bops, z.bops, [&](TOp& e) { if (e.count) e.param += dm; });
+      copy(bmem, a.bops, z.bops, mems);
+      copy(dmems, a.dmems, z.dmems, [&](DMem& e) { e.g += dg; });
+      copy(drefs, a.drefs, z.drefs, [&](DRef& e) { e.mem0 += moved(a.dmems, d.dmems); });
+      copy(druns, a.druns, z.druns, [&](DRun& e) { e.gate += dg; });
+      copy(tabent, a.tabent, z.tabent, [&](DRun& e) { e.gate += dg; });
+      copy(tabs, a.tabs, z.tabs, [&](int4& e) { e.x += moved(a.tabent, d.tabent); });
+      copy(runs, a.tabs, z.tabs, [](int2&) {});
+      copy(gmem, a.gmem, z.gmem, [](GMem&) {});
+      R.cost = regs[r0].cost;
+      marks[r + 1] = here();
+      continue;
+    }
     // gate specs of this register
     const int g0 = (int)gspec.size();
     for (const auto& g : c->gates) {
@@ -2075,6 +2437,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
       tp.phase0 = (int)phases.size();
       tp.drun0 = (int)druns.size();
       tp.run0 = (int)runs.size();
+      tp.mem0 = (int)gmem.size();
       tp.nphase = (int)p.phases.size();
       for (const HostPhase& ph : p.phases) {
         TPhase t;
@@ -2087,9 +2450,31 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
         };
         t.bop0 = (int)bops.size();
         t.fop0 = (int)fops.size();
-        std::vector<int> last(rb, -1);   // forward op index (in fops) open for fusion per phase bit
+        pf.clear();
+        pm.clear();
+        pb.clear();
+        constexpr uint8_t kDead = 0xff;
+        int last[kRB], lastx[kRB], xlast[kRB], blast[kRB];
+        for (int k = 0; k < kRB; ++k) {
+          last[k] = -1;   // forward op (in pf) open for fusion per phase bit
+          lastx[k] = -1;  // forward op (in pf) of the X that was the last gate on a phase bit
+          xlast[k] = 0;   // and its form
+          blast[k] = -1;  // backward run (in pb) open per phase bit
+        }
+        // the run on bit tb comes to the place of the X before it (nothing in between has
+        // touched the bit)
+        auto join_x = [&](int tb, const FMem run) {
+          if (last[tb] >= 0) pf[last[tb]].kind = kDead;
+          TOp& x = pf[lastx[tb]];
+          x.kind = TK_DENSEX;
+          x.cmask = x.cval = 0;
+          x.var = (uint8_t)(FV_DENSEX + 10 * tb + 5 + xlast[tb]);
+          pm[lastx[tb]] = run;
+          last[tb] = lastx[tb];
+          lastx[tb] = -1;
+        };
         int dg = -1;                     // open TK_DIAG16 table of this phase
-        int nval = 0;                    // backward ops with a gradient sum
+        int nval = 0;                    // gradient sums of the backward ops
         // TK_DIAGRUN runs of this phase (complex64 path): the op each opened,
         // its entries, the run open per phase bit and the latest run opened
         std::vector<int> run_op;
@@ -2116,7 +2501,13 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
                 if (v) tval |= 1u << qb;
               }
             }
-          // backward op: one per gate
+          // X with one control in the phase (its value 1) and none outside, or with
+          // controls outside only: renames the outputs of the run before it
+          const bool renames = !plain && g.kind == QS_GATE_X && tb >= 0 && (cm || tmask) &&
+                               (cm == 0 || (tmask == 0 && !(cm & (cm - 1)) && cv == cm));
+          const int xform = cm ? 1 + __builtin_ctz(cm) : 0;
+          // backward op: uncontrolled gates on one phase bit collect in a run (no gate in
+          // between touches the bit); others are ops of their own
           TOp b;
           memset(&b, 0, sizeof(b));
           b.t = (uint8_t)(tb >= 0 ? tb : g.locs[0]);
@@ -2124,24 +2515,47 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
           b.cval = cv;
           b.tmask = tmask;
           b.tval = tval;
-          b.param = g.param;
-          b.gen = g.param >= 0 ? (uint8_t)gen_of(g.kind, &b.cfac2) : GEN_NONE;
+          float cf2 = 0.f;
+          b.gen = g.param >= 0 ? (uint8_t)gen_of(g.kind, &cf2) : GEN_NONE;
           // uncompute kind: the generator picks the structured form (Rx / Ry / diagonal)
           if (tb < 0) b.kind = TK_DIAGOUT;
-          else if (b.gen == GEN_X) b.kind = TK_RX;
-          else if (b.gen == GEN_Y) b.kind = TK_RY;
-          else if (b.gen != GEN_NONE) b.kind = TK_DIAG;
-          else b.kind = g.kind == QS_GATE_X ? TK_SWAP : diag ? TK_DIAG : TK_DENSE;
+          else b.kind = bwd_kind(b.gen, diag, g.kind == QS_GATE_X);
           if (g.param >= 0 && b.gen == GEN_NONE)
             return fail(QS_EUNSUPPORTED, "register %d gate %d: kind %d has no batched gradient", r, gi, g.kind);
-          for (int q = t.bop0; q < (int)bops.size(); ++q)
-            if (bops[q].gen != GEN_NONE && b.gen != GEN_NONE && bops[q].param == b.param) {
-              bops[q].shared = 1;
-              b.shared = 1;
+          {
+            const bool plain = tb >= 0 && !cm && !tmask && g.kind != QS_GATE_X;
+            BGroup* run = tb >= 0 && blast[tb] >= 0 ? &pb[blast[tb]] : nullptr;
+            auto take = [&](BGroup& u, bool pre) {
+              u.op.cmask = cm ? 0 : 1;  // controls outside the phase: tmask / tval
+              u.op.cval = 0;
+              u.op.tmask = tmask;
+              u.op.tval = tval;
+              u.op.t = (uint8_t)tb;
+              u.op.var = (uint8_t)(BV_RUN + 10 * tb + xform + (pre ? 5 : 0));
+              u.x = gi;
+              u.xop = b;
+              u.pre = pre;
+              pb.push_back(u);
+            };
+            if (plain && run && run->count < kMaxRun) {
+              run->gates[run->count++] = gi;  // stays at the run's place: nothing since has touched the bit
+            } else if (renames && run && run->x < 0 && is_run(c, run->gates, run->count)) {
+              const BGroup u = *run;  // moves here with the X
+              run->dead = true;
+              BGroup v = u;
+              take(v, false);
+              blast[tb] = -1;
+            } else if (renames) {
+              BGroup u{b, b, {0}, 0, -1, false, false};  // the next run on the bit may come to this place
+              take(u, true);
+              blast[tb] = (int)pb.size() - 1;
+            } else {
+              pb.push_back(BGroup{b, b, {gi}, 1, -1, false, false});
+              if (tb >= 0) blast[tb] = plain ? (int)pb.size() - 1 : -1;
             }
-          if (b.gen != GEN_NONE) b.pad = (uint8_t)nval++;
-          bops.push_back(b);
-          bgate.push_back(g0 + gi);
+            for (int k = 0; k < rb; ++k)
+              if ((cm >> k) & 1) blast[k] = -1;
+          }
           // forward op.  A diagonal gate with its target outside the phase is a
           // per-thread factor.  Consecutive uncontrolled gates on one target fuse
           // into one 2x2; controlled diagonal gates inside the phase join its open
@@ -2172,20 +2586,36 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
           if (tb < 0) {
             f.kind = TK_DIAGOUT;
             f.t = (uint8_t)g.locs[0];
-            fops.push_back(f);
-            fmem.push_back(fm);
+            pf.push_back(f);
+            pm.push_back(fm);
             for (int k = 0; k < rb; ++k)
-              if ((cm >> k) & 1) last[k] = -1;
+              if ((cm >> k) & 1) last[k] = lastx[k] = -1;
             continue;
           }
           const bool fusable = cm == 0 && tmask == 0 && g.kind != QS_GATE_X;
+          int xat = -1;  // this gate's op if it is an X that a run may come to
           const uint8_t gbits = (uint8_t)(cm | (1u << tb));
           if (!diag) nondiag |= gbits;
           if (!diag) run_open[tb] = -1;  // a run moves no later gate past this one
-          if (fusable && last[tb] >= 0 && fmem[last[tb]].count < 4) {
-            FMem& fmo = fmem[last[tb]];
+          if (fusable && last[tb] >= 0 && pm[last[tb]].count < kMaxRun) {
+            FMem& fmo = pm[last[tb]];
             fmo.g[fmo.count++] = g0 + gi;
-            if (!diag) fops[last[tb]].kind = TK_DENSE;
+            if (!diag && pf[last[tb]].kind == TK_DIAG) {
+              pf[last[tb]].kind = TK_DENSE;
+              if (lastx[tb] >= 0) join_x(tb, pm[last[tb]]);
+            }
+          } else if (fusable && !diag && lastx[tb] >= 0 && last[tb] < 0) {
+            join_x(tb, fm);
+          } else if (renames && last[tb] >= 0 && pf[last[tb]].kind == TK_DENSE) {
+            // the dense op moves here (nothing since has touched its bit) and takes the X along
+            TOp x = pf[last[tb]];
+            x.kind = TK_DENSEX;
+            x.tmask = tmask;
+            x.tval = tval;
+            x.var = (uint8_t)(FV_DENSEX + 10 * tb + xform);
+            pf[last[tb]].kind = kDead;
+            pf.push_back(x);
+            pm.push_back(FMem(pm[last[tb]]));
           } else if (!precise && diag && cm == 0 && tmask != 0) {
             // joins (or opens) the run on its target: diagonal gates commute, and
             // no non-diagonal op on this bit was emitted since the run opened
@@ -2196,11 +2626,11 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
               fm.count = 0;
               run_open[tb] = (int)run_op.size();
               run_last = run_open[tb];
-              run_op.push_back((int)fops.size());
+              run_op.push_back((int)pf.size());
               run_ent.emplace_back();
               run_bit.push_back(tb);
-              fops.push_back(f);
-              fmem.push_back(fm);
+              pf.push_back(f);
+              pm.push_back(fm);
             }
             DRun e;
             memset(&e, 0, sizeof(e));
@@ -2215,8 +2645,8 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
               f.cmask = f.cval = 0;
               f.param = (int)drefs.size();
               fm.count = 0;
-              fops.push_back(f);
-              fmem.push_back(fm);
+              pf.push_back(f);
+              pm.push_back(fm);
               drefs.push_back({(int32_t)dmems.size(), 0});
               dg = (int)drefs.size() - 1;
               nondiag = 0;
@@ -2232,19 +2662,26 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
           } else {
             f.kind = g.kind == QS_GATE_X ? TK_SWAP : diag ? TK_DIAG : TK_DENSE;
             f.t = (uint8_t)tb;
-            fops.push_back(f);
-            fmem.push_back(fm);
-            last[tb] = fusable ? (int)fops.size() - 1 : -1;
+            pf.push_back(f);
+            pm.push_back(fm);
+            if (last[tb] >= 0) lastx[tb] = -1;  // a full run lies between
+            last[tb] = fusable ? (int)pf.size() - 1 : -1;
+            if (renames) {
+              xat = (int)pf.size() - 1;
+              xlast[tb] = xform;
+            }
           }
           // a controlled gate closes fusion on its target and its phase-local controls
           if (cm || tmask) {
             for (int k = 0; k < rb; ++k)
-              if ((cm >> k) & 1) last[k] = -1;
+              if ((cm >> k) & 1) last[k] = lastx[k] = -1;
             last[tb] = -1;
           }
+          if (xat >= 0) lastx[tb] = xat;
+          else if (!fusable) lastx[tb] = -1;
         }
         for (size_t r = 0; r < run_op.size(); ++r) {
-          TOp& ro = fops[run_op[r]];
+          TOp& ro = pf[run_op[r]];
           if (run_ent[r].size() == 1) {
             // a run of one gate stays that gate's own op (its outside controls as tmask)
             const DRun& e = run_ent[r][0];
@@ -2252,8 +2689,8 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
             ro.tmask = e.tmask;
             ro.tval = e.tval;
             ro.param = -1;
-            fmem[run_op[r]].count = 1;
-            fmem[run_op[r]].g[0] = e.gate;
+            pm[run_op[r]].count = 1;
+            pm[run_op[r]].g[0] = e.gate;
             continue;
           }
           // entries by where their qubits lie: lane bits, warp bits, tile-id bits, several
@@ -2297,18 +2734,106 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
           for (int k = 0; k < 2; ++k) tabent.insert(tabent.end(), part[k].begin(), part[k].end());
           for (int k = 2; k < 4; ++k) druns.insert(druns.end(), part[k].begin(), part[k].end());
         }
+        for (size_t k = 0; k < pf.size(); ++k) {
+          if (pf[k].kind == kDead) continue;
+          fops.push_back(pf[k]);
+          fmem.push_back(pm[k]);
+        }
+        // backward ops: a run becomes one op (TK_RUN, or its plain product without
+        // parameters), a run of diagonal gates or of one gate its gates' own ops, as does
+        // a run whose four sums would leave no room for the gates still to come
+        nval = 0;
+        int left = 0;
+        for (const BGroup& u : pb)
+          for (int k = 0; k < u.count; ++k) left += !u.dead && c->gates[u.gates[k]].param >= 0;
+        const int rec0 = (int)gmem.size();
+        auto record = [&](int gi, float c0) {
+          GMem q;
+          memset(&q, 0, sizeof(q));
+          q.param = c->gates[gi].param;
+          q.c[0] = c0;
+          for (int k = rec0; k < (int)gmem.size(); ++k)
+            if (gmem[k].param == q.param) gmem[k].shared = q.shared = 1;
+          gmem.push_back(q);
+        };
+        for (const BGroup& u : pb) {
+          if (u.dead) continue;
+          FMem fm;
+          memset(&fm, 0, sizeof(fm));
+          fm.rec0 = -1;
+          bool diag = true, param = false;
+          for (int k = 0; k < u.count; ++k) {
+            const qs_gate_desc& g = c->gates[u.gates[k]];
+            diag = diag && gate_is_diagonal(c, g);
+            param = param || g.param >= 0;
+            left -= g.param >= 0;
+          }
+          TOp b = u.op;
+          const bool fits = !param || nval + 4 + left <= phase_vals(P->fused_only ? c->nparams : 0);
+          if (u.count > 1 && !diag && fits && (param || u.x < 0)) {
+            for (; fm.count < u.count; ++fm.count) fm.g[fm.count] = g0 + u.gates[fm.count];
+            b.gen = GEN_NONE;
+            b.kind = param ? TK_RUN : TK_DENSE;
+            if (param) {
+              if (u.x < 0) b.var = (uint8_t)(BV_RUN + 10 * b.t);
+              fm.rec0 = b.param = (int)gmem.size();
+              // in the order k_batch_prep meets them: from the run's end
+              for (int k = u.count; k-- > 0;)
+                if (c->gates[u.gates[k]].param >= 0) record(u.gates[k], 0.f);
+              b.count = (uint32_t)((int)gmem.size() - b.param);
+              b.val = (uint8_t)nval;
+              nval += 4;
+            }
+            bops.push_back(b);
+            bmem.push_back(fm);
+            continue;
+          }
+          auto lone_x = [&] {  // the X the run would have taken along
+            fm.count = 1;
+            fm.g[0] = g0 + u.x;
+            bops.push_back(u.xop);
+            bmem.push_back(fm);
+          };
+          if (u.x >= 0 && u.pre) lone_x();
+          for (int k = 0; k < u.count; ++k) {
+            const int gi = u.gates[k];
+            const qs_gate_desc& g = c->gates[gi];
+            TOp o = u.op;
+            float cf2 = 0.f;
+            if (u.count > 1 || u.x >= 0) {  // a gate of a run: uncontrolled, on the run's bit
+              o.cmask = o.cval = o.var = 0;
+              o.tmask = o.tval = 0;
+              o.gen = g.param >= 0 ? (uint8_t)gen_of(g.kind, &cf2) : GEN_NONE;
+              o.kind = bwd_kind(o.gen, gate_is_diagonal(c, g), false);
+            }
+            if (o.gen != GEN_NONE) {
+              gen_of(g.kind, &cf2);
+              o.param = (int)gmem.size();
+              o.count = 1;
+              o.val = (uint8_t)nval++;
+              record(gi, cf2);
+            }
+            fm.count = 1;
+            fm.g[0] = g0 + gi;
+            bops.push_back(o);
+            bmem.push_back(fm);
+          }
+          if (u.x >= 0 && !u.pre) lone_x();
+        }
         t.nbop = (int)bops.size() - t.bop0;
         t.nfop = (int)fops.size() - t.fop0;
         t.nshared = 0;
-        for (int q = t.bop0; q < (int)bops.size(); ++q) t.nshared += bops[q].shared ? 1 : 0;
+        for (int q = rec0; q < (int)gmem.size(); ++q) t.nshared += gmem[q].shared ? 1 : 0;
         phases.push_back(t);
         cost += (double)(1ll << n) * (1 + 0.02 * t.nbop);
       }
       tp.ndrun = (int)druns.size() - tp.drun0;
       tp.nrun = (int)runs.size() - tp.run0;
+      tp.nmem = (int)gmem.size() - tp.mem0;
       passes.push_back(tp);
     }
     R.cost = cost;
+    marks[r + 1] = here();
   }
   for (size_t i = 0; i < fops.size(); ++i) {
     TOp& f = fops[i];
@@ -2341,7 +2866,8 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   QS_TRY(upload(&P->terms, terms));
   QS_TRY(upload(&P->gspec, gspec));
   QS_TRY(upload(&P->fmem, fmem));
-  QS_TRY(upload(&P->bgate, bgate));
+  QS_TRY(upload(&P->bmem, bmem));
+  QS_TRY(upload(&P->gmem, gmem));
   QS_TRY(upload(&P->dmem, dmems));
   QS_TRY(upload(&P->dref, drefs));
   P->ndiag = (int)drefs.size();
@@ -2402,7 +2928,8 @@ static int launch_prep(const qs_batch_program* P, const double* dev_params, bool
   PrepArgs pa;
   pa.gspec = P->gspec;
   pa.fmem = P->fmem;
-  pa.bgate = P->bgate;
+  pa.bmem = P->bmem;
+  pa.gmem = P->gmem;
   pa.flo = P->flo;
   pa.blo = P->blo;
   pa.dtlo = P->dtlo;
@@ -2646,7 +3173,7 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
   qs_batch_program* P = c->fused;
   cudaStream_t st = s->stream;
   const int np = c->nparams;
-  size_t smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + sizeof(float) * kMaxPhaseOps * kWarps +
+  size_t smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + sizeof(float) * phase_vals(c->nparams) * kWarps +
                 sizeof(double) * ((np + 1) & ~1) + 2 * sizeof(float2) * (1ull << m);
   if (smem > 227 * 1024) return fail(QS_EUNSUPPORTED, "%d parameters do not fit the tiled backward's shared memory", np);
   const bool stage = smem + kStageBytes <= 227 * 1024;
@@ -2705,6 +3232,8 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
   a.wlam = wlam;
   a.phases = P->phases;
   a.bops = P->bops;
+  a.gmem = P->gmem;
+  a.vals = phase_vals(np);
   a.m = m;
   a.g = g;
   a.nparam = np;
@@ -2796,6 +3325,28 @@ int qs_batch_program_create(int nreg, const qs_circuit* const* circuits, const q
   *out = P;
   return QS_OK;
 }
+
+}  // extern "C"
+
+// A program whose forward pass applies the gates without moving a run past gates on other
+// qubits to an X that it could take along, in phases cut at the same gates whatever the
+// later engine's limits: the last bits of its amplitudes, and with them the samples that a
+// shot-based estimate counts, are those of the plain order.
+int qs::batch_program_plain(int nreg, const qs_circuit* const* circuits, const qs_observable* const* observables,
+                            qs_batch_program** out) {
+  *out = nullptr;
+  qs_batch_program* P = new qs_batch_program();
+  const int rc = build_program(nreg, circuits, observables, 0, P, kRB, false, true);
+  if (rc != QS_OK) {
+    const std::string msg = qs_last_error();
+    free_program(P);
+    return fail(rc, "%s", msg.c_str());
+  }
+  *out = P;
+  return QS_OK;
+}
+
+extern "C" {
 
 int qs_batch_program_create_ex(int nreg, const qs_circuit* const* circuits, const qs_observable* const* observables,
                                int tile_qubits, int phase_qubits, int flags, qs_batch_program** out) {
@@ -2930,6 +3481,7 @@ int qs_batch_run(qs_state* s, const qs_batch_program* p, const double* dev_param
   a.phases = p->phases;
   a.fops = p->fops;
   a.bops = p->bops;
+  a.gmem = p->gmem;
   a.terms = p->terms;
   a.loss = dev_loss;
   a.grad = dev_grad;

@@ -299,6 +299,9 @@ int expect_raw(const void* data, int dtype, int n, int nreg, const qs_observable
 int fused_forward(qs_state* s, const qs_circuit* c, const double* host_params, int tile_qubits);
 int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, const qs_observable* o,
                    void* dev_work, double* host_grad, double* host_loss, int tile_qubits);
+// a batch program (complex64, default shape) with the gates in plain order (batch.cu)
+int batch_program_plain(int nreg, const qs_circuit* const* circuits, const qs_observable* const* observables,
+                        qs_batch_program** out);
 void free_fused(qs_batch_program* p);
 int schedule_info(const qs_circuit* c, int tile_qubits, int* npasses, int* nphases);
 // the scheduler's gate order (expanded SWAPs) and pass of each gate, host only (batch.cu)

@@ -417,7 +417,7 @@ int qs_faithful_gradient(const qs_circuit* c, const double* params, const qs_obs
     qs_observable empty;
     std::vector<const qs_observable*> os(R, &empty);
     qs_batch_program* prog = nullptr;
-    if (qs_batch_program_create(R, cs.data(), os.data(), 0, &prog) == QS_OK) {
+    if (batch_program_plain(R, cs.data(), os.data(), &prog) == QS_OK) {
       double* dparams = nullptr;
       if (cudaMalloc(&dparams, sizeof(double) * (pm.size() + R)) == cudaSuccess) {
         rc = qs_state_reset(st, nullptr);

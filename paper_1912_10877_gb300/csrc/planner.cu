@@ -32,14 +32,15 @@ bool gate_is_diagonal(const qs_circuit* c, const qs_gate_desc& g) {
 
 // greedy scan: take gates (in order) whose `fit` bits fit in `set` grown up to
 // `cap` bits, skipping (and blocking all qubits of) gates that do not fit or
-// depend on a skipped gate; at most `limit` gates with a parameter are taken
-static void scan(const qs_circuit* c, const std::vector<int>& rem, const std::vector<uint64_t>& dep,
+// depend on a skipped gate; at most `limit` gates (plain: of any kind, else those with a
+// parameter) are taken
+static void scan(const qs_circuit* c, bool plain, const std::vector<int>& rem, const std::vector<uint64_t>& dep,
                  const std::vector<uint64_t>& fit, uint64_t& set, int cap, size_t limit, std::vector<int>& taken,
                  std::vector<int>& left) {
   uint64_t blocked = 0;
-  size_t params = 0;
+  size_t counted = 0;
   for (int gi : rem) {
-    if ((dep[gi] & blocked) || params >= limit) {
+    if ((dep[gi] & blocked) || counted >= limit) {
       blocked |= dep[gi];
       left.push_back(gi);
       continue;
@@ -47,7 +48,7 @@ static void scan(const qs_circuit* c, const std::vector<int>& rem, const std::ve
     const uint64_t u = set | fit[gi];
     if (__builtin_popcountll(u) <= cap) {
       set = u;
-      params += c->gates[gi].param >= 0;
+      counted += plain || c->gates[gi].param >= 0;
       taken.push_back(gi);
     } else {
       blocked |= dep[gi];
@@ -63,7 +64,8 @@ static std::vector<int> bits_of(uint64_t m) {
   return v;
 }
 
-int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::vector<HostPass>& out, int rb) {
+int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::vector<HostPass>& out, int rb,
+                bool plain) {
   out.clear();
   if (m < kRowBits || m > n || m > kMaxTileBits)
     return fail(QS_EINVAL, "tile of %d qubits for a register of %d", m, n);
@@ -78,13 +80,24 @@ int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::ve
     dep[i] = qubits_of(g);
     fit[i] = gate_is_diagonal(c, g) ? 0ull : (1ull << g.locs[0]);
   }
+  // An uncontrolled diagonal gate that starts a run of gates on its qubit with a
+  // non-diagonal one in it stays with that run: the run is one op, the gate taken early
+  // into a phase without its qubit an op of its own over every amplitude (one a phase in
+  // the batch of variational circuits).
+  uint64_t run = 0;  // qubits whose next gate, going backwards, is of such a run
+  for (int i = G - 1; i >= 0 && !plain; --i) {
+    const qs_gate_desc& g = c->gates[i];
+    if (g.ctrl_mask || g.kind == QS_GATE_X) run &= ~dep[i];
+    else if (fit[i]) run |= fit[i];
+    else if (run & dep[i]) fit[i] = dep[i];
+  }
   const uint64_t seed = (1ull << kRowBits) - 1ull;  // register qubits 0..4: contiguous tile rows
   std::vector<int> rem(G);
   for (int i = 0; i < G; ++i) rem[i] = i;
   while (!rem.empty()) {
     uint64_t B = seed;
     std::vector<int> taken, left;
-    scan(c, rem, dep, fit, B, m, (size_t)-1, taken, left);
+    scan(c, plain, rem, dep, fit, B, m, (size_t)-1, taken, left);
     if (taken.empty()) return fail(QS_EUNSUPPORTED, "no gate fits a %d-qubit tile", m);
     for (int b = 0; __builtin_popcountll(B) < m && b < n; ++b) B |= 1ull << b;  // pad with low qubits
     HostPass P;
@@ -93,7 +106,7 @@ int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::ve
     while (!prem.empty()) {
       uint64_t R = 0;
       std::vector<int> pt, pl;
-      scan(c, prem, dep, fit, R, rb, (size_t)max_phase_params, pt, pl);
+      scan(c, plain, prem, dep, fit, R, rb, (size_t)max_phase_params, pt, pl);
       for (int b : P.tbits) {
         if (__builtin_popcountll(R) >= rb) break;
         R |= 1ull << b;

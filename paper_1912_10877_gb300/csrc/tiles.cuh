@@ -37,14 +37,15 @@ struct TOp {
   uint8_t cmask;  // phase-local control bits
   uint8_t cval;   // their required values
   uint8_t gen;    // backward ops: generator code (GEN_*), 0 = no parameter
-  uint8_t shared; // backward ops: the parameter also appears in another op of the phase
-  uint8_t var;    // forward ops: the specialised form (fwd_variant), one jump per op
-  uint8_t pad;    // backward ops with a generator: their place among the phase's gradient sums
-  int32_t param;  // register-local parameter index (forward TK_DIAG16: table index), -1 = none
-  float cfac2;    // 2 c for U = exp(-i theta c H)
+  uint8_t shared; // TK_DIAGRUN: the tile-id entries
+  uint8_t var;    // the specialised form (fwd_variant, bwd_variant), one jump per op
+  uint8_t val;    // backward ops: first of its sums in the phase's list (TK_RUN: 4, others with a generator: 1)
+  int32_t param;  // forward TK_DIAG16: table index, TK_DIAGRUN: first entry; backward: first of its GMem records
+  float cfac2;    // TK_DIAGRUN: the run's number in the pass (integer bits)
   uint32_t tmask; // controls outside the phase (register qubit bits)
   uint32_t tval;
-  uint32_t count; // TK_DIAGRUN: entries (param: the first, relative to the pass's drun0)
+  uint32_t count; // TK_DIAGRUN: entries (param: the first, relative to the pass's drun0); backward: GMem records
+  uint32_t pad;
   float2 u[4];    // forward: U; backward: U^dagger (row-major 2x2)
 };
 
@@ -59,7 +60,15 @@ struct TOp {
 // bit t is 0 by one factor and those whose bit t is 1 by another (a scalar when
 // its target is outside the phase); the products are formed per thread and
 // applied to the amplitudes once
-enum { TK_DENSE = 0, TK_SWAP = 1, TK_DIAG = 2, TK_RX = 3, TK_RY = 4, TK_DIAG16 = 5, TK_DIAGOUT = 6, TK_DIAGRUN = 7 };
+// TK_DENSEX (forward): a run of uncontrolled gates on one phase bit as one 2x2 with an X
+// on it before or after (var), controlled by a phase bit (var) or by qubits outside
+// (tmask / tval): the X only renames the inputs or outputs
+// TK_RUN (backward): a run of two or more uncontrolled gates on one phase bit, some with
+// a parameter, with or without such an X (cmask = 1: controlled by qubits outside): takes
+// the four sums that every member's derivative is a combination of, uncomputes the run
+// and the X
+enum { TK_DENSE = 0, TK_SWAP = 1, TK_DIAG = 2, TK_RX = 3, TK_RY = 4, TK_DIAG16 = 5, TK_DIAGOUT = 6, TK_DIAGRUN = 7,
+       TK_DENSEX = 8, TK_RUN = 9 };
 
 constexpr int kRunTab = 48;  // entries of a run's table: 32 lanes, then 16 warps (products for bit t = 0 and 1)
 
@@ -69,6 +78,18 @@ struct DRun {
   uint32_t tq;           // target register qubit when outside the phase (scalar entry), else 0xffffffff
   float2 u0, u3;         // the gate's diagonal
 };
+// Where a parameterised gate's derivative comes from: c . (its op's sums).  An op with
+// one gate has one sum, Im<lambda|H|psi>, and c[0] = 2 c of U = exp(-i theta c H); a
+// TK_RUN has Im sum conj(l0) x0, Im sum conj(l1) x1, and the same of X and Y, and c is
+// twice the factor times the Pauli decomposition of the generator carried to the end of
+// the run.
+struct GMem {
+  int32_t param;    // register-local parameter index
+  uint32_t shared;  // the parameter appears in another record of the phase
+  float c[4];
+  uint32_t pad[2];
+};
+
 enum { GEN_NONE = 0, GEN_X = 1, GEN_Y = 2, GEN_Z = 3, GEN_P1 = 4, GEN_I = 5 };
 
 struct TPhase {
@@ -77,8 +98,8 @@ struct TPhase {
   uint16_t keep[kRB];       // bits below each register bit (phase_base)
   uint16_t sroff[1 << kRB]; // swz(register offset of amplitude j): slot = swz(base) ^ sroff[j]
   int32_t fop0, nfop;       // forward ops (fused), applied in order
-  int32_t bop0, nbop;       // backward ops (unfused), applied in reverse order
-  int32_t nshared;          // backward ops whose parameter another op of the phase shares
+  int32_t bop0, nbop;       // backward ops, applied in reverse order
+  int32_t nshared;          // their records whose parameter another one of the phase shares
 };
 
 struct TPass {
@@ -87,6 +108,7 @@ struct TPass {
   int32_t phase0, nphase;
   int32_t drun0, ndrun;     // the pass's TK_DIAGRUN entries
   int32_t run0, nrun;       // the pass's TK_DIAGRUN ops
+  int32_t mem0, nmem;       // the pass's GMem records
 };
 
 struct HostPhase {
@@ -102,9 +124,11 @@ struct HostPass {
 // Greedy commutation-aware scheduling: passes of m qubits (always containing
 // register qubits 0..4, so tile rows are contiguous), phases of exactly rb of
 // the pass's qubits with at most max_phase_params parameterised gates.  Gates must be single-target; a non-diagonal gate's target
-// lies in its phase, its controls and diagonal gates may be anywhere.  Returns
+// lies in its phase, its controls and diagonal gates may be anywhere.  plain: no gate is
+// held back for the run it starts and every gate counts towards a phase's limit.  Returns
 // QS_OK or QS_EUNSUPPORTED.
-int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::vector<HostPass>& out, int rb = kRB);
+int plan_passes(const qs_circuit* c, int n, int m, int max_phase_params, std::vector<HostPass>& out, int rb = kRB,
+                bool plain = false);
 
 // diagonal gates (fit in any phase: they only multiply amplitudes)
 bool gate_is_diagonal(const qs_circuit* c, const qs_gate_desc& g);
