@@ -14,6 +14,7 @@
 // stream order.  The uncompute runs in FP64 (complex128 work buffers) whatever
 // the forward precision; checkpoints taken during the forward replace psi at
 // segment boundaries so that uncompute drift cannot accumulate across segments.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -166,6 +167,98 @@ k_adjoint_param1(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t 
   adj_finish(acc, out);
 }
 
+// A run of uncontrolled single-qubit gates on one qubit, some with a parameter, as one
+// pass, with the controlled X before (pre) or after it that only renames the pair.
+// With (a, b) the pair at the end of the run the pass sums Im conj(l_a) x_a,
+// Im conj(l_b) x_b, Im<l|X|x> and Im<l|Y|x>; a member's derivative is 2 c times its
+// generator carried to the run's end, decomposed over those four (AdjRun::coef).
+//   bound: the FP64 rate.  12 operations a pair for the sums and 32 for U^dag on psi and
+//   lambda, where Rz, Rx, Rz took 64 in three passes and the X a fourth pass.  The pairs
+//   are cut into equal contiguous ranges, four CTAs an SM: a grid-stride loop left a
+//   sixth of the FP64 units idle in its last round.  Measured in the differentiation
+//   workload (n = 20): 62 us a run and its X, 121 us as four passes.
+constexpr int kAdjMembers = 8;
+constexpr int kAdjRunBlocks = 608;  // 4 per SM on 152 SMs
+
+struct AdjRun {
+  double2 ud[4];             // U^dag of the run
+  uint64_t off1;             // offset of its bit
+  uint64_t xmask, xval;      // the X's controls and their values (xmask = 0: no X)
+  int pre, members;
+  int param[kAdjMembers];
+  double coef[kAdjMembers][4];
+};
+
+__global__ void __launch_bounds__(kAdjThreads, 4)
+k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nitems, int t,
+              const __grid_constant__ AdjRun F, double* __restrict__ partials, unsigned* __restrict__ counter,
+              double* __restrict__ grad) {
+  const uint64_t lo = nitems * blockIdx.x / gridDim.x, hi = nitems * (blockIdx.x + 1) / gridDim.x;
+  const uint64_t below = F.off1 - 1;
+  double va = 0.0, vb = 0.0, vx = 0.0, vy = 0.0;
+  for (uint64_t it = lo + threadIdx.x; it < hi; it += kAdjThreads) {
+    const uint64_t b0 = it + (it & ~below), b1 = b0 + F.off1;
+    const bool on = F.xmask && (b0 & F.xmask) == F.xval;
+    const bool in = on && !F.pre, out = on && F.pre;
+    const uint64_t ia = in ? b1 : b0, ib = in ? b0 : b1;
+    const double2 xa = psi[ia], xb = psi[ib], la = lam[ia], lb = lam[ib];
+    va = fma(la.x, xa.y, fma(-la.y, xa.x, va));
+    vb = fma(lb.x, xb.y, fma(-lb.y, xb.x, vb));
+    vx = fma(la.x, xb.y, fma(-la.y, xb.x, vx));
+    vy = fma(lb.x, xa.x, fma(lb.y, xa.y, vy));
+    vx = fma(lb.x, xa.y, fma(-lb.y, xa.x, vx));
+    vy = fma(-la.x, xb.x, fma(-la.y, xb.y, vy));
+    const uint64_t oa = out ? b1 : b0, ob = out ? b0 : b1;
+    psi[oa] = cfma(F.ud[1], xb, cmul(F.ud[0], xa));
+    psi[ob] = cfma(F.ud[3], xb, cmul(F.ud[2], xa));
+    lam[oa] = cfma(F.ud[1], lb, cmul(F.ud[0], la));
+    lam[ob] = cfma(F.ud[3], lb, cmul(F.ud[2], la));
+  }
+  // CTA sums, then the CTA that arrives last folds all of them (in an order that does not
+  // depend on which it is) and adds every member's derivative
+  __shared__ double red[4][kAdjThreads / 32];
+  __shared__ double tot[4];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  auto cta_sums = [&](double (&v)[4]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane < 4) red[lane][warp] = lane == 0 ? v[0] : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3];
+    __syncthreads();
+    if (threadIdx.x < 4) {
+      static_assert(kAdjThreads / 32 == 8, "CTA tree below is written for 8 warps");
+      const double* r = red[threadIdx.x];
+      tot[threadIdx.x] = ((r[0] + r[1]) + (r[2] + r[3])) + ((r[4] + r[5]) + (r[6] + r[7]));
+    }
+    __syncthreads();
+  };
+  double v[4] = {va, vb, vx, vy};
+  cta_sums(v);
+  if (threadIdx.x < 4) partials[threadIdx.x * gridDim.x + blockIdx.x] = tot[threadIdx.x];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(counter, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kAdjThreads) v[k] += __ldcg(partials + k * gridDim.x + i);
+  }
+  __syncthreads();
+  cta_sums(v);
+  if (threadIdx.x == 0) {
+    for (int m = 0; m < F.members; ++m) {
+      const double* c = F.coef[m];
+      grad[F.param[m]] += (c[0] * tot[0] + c[1] * tot[1]) + (c[2] * tot[2] + c[3] * tot[3]);
+    }
+    *counter = 0u;
+  }
+}
+
 // the structured form of a single-target gate, or -1
 static int adj_form1(const std::vector<cd>& G, const std::vector<cd>& Ud, AdjForm1* F) {
   const cd z(0, 0);
@@ -250,6 +343,164 @@ int gate_generator(const qs_gate_desc& g, std::vector<cd>& G, double* cfac) {
   return fail(QS_EUNSUPPORTED, "gate kind %d has no parameter gradient", g.kind);
 }
 
+// One pass of the backward walk: a gate, or a run of gates on one qubit (with the
+// controlled X taken along before or after it).
+struct AdjStep {
+  std::vector<int> gates;
+  int x = -1;
+  bool pre = false, dead = false;
+};
+
+static bool diagonal_gate(const qs_circuit* c, const qs_gate_desc& g) {
+  switch (g.kind) {
+    case QS_GATE_RX: case QS_GATE_RY: case QS_GATE_X: case QS_GATE_Y: case QS_GATE_H: return false;
+    case QS_GATE_ROT: return g.paulis[0] == 3;
+    case QS_GATE_MATRIX: return c->mats[g.mat_offset + 1] == cd(0, 0) && c->mats[g.mat_offset + 2] == cd(0, 0);
+  }
+  return true;
+}
+
+// Whether a run is worth its own pass (44 FP64 operations a pair): two gates or more,
+// one with a parameter, not all diagonal (those take 20 each).
+static bool adj_run(const qs_circuit* c, const AdjStep& u) {
+  bool diag = true, param = false;
+  for (int k : u.gates) {
+    diag = diag && diagonal_gate(c, c->gates[k]);
+    param = param || (c->gates[k].param >= 0 && c->gates[k].kind != QS_GATE_MATRIX);
+  }
+  return u.gates.size() > 1 && param && !diag;
+}
+
+// Gates first .. last - 1 as steps, in circuit order: uncontrolled single-qubit gates on
+// one qubit collect in a run (at the place of its first gate: nothing in between touches
+// the qubit); a controlled X on a run's qubit right after it, or right before it, goes
+// along with it (the run moves to the X's place, past gates on other qubits only).
+static void adj_steps(const qs_circuit* c, int first, int last, std::vector<AdjStep>& out) {
+  out.clear();
+  std::vector<int> open(c->nqubits, -1);  // the run on each qubit that takes further gates
+  for (int k = first; k < last; ++k) {
+    const qs_gate_desc& g = c->gates[k];
+    const int t = g.locs[0];
+    const bool one = g.nlocs == 1 && g.ctrl_mask == 0;
+    const bool cx = g.nlocs == 1 && g.ctrl_mask && g.kind == QS_GATE_X;
+    AdjStep* run = g.nlocs == 1 && open[t] >= 0 ? &out[open[t]] : nullptr;
+    if (one && run && (int)run->gates.size() < kAdjMembers) {
+      run->gates.push_back(k);
+      continue;
+    }
+    AdjStep u;
+    if (cx && run && run->x < 0 && adj_run(c, *run)) {
+      u = *run;
+      run->dead = true;
+    }
+    if (cx) {
+      u.x = k;
+      u.pre = u.gates.empty();
+    } else {
+      u.gates.push_back(k);
+    }
+    for (int j = 0; j < g.nlocs; ++j) open[g.locs[j]] = -1;
+    for (int q = 0; q < c->nqubits; ++q)
+      if ((g.ctrl_mask >> q) & 1) open[q] = -1;
+    if (one || (cx && u.pre)) open[t] = (int)out.size();
+    out.push_back(std::move(u));
+  }
+}
+
+namespace {
+
+struct AdjWalk {
+  qs_state* s;
+  const qs_circuit* c;
+  const double* params;
+  int n;
+  double2 *psi, *lam;
+  double *dgrad, *partials;
+  unsigned* counter;
+  std::vector<cd> U, G;
+
+  int gate(int k) {
+    const qs_gate_desc& g = c->gates[k];
+    cudaStream_t st = s->stream;
+    QS_TRY(gate_matrix(c, g, params, U));
+    dagger(U, g.nlocs);
+    if (g.param >= 0 && g.kind != QS_GATE_MATRIX) {
+      double cfac = 0;
+      QS_TRY(gate_generator(g, G, &cfac));
+      switch (g.nlocs) {
+        case 1: return launch_adjoint_param<1>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st);
+        case 2: return launch_adjoint_param<2>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st);
+        case 3: return launch_adjoint_param<3>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st);
+      }
+      return fail(QS_EUNSUPPORTED, "parameterised gate on %d targets", g.nlocs);
+    }
+    // psi and lambda are adjacent in the work buffer: one launch over both as
+    // a batch of two registers
+    Plan p;
+    QS_TRY(plan_gate(U.data(), g.nlocs, g.locs, g.ctrl_mask, g.ctrl_vals, &p));
+    return launch_plan_on(psi, QS_C128, n, 2, 1ll << n, p, s);
+  }
+
+  int run(const AdjStep& u) {
+    AdjRun F;
+    memset(&F, 0, sizeof(F));
+    // from the run's end: E is the product of the gates passed; E H E^dag is a gate's
+    // generator at the end of the run
+    cd E[4] = {1, 0, 0, 1};
+    for (size_t q = u.gates.size(); q-- > 0;) {
+      const qs_gate_desc& g = c->gates[u.gates[q]];
+      if (g.param >= 0 && g.kind != QS_GATE_MATRIX) {
+        double cfac = 0;
+        QS_TRY(gate_generator(g, G, &cfac));
+        cd M[4];
+        for (int i = 0; i < 2; ++i)
+          for (int j = 0; j < 2; ++j) {
+            cd v = 0;
+            for (int a = 0; a < 2; ++a)
+              for (int b = 0; b < 2; ++b) v += E[2 * i + a] * G[2 * a + b] * std::conj(E[2 * j + b]);
+            M[2 * i + j] = v;
+          }
+        const double f = 2.0 * cfac;
+        double* co = F.coef[F.members];
+        co[0] = f * M[0].real();
+        co[1] = f * M[3].real();
+        co[2] = f * M[1].real();
+        co[3] = -f * M[1].imag();
+        F.param[F.members++] = g.param;
+      }
+      QS_TRY(gate_matrix(c, g, params, U));
+      const cd A[4] = {E[0] * U[0] + E[1] * U[2], E[0] * U[1] + E[1] * U[3], E[2] * U[0] + E[3] * U[2],
+                       E[2] * U[1] + E[3] * U[3]};
+      std::copy(A, A + 4, E);
+    }
+    for (int i = 0; i < 2; ++i)
+      for (int j = 0; j < 2; ++j) F.ud[2 * i + j] = make_double2(E[2 * j + i].real(), -E[2 * j + i].imag());
+    const int t = c->gates[u.gates[0]].locs[0];
+    F.off1 = 1ull << t;
+    if (u.x >= 0) {
+      F.xmask = c->gates[u.x].ctrl_mask;
+      F.xval = c->gates[u.x].ctrl_vals & F.xmask;
+      F.pre = u.pre ? 1 : 0;
+    }
+    const uint64_t items = 1ull << (n - 1);
+    const int nblk = (int)std::min<uint64_t>(kAdjRunBlocks, std::max<uint64_t>(1, items / kAdjThreads));
+    k_adjoint_run<<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, t, F, partials, counter, dgrad);
+    QS_LAUNCHED();
+    return QS_OK;
+  }
+
+  int step(const AdjStep& u) {
+    if (u.dead) return QS_OK;
+    if (adj_run(c, u)) return run(u);
+    if (u.x >= 0 && !u.pre) QS_TRY(gate(u.x));
+    for (size_t q = u.gates.size(); q-- > 0;) QS_TRY(gate(u.gates[q]));
+    if (u.x >= 0 && u.pre) QS_TRY(gate(u.x));
+    return QS_OK;
+  }
+};
+
+}  // namespace
+
 int backward(qs_state* s, const qs_circuit* c, const double* params, const qs_observable* o, int ckpt_every,
              const void* ckpts, void* work, double* host_grad, double* host_loss) {
   if (s->nreg != 1) return fail(QS_EUNSUPPORTED, "qs_backward takes a single register");
@@ -263,43 +514,27 @@ int backward(qs_state* s, const qs_circuit* c, const double* params, const qs_ob
   double2* lam = psi + dim;
   const int np = std::max(1, c->nparams);
   if (host_loss) QS_TRY(expect_raw(s->data, s->dtype, n, 1, o, s, host_loss));
-  // scratch: grad[np] | partials[kAdjMaxBlocks]
-  QS_TRY(ensure_ws(s, s->ws, sizeof(double) * (np + kAdjMaxBlocks) + 256));
+  // scratch: grad[np] | partials | counter
+  constexpr int kPartials = std::max(kAdjMaxBlocks, 4 * kAdjRunBlocks);
+  QS_TRY(ensure_ws(s, s->ws, sizeof(double) * (np + kPartials) + 256));
   double* dgrad = (double*)s->ws.ptr;
   double* partials = dgrad + np;
-  unsigned* counter = reinterpret_cast<unsigned*>(partials + kAdjMaxBlocks);
+  unsigned* counter = reinterpret_cast<unsigned*>(partials + kPartials);
   QS_CUDA(cudaMemsetAsync(dgrad, 0, sizeof(double) * np, st));
   QS_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned), st));
   QS_TRY(promote_to_c128(s->data, s->dtype, psi, dim, st));
   QS_TRY(apply_observable_c128(psi, lam, n, o, st));
   const size_t ab = amp_bytes(s->dtype);
-  std::vector<cd> U, G;
-  for (int k = (int)c->gates.size() - 1; k >= 0; --k) {
-    const qs_gate_desc& g = c->gates[k];
-    if (ckpt_every > 0 && (k + 1) % ckpt_every == 0 && k + 1 < (int)c->gates.size()) {
-      const int slot = (k + 1) / ckpt_every - 1;
-      QS_TRY(promote_to_c128((const char*)ckpts + ab * dim * slot, s->dtype, psi, dim, st));
-    }
-    QS_TRY(gate_matrix(c, g, params, U));
-    dagger(U, g.nlocs);
-    if (g.param >= 0 && g.kind != QS_GATE_MATRIX) {
-      double cfac = 0;
-      QS_TRY(gate_generator(g, G, &cfac));
-      int rc;
-      switch (g.nlocs) {
-        case 1: rc = launch_adjoint_param<1>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st); break;
-        case 2: rc = launch_adjoint_param<2>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st); break;
-        case 3: rc = launch_adjoint_param<3>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st); break;
-        default: rc = fail(QS_EUNSUPPORTED, "parameterised gate on %d targets", g.nlocs);
-      }
-      QS_TRY(rc);
-    } else {
-      // psi and lambda are adjacent in the work buffer: one launch over both as
-      // a batch of two registers
-      Plan p;
-      QS_TRY(plan_gate(U.data(), g.nlocs, g.locs, g.ctrl_mask, g.ctrl_vals, &p));
-      QS_TRY(launch_plan_on(psi, QS_C128, n, 2, dim, p, s));
-    }
+  AdjWalk w{s, c, params, n, psi, lam, dgrad, partials, counter, {}, {}};
+  // segments between checkpoints, last first: psi restarts from the checkpoint at a
+  // segment's end, so no run spans one
+  const int ng = (int)c->gates.size(), every = ckpt_every > 0 ? ckpt_every : std::max(1, ng);
+  std::vector<AdjStep> steps;
+  for (int seg = ng > 0 ? (ng - 1) / every : -1; seg >= 0; --seg) {
+    const int first = seg * every, last = std::min(ng, first + every);
+    if (last < ng) QS_TRY(promote_to_c128((const char*)ckpts + ab * dim * seg, s->dtype, psi, dim, st));
+    adj_steps(c, first, last, steps);
+    for (size_t k = steps.size(); k-- > 0;) QS_TRY(w.step(steps[k]));
   }
   QS_CUDA(cudaMemcpyAsync(host_grad, dgrad, sizeof(double) * c->nparams, cudaMemcpyDeviceToHost, st));
   QS_CUDA(cudaStreamSynchronize(st));
