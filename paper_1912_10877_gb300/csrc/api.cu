@@ -111,7 +111,27 @@ struct Fuser {
   std::vector<std::vector<cd>> pend;
   std::vector<bool> has;
   bool precise = false;
+  bool small = false;       // collect plans for apply_small
+  std::vector<Plan> plans;
   explicit Fuser(qs_state* st, int n) : s(st), pend(n), has(n, false) {}
+  // applies a plan: at once, or with the others collected before the next one that the
+  // small-register path does not take
+  int emit(const Plan& p) {
+    if (!small) return launch_plan(s, p);
+    if (p.op == OP_NOP) return QS_OK;
+    if (small_plan(p)) {
+      plans.push_back(p);
+      return QS_OK;
+    }
+    QS_TRY(drain());
+    return launch_plan(s, p);
+  }
+  int drain() {
+    if (plans.empty()) return QS_OK;
+    const int rc = apply_small(s->data, s->dtype, s->nq[0], s->nreg, plans, s->stream);
+    plans.clear();
+    return rc;
+  }
   int flush(int q) {
     if (!has[q]) return QS_OK;
     has[q] = false;
@@ -119,7 +139,7 @@ struct Fuser {
     int loc = q;
     QS_TRY(plan_gate(pend[q].data(), 1, &loc, 0, 0, &p));
     p.precise = precise;
-    return launch_plan(s, p);
+    return emit(p);
   }
   int flush_mask(uint64_t m) {
     for (int q = 0; q < (int)has.size(); ++q)
@@ -194,6 +214,7 @@ static int apply_circuit_impl(qs_state* s, const qs_circuit* c, const double* pa
   }
   Fuser fz(s, c->nqubits);
   fz.precise = precise;
+  fz.small = !unfused && ckpt_every == 0 && !precise && s->uniform && small_register(s->nq[0], s->nreg);
   const size_t ab = amp_bytes(s->dtype);
   for (int k = 0; k < ng; ++k) {
     const qs_gate_desc& g = c->gates[k];
@@ -207,7 +228,7 @@ static int apply_circuit_impl(qs_state* s, const qs_circuit* c, const double* pa
       Plan p;
       QS_TRY(plan_gate(U.data(), g.nlocs, g.locs, g.ctrl_mask, g.ctrl_vals, &p));
       p.precise = precise;
-      QS_TRY(launch_plan(s, p));
+      QS_TRY(fz.emit(p));
     }
     if (ckpt_every > 0 && (k + 1) % ckpt_every == 0 && k + 1 < ng) {
       QS_TRY(fz.flush_all());  // the checkpoint holds the state after gate k exactly
@@ -216,7 +237,8 @@ static int apply_circuit_impl(qs_state* s, const qs_circuit* c, const double* pa
                               cudaMemcpyDeviceToDevice, s->stream));
     }
   }
-  return fz.flush_all();
+  QS_TRY(fz.flush_all());
+  return fz.drain();
 }
 
 }  // namespace qs

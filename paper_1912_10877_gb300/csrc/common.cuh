@@ -261,6 +261,12 @@ int launch_plan(qs_state* s, const Plan& p);
 int launch_plan_on(void* data, int dtype, int n, int nreg, int64_t reg_stride, const Plan& p,
                    qs_state* owner);
 
+// gate-by-gate application of small registers, many plans a launch (small.cu): registers
+// that take the path, plans that it applies, and the call (n <= 14)
+bool small_register(int n, int nreg);
+bool small_plan(const Plan& p);
+int apply_small(void* data, int dtype, int n, int nreg, const std::vector<Plan>& plans, cudaStream_t st);
+
 // gate matrices (FP64, row-major), generators and daggers
 int named_matrix(int kind, int k, const int32_t* paulis, double theta, std::vector<cd>& U);
 int gate_matrix(const qs_circuit* c, const qs_gate_desc& g, const double* params, std::vector<cd>& U);
