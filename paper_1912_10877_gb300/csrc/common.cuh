@@ -232,7 +232,8 @@ enum OpClass {
   OP_RXLIKE1,   // OP_DENSE1 with real diagonal, imaginary off-diagonal (Rx): half the multiply-adds
   OP_DIAGK,     // amplitude *= d[m], m = gathered target bits
   OP_PERMK,     // y[m] = v[m] x[perm[m]]
-  OP_DENSEK     // y = U x over 2^k tuples
+  OP_DENSEK,    // y = U x over 2^k tuples
+  OP_HLIKE1     // OP_REAL1 with U[0] = U[2] (H)
 };
 
 struct Plan {

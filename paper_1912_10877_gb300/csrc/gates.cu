@@ -93,6 +93,17 @@ __device__ __forceinline__ void pair_op(c2_t<R>& a, c2_t<R>& b, const U4<R>& u) 
     T na = cmul(u.m[1], b);
     T nb = cmul(u.m[2], a);
     a = na; b = nb;
+  } else if constexpr (OP == OP_HLIKE1) {
+    // u real with u0 = u2 (H): the product u0 a serves both outputs, 3 operations for two
+    // components instead of 4, with the same rounding (complex128 is bound by the FP64
+    // rate: H at n = 25 264 -> 201 us)
+    T na, nb;
+    const auto px = u.m[0].x * a.x, py = u.m[0].x * a.y;
+    na.x = fma(u.m[1].x, b.x, px);
+    na.y = fma(u.m[1].x, b.y, py);
+    nb.x = fma(u.m[3].x, b.x, px);
+    nb.y = fma(u.m[3].x, b.y, py);
+    a = na; b = nb;
   } else if constexpr (OP == OP_REAL1) {  // u real: 2 operations per component
     T na, nb;
     na.x = fma(u.m[1].x, b.x, u.m[0].x * a.x);
@@ -555,6 +566,9 @@ static int launch_typed(c2_t<R>* psi, int n, int nreg, const Plan& p, cudaStream
     case OP_PERM1: return launch_1<R, OP_PERM1>(psi, n, nreg, p, st);
     case OP_DENSE1: return launch_1<R, OP_DENSE1>(psi, n, nreg, p, st);
     case OP_REAL1: return launch_1<R, OP_REAL1>(psi, n, nreg, p, st);
+    case OP_HLIKE1:  // complex64 is bound by HBM in either form
+      if constexpr (std::is_same<R, double>::value) return launch_1<R, OP_HLIKE1>(psi, n, nreg, p, st);
+      else return launch_1<R, OP_REAL1>(psi, n, nreg, p, st);
     case OP_RXLIKE1: return launch_1<R, OP_RXLIKE1>(psi, n, nreg, p, st);
     case OP_DIAGK: return launch_k_op<R, OP_DIAGK>(psi, n, nreg, p, st);
     case OP_PERMK: return launch_k_op<R, OP_PERMK>(psi, n, nreg, p, st);
@@ -568,7 +582,8 @@ int launch_plan_on(void* data, int dtype, int n, int nreg, int64_t reg_stride, c
   (void)reg_stride;
   cudaStream_t st = owner ? owner->stream : nullptr;
   if (dtype == QS_C64 && p.precise &&
-      (p.op == OP_DIAG1 || p.op == OP_DENSE1 || p.op == OP_REAL1 || p.op == OP_RXLIKE1 || p.op == OP_PERM1 ||
+      (p.op == OP_DIAG1 || p.op == OP_DENSE1 || p.op == OP_REAL1 || p.op == OP_HLIKE1 ||
+       p.op == OP_RXLIKE1 || p.op == OP_PERM1 ||
        ((p.op == OP_DENSEK || p.op == OP_DIAGK || p.op == OP_PERMK) && p.k >= 2 && p.k <= 5)))
     return launch_prec((float2*)data, n, nreg, p, st);
   if (use_block_tc(dtype, p)) return launch_block_tc((float2*)data, n, nreg, p, st);
@@ -662,7 +677,7 @@ int plan_gate(const cd* U, int k, const int* locs, uint64_t ctrl_mask, uint64_t 
     if (perm) {
       P.op = (U[1] == cd(1, 0) && U[2] == cd(1, 0)) ? OP_SWAP1 : OP_PERM1;
     } else if (U[0].imag() == 0 && U[1].imag() == 0 && U[2].imag() == 0 && U[3].imag() == 0) {
-      P.op = OP_REAL1;
+      P.op = U[0] == U[2] ? OP_HLIKE1 : OP_REAL1;
     } else if (U[0].imag() == 0 && U[3].imag() == 0 && U[1].real() == 0 && U[2].real() == 0) {
       P.op = OP_RXLIKE1;
     } else {

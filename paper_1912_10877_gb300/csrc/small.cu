@@ -197,7 +197,7 @@ bool small_op(const Plan& p, SmallOp<R>* o) {
       return true;
     case OP_SWAP1: o->kind = SM_SWAP; break;
     case OP_PERM1: o->kind = SM_PERM; break;
-    case OP_REAL1: o->kind = SM_REAL; break;
+    case OP_REAL1: case OP_HLIKE1: o->kind = SM_REAL; break;
     case OP_RXLIKE1: o->kind = SM_RX; break;
     case OP_DENSE1: o->kind = SM_DENSE; break;
     default: return false;
