@@ -395,7 +395,11 @@ int qs_apply_circuit(qs_state* s, const qs_circuit* c, const double* host_params
  * dev_out[0] (device).  Every grid-barrier wait is bounded; a wait that gives
  * up leaves the state unspecified and makes the next qs_state_sync return
  * QS_ETIMEDOUT.  Asynchronous on s's stream; uses s's scratch (a second state
- * buffer and the block tables). */
+ * buffer and the block tables).  With grid_ctas = 0 a circuit of single-target
+ * gates (controls allowed, a gate spanning at most QS_MAXK qubits) and
+ * uncontrolled SWAPs on up to 14 qubits runs in one thread-block cluster
+ * instead, gate by gate (runs of uncontrolled gates fused, kmax unused;
+ * complex64 gates compensated as with QS_APPLY_PRECISE), without scratch. */
 int qs_run_circuit_one_launch(qs_state* s, const qs_circuit* c, const double* host_params, int kmax,
                               const qs_observable* o, int grid_ctas, double* dev_out);
 

@@ -419,6 +419,7 @@ int qs_circuit_destroy(qs_circuit* c) {
   if (c && c->fused) free_fused(c->fused);
   if (c) free_blocks(c);
   if (c) free_onelaunch(c);
+  if (c) free_smallrun(c);
   delete c;
   return QS_OK;
 }

@@ -206,6 +206,8 @@ struct qs_circuit {
   // device tables of the one-launch path (built on first use, rebuilt when the
   // block width, dtype, device or parameters change)
   mutable void* onelaunch = nullptr;
+  // fused ops of the one-cluster path (rebuilt as the above)
+  mutable void* smallrun = nullptr;
 };
 
 struct qs_observable {
@@ -282,6 +284,10 @@ bool use_block_tc(int dtype, const Plan& p);
 int launch_block_tc(float2* psi, int n, int nreg, const Plan& p, cudaStream_t st);
 int tc_status_take();  // QS_ETIMEDOUT (and clears it) if a bounded device wait gave up
 int tc_status_address(int** out);  // device address of that status word (current device)
+// a circuit of single-target gates on a small register in one cluster (smallrun.cu)
+int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* params, const qs_observable* o,
+                      double* dev_out, cudaStream_t st);
+void free_smallrun(const qs_circuit* c);
 void free_onelaunch(const qs_circuit* c);  // releases the one-launch tables of a circuit
 // real Gram matrix sum_x psi_x^T lambda_x of a 4/5-qubit support on the tensor cores
 // (interleaved re/im layout), per-CTA partials [grid][W][W]

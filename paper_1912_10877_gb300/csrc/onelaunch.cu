@@ -342,6 +342,11 @@ int qs_run_circuit_one_launch(qs_state* s, const qs_circuit* c, const double* ho
       ++a.nterm;
     }
   }
+  // single-target gates on up to 14 qubits, every SM asked for: one cluster
+  if (grid_ctas <= 0) {
+    const int rc = run_small_circuit(s->data, s->dtype, c, host_params, o, dev_out, s->stream);
+    if (rc != QS_EUNSUPPORTED) return rc;
+  }
   OLCache* k = nullptr;
   QS_TRY(onelaunch_tables(s, c, host_params, kmax, &k));
   const int nb = k->nb;
