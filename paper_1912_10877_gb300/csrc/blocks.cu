@@ -171,6 +171,23 @@ void left_multiply(std::vector<cd>& M, int w, const std::vector<cd>& U, int k, c
   for (int m = 0; m < Dk; ++m)
     for (int j = 0; j < k; ++j)
       if ((m >> j) & 1) off[m] |= 1u << tpos[j];
+  if (k == 1) {  // two rows at a time, in plain arithmetic along them
+    const double a = U[0].real(), ai = U[0].imag(), b = U[1].real(), bi = U[1].imag();
+    const double c = U[2].real(), ci = U[2].imag(), d = U[3].real(), di = U[3].imag();
+    for (uint32_t x = 0; x < (uint32_t)Dw; ++x) {
+      if ((x & tmask) || (x & cmask) != cval) continue;
+      double* r0 = reinterpret_cast<double*>(&M[(size_t)x * Dw]);
+      double* r1 = reinterpret_cast<double*>(&M[(size_t)(x | tmask) * Dw]);
+      for (int j = 0; j < 2 * Dw; j += 2) {
+        const double p = r0[j], pi = r0[j + 1], q = r1[j], qi = r1[j + 1];
+        r0[j] = (a * p - ai * pi) + (b * q - bi * qi);
+        r0[j + 1] = (a * pi + ai * p) + (b * qi + bi * q);
+        r1[j] = (c * p - ci * pi) + (d * q - di * qi);
+        r1[j + 1] = (c * pi + ci * p) + (d * qi + di * q);
+      }
+    }
+    return;
+  }
   std::vector<cd> v(Dk);
   for (int col = 0; col < Dw; ++col)
     for (uint32_t x = 0; x < (uint32_t)Dw; ++x) {
@@ -640,6 +657,95 @@ int gram(int w, const void* psi, const void* lam, int n, const std::vector<int>&
   return fail(QS_EUNSUPPORTED, "block of %d qubits", w);
 }
 
+// ---- a block's gradients from its rho, on the device
+//
+// The host walked every block's gates over its rho after the last launch, some 8 us a
+// gate with the GPU idle (10 ms for the brickwork of 26 qubits).  Blocks of single-target
+// gates walk theirs in one launch, a CTA a block, all blocks at once: rho in shared
+// memory, in FP64 as there.  Bound by the FP64 rate of one SM a block (16 K operations a
+// dense gate on 5 qubits, 5 us).
+struct BGate {
+  double2 u[4];       // the gate
+  double2 h[4];       // its generator
+  double f;           // 2 c
+  uint32_t cmask, cval;
+  int t, out, diag;   // block bit; place of its derivative (-1: no parameter)
+  int pad;
+};
+struct BRho {
+  int64_t off;        // into the Gram matrices
+  int w, tc, g0, ng;  // width, layout, its gates
+};
+
+__global__ void __launch_bounds__(256) k_block_grads(const double* __restrict__ grams, const BRho* __restrict__ blocks,
+                                                     const BGate* __restrict__ gates, double* __restrict__ out) {
+  __shared__ double2 rho[32 * 32];
+  const BRho B = blocks[blockIdx.x];
+  const int w = B.w, D = 1 << w, W2 = 2 * D, tid = threadIdx.x;
+  const double* g2 = grams + B.off;
+  auto re = [&](int p) { return B.tc ? 2 * p : p; };
+  auto im = [&](int p) { return B.tc ? 2 * p + 1 : D + p; };
+  for (int e = tid; e < D * D; e += 256) {
+    const int p = e >> w, q = e & (D - 1);
+    rho[e] = make_double2(g2[re(p) * W2 + re(q)] + g2[im(p) * W2 + im(q)],
+                          g2[im(p) * W2 + re(q)] - g2[re(p) * W2 + im(q)]);
+  }
+  __syncthreads();
+  for (int k = B.ng - 1; k >= 0; --k) {
+    const BGate& g = gates[B.g0 + k];
+    const int t = g.t, bit = 1 << t;
+    const uint32_t cm = g.cmask, cv = g.cval;
+    auto at = [&](int j) { return ((j >> t) << (t + 1)) | (j & (bit - 1)); };  // j-th index with bit t = 0
+    if (g.out >= 0 && tid < 32) {  // Im Tr(H rho) over the pairs where the controls hold
+      double v = 0.0;
+      if (tid < D / 2) {
+        const int x = at(tid), y = x | bit;
+        if ((x & cm) == cv) {
+          const double2 a = cmul(g.h[0], rho[x * D + x]), b = cmul(g.h[1], rho[y * D + x]);
+          const double2 c = cmul(g.h[2], rho[x * D + y]), d = cmul(g.h[3], rho[y * D + y]);
+          v = (a.y + b.y) + (c.y + d.y);
+        }
+      }
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (tid == 0) out[g.out] = g.f * v;
+    }
+    if (k == 0) break;
+    __syncthreads();
+    // rho <- G^dag rho G
+    if (g.diag) {
+      for (int e = tid; e < D * D; e += 256) {
+        const int p = e >> w, q = e & (D - 1);
+        double2 v = rho[e];
+        if ((p & cm) == cv) {
+          const double2 d = (p & bit) ? g.u[3] : g.u[0];
+          v = cmul(make_double2(d.x, -d.y), v);
+        }
+        if ((q & cm) == cv) v = cmul((q & bit) ? g.u[3] : g.u[0], v);
+        rho[e] = v;
+      }
+      __syncthreads();
+      continue;
+    }
+    auto conj = [](double2 v) { return make_double2(v.x, -v.y); };
+    for (int e = tid; e < D * D / 2; e += 256) {
+      const int q = e & (D - 1), p = at(e >> w);
+      if ((p & cm) != cv) continue;
+      const double2 a = rho[p * D + q], b = rho[(p | bit) * D + q];
+      rho[p * D + q] = cfma(conj(g.u[2]), b, cmul(conj(g.u[0]), a));
+      rho[(p | bit) * D + q] = cfma(conj(g.u[3]), b, cmul(conj(g.u[1]), a));
+    }
+    __syncthreads();
+    for (int e = tid; e < D * D / 2; e += 256) {
+      const int p = e & (D - 1), q = at(e >> w);
+      if ((q & cm) != cv) continue;
+      const double2 a = rho[p * D + q], b = rho[p * D + (q | bit)];
+      rho[p * D + q] = cfma(g.u[2], b, cmul(g.u[0], a));
+      rho[p * D + (q | bit)] = cfma(g.u[3], b, cmul(g.u[1], a));
+    }
+    __syncthreads();
+  }
+}
+
 // H embedded in the block space: acts as H on the targets where the controls
 // match, and as zero elsewhere (the control projector)
 void embed_generator(const std::vector<cd>& H, int k, const int* tpos, uint32_t cmask, uint32_t cval, int w,
@@ -687,9 +793,16 @@ int backward_blocks(qs_state* s, const qs_circuit* c, const double* params, cons
   if (c->nparams > 0 && !params) return fail(QS_EINVAL, "params is NULL");
   const std::vector<Block>& blocks = cached_blocks(c, kmax);
   const int nb = (int)blocks.size();
+  const bool f32 = s->dtype == QS_C64;
   // which blocks need rho, and where it goes in device scratch
   std::vector<int64_t> rho_off(nb, -1);
   std::vector<char> rho_tc(nb, 0);  // rho of this block came from the tensor cores (interleaved layout)
+  std::vector<char> on_gpu(nb, 0);  // its gradients are worked out by k_block_grads
+  std::vector<BGate> bgates;
+  std::vector<BRho> brhos;
+  std::vector<int> bparam;          // parameter of each derivative k_block_grads writes
+  std::vector<cd> U, H;
+  bool host_rho = false;
   int64_t rho_total = 0;
   for (int bi = 0; bi < nb; ++bi) {
     const Block& b = blocks[bi];
@@ -699,10 +812,43 @@ int backward_blocks(qs_state* s, const qs_circuit* c, const double* params, cons
     if (has_param) {
       rho_off[bi] = rho_total;
       rho_total += (int64_t)4 << (2 * popc(b.support));
+      bool single = true;
+      for (int gi : b.gates) single = single && c->gates[gi].nlocs == 1;
+      on_gpu[bi] = single;
+      host_rho = host_rho || !single;
+      if (!single) continue;
+      int pos[64], w = 0;
+      for (int q = 0; q < 64; ++q)
+        if ((b.support >> q) & 1ull) pos[q] = w++;
+      brhos.push_back(BRho{rho_off[bi], w, f32 && (w == 4 || w == 5) && tensor_cores_enabled(), (int)bgates.size(),
+                           (int)b.gates.size()});
+      for (int gi : b.gates) {
+        const qs_gate_desc& g = c->gates[gi];
+        BGate o;
+        std::memset(&o, 0, sizeof(o));
+        QS_TRY(gate_matrix(c, g, params, U));
+        for (int k = 0; k < 4; ++k) o.u[k] = make_double2(U[k].real(), U[k].imag());
+        o.diag = U[1] == cd(0, 0) && U[2] == cd(0, 0);
+        o.t = pos[g.locs[0]];
+        o.out = -1;
+        for (int q = 0; q < 64; ++q)
+          if ((g.ctrl_mask >> q) & 1ull) {
+            o.cmask |= 1u << pos[q];
+            if ((g.ctrl_vals >> q) & 1ull) o.cval |= 1u << pos[q];
+          }
+        if (g.param >= 0 && g.kind != QS_GATE_MATRIX) {
+          double cfac = 0;
+          QS_TRY(gate_generator(g, H, &cfac));
+          for (int k = 0; k < 4; ++k) o.h[k] = make_double2(H[k].real(), H[k].imag());
+          o.f = 2.0 * cfac;
+          o.out = (int)bparam.size();
+          bparam.push_back(g.param);
+        }
+        bgates.push_back(o);
+      }
     }
   }
   cudaStream_t st = s->stream;
-  const bool f32 = s->dtype == QS_C64;
   const uint64_t dim = 1ull << n;
   if (host_loss) QS_TRY(expect_raw(s->data, s->dtype, n, 1, o, s, host_loss));
   void* lam = work;
@@ -711,9 +857,18 @@ int backward_blocks(qs_state* s, const qs_circuit* c, const double* params, cons
   QS_CUDA(cudaGetDevice(&dev));
   QS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const size_t npart = gram_partials_doubles(sms);
-  QS_TRY(ensure_ws(s, s->ws, sizeof(double) * (npart + (size_t)rho_total) + 256));
+  const size_t nout = bparam.size(), gate_off = (sizeof(double) * (npart + (size_t)rho_total + nout) + 15) / 16 * 16;
+  const size_t block_off = gate_off + sizeof(BGate) * bgates.size();
+  QS_TRY(ensure_ws(s, s->ws, block_off + sizeof(BRho) * brhos.size() + 256));
   double* partials = (double*)s->ws.ptr;
   double* rhos = partials + npart;
+  double* dout = rhos + rho_total;
+  const BGate* dgates = (const BGate*)((char*)s->ws.ptr + gate_off);
+  const BRho* dblocks = (const BRho*)((char*)s->ws.ptr + block_off);
+  if (!brhos.empty()) {
+    QS_CUDA(cudaMemcpyAsync((void*)dgates, bgates.data(), sizeof(BGate) * bgates.size(), cudaMemcpyHostToDevice, st));
+    QS_CUDA(cudaMemcpyAsync((void*)dblocks, brhos.data(), sizeof(BRho) * brhos.size(), cudaMemcpyHostToDevice, st));
+  }
   // device pass: per block, rho (if it has parameters) then the uncompute; no host round trip
   std::vector<int> qubits;
   std::vector<cd> M;
@@ -750,16 +905,22 @@ int backward_blocks(qs_state* s, const qs_circuit* c, const double* params, cons
     QS_TRY(launch_plan_on(s->data, s->dtype, n, 1, (int64_t)dim, p, s));
     QS_TRY(launch_plan_on(lam, s->dtype, n, 1, (int64_t)dim, p, s));
   }
-  std::vector<double> G2((size_t)std::max<int64_t>(1, rho_total));
-  if (rho_total > 0)
+  std::vector<double> G2((size_t)std::max<int64_t>(1, host_rho ? rho_total : 0)), dev_out(std::max<size_t>(1, nout));
+  if (!brhos.empty()) {
+    k_block_grads<<<(unsigned)brhos.size(), 256, 0, st>>>(rhos, dblocks, dgates, dout);
+    QS_LAUNCHED();
+    QS_CUDA(cudaMemcpyAsync(dev_out.data(), dout, sizeof(double) * nout, cudaMemcpyDeviceToHost, st));
+  }
+  if (host_rho)
     QS_CUDA(cudaMemcpyAsync(G2.data(), rhos, sizeof(double) * rho_total, cudaMemcpyDeviceToHost, st));
   QS_CUDA(cudaStreamSynchronize(st));
   QS_TRY(tc_status_take());
-  // host: every block's gradients from its rho (FP64)
   std::vector<double> grad(std::max(1, c->nparams), 0.0);
-  std::vector<cd> U, H, Hemb, rho;
+  for (size_t k = 0; k < nout; ++k) grad[bparam[k]] += dev_out[k];
+  // host: the gradients of the blocks with multi-target gates from their rho (FP64)
+  std::vector<cd> Hemb, rho;
   for (int bi = 0; bi < nb; ++bi) {
-    if (rho_off[bi] < 0) continue;
+    if (rho_off[bi] < 0 || on_gpu[bi]) continue;
     const Block& b = blocks[bi];
     qubits.clear();
     for (int q = 0; q < 64; ++q)
