@@ -2130,7 +2130,8 @@ struct qs_batch_program {
   std::vector<int64_t> param_off;    // nreg + 1
   std::vector<int64_t> amp_off;      // nreg + 1
   int64_t work_elems = 0;
-  // device tables
+  // device tables (one allocation)
+  void* tables = nullptr;
   qs::BReg* regs = nullptr;
   int32_t* order = nullptr;
   qs::TPass* passes = nullptr;
@@ -2160,6 +2161,7 @@ struct qs_batch_program {
   int rb = qs::kRB;
   int tile = 0;
   bool precise = false;
+  bool forward_only = false;  // no tables and buffers for a backward pass
   float2* flo = nullptr;   // corrections of the forward ops (4 per op)
   float2* blo = nullptr;   // corrections of the backward ops (4 per op)
   float2* dtlo = nullptr;  // corrections of the diagonal tables (16 per table)
@@ -2198,17 +2200,37 @@ static int gen_of(int kind, float* cfac2) {
   return GEN_NONE;
 }
 
-template <typename T>
-static int upload(T** dst, const std::vector<T>& v) {
-  const size_t bytes = sizeof(T) * std::max<size_t>(1, v.size());
-  if (cudaMalloc((void**)dst, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    *dst = nullptr;
-    return fail(QS_ENOMEM, "cudaMalloc of %zu program bytes failed", bytes);
+// The program's tables in one device allocation (an allocation and a free a table were a
+// third of the time a program of 240 registers took to make)
+struct TableSet {
+  struct Item {
+    void** dst;
+    const void* src;  // NULL: written on the device
+    size_t bytes, at;
+  };
+  std::vector<Item> items;
+  size_t total = 0;
+  template <typename T>
+  void add(T** dst, const std::vector<T>& v) { put((void**)dst, v.empty() ? nullptr : v.data(), sizeof(T) * v.size()); }
+  template <typename T>
+  void room(T** dst, size_t count) { put((void**)dst, nullptr, sizeof(T) * count); }
+  void put(void** dst, const void* src, size_t bytes) {
+    items.push_back(Item{dst, src, bytes, total});
+    total += (std::max<size_t>(bytes, 1) + 255) / 256 * 256;
   }
-  if (!v.empty()) QS_CUDA(cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice));
-  return QS_OK;
-}
+  int upload(void** base) {
+    if (cudaMalloc(base, total) != cudaSuccess) {
+      cudaGetLastError();
+      *base = nullptr;
+      return fail(QS_ENOMEM, "cudaMalloc of %zu program bytes failed", total);
+    }
+    for (const Item& i : items) {
+      *i.dst = (char*)*base + i.at;
+      if (i.src) QS_CUDA(cudaMemcpy(*i.dst, i.src, i.bytes, cudaMemcpyHostToDevice));
+    }
+    return QS_OK;
+  }
+};
 
 static void free_program(qs_batch_program* p) {
   if (!p) return;
@@ -2216,9 +2238,7 @@ static void free_program(qs_batch_program* p) {
   int cur = -1;
   const bool swap = p->device >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != p->device &&
                     cudaSetDevice(p->device) == cudaSuccess;
-  void* ptrs[] = {p->regs, p->order, p->passes, p->phases, p->fops, p->bops, p->terms, p->gspec, p->fmem,
-                  p->bmem, p->gmem, p->dmem, p->dref, p->dtab, p->counter, p->wpsi, p->wlam, p->dparams,
-                  p->flo, p->blo, p->dtlo, p->wpsif, p->wlamf, p->druns, p->tabent, p->tabs, p->runs, p->rtab};
+  void* ptrs[] = {p->tables, p->wpsi, p->wlam, p->dparams, p->flo, p->blo, p->dtlo, p->wpsif, p->wlamf};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   if (swap) cudaSetDevice(cur);
@@ -2757,7 +2777,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
           gmem.push_back(q);
         };
         for (const BGroup& u : pb) {
-          if (u.dead) continue;
+          if (u.dead || plain) continue;  // a plain program runs forward only
           FMem fm;
           memset(&fm, 0, sizeof(fm));
           fm.rec0 = -1;
@@ -2857,30 +2877,33 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   P->npass = (int64_t)passes.size();
   P->nphase = (int64_t)phases.size();
   P->work_elems = work;
-  QS_TRY(upload(&P->regs, regs));
-  QS_TRY(upload(&P->order, order));
-  QS_TRY(upload(&P->passes, passes));
-  QS_TRY(upload(&P->phases, phases));
-  QS_TRY(upload(&P->fops, fops));
-  QS_TRY(upload(&P->bops, bops));
-  QS_TRY(upload(&P->terms, terms));
-  QS_TRY(upload(&P->gspec, gspec));
-  QS_TRY(upload(&P->fmem, fmem));
-  QS_TRY(upload(&P->bmem, bmem));
-  QS_TRY(upload(&P->gmem, gmem));
-  QS_TRY(upload(&P->dmem, dmems));
-  QS_TRY(upload(&P->dref, drefs));
   P->ndiag = (int)drefs.size();
   P->ndrun = (int)druns.size();
   P->nrun = (int)runs.size();
-  QS_TRY(upload(&P->druns, druns.empty() ? std::vector<DRun>(1) : druns));
-  QS_TRY(upload(&P->tabent, tabent));
-  QS_TRY(upload(&P->tabs, tabs));
-  QS_TRY(upload(&P->runs, runs));
-  QS_TRY(upload(&P->rtab, std::vector<float4>((size_t)kRunTab * runs.size())));
-  QS_TRY(upload(&P->dtab, std::vector<float2>(16 * std::max<size_t>(1, drefs.size()))));
-  QS_TRY(upload(&P->counter, std::vector<int>(1, 0)));
-  if (work > 0 && !precise) {
+  TableSet tab;
+  tab.add(&P->regs, regs);
+  tab.add(&P->order, order);
+  tab.add(&P->passes, passes);
+  tab.add(&P->phases, phases);
+  tab.add(&P->fops, fops);
+  tab.add(&P->bops, bops);
+  tab.add(&P->terms, terms);
+  tab.add(&P->gspec, gspec);
+  tab.add(&P->fmem, fmem);
+  tab.add(&P->bmem, bmem);
+  tab.add(&P->gmem, gmem);
+  tab.add(&P->dmem, dmems);
+  tab.add(&P->dref, drefs);
+  tab.add(&P->druns, druns);
+  tab.add(&P->tabent, tabent);
+  tab.add(&P->tabs, tabs);
+  tab.add(&P->runs, runs);
+  tab.room(&P->rtab, (size_t)kRunTab * runs.size());
+  tab.room(&P->dtab, 16 * drefs.size());
+  tab.room(&P->counter, 1);
+  QS_TRY(tab.upload(&P->tables));
+  P->forward_only = plain;
+  if (work > 0 && !precise && !plain) {
     if (cudaMalloc(&P->wpsi, sizeof(float2) * work) != cudaSuccess ||
         cudaMalloc(&P->wlam, sizeof(float2) * work) != cudaSuccess) {
       cudaGetLastError();
@@ -3328,7 +3351,7 @@ int qs_batch_program_create(int nreg, const qs_circuit* const* circuits, const q
 
 }  // extern "C"
 
-// A program whose forward pass applies the gates without moving a run past gates on other
+// A forward-only program that applies the gates without moving a run past gates on other
 // qubits to an X that it could take along, in phases cut at the same gates whatever the
 // later engine's limits: the last bits of its amplitudes, and with them the samples that a
 // shot-based estimate counts, are those of the plain order.
@@ -3456,6 +3479,7 @@ int qs_batch_run(qs_state* s, const qs_batch_program* p, const double* dev_param
   if (p->param_off[p->nreg] > 0 && !dev_params) return fail(QS_EINVAL, "params is NULL");
   const bool grad = (flags & QS_BATCH_GRAD) != 0;
   if (grad && !dev_grad) return fail(QS_EINVAL, "grad is NULL");
+  if (grad && p->forward_only) return fail(QS_EINVAL, "a forward-only program has no gradient");
   int dev = 0;
   QS_CUDA(cudaGetDevice(&dev));
   if (dev != p->device)

@@ -411,27 +411,24 @@ int qs_faithful_gradient(const qs_circuit* c, const double* params, const qs_obs
     }
   int rc = QS_OK;
   bool done = false;
+  qs_batch_program* prog = nullptr;
+  double* dparams = nullptr;
   if (dtype == QS_C64 && n >= 5) {
     // one persistent launch for all 2P registers when the circuit fits the batched engine
     std::vector<const qs_circuit*> cs(R, c);
     qs_observable empty;
     std::vector<const qs_observable*> os(R, &empty);
-    qs_batch_program* prog = nullptr;
     if (batch_program_plain(R, cs.data(), os.data(), &prog) == QS_OK) {
-      double* dparams = nullptr;
       if (cudaMalloc(&dparams, sizeof(double) * (pm.size() + R)) == cudaSuccess) {
-        rc = qs_state_reset(st, nullptr);
-        if (rc == QS_OK && cudaMemcpyAsync(dparams, pm.data(), sizeof(double) * pm.size(), cudaMemcpyHostToDevice,
-                                           (cudaStream_t)stream) != cudaSuccess)
+        if (cudaMemcpyAsync(dparams, pm.data(), sizeof(double) * pm.size(), cudaMemcpyHostToDevice,
+                            (cudaStream_t)stream) != cudaSuccess)
           rc = fail(QS_EDEVICE, "parameter upload failed");
         if (rc == QS_OK) rc = qs_batch_run(st, prog, dparams, dparams + pm.size(), nullptr, QS_BATCH_RESET);
-        if (rc == QS_OK) rc = qs_state_sync(st);
-        cudaFree(dparams);
         done = rc == QS_OK;
       } else {
         cudaGetLastError();
+        dparams = nullptr;
       }
-      qs_batch_program_destroy(prog);
     }
   }
   if (!done && rc == QS_OK) {
@@ -440,7 +437,10 @@ int qs_faithful_gradient(const qs_circuit* c, const double* params, const qs_obs
   }
   std::vector<double> E(R, 0.0);
   if (rc == QS_OK) rc = nshots > 0 ? shot_expect(st, o, host_u, nshots, dev_work, E.data()) : qs_expect(st, o, E.data());
-  qs_state_destroy(st);
+  if (rc == QS_OK && done) rc = qs_state_sync(st);  // the batch's own status
+  qs_state_destroy(st);  // waits for the stream: the program and its parameters are free to go
+  if (dparams) cudaFree(dparams);
+  if (prog) qs_batch_program_destroy(prog);
   if (rc != QS_OK) return rc;
   for (int k = 0; k < P; ++k) host_grad[k] = 0.5 * (E[2 * k] - E[2 * k + 1]);
   return QS_OK;
