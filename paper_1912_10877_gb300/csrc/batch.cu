@@ -276,8 +276,8 @@ struct RunCtx {
 
 // a TK_DIAGRUN op: the products p0, p1 of its entries' factors, then one pass over the
 // amplitudes by phase bit t.  The table look-ups replace up to n - 4 entries tested and
-// multiplied by every thread (QFT of 29 qubits,
-// first pass: 20.7 -> 11.0 ms, with the phases no longer cut at 64 gates).
+// multiplied by every thread (QFT of 29 qubits, first pass: 20.7 -> 11.0 ms, with the
+// phases no longer cut at 64 gates).
 template <int RB>
 __device__ __forceinline__ void diag_run(float2 (&x)[1 << RB], const TOp& op, const RunCtx& rc, uint32_t gb) {
   const int run = __float_as_int(op.cfac2);
@@ -309,6 +309,39 @@ __device__ __forceinline__ void diag_run(float2 (&x)[1 << RB], const TOp& op, co
       case 1: mul_by_bit<RB, 1>(x, p0, p1); break;
       case 2: if constexpr (RB > 2) mul_by_bit<RB, 2>(x, p0, p1); break;
       default: if constexpr (RB > 3) mul_by_bit<RB, 3>(x, p0, p1); break;
+    }
+  }
+}
+
+// A TK_REALRUN op: the layer of one qubit of a QFT (H, then the controlled phases on it) in
+// one dispatch.  Bound by instruction issue: H, table and run as ops of their own took 490
+// instructions a thread for the 16 amplitudes, two thirds of them record loads, jumps and
+// register moves, and multiplied the 8 amplitudes that the table leaves alone as well
+// (QFT of 29 qubits: 26.3 -> 20.6 ms; its passes 11.0, 7.3, 6.4 -> 7.5, 5.1, 5.4).
+template <int RB, int T>
+__device__ __forceinline__ void real_run(float2 (&x)[1 << RB], const TOp& op, const RunCtx& rc, const float2* dtab,
+                                         uint32_t gb) {
+  if constexpr (T < RB) {
+    const int run = __float_as_int(op.cfac2);
+    const float4* tab = rc.tab + run * kRunTab;
+    const float4 a = tab[threadIdx.x & 31], b = tab[32 + (threadIdx.x >> 5)];
+    float2 p = cmulf(make_float2(a.z, a.w), make_float2(b.z, b.w));
+    uint32_t k = 0;
+    if (rc.tile) {
+      const float4 t = rc.tile[run];
+      p = cmulf(p, make_float2(t.z, t.w));
+      k = op.shared;
+    }
+    float2 p0 = make_float2(1.f, 0.f);  // stays 1
+    for (; k < op.count; ++k) run_entry(rc.entries + op.param + k, gb, p0, p);
+    op_fwd<RB, T, TK_REAL, false>(x, op);
+    if (op.pad) {
+      const float2* d = dtab + 16 * (op.pad - 1);
+#pragma unroll
+      for (int j = 1 << T; j < (1 << RB); ++j)
+        if ((j >> T) & 1) x[j] = cmulf(x[j], cmulf(p, __ldg(d + j)));
+    } else {
+      mul_bit1<RB, T>(x, p);
     }
   }
 }
@@ -1015,6 +1048,7 @@ __device__ __forceinline__ TOp load_op(const TOp* p) {
   r.tmask = b.x;
   r.tval = b.y;
   r.count = b.z;
+  r.pad = b.w;
   r.u[0] = make_float2(__uint_as_float(c.x), __uint_as_float(c.y));
   r.u[1] = make_float2(__uint_as_float(c.z), __uint_as_float(c.w));
   r.u[2] = make_float2(__uint_as_float(d.x), __uint_as_float(d.y));
@@ -1121,6 +1155,17 @@ __device__ __forceinline__ void phase_fwd_body(float2* sm, const TPhase* php, co
         continue;
       }
       if (!on) continue;
+      if constexpr (!COMP && !RESLOT) {
+        if (cur.kind == TK_REALRUN) {
+          switch (cur.t) {
+            case 0: real_run<RB, 0>(x, cur, rc, dtab, gb); break;
+            case 1: real_run<RB, 1>(x, cur, rc, dtab, gb); break;
+            case 2: real_run<RB, 2>(x, cur, rc, dtab, gb); break;
+            default: real_run<RB, 3>(x, cur, rc, dtab, gb); break;
+          }
+          continue;
+        }
+      }
       if (cur.kind == TK_DIAGOUT) {
         const bool b1 = (gb >> cur.t) & 1u;
         const float2 f = b1 ? cur.u[3] : cur.u[0];
@@ -2271,6 +2316,24 @@ static uint8_t fwd_variant(const TOp& f) {
   }
 }
 
+// gates whose product is a real 2x2
+static bool real_gates(const std::vector<GSpec>& gspec, const FMem& fm) {
+  for (int k = 0; k < fm.count; ++k) {
+    const GSpec& gs = gspec[fm.g[k]];
+    if (!(gs.kind == QS_GATE_H || gs.kind == QS_GATE_RY || gs.kind == QS_GATE_X || gs.kind == QS_GATE_Z ||
+          gs.kind == QS_GATE_I ||
+          (gs.kind == QS_GATE_MATRIX && gs.mat[0].y == 0 && gs.mat[1].y == 0 && gs.mat[2].y == 0 && gs.mat[3].y == 0)))
+      return false;
+  }
+  return true;
+}
+
+// diagonal gates with the first entry exactly 1: factors on the target's 1 only
+static bool unit_first(int kind) {
+  return kind == QS_GATE_SHIFT || kind == QS_GATE_Z || kind == QS_GATE_S || kind == QS_GATE_SDG || kind == QS_GATE_T ||
+         kind == QS_GATE_TDG || kind == QS_GATE_I;
+}
+
 // Gradient sums a phase may have.  The tiled gradient keeps them beside a double per
 // parameter in shared memory: circuits that nearly fill it keep to one sum a gate.
 static int phase_vals(int nparams) { return nparams > 11000 ? kMaxPhaseOps : kMaxPhaseVals; }
@@ -2737,12 +2800,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
             part[kind == 2 && part[2].size() >= 255 ? 3 : kind].push_back(f);
           }
           bool one0 = true;
-          for (const DRun& e : run_ent[r]) {
-            const int k = gspec[e.gate].kind;
-            one0 = one0 && e.tq == 0xffffffffu &&
-                   (k == QS_GATE_SHIFT || k == QS_GATE_Z || k == QS_GATE_S || k == QS_GATE_SDG || k == QS_GATE_T ||
-                    k == QS_GATE_TDG || k == QS_GATE_I);
-          }
+          for (const DRun& e : run_ent[r]) one0 = one0 && e.tq == 0xffffffffu && unit_first(gspec[e.gate].kind);
           const int run = (int)runs.size() - tp.run0;
           ro.param = (int)druns.size() - tp.drun0;
           ro.count = (uint32_t)(part[2].size() + part[3].size());
@@ -2753,6 +2811,48 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
           tabs.push_back(make_int4((int)tabent.size(), (int)part[0].size(), (int)part[1].size(), 0));
           for (int k = 0; k < 2; ++k) tabent.insert(tabent.end(), part[k].begin(), part[k].end());
           for (int k = 2; k < 4; ++k) druns.insert(druns.end(), part[k].begin(), part[k].end());
+        }
+        // tile engine: a real 2x2, a run on its bit and a table of gates on its bit, next to
+        // each other, become one op when both multiply only where the bit is 1
+        if (P->fused_only && rb == kRB) {
+          int at = -1, tbl = -1, run = -1;  // the 2x2 and what follows it so far
+          auto close = [&] {
+            if (at >= 0 && run >= 0) {
+              TOp& h = pf[at];
+              const TOp& r = pf[run];
+              h.kind = TK_REALRUN;
+              h.param = r.param;
+              h.count = r.count;
+              h.shared = r.shared;
+              h.cfac2 = r.cfac2;
+              h.pad = tbl >= 0 ? pf[tbl].param + 1 : 0;
+              pf[run].kind = kDead;
+              if (tbl >= 0) pf[tbl].kind = kDead;
+            }
+            at = tbl = run = -1;
+          };
+          for (int k = 0; k < (int)pf.size(); ++k) {
+            const TOp& o = pf[k];
+            if (o.kind == kDead) continue;
+            if (at >= 0 && run < 0 && o.kind == TK_DIAGRUN && o.t == pf[at].t && o.gen == 1) {
+              run = k;
+              continue;
+            }
+            if (at >= 0 && tbl < 0 && o.kind == TK_DIAG16) {
+              const DRef d = drefs[o.param];
+              const int bit = 1 << pf[at].t;
+              bool on1 = true;
+              for (int q = d.mem0; q < d.mem0 + d.count; ++q)
+                on1 = on1 && ((dmems[q].cm & dmems[q].cv & bit) || (dmems[q].tb == pf[at].t && unit_first(gspec[dmems[q].g].kind)));
+              if (on1) {
+                tbl = k;
+                continue;
+              }
+            }
+            close();
+            if (o.kind == TK_DENSE && !o.cmask && !o.tmask && real_gates(gspec, pm[k])) at = k;
+          }
+          close();
         }
         for (size_t k = 0; k < pf.size(); ++k) {
           if (pf[k].kind == kDead) continue;
@@ -2858,14 +2958,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   for (size_t i = 0; i < fops.size(); ++i) {
     TOp& f = fops[i];
     f.var = fwd_variant(f);
-    bool real = !precise && f.kind == TK_DENSE && !f.cmask;
-    for (int k = 0; real && k < fmem[i].count; ++k) {
-      const GSpec& gs = gspec[fmem[i].g[k]];
-      real = gs.kind == QS_GATE_H || gs.kind == QS_GATE_RY || gs.kind == QS_GATE_X || gs.kind == QS_GATE_Z ||
-             gs.kind == QS_GATE_I ||
-             (gs.kind == QS_GATE_MATRIX && gs.mat[0].y == 0 && gs.mat[1].y == 0 && gs.mat[2].y == 0 && gs.mat[3].y == 0);
-    }
-    if (real) f.var = (uint8_t)(FV_REAL + f.t);
+    if (!precise && f.kind == TK_DENSE && !f.cmask && real_gates(gspec, fmem[i])) f.var = (uint8_t)(FV_REAL + f.t);
   }
   for (TOp& b : bops) b.var = bwd_variant(b);
   // decreasing cost order

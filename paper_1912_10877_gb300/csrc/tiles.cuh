@@ -45,7 +45,7 @@ struct TOp {
   uint32_t tmask; // controls outside the phase (register qubit bits)
   uint32_t tval;
   uint32_t count; // TK_DIAGRUN: entries (param: the first, relative to the pass's drun0); backward: GMem records
-  uint32_t pad;
+  uint32_t pad;   // TK_REALRUN: its table's index + 1
   float2 u[4];    // forward: U; backward: U^dagger (row-major 2x2)
 };
 
@@ -63,12 +63,15 @@ struct TOp {
 // TK_DENSEX (forward): a run of uncontrolled gates on one phase bit as one 2x2 with an X
 // on it before or after (var), controlled by a phase bit (var) or by qubits outside
 // (tmask / tval): the X only renames the inputs or outputs
+// TK_REALRUN (forward, tile engine): an uncontrolled real 2x2 on phase bit t (u), then a
+// table of the phase's own diagonal gates (pad: its index + 1, 0: none) and a run, both of
+// factors on the amplitudes whose bit t is 1 only
 // TK_RUN (backward): a run of two or more uncontrolled gates on one phase bit, some with
 // a parameter, with or without such an X (cmask = 1: controlled by qubits outside): takes
 // the four sums that every member's derivative is a combination of, uncomputes the run
 // and the X
 enum { TK_DENSE = 0, TK_SWAP = 1, TK_DIAG = 2, TK_RX = 3, TK_RY = 4, TK_DIAG16 = 5, TK_DIAGOUT = 6, TK_DIAGRUN = 7,
-       TK_DENSEX = 8, TK_RUN = 9 };
+       TK_DENSEX = 8, TK_RUN = 9, TK_REALRUN = 10 };
 
 constexpr int kRunTab = 48;  // entries of a run's table: 32 lanes, then 16 warps (products for bit t = 0 and 1)
 

@@ -44,6 +44,34 @@ def test_runs_of_diagonal_gates(n, tile):
     apply_tiles(n, diagonal_runs(n, n), tile)
 
 
+def layers(n, seed):
+    """A real gate on a qubit, then phases on it: inside the phase, outside, both, with
+    controls of either value, and now and then a gate that acts on the 0 as well."""
+    rs = W.rng(seed)
+    gates = []
+    for t in rs.permutation(n):
+        t = int(t)
+        gates.append(W.Gate("H", (t,)) if rs.integers(2) else W.Gate("RY", (t,), theta=float(rs.uniform(-3, 3))))
+        for q in rs.permutation(n)[: rs.integers(2, n)]:
+            if q == t:
+                continue
+            a, b = (t, int(q)) if rs.integers(4) else (int(q), t)
+            gates.append(W.Gate(("SHIFT", "T", "Z", "S")[rs.integers(4)], (a,), (b,), (int(rs.integers(8) > 0),),
+                                theta=float(rs.uniform(-3, 3))))
+        if rs.integers(6) == 0:
+            gates.append(W.Gate("RZ", (t,), (int((t + 1) % n),), (1,), theta=0.4))
+    return gates
+
+
+@pytest.mark.parametrize("n,tile", [(9, 9), (11, 9), (13, 13), (16, 10), (18, 13)])
+def test_real_gates_with_their_phases(n, tile):
+    for seed in (1, 2):
+        apply_tiles(n, layers(n, 10 * n + seed), tile)
+    qft = [g for t in reversed(range(n)) for g in
+           [W.Gate("H", (t,))] + [W.Gate("SHIFT", (t,), (c,), (1,), theta=np.pi / 2 ** (t - c)) for c in range(t)]]
+    apply_tiles(n, qft, tile, 2)
+
+
 def networks(n):
     rs = W.rng(n)
     half = n // 2
