@@ -338,8 +338,12 @@ __device__ __forceinline__ void real_run(float2 (&x)[1 << RB], const TOp& op, co
     if (op.pad) {
       const float2* d = dtab + 16 * (op.pad - 1);
 #pragma unroll
-      for (int j = 1 << T; j < (1 << RB); ++j)
-        if ((j >> T) & 1) x[j] = cmulf(x[j], cmulf(p, __ldg(d + j)));
+      for (int j = 0; j < (1 << RB); j += 2) {
+        if (T > 0 && !((j >> T) & 1)) continue;
+        const float4 f = *reinterpret_cast<const float4*>(d + j);
+        if (T > 0) x[j] = cmulf(x[j], cmulf(p, make_float2(f.x, f.y)));
+        x[j + 1] = cmulf(x[j + 1], cmulf(p, make_float2(f.z, f.w)));
+      }
     } else {
       mul_bit1<RB, T>(x, p);
     }
@@ -1821,7 +1825,33 @@ struct FArgs {
 };
 
 constexpr int kTileRuns = 48;  // runs of a pass whose tables and tile products shared memory holds
-constexpr size_t kRunBytes = sizeof(float4) * kTileRuns * (kRunTab + 2) + sizeof(RunCtx);
+constexpr int kTileTabs = 48;  // TK_DIAG16 tables of a pass that it holds
+constexpr uint32_t kTileBytes = sizeof(float2) << kBatchTile;
+
+// k_fused_pass's shared memory: offsets known to the compiler, so that what the op loop
+// reads costs no pointer and no generic load.  With the diagonal tables here instead of in
+// global memory, and a tile's place found by one OR over the warp instead of a loop over the
+// tile-id bits and a 64-bit division: passes of a QFT of 29 qubits 7.5, 5.1, 5.4 -> 6.6,
+// 4.5, 4.8 ms (a wait for a global or generic load was the first stall).
+constexpr uint32_t kFpBuf = sizeof(uint32_t) << (kMaxTileBits - kRowBits);  // after the rows' offsets: two tiles
+constexpr uint32_t kFpStage = kFpBuf + 2 * kTileBytes;                      // phases, ops, runs' entries (stage_pass)
+constexpr uint32_t kFpOps = kFpStage + (uint32_t)kStagePhaseBytes;
+constexpr uint32_t kFpRuns = kFpOps + (uint32_t)sizeof(TOp) * kStageOps;
+constexpr uint32_t kFpTile = kFpStage + (uint32_t)kStageBytes;  // the runs' tile products, for two tiles
+constexpr uint32_t kFpTab = kFpTile + 2 * sizeof(float4) * kTileRuns;  // the runs' tables
+constexpr uint32_t kFpDiag = kFpTab + sizeof(float4) * kTileRuns * kRunTab;
+constexpr uint32_t kFpCtx = kFpDiag + sizeof(float2) * 16 * kTileTabs;
+constexpr uint32_t kFpBytes = kFpCtx + sizeof(RunCtx);
+static_assert(kFpBytes <= 227 * 1024 && kFpRuns % 16 == 0 && kFpTile % 16 == 0, "a pass's shared memory");
+
+// run_tile_fwd of a pass whose records and tables all lie in shared memory
+__device__ __noinline__ void run_tile_staged(uint32_t sm, int nphase, uint32_t tile, int m, uint32_t tbase) {
+  for (int f = 0; f < nphase; ++f) {
+    const RunCtx rc{sh<DRun>(kFpRuns), sh<float4>(kFpTab), sh<float4>(tile)};
+    phase_fwd_body<kRB, false, false>(sh<float2>(sm), sh<TPhase>(kFpStage) + f, sh<TOp>(kFpOps), sh<float2>(kFpDiag),
+                                      nullptr, nullptr, rc, sh<uint32_t>(0), m, tbase);
+  }
+}
 
 // products of the tile-id entries of the pass's runs for the tile at tb: 16 lanes a run
 __device__ __forceinline__ void tile_products(float4* out, const DRun* entries, const int2* runs, int nrun, uint32_t tb) {
@@ -1848,48 +1878,55 @@ __device__ __forceinline__ void tile_products(float4* out, const DRun* entries, 
 // cp.async (8-byte copies into the swizzled slots) while the phases run on the
 // other, so the pass does not wait on the state's DRAM latency once per tile.
 __global__ void __launch_bounds__(kTileThreads, 1) k_fused_pass(FArgs a) {
-  extern __shared__ __align__(16) unsigned char smraw[];
-  uint32_t* rowoff = reinterpret_cast<uint32_t*>(smraw);
-  float2* sbuf = reinterpret_cast<float2*>(smraw + sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)));
-  unsigned char* stage = reinterpret_cast<unsigned char*>(sbuf + 2 * (1 << kBatchTile));
   const TPass& p = *a.pass;
-  set_rows(rowoff, p, a.m);
-  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, stage, a.druns, nullptr);
+  set_rows(sh<uint32_t>(0), p, a.m);
+  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, sh<unsigned char>(kFpStage), a.druns, nullptr);
   // the runs' tables, and their tile products for this tile and the one before
   const bool held = p.nrun <= kTileRuns;
-  float4* rtile = reinterpret_cast<float4*>(stage + kStageBytes);
-  float4* rtab = rtile + 2 * kTileRuns;
-  RunCtx* rc = reinterpret_cast<RunCtx*>(rtab + kTileRuns * kRunTab);
-  const uint32_t obuf = (uint32_t)(reinterpret_cast<unsigned char*>(sbuf) - smraw);
-  const uint32_t orc = (uint32_t)(reinterpret_cast<unsigned char*>(rc) - smraw);
-  constexpr uint32_t kTileBytes = sizeof(float2) << kBatchTile;
+  const bool staged = held && p.ndt <= kTileTabs && sp.ph != a.phases + p.phase0;
+  float4* rtab = sh<float4>(kFpTab);
+  RunCtx* rc = sh<RunCtx>(kFpCtx);
   if (held)
     for (int i = threadIdx.x; i < p.nrun * kRunTab; i += blockDim.x) rtab[i] = a.rtab[kRunTab * p.run0 + i];
+  if (staged) {
+    const int count = sp.ph[p.nphase - 1].fop0 + sp.ph[p.nphase - 1].nfop;
+    for (int i = threadIdx.x; i < 16 * p.ndt; i += blockDim.x) sh<float2>(kFpDiag)[i] = a.dtab[16 * p.dt0 + i];
+    TOp* ops = sh<TOp>(kFpOps);
+    for (int i = threadIdx.x; i < count; i += blockDim.x) {
+      if (ops[i].kind == TK_DIAG16) ops[i].param -= p.dt0;
+      if (ops[i].kind == TK_REALRUN && ops[i].pad) ops[i].pad -= (uint32_t)p.dt0;
+    }
+  }
   const uint64_t total = a.ntile * (uint64_t)a.nreg;
-  auto tile_src = [&](uint64_t t, uint64_t& tb) {
-    const uint64_t r = t / a.ntile, tl = t - r * a.ntile;
-    tb = tile_base(tl, p, a.g);
-    return a.state + r * a.reg_stride + tb;
+  // a tile's offset in its register: each lane places one bit of the tile's number
+  const int lane = threadIdx.x & 31, gbit = lane < a.g ? p.gbits[lane] : 0;
+  auto tile_src = [&](uint64_t t, uint32_t& tb) {
+    const uint32_t tl = (uint32_t)(t & (a.ntile - 1));
+    tb = __reduce_or_sync(0xffffffffu, lane < a.g ? ((tl >> lane) & 1u) << gbit : 0u);
+    return a.state + (t >> a.g) * a.reg_stride + tb;
   };
-  uint64_t tb = 0;
-  if (blockIdx.x < total) load_tile_async(obuf, tile_src(blockIdx.x, tb), 0, a.m);
+  const int nphase = p.nphase;
+  uint32_t tb = 0;
+  if (blockIdx.x < total) load_tile_async(kFpBuf, tile_src(blockIdx.x, tb), 0, a.m);
   cp_async_commit();
   int i = 0;
   for (uint64_t t = blockIdx.x; t < total; t += gridDim.x, ++i) {
-    const uint32_t sx = obuf + (i & 1) * kTileBytes;
+    const uint32_t sx = kFpBuf + (i & 1) * kTileBytes;
     const uint64_t tn = t + gridDim.x;
     if (tn < total) {
-      uint64_t tbn;
-      load_tile_async(obuf + ((i + 1) & 1) * kTileBytes, tile_src(tn, tbn), 0, a.m);
+      uint32_t tbn;
+      load_tile_async(kFpBuf + ((i + 1) & 1) * kTileBytes, tile_src(tn, tbn), 0, a.m);
     }
     cp_async_commit();
     float2* base = tile_src(t, tb);
-    float4* rt = held ? rtile + (i & 1) * kTileRuns : nullptr;
-    if (held) tile_products(rt, sp.runs, a.runs + p.run0, p.nrun, (uint32_t)tb);
-    if (threadIdx.x == 0) *rc = RunCtx{sp.runs, held ? rtab : a.rtab + kRunTab * p.run0, rt};
+    const uint32_t ot = kFpTile + (i & 1) * (uint32_t)sizeof(float4) * kTileRuns;
+    float4* rt = held ? sh<float4>(ot) : nullptr;
+    if (held) tile_products(rt, sp.runs, a.runs + p.run0, p.nrun, tb);
+    if (threadIdx.x == 0 && !staged) *rc = RunCtx{sp.runs, held ? rtab : a.rtab + kRunTab * p.run0, rt};
     cp_async_wait_prev();  // this tile's copies (all groups but the one just issued)
     __syncthreads();
-    run_tile_fwd<kRB, false, 2>(sx, sp.ph, p.nphase, sp.ops, a.dtab, nullptr, nullptr, orc, 0, a.m, (uint32_t)tb);
+    if (staged) run_tile_staged(sx, nphase, ot, a.m, tb);
+    else run_tile_fwd<kRB, false, 2>(sx, sp.ph, nphase, sp.ops, a.dtab, nullptr, nullptr, kFpCtx, 0, a.m, tb);
     store_tile(sx, base, 0, a.m);
     __syncthreads();
   }
@@ -2469,6 +2506,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
         e.drun0 += moved(a.druns, d.druns);
         e.run0 += moved(a.tabs, d.tabs);
         e.mem0 += dm;
+        e.dt0 += moved(a.drefs, d.drefs);
       });
       copy(phases, a.phases, z.phases, [&](TPhase& e) {
         e.fop0 += moved(a.fops, d.fops);
@@ -2521,6 +2559,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
       tp.drun0 = (int)druns.size();
       tp.run0 = (int)runs.size();
       tp.mem0 = (int)gmem.size();
+      tp.dt0 = (int)drefs.size();
       tp.nphase = (int)p.phases.size();
       for (const HostPhase& ph : p.phases) {
         TPhase t;
@@ -2950,6 +2989,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
       tp.ndrun = (int)druns.size() - tp.drun0;
       tp.nrun = (int)runs.size() - tp.run0;
       tp.nmem = (int)gmem.size() - tp.mem0;
+      tp.ndt = (int)drefs.size() - tp.dt0;
       passes.push_back(tp);
     }
     R.cost = cost;
@@ -3015,8 +3055,7 @@ static int build_program(int nreg, const qs_circuit* const* circs, const qs_obse
   }
   P->host_passes = passes;
   if (P->fused_only) {
-    P->smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + 2 * sizeof(float2) * (1 << kBatchTile) + kStageBytes +
-              kRunBytes;
+    P->smem = kFpBytes;
     QS_CUDA(cudaFuncSetAttribute(k_fused_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P->smem));
     int dev = 0, sms = 0, per_sm = 0;
     QS_CUDA(cudaGetDevice(&dev));

@@ -112,6 +112,7 @@ struct TPass {
   int32_t drun0, ndrun;     // the pass's TK_DIAGRUN entries
   int32_t run0, nrun;       // the pass's TK_DIAGRUN ops
   int32_t mem0, nmem;       // the pass's GMem records
+  int32_t dt0, ndt;         // the pass's TK_DIAG16 tables
 };
 
 struct HostPhase {
