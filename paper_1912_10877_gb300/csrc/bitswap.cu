@@ -11,7 +11,8 @@
 //
 // Bound by HBM: the state once in and once out.  As three controlled X gates a SWAP
 // inside tile passes the network of 29 qubits took two further passes of 3.7 ms and
-// half of a third; this takes 2.6 ms (half the copy rate).
+// half of a third; this takes 2.3 ms (3.7 TB/s; 2.6 ms with the slots' banks in conflict,
+// 2.9 ms with 512 threads).
 #include <algorithm>
 #include <cstring>
 
@@ -37,7 +38,10 @@ struct SwapArgs {
   uint8_t pa[32], pb[32];      // swapped outer index bits
 };
 
-__device__ __forceinline__ uint32_t swap_slot(uint32_t l) { return l ^ ((l >> 5) & 31u); }
+// Half a warp reads or writes 16 amplitudes of 8 bytes at a time, one in each pair of
+// banks: the lowest four bits of a slot take the XOR of every nibble, so that four lane bits
+// that a network sends to neighbouring high bits spread over the banks as they do at home
+__device__ __forceinline__ uint32_t swap_slot(uint32_t l) { return l ^ (((l >> 4) ^ (l >> 8)) & 15u); }
 
 __global__ void __launch_bounds__(kSwapThreads) k_bitswap(const __grid_constant__ SwapArgs a) {
   extern __shared__ __align__(16) float2 sm[];
@@ -67,6 +71,7 @@ __global__ void __launch_bounds__(kSwapThreads) k_bitswap(const __grid_constant_
     return b;
   };
   auto store = [&](float2* dst, const float2* src) {
+#pragma unroll 4
     for (uint32_t q = threadIdx.x; q < nq; q += kSwapThreads) {
       const uint32_t l = 2 * q, row = rowperm[l >> 5];
       const float2 u = src[swap_slot(row | colperm[l & 31])], v = src[swap_slot(row | colperm[(l + 1) & 31])];
