@@ -104,6 +104,11 @@ static int make_state(int nreg, const int32_t* nq, int dtype, void* dev_buf, voi
   return QS_OK;
 }
 
+// a compensated gate that an X after it on its target can ride on (Plan::xmask)
+static bool takes_x(const Plan& p) {
+  return p.op == OP_DENSE1 || p.op == OP_REAL1 || p.op == OP_HLIKE1 || p.op == OP_RXLIKE1 || p.op == OP_PERM1;
+}
+
 // same-qubit single-qubit fusion: a pending 2x2 per qubit; gates that touch a
 // qubit flush its pending matrix first (gates on other qubits commute with it)
 struct Fuser {
@@ -139,6 +144,23 @@ struct Fuser {
     int loc = q;
     QS_TRY(plan_gate(pend[q].data(), 1, &loc, 0, 0, &p));
     p.precise = precise;
+    return emit(p);
+  }
+  // A compensated gate pending on the target of a controlled X takes the X along: one pass
+  // for both.  Returns whether it did.
+  int flush_with_x(const qs_gate_desc& g, bool* done) {
+    const int q = g.locs[0];
+    *done = false;
+    if (!precise || g.kind != QS_GATE_X || !g.ctrl_mask || !has[q]) return QS_OK;
+    Plan p;
+    QS_TRY(plan_gate(pend[q].data(), 1, &q, 0, 0, &p));
+    if (!takes_x(p)) return QS_OK;
+    QS_TRY(flush_mask(g.ctrl_mask));
+    has[q] = false;
+    p.precise = true;
+    p.xmask = g.ctrl_mask;
+    p.xvals = g.ctrl_vals & g.ctrl_mask;
+    *done = true;
     return emit(p);
   }
   int flush_mask(uint64_t m) {
@@ -224,11 +246,15 @@ static int apply_circuit_impl(qs_state* s, const qs_circuit* c, const double* pa
     if (g.nlocs == 1 && g.ctrl_mask == 0 && !unfused) {
       fz.push(g.locs[0], U);
     } else {
-      QS_TRY(fz.flush_mask(locmask | g.ctrl_mask));
-      Plan p;
-      QS_TRY(plan_gate(U.data(), g.nlocs, g.locs, g.ctrl_mask, g.ctrl_vals, &p));
-      p.precise = precise;
-      QS_TRY(fz.emit(p));
+      bool done = false;
+      if (!unfused) QS_TRY(fz.flush_with_x(g, &done));
+      if (!done) {
+        QS_TRY(fz.flush_mask(locmask | g.ctrl_mask));
+        Plan p;
+        QS_TRY(plan_gate(U.data(), g.nlocs, g.locs, g.ctrl_mask, g.ctrl_vals, &p));
+        p.precise = precise;
+        QS_TRY(fz.emit(p));
+      }
     }
     if (ckpt_every > 0 && (k + 1) % ckpt_every == 0 && k + 1 < ng) {
       QS_TRY(fz.flush_all());  // the checkpoint holds the state after gate k exactly

@@ -249,6 +249,9 @@ struct Plan {
   cd d0 = 1, d1 = 1;
   cd u[4];
   bool precise = false;             // complex64: compensated matrix, each output rounded once
+  // precise 1-qubit dense forms: an X on the target after the gate where these controls hold
+  // (xmask = 0: none)
+  uint64_t xmask = 0, xvals = 0;
   // k-qubit forms (row-major 2^k x 2^k; perm / diag tables)
   std::vector<cd> U;
   int perm[1 << QS_MAXK];

@@ -163,10 +163,13 @@ k_gate1(c2_t<R>* __restrict__ psi, uint64_t nitems, IdxSpec s, int t, U4<R> u, i
 }
 
 // complex64 1-qubit gate with its FP64 matrix held as hi + lo and every output
-// rounded once (Plan::precise): the same item layout as k_gate1
+// rounded once (Plan::precise): the same item layout as k_gate1.  An X after it on the same
+// target (xmask: its controls, 0 for none) renames the outputs; a launch of its own cost 4.3
+// us beside the 7.2 us of the gate (20 qubits, both bound by the L2 and the launch).
 template <bool T0>
 __global__ void __launch_bounds__(kThreads)
-k_gate1_prec(float2* __restrict__ psi, uint64_t nitems, IdxSpec s, int t, U4<float> uh, U4<float> ul, int lane_sel) {
+k_gate1_prec(float2* __restrict__ psi, uint64_t nitems, IdxSpec s, int t, U4<float> uh, U4<float> ul, int lane_sel,
+             uint64_t xmask, uint64_t xvals) {
   const uint64_t first = (uint64_t)blockIdx.x * (blockDim.x * kIPT) + threadIdx.x;
   uint64_t idx[kIPT];
   float2 a0[kIPT], a1[kIPT], b0[kIPT], b1[kIPT];
@@ -179,22 +182,23 @@ k_gate1_prec(float2* __restrict__ psi, uint64_t nitems, IdxSpec s, int t, U4<flo
     ld_pair(psi + idx[v], a0[v], a1[v]);
     if (!T0) ld_pair(psi + idx[v] + stride, b0[v], b1[v]);
   }
-  auto op = [&](float2& a, float2& b) {
+  auto op = [&](float2& a, float2& b, uint64_t at) {
     const float2 na = cf_dot2(a, uh.m[0], ul.m[0], b, uh.m[1], ul.m[1]);
     const float2 nb = cf_dot2(a, uh.m[2], ul.m[2], b, uh.m[3], ul.m[3]);
-    a = na;
-    b = nb;
+    const bool x = xmask && (at & xmask) == xvals;
+    a = x ? nb : na;
+    b = x ? na : nb;
   };
 #pragma unroll
   for (int v = 0; v < kIPT; ++v) {
     if (idx[v] == ~0ull) continue;
     if (T0) {
-      op(a0[v], a1[v]);
+      op(a0[v], a1[v], idx[v]);
       st_pair(psi + idx[v], a0[v], a1[v]);
     } else {
       float2 x0 = a0[v], y0 = b0[v], x1 = a1[v], y1 = b1[v];
-      op(x0, y0);
-      op(x1, y1);
+      op(x0, y0, idx[v]);
+      op(x1, y1, idx[v] + 1);
       if (lane_sel == 1) { x0 = a0[v]; y0 = b0[v]; }
       if (lane_sel == 0) { x1 = a1[v]; y1 = b1[v]; }
       st_pair(psi + idx[v], x0, x1);
@@ -456,14 +460,14 @@ static int launch_prec(float2* psi, int n, int nreg, const Plan& p, cudaStream_t
     const uint64_t items = (uint64_t)nreg << s.item_log2;
     if (!items) return QS_OK;
     const int nt = cta_threads(items, kIPT);
-    k_gate1_prec<true><<<blocks_for(items, nt * kIPT), nt, 0, st>>>(psi, items, s, 0, uh, ul, -1);
+    k_gate1_prec<true><<<blocks_for(items, nt * kIPT), nt, 0, st>>>(psi, items, s, 0, uh, ul, -1, p.xmask, p.xvals);
   } else {
     QS_TRY(make_idx(n, 1ull | (1ull << t) | p.ctrl_mask, p.ctrl_vals & ~1ull, &s));
     const uint64_t items = (uint64_t)nreg << s.item_log2;
     if (!items) return QS_OK;
     const int lane = (p.ctrl_mask & 1ull) ? (int)(p.ctrl_vals & 1ull) : -1;
     const int nt = cta_threads(items, kIPT);
-    k_gate1_prec<false><<<blocks_for(items, nt * kIPT), nt, 0, st>>>(psi, items, s, t, uh, ul, lane);
+    k_gate1_prec<false><<<blocks_for(items, nt * kIPT), nt, 0, st>>>(psi, items, s, t, uh, ul, lane, p.xmask, p.xvals);
   }
   QS_LAUNCHED();
   return QS_OK;

@@ -63,3 +63,24 @@ def test_gradient_of_runs(n, every):
         scale = max(1.0, np.max(np.abs(wg)))
         assert abs(loss - wl) < tol * max(1.0, abs(wl))
         assert np.max(np.abs(grad - wg)) < tol * scale, (dtype, np.max(np.abs(grad - wg)) / scale)
+
+
+@pytest.mark.parametrize("n", [2, 5, 9, 13])
+def test_compensated_gate_with_an_x_is_the_two_of_them(n):
+    from paper_1912_10877_gb300 import qsim
+    rs = W.rng(n)
+    psi = W.haar_state(n, seed=n)
+    gates = []
+    for _ in range(40):
+        q = [int(v) for v in rs.permutation(n)]
+        k = int(rs.integers(1, min(4, n)))
+        gates.append(W.Gate(("H", "RX", "RY", "Y", "T", "MATRIX")[rs.integers(6)], (q[0],), theta=float(rs.uniform(-3, 3)),
+                            matrix=W.haar_su2(len(gates))))
+        gates.append(W.Gate("X", (q[0],), tuple(q[1:1 + k]), tuple(int(v) for v in rs.integers(0, 2, k))))
+    fused, apart = qsim.State(n, dtype=torch.complex64), qsim.State(n, dtype=torch.complex64)
+    fused.upload(psi)
+    apart.upload(psi)
+    fused.apply_circuit(qsim.Circuit(gates, n), precise=True)
+    for g in gates:
+        apart.apply_circuit(qsim.Circuit([g], n), precise=True)
+    assert np.array_equal(fused.numpy(), apart.numpy())  # the X only renames
