@@ -25,7 +25,7 @@ namespace qs {
 int expect_raw(const void* data, int dtype, int n, int nreg, const qs_observable* o, qs_state* ws_owner,
                double* host_out);
 int apply_observable_c128(const double2* psi, double2* lam, int n, const qs_observable* o, cudaStream_t st);
-int promote_to_c128(const void* in, int dtype, double2* out, uint64_t dim, cudaStream_t st);
+int promote_to_c128(const void* in, int dtype, double2* out, uint64_t dim, cd f, cudaStream_t st);
 
 constexpr int kAdjThreads = 256;
 constexpr int kAdjMaxBlocks = 1216;  // 8 per SM on 152 SMs
@@ -172,11 +172,17 @@ k_adjoint_param1(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t 
 // With (a, b) the pair at the end of the run the pass sums Im conj(l_a) x_a,
 // Im conj(l_b) x_b, Im<l|X|x> and Im<l|Y|x>; a member's derivative is 2 c times its
 // generator carried to the run's end, decomposed over those four (AdjRun::coef).
-//   bound: the FP64 rate.  12 operations a pair for the sums and 32 for U^dag on psi and
+// The first row of U^dag is divided by its larger entry (its columns traded when that is
+// the second): that entry's products, a quarter of all, are gone.  Psi and lambda then carry
+// the same complex factor, which the host keeps (AdjWalk::phi): derivatives are divided by
+// its square, a checkpoint is multiplied by it, and once it is past 2^100 a run is applied
+// in full (FULL) with the factor taken out.
+//   bound: the FP64 rate.  12 operations a pair for the sums and 24 for U^dag on psi and
 //   lambda, where Rz, Rx, Rz took 64 in three passes and the X a fourth pass.  The pairs
 //   are cut into equal contiguous ranges, four CTAs an SM: a grid-stride loop left a
 //   sixth of the FP64 units idle in its last round.  Measured in the differentiation
-//   workload (n = 20): 62 us a run and its X, 121 us as four passes.
+//   workload (n = 20): 53 us a run and its X, 62 us with every entry of U^dag multiplied, 121
+//   us as four passes.
 constexpr int kAdjMembers = 8;
 constexpr int kAdjRunBlocks = 608;  // 4 per SM on 152 SMs
 
@@ -185,10 +191,12 @@ struct AdjRun {
   uint64_t off1;             // offset of its bit
   uint64_t xmask, xval;      // the X's controls and their values (xmask = 0: no X)
   int pre, members;
+  int swap;                  // columns of U^dag (and the coefficients) are traded
   int param[kAdjMembers];
   double coef[kAdjMembers][4];
 };
 
+template <bool FULL>
 __global__ void __launch_bounds__(kAdjThreads, 4)
 k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nitems, int t,
               const __grid_constant__ AdjRun F, double* __restrict__ partials, unsigned* __restrict__ counter,
@@ -199,7 +207,7 @@ k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nit
   for (uint64_t it = lo + threadIdx.x; it < hi; it += kAdjThreads) {
     const uint64_t b0 = it + (it & ~below), b1 = b0 + F.off1;
     const bool on = F.xmask && (b0 & F.xmask) == F.xval;
-    const bool in = on && !F.pre, out = on && F.pre;
+    const bool in = (on && !F.pre) != (F.swap != 0), out = on && F.pre;
     const uint64_t ia = in ? b1 : b0, ib = in ? b0 : b1;
     const double2 xa = psi[ia], xb = psi[ib], la = lam[ia], lb = lam[ib];
     va = fma(la.x, xa.y, fma(-la.y, xa.x, va));
@@ -209,9 +217,9 @@ k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nit
     vx = fma(lb.x, xa.y, fma(-lb.y, xa.x, vx));
     vy = fma(-la.x, xb.x, fma(-la.y, xb.y, vy));
     const uint64_t oa = out ? b1 : b0, ob = out ? b0 : b1;
-    psi[oa] = cfma(F.ud[1], xb, cmul(F.ud[0], xa));
+    psi[oa] = cfma(F.ud[1], xb, FULL ? cmul(F.ud[0], xa) : xa);
     psi[ob] = cfma(F.ud[3], xb, cmul(F.ud[2], xa));
-    lam[oa] = cfma(F.ud[1], lb, cmul(F.ud[0], la));
+    lam[oa] = cfma(F.ud[1], lb, FULL ? cmul(F.ud[0], la) : la);
     lam[ob] = cfma(F.ud[3], lb, cmul(F.ud[2], la));
   }
   // CTA sums, then the CTA that arrives last folds all of them (in an order that does not
@@ -360,7 +368,7 @@ static bool diagonal_gate(const qs_circuit* c, const qs_gate_desc& g) {
   return true;
 }
 
-// Whether a run is worth its own pass (44 FP64 operations a pair): two gates or more,
+// Whether a run is worth its own pass (36 FP64 operations a pair): two gates or more,
 // one with a parameter, not all diagonal (those take 20 each).
 static bool adj_run(const qs_circuit* c, const AdjStep& u) {
   bool diag = true, param = false;
@@ -418,6 +426,7 @@ struct AdjWalk {
   double *dgrad, *partials;
   unsigned* counter;
   std::vector<cd> U, G;
+  cd phi = 1;  // psi and lambda hold phi times the states
 
   int gate(int k) {
     const qs_gate_desc& g = c->gates[k];
@@ -427,6 +436,7 @@ struct AdjWalk {
     if (g.param >= 0 && g.kind != QS_GATE_MATRIX) {
       double cfac = 0;
       QS_TRY(gate_generator(g, G, &cfac));
+      cfac /= std::norm(phi);
       switch (g.nlocs) {
         case 1: return launch_adjoint_param<1>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st);
         case 2: return launch_adjoint_param<2>(psi, lam, n, g, G, U, partials, counter, dgrad, cfac, st);
@@ -460,7 +470,7 @@ struct AdjWalk {
               for (int b = 0; b < 2; ++b) v += E[2 * i + a] * G[2 * a + b] * std::conj(E[2 * j + b]);
             M[2 * i + j] = v;
           }
-        const double f = 2.0 * cfac;
+        const double f = 2.0 * cfac / std::norm(phi);
         double* co = F.coef[F.members];
         co[0] = f * M[0].real();
         co[1] = f * M[3].real();
@@ -473,8 +483,22 @@ struct AdjWalk {
                        E[2] * U[1] + E[3] * U[3]};
       std::copy(A, A + 4, E);
     }
-    for (int i = 0; i < 2; ++i)
-      for (int j = 0; j < 2; ++j) F.ud[2 * i + j] = make_double2(E[2 * j + i].real(), -E[2 * j + i].imag());
+    cd D[4] = {std::conj(E[0]), std::conj(E[2]), std::conj(E[1]), std::conj(E[3])};
+    F.swap = std::norm(D[1]) > std::norm(D[0]);
+    if (F.swap) {
+      std::swap(D[0], D[1]);
+      std::swap(D[2], D[3]);
+      for (int m = 0; m < F.members; ++m) {
+        std::swap(F.coef[m][0], F.coef[m][1]);
+        F.coef[m][3] = -F.coef[m][3];  // Y with its basis states traded
+      }
+    }
+    // a row without a large entry (a matrix that is not unitary) is applied as it is
+    const double size = std::abs(phi);
+    const bool far = size > 0x1p100 || size < 0x1p-100, full = far || std::norm(D[0]) < 0.25;
+    const cd f = far ? 1.0 / phi : full ? cd(1, 0) : 1.0 / D[0];
+    phi *= f;
+    for (int k = 0; k < 4; ++k) F.ud[k] = make_double2((f * D[k]).real(), (f * D[k]).imag());
     const int t = c->gates[u.gates[0]].locs[0];
     F.off1 = 1ull << t;
     if (u.x >= 0) {
@@ -484,7 +508,8 @@ struct AdjWalk {
     }
     const uint64_t items = 1ull << (n - 1);
     const int nblk = (int)std::min<uint64_t>(kAdjRunBlocks, std::max<uint64_t>(1, items / kAdjThreads));
-    k_adjoint_run<<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, t, F, partials, counter, dgrad);
+    if (full) k_adjoint_run<true><<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, t, F, partials, counter, dgrad);
+    else k_adjoint_run<false><<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, t, F, partials, counter, dgrad);
     QS_LAUNCHED();
     return QS_OK;
   }
@@ -522,7 +547,7 @@ int backward(qs_state* s, const qs_circuit* c, const double* params, const qs_ob
   unsigned* counter = reinterpret_cast<unsigned*>(partials + kPartials);
   QS_CUDA(cudaMemsetAsync(dgrad, 0, sizeof(double) * np, st));
   QS_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned), st));
-  QS_TRY(promote_to_c128(s->data, s->dtype, psi, dim, st));
+  QS_TRY(promote_to_c128(s->data, s->dtype, psi, dim, 1, st));
   QS_TRY(apply_observable_c128(psi, lam, n, o, st));
   const size_t ab = amp_bytes(s->dtype);
   AdjWalk w{s, c, params, n, psi, lam, dgrad, partials, counter, {}, {}};
@@ -532,7 +557,7 @@ int backward(qs_state* s, const qs_circuit* c, const double* params, const qs_ob
   std::vector<AdjStep> steps;
   for (int seg = ng > 0 ? (ng - 1) / every : -1; seg >= 0; --seg) {
     const int first = seg * every, last = std::min(ng, first + every);
-    if (last < ng) QS_TRY(promote_to_c128((const char*)ckpts + ab * dim * seg, s->dtype, psi, dim, st));
+    if (last < ng) QS_TRY(promote_to_c128((const char*)ckpts + ab * dim * seg, s->dtype, psi, dim, w.phi, st));
     adj_steps(c, first, last, steps);
     for (size_t k = steps.size(); k-- > 0;) QS_TRY(w.step(steps[k]));
   }

@@ -919,19 +919,27 @@ int reset_basis(qs_state* s, const uint64_t* host_basis) {
   return QS_OK;
 }
 
-__global__ void k_promote(const float2* __restrict__ in, double2* __restrict__ out, uint64_t dim) {
-  const uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x;
+template <typename C, bool SCALE>
+__global__ void k_promote(const C* __restrict__ in, double2* __restrict__ out, uint64_t dim, double2 f) {
+  const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= dim) return;
-  const float2 v = in[i];
-  out[i] = make_double2((double)v.x, (double)v.y);
+  const C v = in[i];
+  const double2 w = make_double2(v.x, v.y);
+  out[i] = SCALE ? cmul(f, w) : w;
 }
 
-int promote_to_c128(const void* in, int dtype, double2* out, uint64_t dim, cudaStream_t st) {
-  if (dtype == QS_C128) {
+// out = f in
+int promote_to_c128(const void* in, int dtype, double2* out, uint64_t dim, cd f, cudaStream_t st) {
+  const unsigned nb = (unsigned)((dim + 255) / 256);
+  const double2 d = make_double2(f.real(), f.imag());
+  const bool one = f == cd(1, 0);
+  if (dtype == QS_C128 && one) {
     QS_CUDA(cudaMemcpyAsync(out, in, sizeof(double2) * dim, cudaMemcpyDeviceToDevice, st));
     return QS_OK;
   }
-  k_promote<<<(unsigned)((dim + 255) / 256), 256, 0, st>>>((const float2*)in, out, dim);
+  if (dtype == QS_C128) k_promote<double2, true><<<nb, 256, 0, st>>>((const double2*)in, out, dim, d);
+  else if (one) k_promote<float2, false><<<nb, 256, 0, st>>>((const float2*)in, out, dim, d);
+  else k_promote<float2, true><<<nb, 256, 0, st>>>((const float2*)in, out, dim, d);
   QS_LAUNCHED();
   return QS_OK;
 }

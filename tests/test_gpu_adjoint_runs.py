@@ -65,6 +65,33 @@ def test_gradient_of_runs(n, every):
         assert np.max(np.abs(grad - wg)) < tol * scale, (dtype, np.max(np.abs(grad - wg)) / scale)
 
 
+@pytest.mark.parametrize("n,every", [(2, 0), (3, 500), (10, 900)])
+def test_gradient_of_many_runs(n, every):
+    """Runs whose matrices have entries of one size, more than any factor that psi and
+    lambda carry may grow through: the bounds of the short circuits times the gates."""
+    from paper_1912_10877_gb300 import qsim
+    rs = W.rng(n)
+    gates = []
+    for k in range(600):
+        t = k % n
+        gates += [W.Gate("RX", (t,), theta=np.pi / 2 + float(rs.uniform(-0.1, 0.1))), W.Gate("RZ", (t,), param=k)]
+        gates.append(W.Gate("X", (t,), ((t + 1) % n,), (k % 3 > 0,)))
+    params = W.uniform_angles(600, n)
+    terms = W.tfim(n)
+    circ, obs = qsim.Circuit(gates, n, len(params)), qsim.Observable(terms)
+    wl, wg = oracle.gradient(oracle.zero_state(n), n, gates, params, terms)
+    st = qsim.State(n, dtype=torch.complex128)
+    st.reset()
+    ck = qsim.checkpoint_buffer(st, circ, every)
+    if every:
+        qsim.apply_circuit_ckpt(st, circ, params, every, ck)
+    else:
+        st.apply_circuit(circ, params)
+    loss, grad = qsim.backward(st, circ, params, obs, every if ck is not None else 0, ck)
+    assert abs(loss - wl) < 1e-10 * max(1.0, abs(wl))
+    assert np.max(np.abs(grad - wg)) < 1e-10 * max(1.0, np.max(np.abs(wg)))
+
+
 @pytest.mark.parametrize("n", [2, 5, 9, 13])
 def test_compensated_gate_with_an_x_is_the_two_of_them(n):
     from paper_1912_10877_gb300 import qsim
