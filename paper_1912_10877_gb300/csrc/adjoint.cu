@@ -181,8 +181,8 @@ k_adjoint_param1(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t 
 //   lambda, where Rz, Rx, Rz took 64 in three passes and the X a fourth pass.  The pairs
 //   are cut into equal contiguous ranges, four CTAs an SM: a grid-stride loop left a
 //   sixth of the FP64 units idle in its last round.  Measured in the differentiation
-//   workload (n = 20): 53 us a run and its X, 62 us with every entry of U^dag multiplied, 121
-//   us as four passes.
+//   workload (n = 20): 49 us a run and its X (53 us with the four sums reduced one by one, 62
+//   us with every entry of U^dag multiplied as well), 121 us as four passes.
 constexpr int kAdjMembers = 8;
 constexpr int kAdjRunBlocks = 608;  // 4 per SM on 152 SMs
 
@@ -228,12 +228,17 @@ k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nit
   __shared__ double tot[4];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto cta_sums = [&](double (&v)[4]) {
+  // the four sums over a warp in 6 additions a lane (a thread has three or four pairs: 20,
+  // each sum by itself, were a seventh of the kernel's FP64 operations): a lane gives away
+  // two sums, then one, and keeps the sum that bits 4 and 3 of its number say
+  auto cta_sums = [&](const double (&v)[4]) {
+    const bool hi = lane & 16, odd = lane & 8;
+    const double a = (hi ? v[2] : v[0]) + __shfl_xor_sync(0xffffffffu, hi ? v[0] : v[2], 16);
+    const double b = (hi ? v[3] : v[1]) + __shfl_xor_sync(0xffffffffu, hi ? v[1] : v[3], 16);
+    double r = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-    if (lane < 4) red[lane][warp] = lane == 0 ? v[0] : lane == 1 ? v[1] : lane == 2 ? v[2] : v[3];
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if ((lane & 7) == 0) red[lane >> 3][warp] = r;
     __syncthreads();
     if (threadIdx.x < 4) {
       static_assert(kAdjThreads / 32 == 8, "CTA tree below is written for 8 warps");
