@@ -487,7 +487,7 @@ def run_diff_leg(steps: int, warmup: int):
     return {"metric": "fwd+grad seconds (n=20, 8000 gates, 6000 angles)", "unit": "s",
             "value": out["fp64_uncompute_ckpt10"], "tiled_fp32_value": out["tiled_fp32"],
             "backward_s": round(tb, 4),
-            "roofline": {"bound": "alu", "kernel": "FP64 reversible uncompute (k_adjoint_param1 / k_adjoint_param)",
+            "roofline": {"bound": "alu", "kernel": "FP64 reversible uncompute (k_adjoint_run; flops counted gate by gate)",
                          "achieved": round(fp64_flops / tb / 1e12, 3), "peak": fp64_peak, "unit": "TFLOP/s",
                          "frac": round(fp64_flops / tb / 1e12 / fp64_peak, 4), "flops": fp64_flops,
                          "peak_kind": "nominal FP64 rate of GB300 (1.25 TFLOP/s)"},

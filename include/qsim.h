@@ -325,11 +325,13 @@ int qs_circuit_gate_matrices(const qs_circuit* c, int index, const double* host_
 int qs_circuit_schedule_info(const qs_circuit* c, int tile_qubits, int* npasses, int* nphases);
 
 /* The order in which the tile engine applies the circuit's gates for tiles of
- * tile_qubits qubits (0 = 13), host only (no device work).  The engine first
- * rewrites each SWAP(a, b) as X(b) controlled by a, X(a) controlled by b, X(b)
- * controlled by a (each also carrying the SWAP's controls); host_order[i] is
+ * tile_qubits qubits (0 = 13), host only (no device work).  Each SWAP(a, b) is
+ * listed as X(b) controlled by a, X(a) controlled by b, X(b) controlled by a
+ * (each also carrying the SWAP's controls); host_order[i] is
  * the index, in that expanded list, of the i-th gate applied and host_pass[i]
- * its pass.  Inside a pass the engine may still fuse runs of gates on one
+ * its pass.  Uncontrolled SWAPs on disjoint qubits that open or close a circuit of
+ * 16 qubits or more are one pass that permutes the state; other SWAPs are applied
+ * as their three gates.  Inside a pass the engine may still fuse runs of gates on one
  * qubit and apply commuting diagonal gates together; the order here is the
  * scheduler's (Sec. "Representing Quantum Circuits": reordering is valid only
  * between gates on disjoint qubits).  *ngates receives the expanded gate count;
@@ -351,8 +353,11 @@ int qs_circuit_tile_order(const qs_circuit* c, int tile_qubits, int* ngates, int
  * past gates on other qubits), one HBM round trip of the state per pass, with
  * every gate of a pass applied in shared memory / registers.  It takes
  * single-target gates (their controls, tested per amplitude, may sit on any
- * qubit) plus SWAPs (as three CNOTs) on registers of 5..32 qubits; other
- * circuits use the per-gate path.  QS_APPLY_TILES forces the tile engine
+ * qubit) plus SWAPs (qs_circuit_tile_order) on registers of 5..32 qubits; other
+ * circuits use the per-gate path.  Registers of at most 14 qubits and 2^17
+ * amplitudes in all run consecutive gates of the per-gate path in one launch
+ * inside thread-block clusters, with the same results to the bit; QS_APPLY_UNFUSED,
+ * QS_APPLY_PRECISE and checkpointed applies keep a launch a gate.  QS_APPLY_TILES forces the tile engine
  * (QS_EUNSUPPORTED if the circuit does not fit) and QS_APPLY_TILE_QUBITS(m)
  * sets the tile size (9..13; registers smaller than the tile form one tile).  A circuit keeps its
  * schedule and a parameter buffer between calls, so applies of one circuit

@@ -12,7 +12,8 @@
 //
 // Backward (Eq. apply-back): the passes and phases run in reverse; for each
 // gate, in reverse order, a thread adds Im sum conj(lambda) (G psi) over its
-// pairs (FP32 over <= 8 pairs, then FP32 warp shuffles, FP64 from the warp
+// pairs (for a run of gates on one qubit, the four sums that all their derivatives
+// come from) (FP32 over <= 8 pairs, then FP32 warp shuffles, FP64 from the warp
 // level up) and uncomputes psi and lambda with U^dagger in FP32, using the
 // structured Rx / Ry / diagonal forms of the inverse rotations.  The
 // register's gradient lives in shared memory (FP64) and is written once.
