@@ -118,10 +118,24 @@ struct Fuser {
   bool precise = false;
   bool small = false;       // collect plans for apply_small
   std::vector<Plan> plans;
+  Plan held;                // a compensated gate that waits for the next one (launch_prec_pair)
+  bool holding = false;
+  bool pairs = false;       // every plan is compensated, and gates may share a launch
   explicit Fuser(qs_state* st, int n) : s(st), pend(n), has(n, false) {}
   // applies a plan: at once, or with the others collected before the next one that the
   // small-register path does not take
   int emit(const Plan& p) {
+    if (pairs && takes_x(p) && !p.ctrl_mask && p.t >= 1) {
+      if (holding && held.t != p.t) {
+        holding = false;
+        return launch_prec_pair(s, held, p);
+      }
+      QS_TRY(release());
+      held = p;
+      holding = true;
+      return QS_OK;
+    }
+    QS_TRY(release());
     if (!small) return launch_plan(s, p);
     if (p.op == OP_NOP) return QS_OK;
     if (small_plan(p)) {
@@ -130,6 +144,11 @@ struct Fuser {
     }
     QS_TRY(drain());
     return launch_plan(s, p);
+  }
+  int release() {
+    if (!holding) return QS_OK;
+    holding = false;
+    return launch_plan(s, held);
   }
   int drain() {
     if (plans.empty()) return QS_OK;
@@ -168,7 +187,10 @@ struct Fuser {
       if ((m >> q) & 1ull) QS_TRY(flush(q));
     return QS_OK;
   }
-  int flush_all() { return flush_mask(~0ull); }
+  int flush_all() {
+    QS_TRY(flush_mask(~0ull));
+    return release();
+  }
   void push(int q, const std::vector<cd>& U) {
     if (!has[q]) {
       pend[q] = U;
@@ -236,6 +258,7 @@ static int apply_circuit_impl(qs_state* s, const qs_circuit* c, const double* pa
   }
   Fuser fz(s, c->nqubits);
   fz.precise = precise;
+  fz.pairs = precise && !unfused;
   fz.small = !unfused && ckpt_every == 0 && !precise && s->uniform && small_register(s->nq[0], s->nreg);
   const size_t ab = amp_bytes(s->dtype);
   for (int k = 0; k < ng; ++k) {

@@ -263,6 +263,7 @@ int plan_gate(const cd* U, int k, const int* locs, uint64_t ctrl_mask, uint64_t 
 
 // launch a plan on every register of s (uniform: one launch; uneven: per register)
 int launch_plan(qs_state* s, const Plan& p);
+int launch_prec_pair(qs_state* s, const Plan& a, const Plan& b);
 // launch a plan on an explicit single-register buffer (used by the adjoint)
 int launch_plan_on(void* data, int dtype, int n, int nreg, int64_t reg_stride, const Plan& p,
                    qs_state* owner);
