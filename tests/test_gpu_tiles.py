@@ -72,6 +72,13 @@ def test_real_gates_with_their_phases(n, tile):
     apply_tiles(n, qft, tile, 2)
 
 
+@pytest.mark.parametrize("reps", [3, 6, 12, 40])
+def test_passes_that_outgrow_shared_memory(reps):
+    """One pass of more and more phases, ops, runs and tables than its staged area holds."""
+    n = 11
+    apply_tiles(n, [g for k in range(reps) for g in layers(n, 100 + k)], 13)
+
+
 def networks(n):
     rs = W.rng(n)
     half = n // 2
