@@ -2266,11 +2266,6 @@ struct qs_batch_program {
 
 namespace qs {
 
-static bool diag_kind(int k) {
-  return k == QS_GATE_Z || k == QS_GATE_S || k == QS_GATE_SDG || k == QS_GATE_T || k == QS_GATE_TDG ||
-         k == QS_GATE_RZ || k == QS_GATE_SHIFT || k == QS_GATE_PHASE || k == QS_GATE_I;
-}
-
 static int gen_of(int kind, float* cfac2) {
   switch (kind) {
     case QS_GATE_RX: *cfac2 = 1.f; return GEN_X;
