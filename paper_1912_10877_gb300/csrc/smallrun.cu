@@ -92,6 +92,11 @@ k_small_run(c2_t<R>* __restrict__ psi, const __grid_constant__ RunArgs A, const 
   const bool act = tid < area;
   const uint32_t i = (rank << L) | tid;
   T x = act ? psi[i] : cmk<T>(0, 0);
+  // Every amplitude of the cluster is loaded before any is stored: a circuit with SWAPs ends
+  // on other places than it began on, and its ops may need no barrier of their own (lane
+  // targets, diagonal gates, none).  It also lets every CTA start before another touches its
+  // shared memory.
+  cl.sync();
   int turn = 0, rturn = 0;
   for (int o = 0; o < A.nops; ++o) {
     const RunOp<R>& op = ops.op[o];

@@ -76,3 +76,34 @@ def test_gates_wider_than_a_block_stay_refused():
     wide = W.Gate("X", (0,), (1, 2, 3, 4, 5), (1,) * 5)
     with pytest.raises(QsimError):
         qsim.run_one_launch(st, qsim.Circuit([wide], 8), None)
+
+
+@pytest.mark.parametrize("with_obs", [False, True])
+@pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
+@pytest.mark.parametrize("n", [6, 7, 8, 9, 10, 11, 12, 13, 14])
+def test_swaps_with_no_barrier_among_the_gates(dt, n, with_obs):
+    """Qubits that end elsewhere than they began, with no op that needs a barrier: SWAPs alone
+    (exact, many in a row), then with a diagonal gate and gates on lane bits."""
+    from paper_1912_10877_gb300 import qsim
+    far = [W.Gate("SWAP", (0, n - 1))]
+    turn = [W.Gate("SWAP", (q, q + 1)) for q in range(n - 1)]
+    mixed = [W.Gate("T", (n - 1,)), W.Gate("H", (0,)), W.Gate("RX", (4,), (n - 1,), (1,), theta=0.3)]
+    terms = [(0.5, ((0, "Z"),)), (-1.25, ((n - 1, "Z"), (1, "Z")))] if with_obs else []
+    obs = qsim.Observable(terms) if with_obs else None
+    st = qsim.State(n, dtype=dt)
+    psi = st.upload(W.haar_state(n, seed=n)).numpy().astype(np.complex128)
+    tol = 1e-12 if dt == torch.complex128 else 1e-6  # of the path, as above
+    for swaps in (far, turn):
+        for gates, repeats in ((swaps, 101), (mixed + swaps, 3)):
+            st.upload(psi)
+            circ, want = qsim.Circuit(gates, n), psi
+            for _ in range(repeats):
+                out = qsim.run_one_launch(st, circ, None, obs=obs)
+                want = oracle.apply_circuit(want, n, gates)
+            st.sync()
+            if gates is swaps:
+                assert np.array_equal(st.numpy().astype(np.complex128), want)
+            else:
+                assert np.max(np.abs(st.numpy() - want)) < repeats * tol
+            if with_obs:
+                assert abs(float(out.item()) - oracle.expect(want, n, terms)) < 10 * repeats * tol
