@@ -683,13 +683,18 @@ __global__ void __launch_bounds__(kFoldCta) k_sample_fold(const T* __restrict__ 
   const int lane = threadIdx.x & 31;
   const bool folds = (int)(threadIdx.x >> 5) == (int)(blockIdx.x % (kFoldCta / 32)) && lane < G;
   uint64_t r = 0, b = 0;
-  double t = 0.0, acc = 0.0;
+  // the target's bit pattern: sums and values have no sign, so that theirs are in order as
+  // integers, above the pattern of any smaller target.  A target of -0 is 0; infinities and NaNs
+  // of either sign are never exceeded
+  long long tb = 0;
+  double acc = 0.0;
   if (folds) {
     r = (s0 + lane) / a.nshots;
-    t = shot_target(a, s0 + lane, r);
+    const double t = shot_target(a, s0 + lane, r);
     b = shot_block(a, r, t);
     blk[lane] = r * a.nb0 + b;
     acc = start_of(st, r * a.nb0 + b);
+    tb = t == 0.0 ? 0 : t <= 0x1.fffffffffffffp1023 ? __double_as_longlong(t) : 0x7fffffffffffffffll;
   }
   __syncthreads();
   auto first = [&](int g) { return blk[g]; };
@@ -706,10 +711,8 @@ __global__ void __launch_bounds__(kFoldCta) k_sample_fold(const T* __restrict__ 
       for (int j = 0; j < 32; ++j) {
         const double v = row[j];
         acc = __dadd_rn(acc, v);
-        // signs of the comparisons by the bit patterns (none is negative), off the FP64 unit;
-        // a t that is not finite is never exceeded
-        if (found < 0 && __double_as_longlong(acc) > __double_as_longlong(t) && !(__double2hiint(t) >= 0x7ff00000))
-          found = ch * 32 + j;
+        // compared by the bit patterns, off the FP64 unit
+        if (found < 0 && __double_as_longlong(acc) > tb) found = ch * 32 + j;
         const long long vb = __double_as_longlong(v);
         if (vb > 0 && vb <= 0x7ff0000000000000ll) last = ch * 32 + j;
       }

@@ -46,3 +46,26 @@ def test_register_without_weight():
         st = qsim.State(n, dtype=torch.complex64).upload(np.zeros(1 << n))
         u = W.shot_uniforms(8, seed=1)
         assert np.array_equal(st.measure(u)[0], oracle.sample(np.zeros(1 << n, np.complex128), n, u[0]))
+
+
+@pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
+@pytest.mark.parametrize("n,nshots", [(9, 3), (12, 2), (12, 9), (21, 3)])
+def test_targets_that_no_sum_may_exceed(dt, n, nshots):
+    """A target of -0 (amplitudes without weight come first) and a NaN total of either sign: the
+    contract's comparisons are those of floating-point numbers, on every route."""
+    from paper_1912_10877_gb300 import qsim
+    dim = 1 << n
+    u = np.full(nshots, 0.5)
+    u[0] = -0.0
+    first = np.zeros(dim, np.complex128)
+    first[5], first[dim - 3] = 0.6, 0.8
+    states = [first]
+    for nan in (np.nan, np.copysign(np.nan, -1.0)):
+        for at in (2, dim // 2 + 1):
+            psi = first.copy()
+            psi[at] = complex(nan, 0.0)
+            states.append(psi)
+    for k, psi in enumerate(states):
+        st = qsim.State(n, dtype=dt).upload(psi)
+        got = st.measure(u[None])
+        assert np.array_equal(got[0], oracle.sample(st.numpy().astype(np.complex128), n, u)), k
