@@ -303,9 +303,9 @@ int apply_blocks(qs_state* s, const qs_circuit* c, const double* params, int kma
 void free_blocks(const qs_circuit* c);
 
 // samples with device uniforms into device indices (reduce.cu)
-size_t sample_scratch_doubles(int n, int nreg, int nshots);
+size_t sample_scratch_doubles(int n, int nreg, int nshots, bool lean);
 int sample_dev(const void* data, int dtype, int n, int nreg, const double* dev_u, int nshots, int64_t* dev_out,
-               double* scratch, cudaStream_t st);
+               double* scratch, bool lean, cudaStream_t st);
 
 // generator H on a gate's targets and c with U = exp(-i theta c H) (adjoint.cu)
 int gate_generator(const qs_gate_desc& g, std::vector<cd>& G, double* cfac);

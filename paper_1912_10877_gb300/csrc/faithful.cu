@@ -129,12 +129,21 @@ int shot_expect(qs_state* s, const qs_observable* o, const double* host_u, int n
   if (!gs.empty() && (nshots < 1 || !host_u || !work)) return fail(QS_EINVAL, "shots, uniforms and work are needed");
   cudaStream_t st = s->stream;
   const int R = s->nreg;
-  size_t sscr = 0;
-  if (s->uniform) sscr = sample_scratch_doubles(s->nq[0], R, nshots);
-  else
-    for (int r = 0; r < R; ++r) sscr = std::max(sscr, sample_scratch_doubles(s->nq[r], 1, nshots));
   const size_t nsr = (size_t)R * std::max(1, nshots);
-  QS_TRY(ensure_ws(s, s->ws, sizeof(double) * (R + nsr + sscr) + sizeof(int64_t) * nsr + 256));
+  size_t sscr = 0;
+  bool lean = false;
+  auto room = [&] {
+    sscr = 0;
+    for (int r = 0; r < (s->uniform ? 1 : R); ++r)
+      sscr = std::max(sscr, sample_scratch_doubles(s->nq[r], s->uniform ? R : 1, nshots, lean));
+    return ensure_ws(s, s->ws, sizeof(double) * (R + nsr + sscr) + sizeof(int64_t) * nsr + 256);
+  };
+  int rc = room();
+  if (rc == QS_ENOMEM) {
+    lean = true;
+    rc = room();
+  }
+  QS_TRY(rc);
   double* dacc = (double*)s->ws.ptr;
   double* du = dacc + R;
   double* dscr = du + nsr;
@@ -154,11 +163,11 @@ int shot_expect(qs_state* s, const qs_observable* o, const double* host_u, int n
     }
     QS_CUDA(cudaMemcpyAsync(du, host_u + g * nsr, sizeof(double) * nsr, cudaMemcpyHostToDevice, st));
     if (s->uniform) {
-      QS_TRY(sample_dev(work, s->dtype, s->nq[0], R, du, nshots, dsamp, dscr, st));
+      QS_TRY(sample_dev(work, s->dtype, s->nq[0], R, du, nshots, dsamp, dscr, lean, st));
     } else {
       for (int r = 0; r < R; ++r)
         QS_TRY(sample_dev((const char*)work + ab * s->off[r], s->dtype, s->nq[r], 1, du + (size_t)r * nshots, nshots,
-                          dsamp + (size_t)r * nshots, dscr, st));
+                          dsamp + (size_t)r * nshots, dscr, lean, st));
     }
     for (size_t t0 = 0; t0 < G.terms.size(); t0 += kEstTerms) {
       EstTerms e;
@@ -302,9 +311,20 @@ int qs_mmd_gradient(const qs_circuit* c, const double* params, const double* hos
   else if (rc == QS_OK) rc = qs_apply_circuit(s, c, nullptr, 0);
   // device scratch: distributions R x dim, target, kd, Kp - Kq, Kq, diff, dots, samples, uniforms
   const size_t nsr = (size_t)R * std::max(1, nshots);
-  const size_t sscr = nshots > 0 ? sample_scratch_doubles(n, R, nshots) : 0;
-  const size_t doubles = (size_t)R * dim + 5 * dim + (size_t)R + 4 + nsr + sscr;
-  if (rc == QS_OK) rc = ensure_ws(s, s->ws, sizeof(double) * doubles + sizeof(int64_t) * nsr + 256);
+  size_t sscr = 0;
+  bool lean = false;
+  auto room = [&] {
+    sscr = nshots > 0 ? sample_scratch_doubles(n, R, nshots, lean) : 0;
+    const size_t doubles = (size_t)R * dim + 5 * dim + (size_t)R + 4 + nsr + sscr;
+    return ensure_ws(s, s->ws, sizeof(double) * doubles + sizeof(int64_t) * nsr + 256);
+  };
+  if (rc == QS_OK) {
+    rc = room();
+    if (rc == QS_ENOMEM && nshots > 0) {
+      lean = true;
+      rc = room();
+    }
+  }
   if (rc != QS_OK) {
     qs_state_destroy(s);
     return rc;
@@ -325,7 +345,7 @@ int qs_mmd_gradient(const qs_circuit* c, const double* params, const double* hos
     if (nshots > 0) {
       QS_CUDA(cudaMemsetAsync(dist, 0, sizeof(double) * R * dim, st));
       QS_CUDA(cudaMemcpyAsync(du, host_u, sizeof(double) * nsr, cudaMemcpyHostToDevice, st));
-      QS_TRY(sample_dev(s->data, dtype, n, R, du, nshots, dsamp, dscr, st));
+      QS_TRY(sample_dev(s->data, dtype, n, R, du, nshots, dsamp, dscr, lean, st));
       k_hist<<<(unsigned)((nsr + 255) / 256), 256, 0, st>>>(dsamp, nshots, R, dim, (unsigned long long*)dist);
       k_counts_to_dist<<<gb, 256, 0, st>>>(dist, (uint64_t)R * dim, nshots);
     } else if (dtype == QS_C64) {

@@ -741,26 +741,28 @@ __global__ void k_collapse_write(T* psi, uint64_t dim, int64_t x, const double2*
 }
 
 // samples of nreg registers of 2^n amplitudes (back to back) with device uniforms
-// [nreg][nshots] into device indices; scratch: sample_scratch_doubles() doubles
-constexpr uint64_t kRunDoubles = 1ull << 25;  // running sums of the probabilities in scratch: at most 256 MiB
+// [nreg][nshots] into device indices; scratch: sample_scratch_doubles() doubles.  lean: for a
+// device that has no room for the running sums of the probabilities; same samples
+constexpr uint64_t kRunDoubles = 1ull << 25;   // running sums of the probabilities in scratch: at most 256 MiB
+constexpr uint64_t kLeanDoubles = 1ull << 17;  // lean: 1 MiB, those of single-block registers only
 
 // The running sums of every probability cost a second pass over the state and
 // 8 bytes an amplitude, a shot without them folds 1024 probabilities: they are
 // formed once a level-0 block gets a shot or more on the average, or when a
 // register is a single block (whose fold is the running sum).
-static bool keep_runs(int n, int nshots) {
+static bool keep_runs(int n, int nshots, bool lean) {
   const uint64_t dim = 1ull << n, nb0 = (dim + kF - 1) / kF;
-  return nb0 == 1 || (nb0 <= (uint64_t)nshots && dim <= kRunDoubles);
+  return nb0 == 1 || (!lean && nb0 <= (uint64_t)nshots && dim <= kRunDoubles);
 }
 // registers sampled together
-static int sample_group(int n, int nreg) {
-  return (int)std::min<uint64_t>((uint64_t)nreg, std::max<uint64_t>(1, kRunDoubles >> n));
+static int sample_group(int n, int nreg, bool lean) {
+  return (int)std::min<uint64_t>((uint64_t)nreg, std::max<uint64_t>(1, (lean ? kLeanDoubles : kRunDoubles) >> n));
 }
 
-size_t sample_scratch_doubles(int n, int nreg, int nshots) {
+size_t sample_scratch_doubles(int n, int nreg, int nshots, bool lean) {
   const uint64_t dim = 1ull << n, nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF;
   const uint64_t levels = (nb0 > 1 ? 2 * nb0 : 0) + (nb1 > 1 ? 2 * nb1 : 0);
-  return (size_t)((levels + (keep_runs(n, nshots) ? dim : 0)) * (uint64_t)sample_group(n, nreg));
+  return (size_t)((levels + (keep_runs(n, nshots, lean) ? dim : 0)) * (uint64_t)sample_group(n, nreg, lean));
 }
 
 template <typename T, bool RUN>
@@ -781,10 +783,10 @@ static int launch_fold(const T* src, uint64_t nblocks, uint64_t len, const FoldS
 
 template <typename T>
 static int sample_regs(const T* psi, int n, int nreg, const double* dev_u, int nshots, int64_t* dev_out, double* scratch,
-                       cudaStream_t st) {
+                       bool lean, cudaStream_t st) {
   const uint64_t dim = 1ull << n, R = (uint64_t)nreg;
   const uint64_t nb0 = (dim + kF - 1) / kF, nb1 = (nb0 + kF - 1) / kF, len0 = std::min<uint64_t>(dim, kF);
-  const bool runs = keep_runs(n, nshots);
+  const bool runs = keep_runs(n, nshots, lean);
   SampleArgs a;
   memset(&a, 0, sizeof(a));
   a.u = dev_u;
@@ -831,15 +833,15 @@ static int sample_regs(const T* psi, int n, int nreg, const double* dev_u, int n
 }
 
 int sample_dev(const void* data, int dtype, int n, int nreg, const double* dev_u, int nshots, int64_t* dev_out,
-               double* scratch, cudaStream_t st) {
-  const int group = sample_group(n, nreg);
+               double* scratch, bool lean, cudaStream_t st) {
+  const int group = sample_group(n, nreg, lean);
   for (int r = 0; r < nreg; r += group) {
     const int k = std::min(group, nreg - r);
     const char* p = (const char*)data + ((amp_bytes(dtype) * (size_t)r) << n);
     const double* u = dev_u + (size_t)r * nshots;
     int64_t* out = dev_out + (size_t)r * nshots;
-    if (dtype == QS_C64) QS_TRY(sample_regs((const float2*)p, n, k, u, nshots, out, scratch, st));
-    else QS_TRY(sample_regs((const double2*)p, n, k, u, nshots, out, scratch, st));
+    if (dtype == QS_C64) QS_TRY(sample_regs((const float2*)p, n, k, u, nshots, out, scratch, lean, st));
+    else QS_TRY(sample_regs((const double2*)p, n, k, u, nshots, out, scratch, lean, st));
   }
   return QS_OK;
 }
@@ -859,13 +861,32 @@ __global__ void k_seeded_uniforms(uint64_t seed, uint64_t k0, uint64_t nshots, d
 }
 
 // nreg registers of 2^n amplitudes back to back; the uniforms are host_u or drawn
-// from seed (shot j of register r: draw k0 + r nshots + j + 1)
+// from seed (shot j of register r: draw k0 + r nshots + j + 1).  Scratch that the device
+// has no room for: without the running sums, then half the registers at a time.
 int measure_regs(void* data, int dtype, int n, int nreg, const double* host_u, int nshots, int64_t* host_out,
                  int collapse, qs_state* owner, const uint64_t* seed, uint64_t k0) {
   cudaStream_t st = owner->stream;
   const uint64_t dim = 1ull << n;
-  const size_t shots = (size_t)nreg * nshots, scr = sample_scratch_doubles(n, nreg, nshots);
-  QS_TRY(ensure_ws(owner, owner->ws, sizeof(double) * (scr + shots) + sizeof(int64_t) * shots + sizeof(double2) + 256));
+  const size_t shots = (size_t)nreg * nshots;
+  bool lean = false;
+  auto room = [&] {
+    return ensure_ws(owner, owner->ws, sizeof(double) * (sample_scratch_doubles(n, nreg, nshots, lean) + shots) +
+                                           sizeof(int64_t) * shots + sizeof(double2) + 256);
+  };
+  int rc = room();
+  if (rc == QS_ENOMEM) {
+    lean = true;
+    rc = room();
+  }
+  if (rc == QS_ENOMEM && nreg > 1) {
+    const int h = nreg / 2;
+    const size_t k = (size_t)h * nshots;
+    QS_TRY(measure_regs(data, dtype, n, h, host_u, nshots, host_out, collapse, owner, seed, k0));
+    return measure_regs((char*)data + ((amp_bytes(dtype) * (size_t)h) << n), dtype, n, nreg - h,
+                        host_u ? host_u + k : nullptr, nshots, host_out + k, collapse, owner, seed, k0 + k);
+  }
+  QS_TRY(rc);
+  const size_t scr = sample_scratch_doubles(n, nreg, nshots, lean);
   double* dscr = (double*)owner->ws.ptr;
   double* du = dscr + scr;
   int64_t* dout = (int64_t*)(du + shots);
@@ -876,7 +897,7 @@ int measure_regs(void* data, int dtype, int n, int nreg, const double* host_u, i
   } else {
     QS_CUDA(cudaMemcpyAsync(du, host_u, sizeof(double) * shots, cudaMemcpyHostToDevice, st));
   }
-  QS_TRY(sample_dev(data, dtype, n, nreg, du, nshots, dout, dscr, st));
+  QS_TRY(sample_dev(data, dtype, n, nreg, du, nshots, dout, dscr, lean, st));
   QS_CUDA(cudaMemcpyAsync(host_out, dout, sizeof(int64_t) * shots, cudaMemcpyDeviceToHost, st));
   QS_CUDA(cudaStreamSynchronize(st));
   if (!collapse) return QS_OK;

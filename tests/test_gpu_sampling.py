@@ -69,3 +69,35 @@ def test_targets_that_no_sum_may_exceed(dt, n, nshots):
         st = qsim.State(n, dtype=dt).upload(psi)
         got = st.measure(u[None])
         assert np.array_equal(got[0], oracle.sample(st.numpy().astype(np.complex128), n, u)), k
+
+
+def test_device_without_room_for_the_running_sums():
+    """128 MiB left on the device: the running sums of 2^25 probabilities do not fit (256 MiB),
+    nor do 2^24 uniforms with their samples; the same samples as with room."""
+    from paper_1912_10877_gb300 import qsim
+
+    def amplitudes(st, seed):
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        st.buffer.copy_(torch.randn(st.buffer.shape, dtype=st.buffer.dtype, device="cuda", generator=g))
+        return st
+
+    cases = [([25], 1 << 15), ([4] * 4096, 4096)]  # as many shots as level-0 blocks; many shots on many registers
+    states = [amplitudes(qsim.State(sizes, dtype=torch.complex64), k) for k, (sizes, _) in enumerate(cases)]
+    uniforms = [W.shot_uniforms(nshots, seed=k, nreg=len(sizes)) for k, (sizes, nshots) in enumerate(cases)]
+    want = []
+    for (sizes, _), st, u in zip(cases, states, uniforms):
+        other = qsim.State(sizes, dtype=torch.complex64)
+        other.buffer.copy_(st.buffer)
+        other.measure(u[:, :2])  # the kernels of either route are loaded
+        want.append(other.measure(u))
+        del other
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (128 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got = [st.measure(u) for st, u in zip(states, uniforms)]
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    for g, w in zip(got, want):
+        assert np.array_equal(g, w)
