@@ -403,8 +403,9 @@ int qs_apply_circuit(qs_state* s, const qs_circuit* c, const double* host_params
  * buffer and the block tables).  With grid_ctas = 0 a circuit of single-target
  * gates (controls allowed, a gate spanning at most QS_MAXK qubits) and
  * uncontrolled SWAPs on up to 14 qubits runs in one thread-block cluster
- * instead, gate by gate (runs of uncontrolled gates fused, kmax unused;
- * complex64 gates compensated as with QS_APPLY_PRECISE), without scratch. */
+ * instead, gate by gate (runs of uncontrolled gates fused; complex64 gates
+ * compensated as with QS_APPLY_PRECISE), without scratch, unless its blocks of
+ * kmax qubits are estimated to take less (many gates on few qubits). */
 int qs_run_circuit_one_launch(qs_state* s, const qs_circuit* c, const double* host_params, int kmax,
                               const qs_observable* o, int grid_ctas, double* dev_out);
 

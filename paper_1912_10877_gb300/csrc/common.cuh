@@ -289,7 +289,7 @@ int launch_block_tc(float2* psi, int n, int nreg, const Plan& p, cudaStream_t st
 int tc_status_take();  // QS_ETIMEDOUT (and clears it) if a bounded device wait gave up
 int tc_status_address(int** out);  // device address of that status word (current device)
 // a circuit of single-target gates on a small register in one cluster (smallrun.cu)
-int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* params, const qs_observable* o,
+int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* params, int kmax, const qs_observable* o,
                       double* dev_out, cudaStream_t st);
 void free_smallrun(const qs_circuit* c);
 void free_onelaunch(const qs_circuit* c);  // releases the one-launch tables of a circuit

@@ -342,9 +342,9 @@ int qs_run_circuit_one_launch(qs_state* s, const qs_circuit* c, const double* ho
       ++a.nterm;
     }
   }
-  // single-target gates on up to 14 qubits, every SM asked for: one cluster
+  // single-target gates on up to 14 qubits, every SM asked for: one cluster where that takes less
   if (grid_ctas <= 0) {
-    const int rc = run_small_circuit(s->data, s->dtype, c, host_params, o, dev_out, s->stream);
+    const int rc = run_small_circuit(s->data, s->dtype, c, host_params, kmax, o, dev_out, s->stream);
     if (rc != QS_EUNSUPPORTED) return rc;
   }
   OLCache* k = nullptr;

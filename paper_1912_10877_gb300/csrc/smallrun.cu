@@ -332,13 +332,51 @@ void schedule(std::vector<LOp> left, int n, int lc, std::vector<int>& at, std::v
 // ------------------------------------------------------------------ host: launch
 
 struct RunCache {
-  int dtype = -1, device = -1;
+  int dtype = -1, device = -1, kmax = 0;
   bool fits = false, asked = false;
   std::vector<double> params;
   std::vector<RunOp<float>> f;
   std::vector<RunOp<double>> d;
   std::vector<int> place;  // physical bit of each qubit at the end
 };
+
+// Whether the ops take less here than the circuit's blocks of kmax qubits would in the
+// cooperative launch (k_onelaunch, every SM, a grid barrier a block): a block takes the same time
+// whatever the number of its gates, an op grows with the amplitudes that a CTA holds (16 CTAs at
+// most).  Nanoseconds, fitted to 2200 pairs of times over 3 to 14 qubits, kmax 2, 4 and 5, circuits
+// that spread over the register or pile up on two or five qubits (the times of either side within
+// a third of the fit; the path taken at most 1.21 of the better one, in 22 cases over 1.03).
+// Measured, complex64 / complex128: 300 controlled Rx on five of 10 qubits 98 / 143 us here, 13 / 15
+// us as one block; the same over all 14 qubits 182 / 643 us here, 287 / 483 us as blocks for 200 of
+// them; 10 layers of Rz Rx Rz and a CNOT ring on 12 qubits 56 / 97 us here, 151 / 194 us as blocks.
+// A circuit with parameters pays the host for the block matrices whenever its angles change, and
+// a pass with new angles counts as much as one with the same: half of that (18 ns a gate for every
+// row of its block's matrix, 110 ns a gate here) goes to the blocks' side.
+template <typename R>
+bool cluster_pays(const std::vector<RunOp<R>>& ops, const qs_circuit* c, int kmax) {
+  const bool f64 = sizeof(R) == 8;
+  const int n = c->nqubits;
+  const int64_t a = n > 11 ? 1ll << (n - 11) : 1;  // FP64 warps' shares of a CTA's amplitudes
+  int64_t here = 0;
+  for (const RunOp<R>& o : ops) switch (o.kind) {
+      case RU_DIAG: here += f64 ? 120 + 100 * a : 160 + 12 * a; break;
+      case RU_X: here += 180; break;
+      case RU_DENSE: here += f64 ? 190 + 230 * a : 240 + 45 * a; break;
+      default: here += 500 + 200 * a;
+    }
+  int nb = 0;
+  if (qs_circuit_blocks(c, nullptr, kmax, &nb, nullptr, nullptr, nullptr) != QS_OK) return true;
+  std::vector<int32_t> widths(std::max(1, nb));
+  if (qs_circuit_blocks(c, nullptr, kmax, &nb, widths.data(), nullptr, nullptr) != QS_OK) return true;
+  const int64_t block = f64 ? (n < 10 ? 4600 : 5800) + 400 * (a - 1) : 4000 + 200 * (a - 1);
+  int64_t blocks = 2500 + nb * block;
+  if (c->nparams > 0 && nb > 0) {
+    int64_t rows = 0;
+    for (int b = 0; b < nb; ++b) rows += 1ll << widths[b];
+    blocks += 4000 + std::max<int64_t>(0, (9 * rows / nb - 55) * (int64_t)c->gates.size());
+  }
+  return here <= blocks;
+}
 
 // CTAs of the cluster: one for every 128 amplitudes (a warp for each FP64 unit of an SM)
 int rank_bits(int n) { return std::max(0, std::min(4, n - 7)); }
@@ -391,8 +429,9 @@ void free_smallrun(const qs_circuit* c) {
 }
 
 // Runs circuit c on the single register at `data`, <o> (Z strings) to dev_out if not NULL.
-// QS_EUNSUPPORTED, with nothing launched: the circuit is not one of this path's.
-int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* params, const qs_observable* o,
+// QS_EUNSUPPORTED, with nothing launched: the circuit is not one of this path's, or takes
+// less as blocks of kmax qubits.
+int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* params, int kmax, const qs_observable* o,
                       double* dev_out, cudaStream_t st) {
   const int n = c->nqubits;
   if (n > kRunMaxQubits || (o && o->terms.size() > (size_t)kRunTerms)) return QS_EUNSUPPORTED;
@@ -400,13 +439,14 @@ int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* 
   QS_CUDA(cudaGetDevice(&dev));
   RunCache* k = static_cast<RunCache*>(c->smallrun);
   const int np = c->nparams;
-  if (!k || k->dtype != dtype || k->device != dev || (int)k->params.size() != np ||
+  if (!k || k->dtype != dtype || k->device != dev || k->kmax != kmax || (int)k->params.size() != np ||
       (np && std::memcmp(k->params.data(), params, sizeof(double) * np) != 0)) {
     free_smallrun(c);
     k = new RunCache();
     c->smallrun = k;  // owned by the circuit
     k->dtype = dtype;
     k->device = dev;
+    k->kmax = kmax;
     if (np) k->params.assign(params, params + np);
     std::vector<LOp> ops;
     std::vector<int> label, at;
@@ -421,7 +461,8 @@ int run_small_circuit(void* data, int dtype, const qs_circuit* c, const double* 
       else schedule(ops, n, rank_bits(n), at, k->d);
       k->place.resize(n);
       for (int q = 0; q < n; ++q) k->place[q] = at[label[q]];
-      k->fits = std::max(k->f.size(), k->d.size()) <= (size_t)kRunCaps[2];
+      k->fits = std::max(k->f.size(), k->d.size()) <= (size_t)kRunCaps[2] &&
+                (dtype == QS_C64 ? cluster_pays(k->f, c, kmax) : cluster_pays(k->d, c, kmax));
     }
   }
   if (!k->fits) return QS_EUNSUPPORTED;

@@ -107,3 +107,33 @@ def test_swaps_with_no_barrier_among_the_gates(dt, n, with_obs):
                 assert np.max(np.abs(st.numpy() - want)) < repeats * tol
             if with_obs:
                 assert abs(float(out.item()) - oracle.expect(want, n, terms)) < 10 * repeats * tol
+
+
+@pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
+@pytest.mark.parametrize("n,kmax", [(5, 5), (8, 5), (11, 5), (14, 5), (14, 4), (10, 2)])
+def test_gates_piled_on_few_qubits_run_as_blocks(dt, n, kmax):
+    """Hundreds of gates on kmax qubits are one block: the same bits as the block launch that the
+    caller asks for by its CTAs.  A variational circuit keeps to the cluster (its bits differ)."""
+    from paper_1912_10877_gb300 import qsim
+    rs = W.rng(n)
+    piled = []
+    for _ in range(300):
+        a, b = (int(v) for v in rs.permutation(kmax)[:2])
+        piled.append(W.Gate("RX", (a,), (b,), (1,), theta=float(rs.uniform(-3, 3))))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    psi = W.haar_state(n, seed=n)
+    gates, params = W.variational(n, 4, "ring")
+    angles = [W.Gate(g.name, g.locs, g.ctrl_locs, g.ctrl_vals, theta=None if g.param is None else float(params[g.param]))
+              for g in gates]
+    for g, blocks in ((piled, True), (angles, False)):
+        if not blocks and (n == 5 or n == 14):
+            continue  # near the line between the two
+        circ, got = qsim.Circuit(g, n), []
+        for ctas in (0, sms):
+            st = qsim.State(n, dtype=dt).upload(psi)
+            qsim.run_one_launch(st, circ, None, kmax=kmax, grid_ctas=ctas)
+            st.sync()
+            got.append(st.numpy())
+        assert np.array_equal(*got) == blocks
+        want = oracle.apply_circuit(psi, n, g)
+        assert np.max(np.abs(got[0] - want)) < (1e-12 if dt == torch.complex128 else 2e-5)
