@@ -152,6 +152,11 @@ struct Fuser {
   }
   int drain() {
     if (plans.empty()) return QS_OK;
+    if (!small_pays(s->dtype, s->nq[0], plans)) {
+      for (const Plan& p : plans) QS_TRY(launch_plan(s, p));
+      plans.clear();
+      return QS_OK;
+    }
     const int rc = apply_small(s->data, s->dtype, s->nq[0], s->nreg, plans, s->stream);
     plans.clear();
     return rc;

@@ -263,6 +263,28 @@ bool small_plan(const Plan& p) {
   return small_op<float>(p, &o);
 }
 
+// A lone gate is the cheaper launch of its own kernel (10 qubits: 6.0 us a call against 7.6).
+// At 14 qubits complex128 the FP64 arithmetic of a cluster's eight SMs takes about as long as the
+// launch it saves: the first launch's 5 us have to come out of what a list's gates gain (tenths of
+// a microsecond each).  Measured, here and as launches: a dense 2x2 on every qubit 86.0 and 84.0
+// us, H 41 and 57, Rx 57.7 and 57.4; H on two qubits 10.3 and 8.3; two controlled X 6.1 and 7.4, two
+// T 8.2 and 12.4; six controlled Rx 20.5 and 24.6; 2, 6 and 20 controlled dense gates 16.0, 36.9 and
+// 96 against 12.3, 32.8 and 113.
+bool small_pays(int dtype, int n, const std::vector<Plan>& plans) {
+  if (plans.size() < 2) return false;
+  if (dtype == QS_C64 || n < kSmallMaxQubits) return true;
+  int gain = 0;
+  for (const Plan& p : plans) {
+    const bool ctrl = p.ctrl_mask != 0;
+    if (p.op == OP_DENSE1) gain += ctrl ? 7 : 0;
+    else if (p.op == OP_RXLIKE1) gain += ctrl ? 12 : 3;
+    else if (p.op == OP_REAL1 || p.op == OP_HLIKE1) gain += ctrl ? 20 : 15;
+    else gain += 26;
+    if (gain > 50) return true;
+  }
+  return false;
+}
+
 int apply_small(void* data, int dtype, int n, int nreg, const std::vector<Plan>& plans, cudaStream_t st) {
   if (dtype == QS_C64) return run_small<float>((float2*)data, n, nreg, plans, st);
   return run_small<double>((double2*)data, n, nreg, plans, st);

@@ -74,3 +74,19 @@ def test_small_batches_and_per_register_parameters(dt):
     out = st.numpy().reshape(nreg, -1)
     for r in range(nreg):
         assert np.max(np.abs(out[r] - oracle.apply_circuit(psi[r], n, gates, params[0]))) < TOL[dt]
+
+
+@pytest.mark.parametrize("dt", ["c64", "c128"])
+def test_short_lists_and_dense_layers_keep_their_bits(dt):
+    """Lists that go gate by gate (one gate; at 14 qubits complex128 dense gates alone) and their
+    neighbours that do not: the bits of a launch a gate in the same order."""
+    from paper_1912_10877_gb300 import qsim
+    for n in (1, 3, 10, 13, 14):
+        psi = W.haar_state(n, seed=n)
+        layer = [W.Gate("MATRIX", (q,), matrix=W.haar_su2(q)) for q in range(n)]
+        real = [W.Gate("H", (q,)) for q in range(n)]
+        for gates in (layer[:1], real[:1], layer, real, [W.Gate("T", (0,), (n - 1,))] + layer if n > 1 else real):
+            circ, got = qsim.Circuit(gates, n), []
+            for fused in (True, False):
+                got.append(qsim.State(n, dtype=TDT[dt]).upload(psi).apply_circuit(circ, fused=fused).numpy())
+            assert np.array_equal(*got), (n, len(gates))
