@@ -1843,7 +1843,8 @@ constexpr uint32_t kFpTab = kFpTile + 2 * sizeof(float4) * kTileRuns;  // the ru
 constexpr uint32_t kFpDiag = kFpTab + sizeof(float4) * kTileRuns * kRunTab;
 constexpr uint32_t kFpCtx = kFpDiag + sizeof(float2) * 16 * kTileTabs;
 constexpr uint32_t kFpBytes = kFpCtx + sizeof(RunCtx);
-static_assert(kFpBytes <= 227 * 1024 && kFpRuns % 16 == 0 && kFpTile % 16 == 0, "a pass's shared memory");
+constexpr int kMaxSmem = 227 * 1024;  // of a CTA
+static_assert(kFpBytes <= kMaxSmem && kFpRuns % 16 == 0 && kFpTile % 16 == 0, "a pass's shared memory");
 
 // run_tile_fwd of a pass whose records and tables all lie in shared memory
 __device__ __noinline__ void run_tile_staged(uint32_t sm, int nphase, uint32_t tile, int m, uint32_t tbase) {
@@ -3326,8 +3327,8 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
   const int np = c->nparams;
   size_t smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + sizeof(float) * phase_vals(c->nparams) * kWarps +
                 sizeof(double) * ((np + 1) & ~1) + 2 * sizeof(float2) * (1ull << m);
-  if (smem > 227 * 1024) return fail(QS_EUNSUPPORTED, "%d parameters do not fit the tiled backward's shared memory", np);
-  const bool stage = smem + kStageBytes <= 227 * 1024;
+  if (smem > kMaxSmem) return fail(QS_EUNSUPPORTED, "%d parameters do not fit the tiled backward's shared memory", np);
+  const bool stage = smem + kStageBytes <= kMaxSmem;
   if (stage) smem += kStageBytes;
   if (host_loss) QS_TRY(expect_raw(s->data, QS_C64, n, 1, o, s, host_loss));
   if (np > 0) {
@@ -3365,7 +3366,8 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
     QS_LAUNCHED();
   }
   // per-CTA partials and the gradient accumulator in the state's scratch
-  QS_CUDA(cudaFuncSetAttribute(k_fused_bwd_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit belongs to the function: the same for every circuit, as other threads launch theirs
+  QS_CUDA(cudaFuncSetAttribute(k_fused_bwd_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
   int dev = 0, sms = 0, per_sm = 0;
   QS_CUDA(cudaGetDevice(&dev));
   QS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

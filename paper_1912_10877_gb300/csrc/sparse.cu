@@ -183,12 +183,14 @@ __global__ void k_scan_add(int64_t* __restrict__ a, uint64_t n, const int64_t* _
 // shared memory of k_sp_fill: the groups' records, the trie, the tables; then per
 // warp the large groups' leading sums and row values, the entry codes and the small
 // groups' sign patterns of the rows' low bits
-__host__ __device__ inline size_t fill_common(int ngroups) {
+__host__ __device__ constexpr size_t fill_common(int ngroups) {
   return ((size_t)ngroups * (sizeof(SpGroup) + sizeof(uint32_t) + kTab * sizeof(double2)) + 15) & ~(size_t)15;
 }
-__host__ __device__ inline size_t fill_per_warp(int ngroups, int nlarge) {
+__host__ __device__ constexpr size_t fill_per_warp(int ngroups, int nlarge) {
   return (size_t)nlarge * 32 * 2 * sizeof(double2) + (size_t)ngroups * 32 * (sizeof(uint16_t) + 1);
 }
+constexpr size_t kFillSmem = 100 * 1024;  // of a CTA: two an SM
+static_assert(fill_common(kSpMaxGroups) + fill_per_warp(kSpMaxGroups, kSpMaxGroups) <= kFillSmem, "one warp always fits");
 
 __global__ void __launch_bounds__(32 * kFillWarps)
 k_sp_fill(const __grid_constant__ SpTerms T, const __grid_constant__ SpTable tables, uint64_t dim, int segs,
@@ -387,9 +389,10 @@ int qs_observable_csr_fill(const qs_observable* o, int nqubits, const int64_t* d
   // warps of a CTA: as many as keep two CTAs on an SM, at least one
   const size_t common = fill_common(T.ngroups), per = fill_per_warp(T.ngroups, T.nlarge);
   int warps = kFillWarps;
-  while (warps > 1 && common + warps * per > 100 * 1024) warps >>= 1;
+  while (warps > 1 && common + warps * per > kFillSmem) warps >>= 1;
   const size_t smem = common + warps * per;
-  QS_CUDA(cudaFuncSetAttribute(k_sp_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit belongs to the function: the same for every observable, as other threads launch theirs
+  QS_CUDA(cudaFuncSetAttribute(k_sp_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFillSmem));
   const uint64_t rows = (dim / segs + 31) / 32;
   k_sp_fill<<<(unsigned)((rows + warps - 1) / warps), 32 * warps, smem, st>>>(T, tab, dim, segs, dev_rowptr, dev_cols,
                                                                            (double2*)dev_vals);
