@@ -1072,12 +1072,16 @@ __device__ __forceinline__ TOp load_op(const TOp* p) {
 // indices rebased to the pass's first op.  A pass larger than the staging
 // area keeps reading global memory.
 constexpr int kStagePhases = 32;
-constexpr int kStageOps = 480;
-constexpr int kStageRecs = 256;  // forward: TK_DIAGRUN entries; backward: GMem records
+constexpr int kStageOps = 512;
+// forward: TK_DIAGRUN entries; backward: GMem records.  Where shared memory does not hold that many
+// beside the rest (precise path, tiled gradients with thousands of parameters), fewer
+constexpr int kStageRecs = 256, kStageRecsPrec = 224;
 static_assert(sizeof(TOp) == 64 && sizeof(TOp) % 16 == 0, "TOp is copied as 16-byte words");
 static_assert(sizeof(DRun) == 32 && sizeof(GMem) == 32, "records are copied as 16-byte words");
 constexpr size_t kStagePhaseBytes = (sizeof(TPhase) * kStagePhases + 15) & ~size_t(15);
-constexpr size_t kStageBytes = kStagePhaseBytes + sizeof(TOp) * kStageOps + sizeof(DRun) * kStageRecs;
+constexpr size_t stage_bytes(int recs) { return kStagePhaseBytes + sizeof(TOp) * kStageOps + sizeof(DRun) * recs; }
+constexpr size_t kStageBytes = stage_bytes(kStageRecs);
+constexpr int kMaxSmem = 227 * 1024;  // of a CTA
 
 struct StagedPass {
   const TPhase* ph;  // the pass's first phase
@@ -1088,14 +1092,14 @@ struct StagedPass {
 };
 
 // FWD: the forward ops (fop0 / nfop), else the backward ops (bop0 / nbop).
-// buf: kStageBytes of shared memory, or nullptr.  Every thread of the CTA
+// buf: stage_bytes(room) of shared memory, or nullptr.  Every thread of the CTA
 // calls this (it ends with a barrier when it copies).
 template <bool FWD>
-__device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp* ops, unsigned char* buf,
+__device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp* ops, unsigned char* buf, int room,
                                  const DRun* druns, const GMem* gmem) {
   StagedPass r{phases + p.phase0, ops, 0, FWD ? druns + p.drun0 : nullptr, gmem};
   if (!buf || p.nphase <= 0 || p.nphase > kStagePhases) return r;
-  if (FWD && p.ndrun > kStageRecs) return r;
+  if (FWD && p.ndrun > room) return r;
   const TPhase& f0 = phases[p.phase0];
   const TPhase& fl = phases[p.phase0 + p.nphase - 1];
   const int first = FWD ? f0.fop0 : f0.bop0;
@@ -1115,7 +1119,7 @@ __device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp
   }
   // a pass with more GMem records than the area holds reads those from global memory
   uint4* rd = reinterpret_cast<uint4*>(buf + kStagePhaseBytes + sizeof(TOp) * kStageOps);
-  const bool recs = FWD || p.nmem <= kStageRecs;
+  const bool recs = FWD || p.nmem <= room;
   const uint4* rs = FWD ? reinterpret_cast<const uint4*>(druns + p.drun0) : reinterpret_cast<const uint4*>(gmem + p.mem0);
   for (int i = threadIdx.x; recs && i < (FWD ? p.ndrun : p.nmem) * 2; i += blockDim.x) rd[i] = rs[i];
   __syncthreads();
@@ -1594,7 +1598,7 @@ __device__ __noinline__ void batch_bwd_streamed(uint32_t sx, uint32_t sl, const 
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, nullptr, gmem);
+    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, kStageRecs, nullptr, gmem);
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
       load_tiles<true>(sx, wp + tb, sl, wl + tb, rows, m);
@@ -1615,7 +1619,7 @@ __device__ __noinline__ void batch_bwd_streamed_ff(uint32_t sx, uint32_t sl, con
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, nullptr, gmem);
+    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, kStageRecsPrec, nullptr, gmem);
     const float2* lo = blo + 4 * (size_t)sp.first;
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
@@ -1658,7 +1662,7 @@ __device__ __noinline__ void batch_fwd_streamed(uint32_t sx, uint32_t sx2, float
   for (int pi = 0; pi < npass; ++pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<true>(p, phases, fops, stage, druns, nullptr);
+    const StagedPass sp = stage_pass<true>(p, phases, fops, stage, COMP ? kStageRecsPrec : kStageRecs, druns, nullptr);
     const float2* lo = COMP ? flo + 4 * (size_t)sp.first : nullptr;
     if (threadIdx.x == 0) *sh<RunCtx>(rc) = RunCtx{sp.runs, rtab + kRunTab * p.run0, nullptr};
     // two tile buffers (sx, sx2): the next tile's copies are in flight while
@@ -1792,10 +1796,11 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
 }
 
 // bytes of dynamic shared memory of k_batch<RB, PREC>
-static size_t batch_smem(int rb, bool prec) {
+static constexpr size_t batch_smem(int rb, bool prec) {
   const size_t mt = (size_t)1 << (9 + rb);
-  return ((sizeof(BShared) + 255) & ~size_t(255)) + (prec ? (8 + 32) * mt : 16 * mt) + kStageBytes;
+  return ((sizeof(BShared) + 255) & ~size_t(255)) + (prec ? (8 + 32) * mt + stage_bytes(kStageRecsPrec) : 16 * mt + kStageBytes);
 }
+static_assert(batch_smem(kRB, false) <= kMaxSmem && batch_smem(3, true) <= kMaxSmem, "a register's shared memory");
 
 // the instantiation of k_batch for a phase width and path
 static const void* batch_kernel(int rb, bool prec) {
@@ -1843,7 +1848,6 @@ constexpr uint32_t kFpTab = kFpTile + 2 * sizeof(float4) * kTileRuns;  // the ru
 constexpr uint32_t kFpDiag = kFpTab + sizeof(float4) * kTileRuns * kRunTab;
 constexpr uint32_t kFpCtx = kFpDiag + sizeof(float2) * 16 * kTileTabs;
 constexpr uint32_t kFpBytes = kFpCtx + sizeof(RunCtx);
-constexpr int kMaxSmem = 227 * 1024;  // of a CTA
 static_assert(kFpBytes <= kMaxSmem && kFpRuns % 16 == 0 && kFpTile % 16 == 0, "a pass's shared memory");
 
 // run_tile_fwd of a pass whose records and tables all lie in shared memory
@@ -1882,7 +1886,7 @@ __device__ __forceinline__ void tile_products(float4* out, const DRun* entries, 
 __global__ void __launch_bounds__(kTileThreads, 1) k_fused_pass(FArgs a) {
   const TPass& p = *a.pass;
   set_rows(sh<uint32_t>(0), p, a.m);
-  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, sh<unsigned char>(kFpStage), a.druns, nullptr);
+  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, sh<unsigned char>(kFpStage), kStageRecs, a.druns, nullptr);
   // the runs' tables, and their tile products for this tile and the one before
   const bool held = p.nrun <= kTileRuns;
   const bool staged = held && p.ndt <= kTileTabs && sp.ph != a.phases + p.phase0;
@@ -1949,7 +1953,7 @@ struct FBArgs {
   const GMem* gmem;
   int vals;              // gradient sums of a phase, at most
   int m, g, nparam;
-  int stage;             // 1: kStageBytes of shared memory after the tiles hold the pass's records
+  int stage;             // GMem records that stage_pass's area after the tiles has room for (-1: no area)
   uint64_t ntile;
   double* partials;      // [gridDim.x][nparam]
 };
@@ -1961,11 +1965,11 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_bwd_pass(FBArgs a) {
   double* gacc = reinterpret_cast<double*>(red + a.vals * kWarps);
   float2* sx = reinterpret_cast<float2*>(gacc + ((a.nparam + 1) & ~1));
   float2* sl = sx + (1 << a.m);
-  unsigned char* stage = a.stage ? reinterpret_cast<unsigned char*>(sl + (1 << a.m)) : nullptr;
+  unsigned char* stage = a.stage >= 0 ? reinterpret_cast<unsigned char*>(sl + (1 << a.m)) : nullptr;
   const TPass& p = *a.pass;
   for (int i = threadIdx.x; i < a.nparam; i += blockDim.x) gacc[i] = 0.0;
   set_rows(rowoff, p, a.m);
-  const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage, nullptr, a.gmem);
+  const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage, a.stage, nullptr, a.gmem);
   auto at = [&](const void* q) { return (uint32_t)((const unsigned char*)q - smraw); };
   for (uint64_t t = blockIdx.x; t < a.ntile; t += gridDim.x) {
     const uint64_t tb = tile_base(t, p, a.g);
@@ -3328,8 +3332,9 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
   size_t smem = sizeof(uint32_t) * (1 << (kMaxTileBits - kRowBits)) + sizeof(float) * phase_vals(c->nparams) * kWarps +
                 sizeof(double) * ((np + 1) & ~1) + 2 * sizeof(float2) * (1ull << m);
   if (smem > kMaxSmem) return fail(QS_EUNSUPPORTED, "%d parameters do not fit the tiled backward's shared memory", np);
-  const bool stage = smem + kStageBytes <= kMaxSmem;
-  if (stage) smem += kStageBytes;
+  // without room for the records those are read from global memory, once a phase
+  const int stage = smem + kStageBytes <= kMaxSmem ? kStageRecs : smem + stage_bytes(0) <= kMaxSmem ? 0 : -1;
+  if (stage >= 0) smem += stage_bytes(stage);
   if (host_loss) QS_TRY(expect_raw(s->data, QS_C64, n, 1, o, s, host_loss));
   if (np > 0) {
     if (P->dparams_n < np) {
@@ -3390,7 +3395,7 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
   a.m = m;
   a.g = g;
   a.nparam = np;
-  a.stage = stage ? 1 : 0;
+  a.stage = stage;
   a.ntile = ntile;
   a.partials = partials;
   auto swaps = [&](const std::vector<std::pair<int, int>>& net) -> int {  // its own inverse, on psi and lambda
