@@ -870,7 +870,7 @@ __device__ __forceinline__ T* sh(uint32_t off) {
 
 struct BShared {
   double grad[kMaxRegParams];
-  float red[kMaxPhaseVals * kWarps];
+  alignas(16) float red[kMaxPhaseVals * kWarps];  // in the forward: a pass's TK_DIAGRUN entries
   double lred[kWarps];
   uint32_t rowoff[1 << (kMaxTileBits - kRowBits)];  // register offset of each 32-amplitude tile row (current pass)
   RunCtx rc;
@@ -1073,14 +1073,14 @@ __device__ __forceinline__ TOp load_op(const TOp* p) {
 // area keeps reading global memory.
 constexpr int kStagePhases = 32;
 constexpr int kStageOps = 512;
-// forward: TK_DIAGRUN entries; backward: GMem records.  Where shared memory does not hold that many
-// beside the rest (precise path, tiled gradients with thousands of parameters), fewer
-constexpr int kStageRecs = 256, kStageRecsPrec = 224;
+constexpr int kStageRuns = 256;  // forward: TK_DIAGRUN entries
+constexpr int kStageMems = 224;  // backward: GMem records
 static_assert(sizeof(TOp) == 64 && sizeof(TOp) % 16 == 0, "TOp is copied as 16-byte words");
 static_assert(sizeof(DRun) == 32 && sizeof(GMem) == 32, "records are copied as 16-byte words");
+static_assert(sizeof(DRun) * kStageRuns <= sizeof(BShared::red), "a pass's entries in the forward");
 constexpr size_t kStagePhaseBytes = (sizeof(TPhase) * kStagePhases + 15) & ~size_t(15);
-constexpr size_t stage_bytes(int recs) { return kStagePhaseBytes + sizeof(TOp) * kStageOps + sizeof(DRun) * recs; }
-constexpr size_t kStageBytes = stage_bytes(kStageRecs);
+constexpr size_t kStageBytes = kStagePhaseBytes + sizeof(TOp) * kStageOps;  // then the records
+constexpr size_t kStageMemBytes = sizeof(GMem) * kStageMems;
 constexpr int kMaxSmem = 227 * 1024;  // of a CTA
 
 struct StagedPass {
@@ -1092,11 +1092,11 @@ struct StagedPass {
 };
 
 // FWD: the forward ops (fop0 / nfop), else the backward ops (bop0 / nbop).
-// buf: stage_bytes(room) of shared memory, or nullptr.  Every thread of the CTA
-// calls this (it ends with a barrier when it copies).
+// buf: kStageBytes of shared memory, or nullptr; rec: `room` records of it.  Every thread of
+// the CTA calls this (it ends with a barrier when it copies).
 template <bool FWD>
-__device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp* ops, unsigned char* buf, int room,
-                                 const DRun* druns, const GMem* gmem) {
+__device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp* ops, unsigned char* buf, void* rec,
+                                 int room, const DRun* druns, const GMem* gmem) {
   StagedPass r{phases + p.phase0, ops, 0, FWD ? druns + p.drun0 : nullptr, gmem};
   if (!buf || p.nphase <= 0 || p.nphase > kStagePhases) return r;
   if (FWD && p.ndrun > room) return r;
@@ -1118,7 +1118,7 @@ __device__ StagedPass stage_pass(const TPass& p, const TPhase* phases, const TOp
     sph[threadIdx.x] = q;
   }
   // a pass with more GMem records than the area holds reads those from global memory
-  uint4* rd = reinterpret_cast<uint4*>(buf + kStagePhaseBytes + sizeof(TOp) * kStageOps);
+  uint4* rd = reinterpret_cast<uint4*>(rec);
   const bool recs = FWD || p.nmem <= room;
   const uint4* rs = FWD ? reinterpret_cast<const uint4*>(druns + p.drun0) : reinterpret_cast<const uint4*>(gmem + p.mem0);
   for (int i = threadIdx.x; recs && i < (FWD ? p.ndrun : p.nmem) * 2; i += blockDim.x) rd[i] = rs[i];
@@ -1598,7 +1598,7 @@ __device__ __noinline__ void batch_bwd_streamed(uint32_t sx, uint32_t sl, const 
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, kStageRecs, nullptr, gmem);
+    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, stage + kStageBytes, kStageMems, nullptr, gmem);
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
       load_tiles<true>(sx, wp + tb, sl, wl + tb, rows, m);
@@ -1619,7 +1619,7 @@ __device__ __noinline__ void batch_bwd_streamed_ff(uint32_t sx, uint32_t sl, con
   for (int pi = npass - 1; pi >= 0; --pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, kStageRecsPrec, nullptr, gmem);
+    const StagedPass sp = stage_pass<false>(p, phases, bops, stage, stage + kStageBytes, kStageMems, nullptr, gmem);
     const float2* lo = blo + 4 * (size_t)sp.first;
     for (uint64_t t = 0; t < ntile; ++t) {
       const uint64_t tb = tile_base(t, p, g);
@@ -1662,7 +1662,8 @@ __device__ __noinline__ void batch_fwd_streamed(uint32_t sx, uint32_t sx2, float
   for (int pi = 0; pi < npass; ++pi) {
     const TPass& p = P[pi];
     set_rows(sh<uint32_t>(rows), p, m);
-    const StagedPass sp = stage_pass<true>(p, phases, fops, stage, COMP ? kStageRecsPrec : kStageRecs, druns, nullptr);
+    const StagedPass sp = stage_pass<true>(p, phases, fops, stage, sh<float>((uint32_t)offsetof(BShared, red)), kStageRuns,
+                                           druns, nullptr);
     const float2* lo = COMP ? flo + 4 * (size_t)sp.first : nullptr;
     if (threadIdx.x == 0) *sh<RunCtx>(rc) = RunCtx{sp.runs, rtab + kRunTab * p.run0, nullptr};
     // two tile buffers (sx, sx2): the next tile's copies are in flight while
@@ -1798,9 +1799,11 @@ __global__ void __launch_bounds__(kTileThreads, kBatchMinBlocks<RB, PREC>) k_bat
 // bytes of dynamic shared memory of k_batch<RB, PREC>
 static constexpr size_t batch_smem(int rb, bool prec) {
   const size_t mt = (size_t)1 << (9 + rb);
-  return ((sizeof(BShared) + 255) & ~size_t(255)) + (prec ? (8 + 32) * mt + stage_bytes(kStageRecsPrec) : 16 * mt + kStageBytes);
+  return ((sizeof(BShared) + 255) & ~size_t(255)) + (prec ? (8 + 32) * mt : 16 * mt) + kStageBytes + kStageMemBytes;
 }
-static_assert(batch_smem(kRB, false) <= kMaxSmem && batch_smem(3, true) <= kMaxSmem, "a register's shared memory");
+// 195 KB leave 60 KB of L1, a byte more 28 (the state's tiles stream through it: batch of 1024
+// registers 91.4 ms, 93.9 with 2 KB more)
+static_assert(batch_smem(kRB, false) <= 195 * 1024 && batch_smem(3, true) <= kMaxSmem, "a register's shared memory");
 
 // the instantiation of k_batch for a phase width and path
 static const void* batch_kernel(int rb, bool prec) {
@@ -1843,7 +1846,7 @@ constexpr uint32_t kFpBuf = sizeof(uint32_t) << (kMaxTileBits - kRowBits);  // a
 constexpr uint32_t kFpStage = kFpBuf + 2 * kTileBytes;                      // phases, ops, runs' entries (stage_pass)
 constexpr uint32_t kFpOps = kFpStage + (uint32_t)kStagePhaseBytes;
 constexpr uint32_t kFpRuns = kFpOps + (uint32_t)sizeof(TOp) * kStageOps;
-constexpr uint32_t kFpTile = kFpStage + (uint32_t)kStageBytes;  // the runs' tile products, for two tiles
+constexpr uint32_t kFpTile = kFpRuns + (uint32_t)sizeof(DRun) * kStageRuns;  // the runs' tile products, for two tiles
 constexpr uint32_t kFpTab = kFpTile + 2 * sizeof(float4) * kTileRuns;  // the runs' tables
 constexpr uint32_t kFpDiag = kFpTab + sizeof(float4) * kTileRuns * kRunTab;
 constexpr uint32_t kFpCtx = kFpDiag + sizeof(float2) * 16 * kTileTabs;
@@ -1886,7 +1889,8 @@ __device__ __forceinline__ void tile_products(float4* out, const DRun* entries, 
 __global__ void __launch_bounds__(kTileThreads, 1) k_fused_pass(FArgs a) {
   const TPass& p = *a.pass;
   set_rows(sh<uint32_t>(0), p, a.m);
-  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, sh<unsigned char>(kFpStage), kStageRecs, a.druns, nullptr);
+  const StagedPass sp = stage_pass<true>(p, a.phases, a.fops, sh<unsigned char>(kFpStage), sh<DRun>(kFpRuns), kStageRuns,
+                                       a.druns, nullptr);
   // the runs' tables, and their tile products for this tile and the one before
   const bool held = p.nrun <= kTileRuns;
   const bool staged = held && p.ndt <= kTileTabs && sp.ph != a.phases + p.phase0;
@@ -1969,7 +1973,8 @@ __global__ void __launch_bounds__(kTileThreads, 1) k_fused_bwd_pass(FBArgs a) {
   const TPass& p = *a.pass;
   for (int i = threadIdx.x; i < a.nparam; i += blockDim.x) gacc[i] = 0.0;
   set_rows(rowoff, p, a.m);
-  const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage, a.stage, nullptr, a.gmem);
+  const StagedPass sp = stage_pass<false>(p, a.phases, a.bops, stage, stage ? stage + kStageBytes : nullptr, a.stage,
+                                        nullptr, a.gmem);
   auto at = [&](const void* q) { return (uint32_t)((const unsigned char*)q - smraw); };
   for (uint64_t t = blockIdx.x; t < a.ntile; t += gridDim.x) {
     const uint64_t tb = tile_base(t, p, a.g);
@@ -3333,8 +3338,8 @@ int fused_backward(qs_state* s, const qs_circuit* c, const double* host_params, 
                 sizeof(double) * ((np + 1) & ~1) + 2 * sizeof(float2) * (1ull << m);
   if (smem > kMaxSmem) return fail(QS_EUNSUPPORTED, "%d parameters do not fit the tiled backward's shared memory", np);
   // without room for the records those are read from global memory, once a phase
-  const int stage = smem + kStageBytes <= kMaxSmem ? kStageRecs : smem + stage_bytes(0) <= kMaxSmem ? 0 : -1;
-  if (stage >= 0) smem += stage_bytes(stage);
+  const int stage = smem + kStageBytes + kStageMemBytes <= kMaxSmem ? kStageMems : smem + kStageBytes <= kMaxSmem ? 0 : -1;
+  if (stage >= 0) smem += kStageBytes + sizeof(GMem) * stage;
   if (host_loss) QS_TRY(expect_raw(s->data, QS_C64, n, 1, o, s, host_loss));
   if (np > 0) {
     if (P->dparams_n < np) {
