@@ -70,7 +70,8 @@ struct TOp {
 // a parameter, with or without such an X (cmask = 1: controlled by qubits outside): takes
 // the four sums that every member's derivative is a combination of, uncomputes the run
 // and the X
-enum { TK_DENSE = 0, TK_SWAP = 1, TK_DIAG = 2, TK_RX = 3, TK_RY = 4, TK_DIAG16 = 5, TK_DIAGOUT = 6, TK_DIAGRUN = 7,
+// (the kinds up to TK_DIAGRUN are the ones that the forward applies by their form alone)
+enum { TK_DENSE = 0, TK_SWAP = 1, TK_DIAG = 2, TK_RX = 3, TK_RY = 4, TK_DIAGRUN = 5, TK_DIAG16 = 6, TK_DIAGOUT = 7,
        TK_DENSEX = 8, TK_RUN = 9, TK_REALRUN = 10 };
 
 constexpr int kRunTab = 48;  // entries of a run's table: 32 lanes, then 16 warps (products for bit t = 0 and 1)

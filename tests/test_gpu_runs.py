@@ -116,3 +116,39 @@ def test_registers_of_one_circuit(precise):
         assert abs(loss[r] - wl) < 1e-5, r
         assert np.max(np.abs(grad[off:off + len(wg)] - wg)) < 1e-5 * max(1.0, np.max(np.abs(wg))), r
         off += len(wg)
+
+
+@pytest.mark.parametrize("count", [223, 255, 480, 511, 512, 513])
+def test_passes_at_the_edges_of_their_staged_area(count):
+    """One pass of gates that are an op and a gradient record each, up to and past the ops (512) and
+    records (224) that its area in shared memory holds: batches of both paths and the tiled gradient.
+    Tolerance: 3 x 512 gates (forward, psi and lambda back) of FP32 roundings, 6e-8 each, add up to
+    3e-6 at random; six times that."""
+    from paper_1912_10877_gb300 import qsim
+    n = 14
+    rs = W.rng(count)
+    gates = []
+    for k in range(count):  # four qubits at a time: few phases
+        a, b = (int(v) for v in rs.permutation(4)[:2])
+        base = 4 * (3 * k // count)
+        gates.append(W.Gate("RX", (base + a,), (base + b,), (1,), param=k))
+    gates = [W.Gate("H", (q,)) for q in range(n)] + gates
+    params, terms = W.uniform_angles(count, count), W.zz_chain(n) + [(0.7, ((2, "Z"),))]
+    psi = oracle.apply_circuit(oracle.zero_state(n), n, gates, params)
+    wl, wg = oracle.gradient(oracle.zero_state(n), n, gates, params, terms)
+    circ, obs = qsim.Circuit(gates, n), qsim.Observable(terms)
+    for precise in (False, True):
+        st = qsim.State([n, n], dtype=torch.complex64)
+        prog = qsim.BatchProgram([circ, circ], [obs, obs], precise=precise)
+        loss, grad = prog.run(st, torch.tensor(np.tile(params, 2), device="cuda"), grad=True)
+        for r in range(2):
+            assert np.max(np.abs(st.register(r).cpu().numpy() - psi)) < 2e-5
+            assert abs(float(loss[r]) - wl) < 2e-5
+            assert np.max(np.abs(grad[r * count:(r + 1) * count].cpu().numpy() - wg)) < 2e-5 * max(1.0, np.max(np.abs(wg)))
+    st = qsim.State(n, dtype=torch.complex64)
+    st.reset()
+    st.apply_circuit(circ, params, tiles=True)
+    assert np.max(np.abs(st.numpy() - psi)) < 2e-5
+    loss, grad = qsim.backward_tiled(st, circ, params, obs)
+    assert abs(loss - wl) < 2e-5
+    assert np.max(np.abs(grad - wg)) < 2e-5 * max(1.0, np.max(np.abs(wg)))
