@@ -325,7 +325,7 @@ int build_terms(const qs_observable* o, int n, SpTerms* T, SpTable* tab) {
       continue;
     }
     for (int k = 0; k < G.nt; ++k) G.z[k] = T->z[G.t0 + k];
-    for (int q = 0; q < segments(n); ++q)
+    for (int q = 1; q < segments(n); ++q)  // segment 0 has no top bits
       for (int k = 0; k < G.nt; ++k)
         G.seg |= (uint64_t)(__builtin_popcountll(((uint64_t)q << (n - kSegBits)) & G.z[k] & top) & 1) << (kSmallTerms * q + k);
     for (int p = 0; p < kTab; ++p) {
