@@ -198,7 +198,7 @@ struct AdjRun {
 
 template <bool FULL>
 __global__ void __launch_bounds__(kAdjThreads, 4)
-k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nitems, int t,
+k_adjoint_run(double2* __restrict__ psi, double2* __restrict__ lam, uint64_t nitems,
               const __grid_constant__ AdjRun F, double* __restrict__ partials, unsigned* __restrict__ counter,
               double* __restrict__ grad) {
   const uint64_t lo = nitems * blockIdx.x / gridDim.x, hi = nitems * (blockIdx.x + 1) / gridDim.x;
@@ -513,8 +513,8 @@ struct AdjWalk {
     }
     const uint64_t items = 1ull << (n - 1);
     const int nblk = (int)std::min<uint64_t>(kAdjRunBlocks, std::max<uint64_t>(1, items / kAdjThreads));
-    if (full) k_adjoint_run<true><<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, t, F, partials, counter, dgrad);
-    else k_adjoint_run<false><<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, t, F, partials, counter, dgrad);
+    if (full) k_adjoint_run<true><<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, F, partials, counter, dgrad);
+    else k_adjoint_run<false><<<nblk, kAdjThreads, 0, s->stream>>>(psi, lam, items, F, partials, counter, dgrad);
     QS_LAUNCHED();
     return QS_OK;
   }

@@ -79,7 +79,7 @@ __device__ __forceinline__ c2_t<R> small_out(int kind, const c2_t<R>* u, c2_t<R>
   }
 }
 
-// E amplitudes a thread; threads and CTAs as the launch has them
+// E (1 or 2) amplitudes a thread; threads and CTAs as the launch has them
 template <typename R, int E, int CAP>
 __global__ void __launch_bounds__(kSmallThreads)
 k_small(c2_t<R>* __restrict__ psi, int n, int nops, const __grid_constant__ SmallOps<R, CAP> ops) {
@@ -89,7 +89,8 @@ k_small(c2_t<R>* __restrict__ psi, int n, int nops, const __grid_constant__ Smal
   cg::cluster_group cl = cg::this_cluster();
   const unsigned cs = cl.num_blocks(), rank = cl.block_rank();
   const int lc = 31 - __clz((int)cs), L = n - lc;  // bits of a CTA's amplitudes
-  const uint32_t nt = 1u << (L - (E == 1 ? 0 : E == 2 ? 1 : 2));  // threads that hold amplitudes (may be below a warp)
+  const uint32_t nt = 1u << (L - (E - 1));  // threads that hold amplitudes (may be below a warp)
+  static_assert(E == 1 || E == 2, "an own partner is the other amplitude");
   const int lt = 31 - __clz((int)nt);
   const uint32_t tid = threadIdx.x, hi = rank << L, area = 1u << L;
   const bool act = tid < nt;
@@ -133,7 +134,7 @@ k_small(c2_t<R>* __restrict__ psi, int n, int nops, const __grid_constant__ Smal
       rturn ^= 1;
     } else if (t >= lt) {
 #pragma unroll
-      for (int e = 0; e < E; ++e) y[e] = E == 1 ? x[e] : E == 2 || t == lt ? x[e ^ (E > 1 ? 1 : 0)] : x[e ^ (E > 2 ? 2 : 0)];
+      for (int e = 0; e < E; ++e) y[e] = x[e ^ (E - 1)];
     } else if (t < 5) {
 #pragma unroll
       for (int e = 0; e < E; ++e) y[e] = shfl2(x[e], 1 << t);
