@@ -3644,7 +3644,7 @@ int qs_batch_run(qs_state* s, const qs_batch_program* p, const double* dev_param
   if (dev != p->device)
     return fail(QS_EINVAL, "the program was built on device %d; the current device is %d", p->device, dev);
   cudaStream_t st = s->stream;
-  QS_TRY(launch_prep(p, dev_params, true, st));
+  QS_TRY(launch_prep(p, dev_params, grad, st));  // without gradients the backward's records are not read
   QS_CUDA(cudaMemsetAsync(p->counter, 0, sizeof(int), st));
   BArgs a;
   a.state = (float2*)s->data;
