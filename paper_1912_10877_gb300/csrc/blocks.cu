@@ -48,9 +48,11 @@ uint64_t gate_qubits(const qs_gate_desc& g) {
   return m;
 }
 
+// GATES: with each block's gates, else its support only
+template <bool GATES>
 void plan_blocks(const qs_circuit* c, int kmax, std::vector<Block>& out) {
   out.clear();
-  std::vector<Block> open;
+  std::vector<Block> open, rest;
   for (int gi = 0; gi < (int)c->gates.size(); ++gi) {
     const uint64_t q = gate_qubits(c->gates[gi]);
     uint64_t s = q;
@@ -59,12 +61,12 @@ void plan_blocks(const qs_circuit* c, int kmax, std::vector<Block>& out) {
     if (popc(s) <= kmax) {
       Block merged;
       merged.support = s;
-      std::vector<Block> rest;
+      rest.clear();
       for (Block& b : open) {
-        if (b.support & q) merged.gates.insert(merged.gates.end(), b.gates.begin(), b.gates.end());
-        else rest.push_back(std::move(b));
+        if (!(b.support & q)) rest.push_back(std::move(b));
+        else if (GATES) merged.gates.insert(merged.gates.end(), b.gates.begin(), b.gates.end());
       }
-      merged.gates.push_back(gi);
+      if (GATES) merged.gates.push_back(gi);
       rest.push_back(std::move(merged));
       open.swap(rest);
       continue;
@@ -78,7 +80,7 @@ void plan_blocks(const qs_circuit* c, int kmax, std::vector<Block>& out) {
       if ((open[i].support & q) && popc(open[i].support | q) <= kmax &&
           (keep < 0 || popc(open[i].support) > popc(open[(size_t)keep].support)))
         keep = (long)i;
-    std::vector<Block> rest;
+    rest.clear();
     for (size_t i = 0; i < open.size(); ++i) {
       Block& b = open[i];
       if ((long)i == keep) continue;
@@ -88,12 +90,12 @@ void plan_blocks(const qs_circuit* c, int kmax, std::vector<Block>& out) {
     if (keep >= 0) {
       Block kb = std::move(open[(size_t)keep]);
       kb.support |= q;
-      kb.gates.push_back(gi);
+      if (GATES) kb.gates.push_back(gi);
       rest.push_back(std::move(kb));
     } else {
       Block nb;
       nb.support = q;
-      nb.gates.push_back(gi);
+      if (GATES) nb.gates.push_back(gi);
       if (popc(q) > kmax) out.push_back(std::move(nb));  // wider than k: stays a gate of its own
       else rest.push_back(std::move(nb));
     }
@@ -129,7 +131,7 @@ void plan_blocks(const qs_circuit* c, int kmax, std::vector<Block>& out) {
       if (best >= 0) {
         Block& t = out[(size_t)best];
         t.support |= sj;
-        t.gates.insert(t.gates.end(), out[j].gates.begin(), out[j].gates.end());
+        if (GATES) t.gates.insert(t.gates.end(), out[j].gates.begin(), out[j].gates.end());
         out.erase(out.begin() + (long)j);
         changed = true;
       } else {
@@ -152,7 +154,7 @@ void plan_blocks(const qs_circuit* c, int kmax, std::vector<Block>& out) {
       if (best >= 0) {
         Block& t = out[(size_t)best];
         t.support |= si;
-        t.gates.insert(t.gates.begin(), out[(size_t)i].gates.begin(), out[(size_t)i].gates.end());
+        if (GATES) t.gates.insert(t.gates.begin(), out[(size_t)i].gates.begin(), out[(size_t)i].gates.end());
         out.erase(out.begin() + i);
         changed = true;
       }
@@ -232,7 +234,7 @@ int block_matrix(const qs_circuit* c, const Block& b, const double* params, std:
 const std::vector<Block>& cached_blocks(const qs_circuit* c, int kmax) {
   if (c->block_k != kmax || !c->blocks) {
     auto* v = new std::vector<Block>();
-    plan_blocks(c, kmax, *v);
+    plan_blocks<true>(c, kmax, *v);
     delete static_cast<std::vector<Block>*>(c->blocks);
     c->blocks = v;
     c->block_k = kmax;
@@ -241,6 +243,14 @@ const std::vector<Block>& cached_blocks(const qs_circuit* c, int kmax) {
 }
 
 }  // namespace
+
+void block_widths(const qs_circuit* c, int kmax, std::vector<int>& widths) {
+  std::vector<Block> planned;
+  const bool known = c->blocks && c->block_k == kmax;
+  if (!known) plan_blocks<false>(c, kmax, planned);
+  widths.clear();
+  for (const Block& b : known ? cached_blocks(c, kmax) : planned) widths.push_back(popc(b.support));
+}
 
 void free_blocks(const qs_circuit* c) {
   delete static_cast<std::vector<Block>*>(c->blocks);

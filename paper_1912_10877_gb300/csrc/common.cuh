@@ -303,6 +303,7 @@ int gram_tc(int w, const float2* psi, const float2* lam, int n, const int* qubit
 // the circuit fused into blocks of at most kmax qubits, gate-by-gate path (blocks.cu)
 int apply_blocks(qs_state* s, const qs_circuit* c, const double* params, int kmax, bool precise);
 void free_blocks(const qs_circuit* c);
+void block_widths(const qs_circuit* c, int kmax, std::vector<int>& widths);  // of the planner's blocks, in order
 
 // samples with device uniforms into device indices (reduce.cu)
 size_t sample_scratch_doubles(int n, int nreg, int nshots, bool lean);

@@ -364,10 +364,9 @@ bool cluster_pays(const std::vector<RunOp<R>>& ops, const qs_circuit* c, int kma
       case RU_DENSE: here += f64 ? 190 + 230 * a : 240 + 45 * a; break;
       default: here += 500 + 200 * a;
     }
-  int nb = 0;
-  if (qs_circuit_blocks(c, nullptr, kmax, &nb, nullptr, nullptr, nullptr) != QS_OK) return true;
-  std::vector<int32_t> widths(std::max(1, nb));
-  if (qs_circuit_blocks(c, nullptr, kmax, &nb, widths.data(), nullptr, nullptr) != QS_OK) return true;
+  std::vector<int> widths;
+  block_widths(c, kmax, widths);
+  const int nb = (int)widths.size();
   const int64_t block = f64 ? (n < 10 ? 4600 : 5800) + 400 * (a - 1) : 4000 + 200 * (a - 1);
   int64_t blocks = 2500 + nb * block;
   if (c->nparams > 0 && nb > 0) {
