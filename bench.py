@@ -478,16 +478,15 @@ def run_diff_leg(steps: int, warmup: int):
     t0 = time.perf_counter()
     qsim.backward(st, circ, params, obs, every, ck, work)
     tb = time.perf_counter() - t0
-    # FP64 roofline of the backward: per rotation and amplitude pair, uncompute psi and lambda
-    # (Rz^dag: two complex-by-phase products, 6 flops each, per state; Rx^dag: c a + i s b, 6 flops
-    # per amplitude, per state) and Im<lambda|G|psi> (8 flops per pair): 32 FP64 flops per pair,
-    # 16 per amplitude; CNOTs move amplitudes (0 flops)
-    fp64_flops = 6000 * 16.0 * (1 << n)
+    # FP64 roofline of the backward, as executed: a run Rz Rx Rz takes 36 FP64 instructions an
+    # amplitude pair (12 multiply-adds for its four sums; 12 for U^dag on psi and as many on lambda,
+    # two of them plain products), 68 flops with a multiply-add as two; CNOTs move amplitudes (0 flops)
+    fp64_flops = 2000 * 34.0 * (1 << n)
     fp64_peak = 1.25  # TFLOP/s, nominal FP64 of GB300
     return {"metric": "fwd+grad seconds (n=20, 8000 gates, 6000 angles)", "unit": "s",
             "value": out["fp64_uncompute_ckpt10"], "tiled_fp32_value": out["tiled_fp32"],
             "backward_s": round(tb, 4),
-            "roofline": {"bound": "alu", "kernel": "FP64 reversible uncompute (k_adjoint_run; flops counted gate by gate)",
+            "roofline": {"bound": "alu", "kernel": "FP64 reversible uncompute (k_adjoint_run; flops it executes)",
                          "achieved": round(fp64_flops / tb / 1e12, 3), "peak": fp64_peak, "unit": "TFLOP/s",
                          "frac": round(fp64_flops / tb / 1e12 / fp64_peak, 4), "flops": fp64_flops,
                          "peak_kind": "nominal FP64 rate of GB300 (1.25 TFLOP/s)"},
@@ -500,9 +499,9 @@ def run_diff_leg(steps: int, warmup: int):
 def run_large_leg(steps: int, warmup: int):
     """n = 32 (32 GiB complex64): QFT with swap network on a seeded basis state, depth-20
     brickwork of Rz + Haar SU(2) + CZ, reversible gradient of <Z_1> w.r.t. the 640 angles.
-    The QFT runs on the tile engine (6 passes: its controlled phases fuse); the brickwork
+    The QFT runs on the tile engine (its controlled phases fuse); the brickwork
     forward runs both ways, on the tile engine and as fused 5-qubit blocks (dense ones on
-    the tensor cores), and the faster one counts; the gradient runs on the tile engine."""
+    the tensor cores), and the faster one counts, as for the gradient."""
     import torch
     from paper_1912_10877_gb300 import qsim
     n, depth = 32, 20
@@ -632,7 +631,7 @@ def run_small_leg(reps: int = 50):
     st.reset()
     cap.replay()
     e = float(st.expect(obs)[0])
-    # the whole circuit and <sum ZZ> in one cooperative launch, per block width and grid size
+    # the whole circuit and <sum ZZ> in one launch, per block width and grid size (gridsms: one cluster)
     one = {}
     out = torch.empty(1, dtype=torch.float64, device="cuda")
     for k in (3, 4, 5):
@@ -648,8 +647,8 @@ def run_small_leg(reps: int = 50):
             "value": round(best, 1), "gate_by_gate_us": round(t_unf, 1), "default_us": round(t_def, 1),
             "graph_replay_us": round(t_graph, 1), "blocks_graph_replay": blocks,
             "one_launch_us": {"best": best_one, "by_shape": one,
-                              "note": "circuit and <sum ZZ> in one cooperative launch (fused blocks of k qubits, "
-                                      "grid barrier between blocks)"},
+                              "note": "circuit and <sum ZZ> in one launch (gridsms: one thread-block cluster, gate "
+                                      "by gate; else fused blocks of k qubits, grid barrier between blocks)"},
             "roofline": {"bound": "latency", "achieved": round(best, 1), "unit": "us per circuit",
                          "note": "a 64 KiB register: launch and barrier latency and the FP64 rate of the SMs it "
                                  "reaches bound it, not HBM"},

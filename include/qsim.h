@@ -500,9 +500,10 @@ int qs_backward(qs_state* s, const qs_circuit* c, const double* host_params,
  * Sec. "Reverse Mode" with a fused block as the unit: walking the blocks from
  * last to first, one pass forms rho = sum_x psi_x lambda_x^dag over the
  * block's tuples (FP32 products per 128 tuples for complex64, FP64 sums), the
- * gradients of the block's gates follow on the host in FP64 as
+ * gradients of the block's gates follow in FP64 as
  * 2 c Im Tr(E H E^dag rho) (E: the block's later gates, H: the generator with
- * its control projector), then psi and lambda are uncomputed by the block's
+ * its control projector), on the device for blocks of single-target gates and
+ * on the host for the others, then psi and lambda are uncomputed by the block's
  * adjoint.  s holds the final state of a single register (complex64 or
  * complex128) and holds the uncomputed initial state on return.  dev_work:
  * qs_backward_blocks_work_bytes() bytes (lambda).  host_grad: nparams doubles

@@ -6,10 +6,13 @@
 // <psi|P|psi> = sum_i ph(i) conj(psi_{i^x}) psi_i.  Terms are grouped by their
 // x mask; each group reads each amplitude (or each pair (i, i^x) once, counting
 // it twice) and adds it weighted with the group's coefficients in FP64.  The sum
-// is pairwise: a thread adds at most 16 items in order (the serial base case),
+// is pairwise: a thread adds at most 16 items in order to each of its sums (32
+// where a unit has odd and even numbers of Y factors; the serial base case),
 // threads, warps and blocks combine by balanced trees, and a second kernel folds
-// the per-block partials (64 at most in order) and the groups by balanced trees
-// as well (fixed shapes, so results are reproducible run to run).
+// the per-block partials (16 at most in order) and the groups by balanced trees
+// as well (fixed shapes, so results are reproducible run to run).  qs_expect_static
+// has room for 65536 partial sums: with nblk blocks for 2^n amplitudes a thread
+// adds 16 ceil(2^n / kBlockAmps / nblk) items in order.
 //
 // measure (Sec. "Instructions on Quantum Registers"): the deterministic
 // contract of qsim.h -- FP64 probabilities with separately rounded multiply

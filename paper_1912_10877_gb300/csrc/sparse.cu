@@ -24,7 +24,7 @@
 //    the children swapped where the row's bit is 1;
 //  - a warp stages its rows' entries as 2-byte codes in shared memory and writes
 //    columns and values in order.
-// heisenberg(20) (11.5 M nonzeros, 285 MB): counts 40 us, scan 10, fill 135 (bound by
+// heisenberg(20) (11.2 M nonzeros, 276 MB): counts 40 us, scan 10, fill 135 (bound by
 // the walks' chains of dependent shared-memory loads; its stores alone would take
 // 42).  Before, with every sum in FP64, a selection of the next column among all and
 // a thread's rows stored one by one: 313, 80 and 629 us.

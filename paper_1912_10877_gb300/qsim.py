@@ -573,8 +573,9 @@ def backward_blocks(state: State, circuit: Circuit, params, obs: Observable, kma
 
 def run_one_launch(state: State, circuit: Circuit, params=None, kmax: int = 4, obs: "Observable | None" = None,
                    grid_ctas: int = 0, out: torch.Tensor | None = None):
-    """The whole circuit on one small register in a single cooperative launch
-    (qs_run_circuit_one_launch), with <obs> (diagonal) evaluated in the same launch into
+    """The whole circuit on one small register in a single launch
+    (qs_run_circuit_one_launch: a thread-block cluster, or a cooperative launch of its
+    blocks of kmax qubits where those take less), with <obs> (diagonal) evaluated in the same launch into
     `out` (a float64 CUDA tensor of one element, returned).  Asynchronous."""
     p = _params_array(params, circuit.nparams)
     if obs is not None and out is None:
