@@ -155,8 +155,9 @@ int launch_bitswap(float2* psi, int n, int nreg, const std::vector<std::pair<int
   const size_t smem = sizeof(float2) * 2 << a.m;
   // the limit belongs to the function: always the largest tile's, never one that another thread's
   // launch exceeds
-  QS_CUDA(cudaFuncSetAttribute(k_bitswap, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)(sizeof(float2) * 2 << kSwapTileMax)));
+  if (smem > 48 * 1024)
+    QS_CUDA(cudaFuncSetAttribute(k_bitswap, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(float2) * 2 << kSwapTileMax)));
   int dev = 0, sms = 0, per_sm = 0;
   QS_CUDA(cudaGetDevice(&dev));
   QS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));

@@ -103,7 +103,10 @@ k_sp_rows(const __grid_constant__ SpTerms T, uint64_t dim, int segs, int64_t* __
   int c[kSegs];
 #pragma unroll
   for (int s = 0; s < kSegs; ++s) c[s] = 0;
-  for (int g = 0; g < T.ngroups; ++g) {
+  // a warp without rows does not queue for the FP64 unit (one qubit, 40 terms in two large groups:
+  // the call 56 us, 34 without its 31 idle warps)
+  const int ngroups = low - lane < dim ? T.ngroups : 0;
+  for (int g = 0; g < ngroups; ++g) {
     const SpGroup& G = T.g[g];
     if (G.large < 0) {
       const uint32_t p = signs(G, low ^ G.x);
@@ -392,7 +395,7 @@ int qs_observable_csr_fill(const qs_observable* o, int nqubits, const int64_t* d
   while (warps > 1 && common + warps * per > kFillSmem) warps >>= 1;
   const size_t smem = common + warps * per;
   // the limit belongs to the function: the same for every observable, as other threads launch theirs
-  QS_CUDA(cudaFuncSetAttribute(k_sp_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFillSmem));
+  if (smem > 48 * 1024) QS_CUDA(cudaFuncSetAttribute(k_sp_fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFillSmem));
   const uint64_t rows = (dim / segs + 31) / 32;
   k_sp_fill<<<(unsigned)((rows + warps - 1) / warps), 32 * warps, smem, st>>>(T, tab, dim, segs, dev_rowptr, dev_cols,
                                                                            (double2*)dev_vals);
