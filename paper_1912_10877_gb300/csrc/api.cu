@@ -152,7 +152,7 @@ struct Fuser {
   }
   int drain() {
     if (plans.empty()) return QS_OK;
-    if (!small_pays(s->dtype, s->nq[0], plans)) {
+    if (!small_pays(s->dtype, s->nq[0], s->nreg, plans)) {
       for (const Plan& p : plans) QS_TRY(launch_plan(s, p));
       plans.clear();
       return QS_OK;

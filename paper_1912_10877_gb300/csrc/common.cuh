@@ -273,7 +273,7 @@ int launch_plan_on(void* data, int dtype, int n, int nreg, int64_t reg_stride, c
 // launches, and the call (n <= 14)
 bool small_register(int n, int nreg);
 bool small_plan(const Plan& p);
-bool small_pays(int dtype, int n, const std::vector<Plan>& plans);
+bool small_pays(int dtype, int n, int nreg, const std::vector<Plan>& plans);
 int apply_small(void* data, int dtype, int n, int nreg, const std::vector<Plan>& plans, cudaStream_t st);
 
 // gate matrices (FP64, row-major), generators and daggers

@@ -270,10 +270,11 @@ bool small_plan(const Plan& p) {
 // a microsecond each).  Measured, here and as launches: a dense 2x2 on every qubit 86.0 and 84.0
 // us, H 41 and 57, Rx 57.7 and 57.4; H on two qubits 10.3 and 8.3; two controlled X 6.1 and 7.4, two
 // T 8.2 and 12.4; six controlled Rx 20.5 and 24.6; 2, 6 and 20 controlled dense gates 16.0, 36.9 and
-// 96 against 12.3, 32.8 and 113.
-bool small_pays(int dtype, int n, const std::vector<Plan>& plans) {
+// 96 against 12.3, 32.8 and 113.  Registers of a batch have a cluster each, launches more to do
+// (eight of them, 60 gates Rx: 61 us here, 86 as launches).
+bool small_pays(int dtype, int n, int nreg, const std::vector<Plan>& plans) {
   if (plans.size() < 2) return false;
-  if (dtype == QS_C64 || n < kSmallMaxQubits) return true;
+  if (dtype == QS_C64 || n < kSmallMaxQubits || nreg > 1) return true;
   int gain = 0;
   for (const Plan& p : plans) {
     const bool ctrl = p.ctrl_mask != 0;
